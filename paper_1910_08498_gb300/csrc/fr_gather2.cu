@@ -71,10 +71,10 @@ int resident_ctas(const void *fn, int threads, size_t smem) {
   return per_sm;
 }
 
-cudaError_t launch_multi(const void *fn, const MultiLaunch &p, int threads, size_t smem,
-                         cudaStream_t st) {
+cudaError_t launch_multi(const void *fn, const MultiLaunch &p, int per_item, int threads,
+                         size_t smem, cudaStream_t st) {
   cudaLaunchConfig_t cfg{};
-  cfg.gridDim = dim3((unsigned)p.nitems);
+  cfg.gridDim = dim3((unsigned)p.nitems * (unsigned)per_item);
   cfg.blockDim = dim3((unsigned)threads);
   cfg.dynamicSmemBytes = smem;
   cfg.stream = st;
@@ -88,8 +88,8 @@ cudaError_t launch_multi(const void *fn, const MultiLaunch &p, int threads, size
 }
 
 size_t gather2_smem_bytes(const GatherShape &sh, int chunk) {
-  const int nw = sh.bx * sh.by / 32;
-  return (size_t)nw * (sh.zc == 8 ? gather2_warp_smem<8>(chunk) : gather2_warp_smem<16>(chunk));
+  (void)sh;  // one warp per CTA
+  return gather2_warp_smem<8, 0>(chunk);
 }
 
 // brick shapes: columns in x, columns in y, voxels per column (z)

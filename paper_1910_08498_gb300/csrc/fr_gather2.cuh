@@ -1,437 +1,641 @@
 // fr_gather2.cuh -- the direct-drain gather insertion kernel.
 //
-// Same decomposition as the per-voxel gather of fr_gather.cuh (a warp owns an
-// 8 x 4 x ZC footprint of voxel columns, culls the images of its work unit
-// into a shared-memory list, and accumulates (image, voxel) items into
-// shared-memory partial sums that are folded into HBM with TwoSum), with far
-// fewer instructions spent per item:
+// A warp owns a footprint of 8 x 8 x 8 voxels (4 x 8 x 8 in the fold columns),
+// culls the images of its work unit into a list, and accumulates (image, voxel)
+// items into shared-memory partial sums that are folded into HBM with TwoSum;
+// warps never wait for one another.  Per list entry (an image, in one of the two
+// orientations of its half plane):
 //
-//  * item generation: for each list image every lane marks the run of z
-//    levels of its column that lie within a of the plane (u_z is linear in z,
-//    so the run is contiguous) and appends one 16-bit tag per item (list entry,
-//    column, z level) to the warp's tag queue, at lane-major positions found
-//    with one ballot per bit of the run length (8- or 16-deep columns);
-//  * evaluation: each full round of 32 tags (one item per lane) forms
-//    u = R^T v from the footprint centre's compensated projection, reflects
-//    u through the origin when it lies in the mirrored half plane (the pixel is
-//    then read at -c and conjugated: Hermitian symmetry), puts the 4 x 4
-//    candidate box at ceil(u - a) clamped into the stored half plane
-//    kx in [0, H], ky in [-H, H - 1] (box rows and columns moved in by the
-//    clamp lie outside the blob and are masked), reads each box row as two
-//    two-pixel loads, evaluates the Chebyshev weight polynomial in
-//    x = 2 r^2 / a^2 - 1 for two candidates at a time with packed FP32x2
-//    FMAs (masked to 0 outside r <= a) and adds the complex and weight sums to
-//    the voxel's partial sums with shared-memory atomics.
+//  * patch: the pixels that the footprint's voxels can meet, a rectangle of at
+//    most PW x PW stored pixels, are copied into one of the warp's two
+//    shared-memory patches while the previous entry is evaluated (cp.async;
+//    FP16 pixels go through registers and are converted on the way).  A row of
+//    20 eight-byte pixels puts pixel (x, y) in bank pair x + 4 y modulo 16, so
+//    that any 4 x 4 block of pixels is free of bank conflicts;
+//  * item generation: a lane computes the run of z levels of each of its
+//    columns that lie within a of the plane (u_z is linear in z) and writes one
+//    8-bit tag per item (column, z level) at positions from a warp scan;
+//  * evaluation: 32 items a round, one per lane: u = R^T v from the footprint
+//    centre's compensated projection, the 4 x 4 candidate box at rint(u - 1.5)
+//    (it covers [u - a, u + a] for every a < 2), clamped into the patch (rows
+//    and columns moved in by the clamp lie outside the blob and are masked), its
+//    16 pixels from the patch, the Chebyshev weight polynomial in
+//    x = 2 r^2 / a^2 - 1 for two candidates at a time with packed FP32x2 FMAs
+//    (masked to 0 outside r <= a), and the complex and weight sums added to the
+//    voxel's partial sums with plain loads and stores: the items of one entry
+//    are distinct voxels.
 //
-// An item whose box crosses the column kx = 0 is evaluated twice: the box
-// clamped to kx >= 0 read directly, and the point-reflected box clamped to
-// kx >= 0 read conjugated (its tag is queued again with the half forced).  Away
-// from the fold columns every point of the extended plane within a of the
-// voxel has (R c)_x > 0, so a column c_x > 0 receives the stored pixel c, a
-// column c_x < 0 the stored -c conjugated, and the column c_x = 0 both (0, c_y)
-// and, conjugated, (0, -c_y): exactly what the two boxes read.  The bricks of
-// this kernel's main launch tile x >= floor(a) + 1.  The fold columns |x| <=
-// floor(a), where the fold predicate itself has to be evaluated per pixel,
-// are computed by a second instantiation over those columns only (FOLD), in
-// footprints 4 columns wide so that three of four lanes hold fold columns:
-// there a stored pixel k counts in the directly read box when it is not
-// folded and in the reflected box when it is (exact sign of R00 k_x + R01
-// k_y).  Polynomial weights only, 4 x 4 boxes only (a < 2).
+// What bounds it.  Reading the boxes straight from global memory through L1 cost
+// 128 data-pipe wavefronts a round (32 boxes lie in about nine image rows) and
+// kept that pipe 90 % busy at 63 % issue: 13.4 ms for 5000 FP32 images of 256^2.
+// From the patches a round costs 51, and one 512-voxel footprint a warp (137
+// items an entry) halves the work per entry against 256 voxels: 9.6 ms, the
+// data pipe 71 %, FMA pipe 63 %, issue 65 % busy, about one third of the time in
+// the per-entry work (items, patch copies), the rest in the rounds.
+//
+// Half planes.  A stored pixel k sits at R k or, point-reflected and
+// conjugated, at -R k.  An image whose patch lies in k_x > 0 (or its mirror)
+// makes one list entry: as stored, or with the in-plane axes negated (u -> -u)
+// and the sums conjugated.  One whose patch crosses k_x = 0 makes both, and
+// each item is evaluated once per half it reaches.  Away from the fold columns
+// every point of the extended plane within a of the voxel has (R c)_x > 0, so
+// a column c_x > 0 receives the stored pixel c, a column c_x < 0 the stored -c
+// conjugated, and the column c_x = 0 both (0, c_y) and, conjugated, (0, -c_y):
+// exactly what the two entries read.  The bricks of this kernel's main launch
+// tile x >= floor(a) + 1.  The fold columns |x| <= floor(a), where the fold
+// predicate itself has to be evaluated per pixel, are computed by a second
+// instantiation over those columns only (FOLD), in footprints 4 columns wide so
+// that three of four lanes hold fold columns: there a stored pixel k counts in
+// the entry as stored when it is not folded and in the reflected entry when it
+// is (exact sign of R00 k_x + R01 k_y, found once per pixel of the patch and
+// kept as one bit).  Polynomial weights only, 4 x 4 boxes only (a < 2).
 #pragma once
 
 #include "fr_gather.cuh"
 
 namespace fr {
 
-constexpr int G2_T2CAP = 64;  // forced second halves: < 32 carried over + <= 32 per round
+constexpr int G2_ENTRIES = 16;  // records built and processed at a time
+constexpr int G2_REC = 16;      // floats of a record
 
-// tags of one list image (<= 32 columns x ZC levels) + < 32 carried over
-template <int ZC>
-__host__ __device__ constexpr int g2_tcap() {
-  return 32 * ZC + 32;
-}
+// Geometry of the warp footprint FW x 8 x 8 and of its pixel patches.
+template <int FW>
+struct G2Shape {
+  static constexpr int FH = 8, ZC = 8;
+  static constexpr int NC = FW * FH / 32;               // columns per lane
+  static constexpr int WV = FW * FH * ZC;               // voxels
+  static constexpr float HX = 0.5f * (FW - 1), HY = 0.5f * (FH - 1), HZ = 0.5f * (ZC - 1);
+  // a box reaches 2 pixels past u, and u lies within the footprint's radius
+  // (6.07; 5.17 for FW = 4) of the centre: at most 17 (15) columns
+  static constexpr int PW = FW == 8 ? 17 : 15;          // patch columns and rows
+  static constexpr int PITCH = 20;                      // = 4 modulo 16 eight-byte banks
+  static constexpr int PATCH = PW * PITCH;              // pixels of a patch
+};
 
-// Per-warp shared memory: image list, partial sums, tag queues, phase counters.
-template <int ZC>
+// Per-warp shared memory: records, partial sums, patches, image list, fold
+// bits, tags.
+template <int FW, int FOLD>
 __host__ __device__ constexpr size_t gather2_warp_smem(int chunk) {
-  return ((size_t)LIST_FIELDS * chunk * 4 + (size_t)3 * (32 * ZC) * 4 + (size_t)G2_T2CAP * 4 +
-          (size_t)g2_tcap<ZC>() * 2 + (size_t)PH_COUNT * 8 + 15) &
+  using SH = G2Shape<FW>;
+  return ((size_t)G2_REC * G2_ENTRIES * 4 + (size_t)3 * SH::WV * 4 + (size_t)2 * SH::PATCH * 8 +
+          (size_t)chunk * 4 + (FOLD ? (size_t)2 * 16 * 4 : 0) + (size_t)(SH::WV + 32) + 15) &
          ~(size_t)15;
 }
 
-// The 4 pixels of a box row starting at `row`, read as two two-pixel loads
-// from the aligned unit at or before `row` (the images are 16-byte aligned,
-// so every image's storage row 0 starts aligned and the unit before an
-// unaligned row start lies in the image's previous storage row), plus one
-// single-pixel load when `row` is not aligned: no load leaves the images.
-template <int F16>
-__device__ __forceinline__ void load_row4(const unsigned char *row, float2 &p0, float2 &p1,
-                                          float2 &p2, float2 &p3) {
-  const uintptr_t u = reinterpret_cast<uintptr_t>(row);
-  if (!F16) {
-    const bool odd = (u & 8) != 0;
-    const float4 *al = reinterpret_cast<const float4 *>(u & ~(uintptr_t)15);
-    const float4 A = __ldg(al), B = __ldg(al + 1);
-    float2 C = make_float2(0.f, 0.f);
-    if (odd) C = __ldg(reinterpret_cast<const float2 *>(al + 2));
-    p0 = odd ? make_float2(A.z, A.w) : make_float2(A.x, A.y);
-    p1 = odd ? make_float2(B.x, B.y) : make_float2(A.z, A.w);
-    p2 = odd ? make_float2(B.z, B.w) : make_float2(B.x, B.y);
-    p3 = odd ? C : make_float2(B.z, B.w);
-  } else {
-    const bool odd = (u & 4) != 0;
-    const uint2 *al = reinterpret_cast<const uint2 *>(u & ~(uintptr_t)7);
-    const uint2 A = __ldg(al), B = __ldg(al + 1);
-    unsigned C = 0u;
-    if (odd) C = __ldg(reinterpret_cast<const unsigned *>(al + 2));
-    const unsigned h0 = odd ? A.y : A.x, h1 = odd ? B.x : A.y, h2 = odd ? B.y : B.x,
-                   h3 = odd ? C : B.y;
-    p0 = __half22float2(*reinterpret_cast<const __half2 *>(&h0));
-    p1 = __half22float2(*reinterpret_cast<const __half2 *>(&h1));
-    p2 = __half22float2(*reinterpret_cast<const __half2 *>(&h2));
-    p3 = __half22float2(*reinterpret_cast<const __half2 *>(&h3));
+__device__ __forceinline__ void cp_async8(uint32_t dst, const void *src) {
+  asm volatile("cp.async.ca.shared.global [%0], [%1], 8;" ::"r"(dst), "l"(src) : "memory");
+}
+__device__ __forceinline__ void cp_async_wait_all() { asm volatile("cp.async.wait_all;" ::: "memory"); }
+
+// The 4 x 4 box of an item: pixels p[l * PITCH + j], u at (dx, dy) from pixel
+// (0, 0), u_z^2 = uz2; returns the sums of w p (complex) and of w over the
+// candidates with r <= a.  FOLD: candidate (j, l) counts only if bit j of
+// rows[l] >> shift is set.
+template <int PITCH, int FOLD>
+__device__ __forceinline__ void g2_box(const float2 *cp, const float2 *p, float dx, float dy,
+                                       float uz2, float cs, float sq, float &ar, float &ai,
+                                       float &aw, const unsigned *rows, int shift) {
+  constexpr int NP = POLY_N;
+  // cp: coefficient pairs (c_k, c_k), kernel-parameter constants
+  // scaled column offsets sq (dx - j): x = (sq dx)^2 + cs (dy^2 + u_z^2) - 1
+  const float2 S2 = make_float2(sq, sq), C2 = make_float2(cs, cs);
+  const float2 DX = make_float2(dx, dx), DY = make_float2(dy, dy);
+  const float2 d01 = __fmul2_rn(__fadd2_rn(DX, make_float2(0.0f, -1.0f)), S2);
+  const float2 d23 = __fmul2_rn(__fadd2_rn(DX, make_float2(-2.0f, -3.0f)), S2);
+  const float U = fmaf(cs, uz2, -1.0f);
+  const float2 UU = make_float2(U, U);
+  // all 16 polynomials advance together: eight independent chains of packed
+  // FMAs (row by row, two chains, the FMA pipe waits for their latency)
+  float2 x[8], h[8];
+#pragma unroll
+  for (int r = 0; r < 4; ++r) {
+    const float2 EY = r ? __fadd2_rn(DY, make_float2(-(float)r, -(float)r)) : DY;
+    const float2 YY = __ffma2_rn(__fmul2_rn(C2, EY), EY, UU);
+    x[2 * r] = __ffma2_rn(d01, d01, YY);
+    x[2 * r + 1] = __ffma2_rn(d23, d23, YY);
+  }
+#pragma unroll
+  for (int i = 0; i < 8; ++i) h[i] = __ffma2_rn(cp[NP - 1], x[i], cp[NP - 2]);
+#pragma unroll
+  for (int k = NP - 3; k >= 0; --k)
+#pragma unroll
+    for (int i = 0; i < 8; ++i) h[i] = __ffma2_rn(h[i], x[i], cp[k]);
+  ar = 0.f;
+  ai = 0.f;
+  aw = 0.f;
+#pragma unroll
+  for (int r = 0; r < 4; ++r) {
+    const float2 p0 = p[r * PITCH], p1 = p[r * PITCH + 1], p2 = p[r * PITCH + 2],
+                 p3 = p[r * PITCH + 3];
+    bool i0 = x[2 * r].x <= 1.0f, i1 = x[2 * r].y <= 1.0f, i2 = x[2 * r + 1].x <= 1.0f,
+         i3 = x[2 * r + 1].y <= 1.0f;
+    if (FOLD) {
+      const unsigned m = rows[r] >> shift;
+      i0 = i0 && (m & 1u);
+      i1 = i1 && (m & 2u);
+      i2 = i2 && (m & 4u);
+      i3 = i3 && (m & 8u);
+    }
+    // predicated accumulation: no select, and no pixel outside the blob is used
+    const float2 wa = h[2 * r], wb = h[2 * r + 1];
+    if (i0) { ar = fmaf(wa.x, p0.x, ar); ai = fmaf(wa.x, p0.y, ai); aw += wa.x; }
+    if (i1) { ar = fmaf(wa.y, p1.x, ar); ai = fmaf(wa.y, p1.y, ai); aw += wa.y; }
+    if (i2) { ar = fmaf(wb.x, p2.x, ar); ai = fmaf(wb.x, p2.y, ai); aw += wb.x; }
+    if (i3) { ar = fmaf(wb.y, p3.x, ar); ai = fmaf(wb.y, p3.y, ai); aw += wb.y; }
   }
 }
 
-// The 4 x 4 box of an item: candidates (kx0 + j, ky0 + l) of the stored half
-// plane (ibase points at pixel kx0 of the image), u at (kx0 + fx, ky0 + fy),
-// u_z^2 = uz2; returns the sums of w p (complex) and of w over the candidates
-// with r <= a.  FOLD: a stored pixel k is inserted at R k when it is not
-// folded and at -R k (conjugated) when it is, folded meaning R00 k_x + R01 k_y
-// < 0 (exact sign; r00, r01 = R00, R01): the box read directly (refl = 0)
-// keeps the candidates that are not folded, the point-reflected box (refl =
-// 1) those that are.  Away from the fold columns that test always passes.
-template <int F16, int FOLD = 0>
-__device__ __forceinline__ void g2_box(const InsertArgs &args, const float2 *cp,
-                                       const unsigned char *ibase, int kx0, int ky0, float fx,
-                                       float fy, float uz2, float cs, float sq, float2 &acc,
-                                       float &aw, float r00 = 0.f, float r01 = 0.f,
-                                       bool refl = false) {
-  constexpr int NP = POLY_N;
-  constexpr int ESZ = F16 ? 4 : 8;
+// Fold a warp's partial sums (s_acc: [3][WV], slot (y FW + x) 8 + z) into HBM
+// and clear them: straight into the double-float accumulators (error-free
+// TwoSum) when the warp is the only writer of its voxels, else into the float4
+// scratch with atomics (merged after the launch).  The loads of four z levels
+// are issued together: one after the other, their latency made a flush take
+// four times as long.
+template <int FW>
+__device__ __noinline__ void g2_flush(const InsertArgs &args, float *s_acc, int fx0, int fy0,
+                                      int z0, bool to_scratch) {
+  using SH = G2Shape<FW>;
+  constexpr int WV = SH::WV, ZC = SH::ZC, ZG = 4;
   const Geom &g = args.g;
-  // cp: coefficient pairs (c_k, c_k), kernel-parameter constants
-  const int row_bytes = g.NX * ESZ;
-  // scaled column offsets sq (fx - j): x = (sq dx)^2 + cs (dy^2 + u_z^2) - 1
-  const float2 d01 = make_float2(sq * fx, sq * (fx - 1.0f));
-  const float2 d23 = make_float2(sq * (fx - 2.0f), sq * (fx - 3.0f));
-  const float U = fmaf(cs, uz2, -1.0f);
-  float2 a2 = make_float2(0.f, 0.f), w2 = make_float2(0.f, 0.f);
+  const int lane = threadIdx.x & 31;
+  __syncwarp();
+#pragma unroll 1
+  for (int k = 0; k < SH::NC * ZC / ZG; ++k) {
+    const int col = (k / (ZC / ZG)) * 32 + lane, t0 = k % (ZC / ZG) * ZG;
+    const int vx = fx0 + col % FW, vy = fy0 + col / FW;
+    if (vx > g.H || vy > g.H) continue;
+    const float *s = s_acc + col * ZC + t0;
+    const size_t slice = (size_t)g.D * g.NXa;
+    const size_t v0 = ((size_t)(z0 + t0 + g.H) * g.D + (size_t)(vy + g.H)) * g.NXa + (size_t)(vx - g.xa0);
+    if (to_scratch) {
 #pragma unroll
-  for (int r = 0; r < 4; ++r) {
-    int ky = ky0 + r;
-    ky += ky < 0 ? g.S : 0;
-    float2 p0, p1, p2, p3;
-    load_row4<F16>(ibase + ky * row_bytes, p0, p1, p2, p3);
-    const float dy = fy - (float)r;
-    const float Y = fmaf(cs * dy, dy, U);
-    const float2 YY = make_float2(Y, Y);
-    const float2 xa = __ffma2_rn(d01, d01, YY), xb = __ffma2_rn(d23, d23, YY);
-    float2 ha = cp[NP - 1], hb = cp[NP - 1];
+      for (int t = 0; t < ZG; ++t) {
+        const float4 v = make_float4(s[t], s[WV + t], s[2 * WV + t], 0.f);
+        if (z0 + t0 + t <= g.H && (v.x != 0.f || v.y != 0.f || v.z != 0.f))
+          atomicAdd(args.scratch + v0 + t * slice, v);
+      }
+    } else {
+      float h[3 * ZG], l[3 * ZG];
 #pragma unroll
-    for (int k = NP - 2; k >= 0; --k) {
-      ha = __ffma2_rn(ha, xa, cp[k]);
-      hb = __ffma2_rn(hb, xb, cp[k]);
+      for (int t = 0; t < ZG; ++t)
+#pragma unroll
+        for (int c = 0; c < 3; ++c) {
+          const bool in = z0 + t0 + t <= g.H;
+          const float *q = args.acc + c * args.plane + v0 + t * slice;
+          h[3 * t + c] = in ? q[0] : 0.f;
+          l[3 * t + c] = in ? q[3 * args.plane] : 0.f;
+        }
+#pragma unroll
+      for (int t = 0; t < ZG; ++t) {
+        const float add[3] = {s[t], s[WV + t], s[2 * WV + t]};
+        if (z0 + t0 + t > g.H || (add[0] == 0.f && add[1] == 0.f && add[2] == 0.f)) continue;
+#pragma unroll
+        for (int c = 0; c < 3; ++c) {
+          float *q = args.acc + c * args.plane + v0 + t * slice;
+          dd_add(h[3 * t + c], l[3 * t + c], add[c]);
+          q[0] = h[3 * t + c];
+          q[3 * args.plane] = l[3 * t + c];
+        }
+      }
     }
-    float w0 = xa.x <= 1.0f ? ha.x : 0.0f, w1 = xa.y <= 1.0f ? ha.y : 0.0f;
-    float w2_ = xb.x <= 1.0f ? hb.x : 0.0f, w3 = xb.y <= 1.0f ? hb.y : 0.0f;
-    if (FOLD) {
-      const int kyr = ky0 + r;
-      if (fold_pred(r00, r01, kx0, kyr) != refl) w0 = 0.f;
-      if (fold_pred(r00, r01, kx0 + 1, kyr) != refl) w1 = 0.f;
-      if (fold_pred(r00, r01, kx0 + 2, kyr) != refl) w2_ = 0.f;
-      if (fold_pred(r00, r01, kx0 + 3, kyr) != refl) w3 = 0.f;
-    }
-    a2 = __ffma2_rn(make_float2(w0, w0), p0, a2);
-    a2 = __ffma2_rn(make_float2(w1, w1), p1, a2);
-    a2 = __ffma2_rn(make_float2(w2_, w2_), p2, a2);
-    a2 = __ffma2_rn(make_float2(w3, w3), p3, a2);
-    w2 = __fadd2_rn(w2, make_float2(w0 + w2_, w1 + w3));
   }
-  acc = a2;
-  aw = w2.x + w2.y;
+  __syncwarp();
+  for (int i = lane; i < 3 * WV; i += 32) s_acc[i] = 0.f;
+  __syncwarp();
+}
+
+// The warp footprints of a BX x BY x BZ brick, FW x 8 x 8 voxels each.
+template <int BX, int BY, int BZ, int FW>
+__host__ __device__ constexpr int g2_warps() {
+  return (BX / FW) * (BY / 8) * (BZ / 8);
 }
 
 // One warp's share of one work unit (see gather_warp for the unit word).
 // args: the batch's arguments; cst: the arguments its launch shares (geometry,
 // weight polynomial, list capacity) and images the batch's images, both read
-// in the inner loops.  The warp footprint is FW x (32 / FW) columns (8 x 4,
-// or 4 x 8 for the fold columns).  FOLD = 0: the bricks tile x >= floor(a) +
-// 1; FOLD = 1: they tile x >= -floor(a) and only the fold columns |x| <=
-// floor(a) are computed, with the fold predicate tested per candidate.
-template <int BX, int BY, int ZC, int F16, int FW = 8, int FOLD = 0>
+// in the inner loops.  FOLD = 0: the bricks tile x >= floor(a) + 1; FOLD = 1:
+// they tile x >= -floor(a) and only the fold columns |x| <= floor(a) are
+// computed, with the fold predicate tested per candidate.
+template <int BX, int BY, int BZ, int F16, int FW = 8, int FOLD = 0>
 __device__ __forceinline__ void gather2_warp(const InsertArgs &args, const InsertArgs &cst,
                                              const void *images, unsigned char *wsmem,
                                              const int4 unit, const int warp) {
-  constexpr int FH = 32 / FW;  // footprint height in y
-  static_assert((FW == 8 || FW == 4) && BX % FW == 0 && BY % FH == 0 && (BX * BY) % 32 == 0,
-                "warp footprint is 8 x 4 or 4 x 8 columns");
-  static_assert(ZC == 8 || ZC == 16, "tags hold 4 bits of z");
-  constexpr int WV = 32 * ZC;
+  using SH = G2Shape<FW>;
+  constexpr int FH = SH::FH, ZC = SH::ZC, WV = SH::WV, PW = SH::PW, PITCH = SH::PITCH,
+                NC = SH::NC;
+  static_assert((FW == 8 || FW == 4) && BX % FW == 0 && BY % FH == 0 && BZ % ZC == 0,
+                "warp footprints are 8 x 8 x 8 or 4 x 8 x 8 voxels");
+  static_assert(PW <= 17 && PW <= PITCH && (!FOLD || PW <= 16), "patch rows");
   constexpr int ESZ = F16 ? 4 : 8;
-  constexpr float HX = 0.5f * (FW - 1), HY = 0.5f * (FH - 1);  // footprint half extents
+  constexpr float HX = SH::HX, HY = SH::HY, HZ = SH::HZ;
+  constexpr unsigned FULL = 0xffffffffu;
   const Geom &g = cst.g;
-  const int lane = threadIdx.x & 31;
-  const int wx = warp % (BX / FW), wy = warp / (BX / FW);
+  int lane;  // read once: the special register is slow
+  asm volatile("mov.u32 %0, %%laneid;" : "=r"(lane));
+  const int wx = warp % (BX / FW), wy = warp / (BX / FW) % (BY / FH), wz = warp / (BX / FW * (BY / FH));
   const int fx0 = (FOLD ? g.xa0 : 1 - g.xa0) + unit.x * BX + wx * FW;
   const int fy0 = -g.H + unit.y * BY + wy * FH;
-  const int z0 = -g.H + unit.z * ZC;
+  const int z0 = -g.H + unit.z * BZ + wz * ZC;
   const int lcap = cst.chunk;
-  if (lcap > 64) {  // list entries are 6 bits of the tags
+  if (lcap < 32 || lcap > 64) {  // the image list holds lcap entries
     if (lane == 0) set_err(args.err, DERR_RANGE);
     return;
   }
-  float *s_list = reinterpret_cast<float *>(__builtin_assume_aligned(wsmem, 16));
-  float *s_acc = s_list + (size_t)LIST_FIELDS * lcap;                               // [3][WV]
-  unsigned *s_tag2 = reinterpret_cast<unsigned *>(s_acc + 3 * WV);                  // [G2_T2CAP]
-  unsigned long long *s_ph = reinterpret_cast<unsigned long long *>(s_tag2 + G2_T2CAP);  // [PH_COUNT]
-  unsigned short *s_tag = reinterpret_cast<unsigned short *>(s_ph + PH_COUNT);      // [g2_tcap]
+  if (fx0 > g.H || fy0 > g.H || z0 > g.H) return;  // no voxel of the volume
+  float4 *s_rec = reinterpret_cast<float4 *>(__builtin_assume_aligned(wsmem, 16));  // [G2_ENTRIES][4]
+  float *s_acc = reinterpret_cast<float *>(s_rec + G2_REC / 4 * G2_ENTRIES);        // [3][WV]
+  float2 *s_patch = reinterpret_cast<float2 *>(s_acc + 3 * WV);                     // [2][PATCH]
+  int *s_idx = reinterpret_cast<int *>(s_patch + 2 * SH::PATCH);                    // [lcap]
+  unsigned *s_bits = reinterpret_cast<unsigned *>(s_idx + lcap);                    // FOLD: [2][16]
+  unsigned char *s_tag = reinterpret_cast<unsigned char *>(s_bits + (FOLD ? 32 : 0));  // [WV + 32]
 
   const int split = unit.w & 0xffff, nsplit = (unit.w >> 16) & 0x3fff;
   const bool to_scratch = nsplit > 1 || ((unit.w >> 30) & 1);
   const int img0 = (int)((long long)args.n * split / nsplit);
   const int img1 = (int)((long long)args.n * (split + 1) / nsplit);
-  const float cx = fx0 + HX, cy = fy0 + HY, cz = z0 + 0.5f * (ZC - 1);  // footprint centre
-  const float hz = 0.5f * (ZC - 1);
-  const float rw = sqrtf(HX * HX + HY * HY + hz * hz);
-  const float a = g.a;
-  // box origin ceil(u - a_box): a spare box cell (KB > floor(2a) + 1) is
-  // shifted down by a margin so a pixel at distance exactly a is never lost
-  // to the rounding of u (the r^2 <= a^2 mask decides it)
-  const float a_box = 4 > (int)floorf(2.0f * a) + 1 ? a + 1e-4f : a;
-  const float a_plane = a + 1e-4f;      // conservative |u_z| <= a test
-  const float reach = (float)g.H + a;   // the extended plane spans [-H, H]^2
-  const float ext = reach + rw + 1.0f;
-  const int vx = fx0 + lane % FW, vy = fy0 + lane / FW;
-  const bool col_in = vx <= g.H && vy <= g.H && (!FOLD || vx <= -g.xa0);
-  const float dvx = (float)(lane % FW) - HX, dvy = (float)(lane / FW) - HY;
+  const float cx = fx0 + HX, cy = fy0 + HY, cz = z0 + HZ;  // footprint centre
+  const float a_plane = g.a + 1e-4f;  // conservative |u_z| <= a test
   const float cs = 2.0f / g.a2, sq = sqrtf(cs);  // the weight polynomial's argument scales
   const unsigned char *imgs = reinterpret_cast<const unsigned char *>(images);
   const size_t img_stride = (size_t)g.S * g.NX * ESZ;
   const unsigned lt = (1u << lane) - 1u;
+  // the lane's columns (x, y), (x, y + 32 / FW): offsets from the centre, last
+  // z level inside the volume (-1: the column is outside)
+  const float dvx = (float)(lane % FW) - HX, dvy = (float)(lane / FW) - HY;
+  int tmax[NC];
+#pragma unroll
+  for (int c = 0; c < NC; ++c) {
+    const int vx = fx0 + lane % FW, vy = fy0 + lane / FW + c * (32 / FW);
+    tmax[c] = vx <= g.H && vy <= g.H && (!FOLD || vx <= -g.xa0) ? min(ZC - 1, g.H - z0) : -1;
+  }
 
   for (int i = lane; i < 3 * WV; i += 32) s_acc[i] = 0.f;
   __syncwarp();
   // optional phase counters (fr_options.debug bit 1): cycles of cull, item
-  // generation (PH_QUEUE), evaluation rounds (PH_DRAIN_FAST) and flushes, item
-  // and round counts; kept in shared memory (lane 0 counts) so that they hold
-  // no registers
+  // generation with the patches (PH_QUEUE), evaluation rounds (PH_DRAIN_FAST)
+  // and flushes, item and round counts, added by lane 0
   const bool prof = args.phase != nullptr;
-  unsigned long long *ph = s_ph;
-  if (prof && lane == 0)
-    for (int k = 0; k < PH_COUNT; ++k) ph[k] = 0;
-  const long long t_start = prof ? clock64() : 0;
   auto tick = [&]() -> long long { return prof ? clock64() : 0; };
-
-  int qt = 0, qt2 = 0;  // queued tags, queued forced second halves
-
-  // One round: lane k evaluates tag q[k] (if k < cnt): li << 9 | column << 4 |
-  // z level, plus bit 16 (half forced) and bit 17 (the reflected half) for
-  // the second halves; an item whose box crosses kx = 0 queues its other half
-  // in s_tag2.
-  auto round = [&](unsigned tag, bool alive) {
-    const int li = (int)((tag >> 9) & 63), src = (int)((tag >> 4) & 31), t = (int)(tag & 15);
-    const bool forced = ((tag >> 16) & 1u) != 0, fneg = ((tag >> 17) & 1u) != 0;
-    const float *L = s_list + li * LIST_FIELDS;
-    const float4 q0 = *reinterpret_cast<const float4 *>(L + LF_MX);   // m, u_z of the centre
-    const float4 q1 = *reinterpret_cast<const float4 *>(L + LF_E1X);  // e1, fractional u_x
-    const float4 q2 = *reinterpret_cast<const float4 *>(L + LF_E2X);  // e2, fractional u_y
-    const int4 q3 = *reinterpret_cast<const int4 *>(L + LF_CIX);      // integer centre, image address
-    const float sdx = (float)(src % FW) - HX, sdy = (float)(src / FW) - HY,
-                sdz = (float)t - hz;
-    const float uz = fmaf(q0.z, sdz, fmaf(q0.y, sdy, fmaf(q0.x, sdx, q0.w)));
-    const float uxr = fmaf(q1.z, sdz, fmaf(q1.y, sdy, fmaf(q1.x, sdx, q1.w)));
-    const float uyr = fmaf(q2.z, sdz, fmaf(q2.y, sdy, fmaf(q2.x, sdx, q2.w)));
-    const float ux = (float)q3.x + uxr, uy = (float)q3.y + uyr;
-    const bool valid = alive && fabsf(ux) <= reach && fabsf(uy) <= reach;
-    // the half plane read: the one u lies in, or the forced one
-    const bool neg = forced ? fneg : ux < 0.f;
-    const float sg = neg ? -1.f : 1.f;
-    const int isg = neg ? -1 : 1;
-    const float vxr = sg * uxr, vyr = sg * uyr;
-    const float ixf = ceilf(vxr - a_box), iyf = ceilf(vyr - a_box);
-    const int kx0 = isg * q3.x + (int)ixf, ky0 = isg * q3.y + (int)iyf;
-    // the box reaches column kx <= 0: the other half as well
-    const bool second = valid && !forced && kx0 < 1;
-    const unsigned m2 = __ballot_sync(0xffffffffu, second);
-    if (second) s_tag2[qt2 + __popc(m2 & lt)] = (tag & 0xffffu) | (1u << 16) | (neg ? 0u : 1u << 17);
-    qt2 += __popc(m2);
-    // clamp the box into the stored half plane [0, H] x [-H, H - 1]
-    const int kxc = min(max(kx0, 0), g.H - 3);
-    const int kyc = min(max(ky0, -g.H), g.H - 4);
-    // an item outside the extended plane (or a dead lane) keeps a box far from u
-    const float fx = valid ? vxr - ixf + (float)(kx0 - kxc) : 64.f;
-    const float fy = vyr - iyf + (float)(ky0 - kyc);
-    float2 acc;
-    float aw;
-    const unsigned char *ibase = reinterpret_cast<const unsigned char *>(
-        (unsigned long long)(unsigned)q3.z | ((unsigned long long)(unsigned)q3.w << 32));
-    g2_box<F16, FOLD>(cst, cst.poly2, ibase + (size_t)kxc * ESZ, kxc,
-                      kyc, fx, fy, uz * uz, cs, sq, acc, aw, q1.x, q2.x, neg);
-    if (valid) {
-      const int slot = src * ZC + t;
-      atomicAdd(&s_acc[slot], acc.x);
-      atomicAdd(&s_acc[WV + slot], neg ? -acc.y : acc.y);
-      atomicAdd(&s_acc[2 * WV + slot], aw);
-    }
-    __syncwarp();
+  auto count = [&](int what, long long v) {
+    if (prof && lane == 0) atomicAdd(args.phase + what, (unsigned long long)v);
   };
+  auto clocked = [&](int what, long long since) {
+    if (prof && lane == 0) atomicAdd(args.phase + what, (unsigned long long)(clock64() - since));
+  };
+  const long long t_start = tick();
+  const float reach = (float)g.H + g.a + 1e-2f;  // the extended plane spans [-H, H]^2
 
-  // evaluate full rounds of both queues (every tag if `all`); the remainders
-  // move to the fronts
-  auto drain = [&](bool all) {
-    const long long t0 = tick();
-    int nr = 0;
-    int head = 0;
-    for (; qt - head >= 32 || (all && qt > head); head += 32) {
-      const bool alive = lane < qt - head;
-      round(alive ? (unsigned)s_tag[head + lane] : 0u, alive);
-      ++nr;
-      if (qt2 >= 32) {
-        const unsigned t2 = s_tag2[lane];
-        __syncwarp();
-        round(t2, true);
-        ++nr;
-        qt2 -= 32;
-        const unsigned v = lane < qt2 ? s_tag2[32 + lane] : 0u;
-        __syncwarp();
-        if (lane < qt2) s_tag2[lane] = v;
-        __syncwarp();
+  // Records of listed images from `head` on, one image per lane, one record
+  // per half plane whose pixels the footprint can meet (each half plane's
+  // pixels lie in k_x >= 0 of the orientation):
+  //   plane normal, u_z of the centre | first in-plane axis, fractional u_x |
+  //   second in-plane axis, fractional u_y |
+  //   first patch pixel relative to the centre's integer part and patch size
+  //   (bytes px, py, pw, ph), first patch pixel (px | py << 16), image, flags
+  //   (bit 0: reflected, bit 1: the image has records for both half planes)
+  // Takes as many images as have G2_ENTRIES records; returns their number, ne
+  // the number of records.
+  auto build = [&](int head, int nl, int &ne) -> int {
+    const bool have = lane < G2_ENTRIES && head + lane < nl;
+    int i = 0;
+    bool direct = false, refl = false;
+    float e1x = 0, e1y = 0, e1z = 0, e2x = 0, e2y = 0, e2z = 0, mx = 0, my = 0, mz = 0;
+    float fx = 0, fy = 0, uz = 0, sx = 0, sy = 0;
+    int cxi = 0, cyi = 0;
+    if (have) {
+      i = s_idx[head + lane];
+      const float *R = args.rot + 9 * (size_t)i;
+      e1x = __ldg(R + 0); e1y = __ldg(R + 3); e1z = __ldg(R + 6);
+      e2x = __ldg(R + 1); e2y = __ldg(R + 4); e2z = __ldg(R + 7);
+      mx = __ldg(R + 2);  my = __ldg(R + 5);  mz = __ldg(R + 8);
+      float hxx, lx, hyy, ly, hzz, lz;
+      dot3_dd(e1x, e1y, e1z, cx, cy, cz, hxx, lx);
+      dot3_dd(e2x, e2y, e2z, cx, cy, cz, hyy, ly);
+      dot3_dd(mx, my, mz, cx, cy, cz, hzz, lz);
+      const float rx = rintf(hxx), ry = rintf(hyy);
+      fx = (hxx - rx) + lx;  // hxx - rx is exact
+      fy = (hyy - ry) + ly;
+      uz = hzz + lz;
+      sx = fabsf(e1x) * HX + fabsf(e1y) * HY + fabsf(e1z) * HZ;
+      sy = fabsf(e2x) * HX + fabsf(e2y) * HY + fabsf(e2z) * HZ;
+      const bool in = fabsf(hxx) <= reach + sx && fabsf(hyy) <= reach + sy;
+      direct = in && hxx + sx + g.a + 1e-2f >= 0.f;
+      refl = in && hxx - sx - g.a - 1e-2f <= 0.f;
+      const float far = 4096.0f;  // bounds for inputs that are no rotation
+      cxi = (int)fminf(fmaxf(rx, -far), far);
+      cyi = (int)fminf(fmaxf(ry, -far), far);
+    }
+    const unsigned bd = __ballot_sync(FULL, direct), br = __ballot_sync(FULL, refl);
+    int o = __popc(bd & lt) + __popc(br & lt);
+    const int mine = (direct ? 1 : 0) + (refl ? 1 : 0);
+    const unsigned taken = __ballot_sync(FULL, have && o + mine <= G2_ENTRIES);
+    const int images_taken = __popc(taken);  // o + mine ascends: the first images
+    ne = __popc(bd & taken) + __popc(br & taken);
+    if (have && o + mine <= G2_ENTRIES) {
+#pragma unroll 1
+      for (int h = 0; h < 2; ++h) {
+        if (h == 0 ? direct : refl) {
+          const float sg = h ? -1.f : 1.f;
+          const float ffx = sg * fx, ffy = sg * fy;
+          const int ccx = h ? -cxi : cxi, ccy = h ? -cyi : cyi;
+          // pixels that the boxes can reach, inside the stored half plane [0, H]
+          // x [-H, H - 1]; at least one whole box, at most PW x PW
+          const float far = 4096.0f, wx_ = sx + 2.01f, wy_ = sy + 2.01f;
+          const int lox = ccx + (int)fminf(fmaxf(ceilf(ffx - wx_), -far), far);
+          const int hix = ccx + (int)fminf(fmaxf(floorf(ffx + wx_), -far), far);
+          const int loy = ccy + (int)fminf(fmaxf(ceilf(ffy - wy_), -far), far);
+          const int hiy = ccy + (int)fminf(fmaxf(floorf(ffy + wy_), -far), far);
+          const int px = max(0, min(lox, g.H + 1 - PW)), py = max(-g.H, min(loy, g.H - PW));
+          const int pw = min(max(min(hix, g.H) - px + 1, 4), min(PW, g.H + 1 - px));
+          const int ph = min(max(min(hiy, g.H - 1) - py + 1, 4), min(PW, g.H - py));
+          const int rpx = max(-127, min(px - ccx, 127)), rpy = max(-127, min(py - ccy, 127));
+          s_rec[o * 4 + 0] = make_float4(mx, my, mz, uz);
+          s_rec[o * 4 + 1] = make_float4(sg * e1x, sg * e1y, sg * e1z, ffx);
+          s_rec[o * 4 + 2] = make_float4(sg * e2x, sg * e2y, sg * e2z, ffy);
+          reinterpret_cast<int4 *>(s_rec)[o * 4 + 3] =
+              make_int4((rpx & 255) | ((rpy & 255) << 8) | (pw << 16) | (ph << 24),
+                        (px & 0xffff) | (py << 16), i, h | (mine == 2 ? 2 : 0));
+          ++o;
+        }
       }
     }
-    if (all && qt2 > 0) {
-      const bool alive = lane < qt2;
-      const unsigned t2 = alive ? s_tag2[lane] : 0u;
-      __syncwarp();
-      qt2 = 0;
-      round(t2, alive);
-      ++nr;
-    }
-    const int rest = qt - head < 0 ? 0 : qt - head;
-    if (head > 0 && rest) {
-      const unsigned short v = lane < rest ? s_tag[head + lane] : (unsigned short)0;
-      __syncwarp();
-      if (lane < rest) s_tag[lane] = v;
-      __syncwarp();
-    }
-    qt = rest;
-    if (prof && lane == 0) {
-      ph[PH_DRAIN_FAST] += (unsigned long long)(clock64() - t0);
-      ph[PH_ROUNDS] += (unsigned long long)nr;
-    }
-  };
-
-  // generate the items of list entry li (tags at the queue's tail): the run
-  // of z levels t with |u_z(t)| <= a of the lane's column, from u_z linear in t
-  auto generate = [&](int li) {
-    const long long tq = tick();
-    const float *L = s_list + li * LIST_FIELDS;
-    const float4 q0 = *reinterpret_cast<const float4 *>(L + LF_MX);
-    const float bz = fmaf(q0.z, -hz, fmaf(q0.y, dvy, fmaf(q0.x, dvx, q0.w)));
-    unsigned near = 0;
-#pragma unroll
-    for (int t = 0; t < ZC; ++t)
-      near |= (fabsf(fmaf(q0.z, (float)t, bz)) <= a_plane ? 1u : 0u) << t;
-    if (!col_in) near = 0;
-    const int c = __popc(near);
-    const int t0 = near ? __ffs(near) - 1 : 0;
-    const unsigned lt_ = lt;
-    int excl = 0, ntag = 0;
-#pragma unroll
-    for (int b = 0; b < 5; ++b) {
-      if (b == 4 && ZC < 16) break;
-      const unsigned bal = __ballot_sync(0xffffffffu, (c >> b) & 1);
-      excl += __popc(bal & lt_) << b;
-      ntag += __popc(bal) << b;
-    }
-    const unsigned base = ((unsigned)li << 9) | ((unsigned)lane << 4);
-    const int p0 = qt + excl;
-#pragma unroll
-    for (int t = 0; t < ZC; ++t)
-      if ((near >> t) & 1u) s_tag[p0 + (t - t0)] = (unsigned short)(base | (unsigned)t);
-    qt += ntag;
     __syncwarp();
-    if (prof && lane == 0) {
-      ph[PH_QUEUE] += (unsigned long long)(clock64() - tq);
-      ph[PH_ITEMS_FAST] += (unsigned long long)ntag;
-    }
+    return images_taken;
   };
 
-  int nl = 0;           // entries in the warp's list
-  int since_flush = 0;  // list entries processed since the last flush
+  // Patch copies: 16 columns x 2 rows a step (rows past the patch repeat its
+  // last row), then column 16.
+  constexpr int RG = (PW + 1) / 2;
+  const int pc = lane & 15, pr = lane >> 4;
+  const int row_bytes = g.NX * ESZ;
+  __half2 stage[F16 ? RG + 1 : 1];
+  // start copying the patch of entry li (FP32: into its patch; FP16: into registers)
+  auto fetch = [&](int li) {
+    const int4 q = reinterpret_cast<const int4 *>(s_rec)[li * 4 + 3];
+    const int pw = (q.x >> 16) & 255, ph1 = (int)((unsigned)q.x >> 24) - 1;
+    const int px = q.y & 0xffff, py = q.y >> 16;
+    const unsigned char *img = imgs + (size_t)(unsigned)q.z * img_stride + px * ESZ;
+    const uint32_t dst = static_cast<uint32_t>(__cvta_generic_to_shared(s_patch + (li & 1) * SH::PATCH)) +
+                         (pr * PITCH + pc) * 8;
+    const int c0 = min(pc, pw - 1) * ESZ;
+    if (py < 0 && py + ph1 >= 0) {  // storage wraps at k_y = 0
+#pragma unroll
+      for (int r = 0; r < RG; ++r) {
+        const int ky = py + min(2 * r + pr, ph1);
+        const unsigned char *src = img + (ky + (ky < 0 ? g.S : 0)) * row_bytes + c0;
+        if (F16) stage[r] = __ldg(reinterpret_cast<const __half2 *>(src));
+        else if (2 * r + 1 < PW || pr == 0) cp_async8(dst + 2 * r * PITCH * 8, src);
+      }
+    } else {
+      const unsigned char *first = img + (py + (py < 0 ? g.S : 0)) * row_bytes + c0;
+#pragma unroll
+      for (int r = 0; r < RG; ++r) {
+        const unsigned char *src = first + (size_t)((unsigned)min(2 * r + pr, ph1) * (unsigned)row_bytes);
+        if (F16) stage[r] = __ldg(reinterpret_cast<const __half2 *>(src));
+        else if (2 * r + 1 < PW || pr == 0) cp_async8(dst + 2 * r * PITCH * 8, src);
+      }
+    }
+    if (PW > 16 && pw > 16) {
+      const int ky = py + min(lane, ph1);
+      const unsigned char *src = img + (ky + (ky < 0 ? g.S : 0)) * row_bytes + 16 * ESZ;
+      if (F16) stage[RG] = __ldg(reinterpret_cast<const __half2 *>(src));
+      else if (lane < PW)
+        cp_async8(dst + (lane * PITCH + 16 - pr * PITCH - pc) * 8, src);
+    }
+  };
+  // FP16: convert the staged pixels into entry li's patch
+  auto land = [&](int li, int pw) {
+    float2 *dst = s_patch + (li & 1) * SH::PATCH + pr * PITCH + pc;
+#pragma unroll
+    for (int r = 0; r < RG; ++r)
+      if (2 * r + 1 < PW || pr == 0) dst[2 * r * PITCH] = __half22float2(stage[r]);
+    if (PW > 16 && pw > 16 && lane < PW)
+      dst[lane * PITCH + 16 - pr * PITCH - pc] = __half22float2(stage[RG]);
+  };
+
+  // one entry: its items, then their rounds
+  auto entry = [&](int li, int ne) {
+    const long long tq = tick();
+    const float4 q0 = s_rec[li * 4], q1 = s_rec[li * 4 + 1], q2 = s_rec[li * 4 + 2];
+    const int4 q3 = reinterpret_cast<const int4 *>(s_rec)[li * 4 + 3];
+    const int rpx = (int)(signed char)(q3.x & 255), rpy = (int)(signed char)((q3.x >> 8) & 255);
+    const int pw = (q3.x >> 16) & 255, ph = (int)((unsigned)q3.x >> 24);
+    const float lox = (float)rpx, hix = (float)(rpx + pw - 4);
+    const float loy = (float)rpy, hiy = (float)(rpy + ph - 4);
+    const float2 *patch = s_patch + (li & 1) * SH::PATCH;
+    if (F16) {
+      land(li, pw);
+      if (li + 1 < ne) fetch(li + 1);
+    }
+    if (FOLD) {
+      // one bit per patch pixel, whether it counts in this entry.  In a row the
+      // sign of R00 k_x + R01 k_y changes at most once: lane r finds where in
+      // row r with five exact evaluations.
+      if (lane < PW) {
+        const bool refl = (q3.w & 1) != 0;
+        const float r00 = refl ? -q1.x : q1.x, r01 = refl ? -q2.x : q2.x;
+        const int px = q3.y & 0xffff, py = q3.y >> 16;
+        const bool up = r00 < 0.f;  // the predicate (folded) turns true along the row, else false
+        int t = 0;                  // columns before the turn, 0 .. 31
+#pragma unroll
+        for (int s = 16; s > 0; s >>= 1)
+          if (fold_pred(r00, r01, px + t + s - 1, py + lane) != up) t += s;
+        const unsigned before = t > 30 ? 0x7fffffffu : (1u << t) - 1u;
+        const unsigned folded = up ? ~before : before;
+        s_bits[(li & 1) * 16 + lane] = refl ? folded : ~folded;
+      }
+    }
+    // z levels t of each column with |u_z| <= a, u_z = b + m_z t: t within a /
+    // |m_z| of -b / m_z (a_plane's margin covers the rounding of the quotients,
+    // and of an m_z too small to divide by)
+    const float iz = __fdividef(1.0f, fabsf(q0.z) < 1e-6f ? 1e-6f : q0.z), az = a_plane * fabsf(iz);
+    float b = fmaf(q0.z, -HZ, fmaf(q0.y, dvy, fmaf(q0.x, dvx, q0.w)));
+    int cnt[NC], first[NC];
+#pragma unroll
+    for (int c = 0; c < NC; ++c) {
+      const float tc = b * iz;
+      int tl = max(__float2int_ru(-tc - az), 0), th = min(__float2int_rd(az - tc), tmax[c]);
+      if (q3.w & 2) {
+        // only the items whose box reaches this entry's half plane: u_x >= -a
+        // (lox is the column k_x = 0 here)
+        const float bx = fmaf(q1.z, -HZ, fmaf(q1.y, dvy + c * (32 / FW), fmaf(q1.x, dvx, q1.w)));
+        const float ez = fabsf(q1.z) < 1e-6f ? 1e-6f : q1.z;
+        const float tb = (lox - a_plane - bx) * __fdividef(1.0f, ez);
+        if (ez > 0.f) tl = max(tl, __float2int_ru(tb));
+        else th = min(th, __float2int_rd(tb));
+      }
+      first[c] = tl;
+      cnt[c] = max(th - tl + 1, 0);
+      b = fmaf(q0.y, (float)(32 / FW), b);
+    }
+    // positions: all first columns, then all second ones
+    int incl = NC == 2 ? cnt[0] | (cnt[NC - 1] << 16) : cnt[0];
+#pragma unroll
+    for (int s = 1; s < 32; s <<= 1)
+      asm volatile(
+          "{\n\t.reg .s32 r;\n\t.reg .pred p;\n\t"
+          "shfl.sync.up.b32 r|p, %0, %1, 0, 0xffffffff;\n\t"
+          "@p add.s32 %0, %0, r;\n\t}"
+          : "+r"(incl)
+          : "r"(s));
+    const int tot = __shfl_sync(FULL, incl, 31);
+    const int tot0 = tot & 0xffff, total = tot0 + (tot >> 16);
+    // a tag is its slot less its position, modulo 256
+#pragma unroll
+    for (int c = 0; c < NC; ++c) {
+      const int p = c == 0 ? (NC == 2 ? incl & 0xffff : incl) - cnt[0]
+                           : (tot & 0xffff) + (incl >> 16) - cnt[c];
+      const unsigned char tag = (unsigned char)(lane * ZC + first[c] - p);
+#pragma unroll
+      for (int s = 0; s < ZC; ++s)
+        if (s < cnt[c]) s_tag[p + s] = tag;
+    }
+    if (!F16) {
+      // this entry's patch has landed; the next one's buffer is free
+      cp_async_wait_all();
+      __syncwarp();
+      if (li + 1 < ne) fetch(li + 1);
+    } else {
+      __syncwarp();
+    }
+    clocked(PH_QUEUE, tq);
+    count(PH_ITEMS_FAST, total);
+    const long long td = tick();
+    const float sgn = (q3.w & 1) ? -1.f : 1.f;
+    // patch address of a pixel: at pixel (ox, oy) relative to the centre's
+    // integer part it is ox + PITCH oy, plus 1.5 2^23 whose significand bits
+    // arrive with it
+    const float kM = 8388608.0f, kR = 12582912.0f;
+    const unsigned base = (unsigned)-(rpy * PITCH + rpx) - 0x4b400000u;
+    // one round ahead: the tags are loaded (their buffer is a round longer)
+    unsigned next = s_tag[lane];
+#pragma unroll 1
+    for (int h = lane, left = total; left > 0; h += 32, left -= 32) {
+      // the slot: of the first columns up to position tot0, of the second after
+      const int slot = (int)((next + h) & 255) + (NC == 2 && h >= tot0 ? 256 : 0);
+      next = s_tag[h + 32];
+      // the partial sums, read before the box: no other item of the entry adds to them
+      const float tr = s_acc[slot], ti = s_acc[WV + slot], tw = s_acc[2 * WV + slot];
+      // voxel offsets from the centre: bit fields of the slot placed in the
+      // significand of 2^23, scaled and shifted (exactly)
+      const float sdz = (__int_as_float(0x4b000000 | (slot & (ZC - 1))) - kM) - HZ;
+      const float sdx = fmaf(__int_as_float(0x4b000000 | (slot & ((FW - 1) * ZC))), 1.0f / ZC,
+                             -(kM / ZC + HX));
+      const float sdy = fmaf(__int_as_float(0x4b000000 | (slot & ((FH - 1) * FW * ZC))),
+                             1.0f / (ZC * FW), -(kM / (ZC * FW) + HY));
+      const float uz = fmaf(q0.z, sdz, fmaf(q0.y, sdy, fmaf(q0.x, sdx, q0.w)));
+      const float ux = fmaf(q1.z, sdz, fmaf(q1.y, sdy, fmaf(q1.x, sdx, q1.w)));
+      const float uy = fmaf(q2.z, sdz, fmaf(q2.y, sdy, fmaf(q2.x, sdx, q2.w)));
+      // box origin: the nearest integer to u - 1.5 (by adding 1.5 2^23), clamped
+      const float ox = fminf(fmaxf(__fadd_rn(__fadd_rn(ux - 1.5f, kR), -kR), lox), hix);
+      const float oy = fminf(fmaxf(__fadd_rn(__fadd_rn(uy - 1.5f, kR), -kR), loy), hiy);
+      const unsigned at = __float_as_uint(fmaf(oy, (float)PITCH, __fadd_rn(ox, kR))) + base;
+      const unsigned *rows = s_bits;
+      int shift = 0;
+      if (FOLD) {
+        shift = (int)(ox - lox);
+        rows += (li & 1) * 16 + (int)(oy - loy);
+      }
+      float ar, ai, aw;
+      g2_box<PITCH, FOLD>(cst.poly2, patch + at, ux - ox, uy - oy, uz * uz, cs, sq, ar, ai, aw,
+                          rows, shift);
+      if (h < total) {
+        s_acc[slot] = tr + ar;
+        s_acc[WV + slot] = fmaf(sgn, ai, ti);
+        s_acc[2 * WV + slot] = tw + aw;
+      }
+    }
+    __syncwarp();
+    count(PH_ROUNDS, (total + 31) / 32);
+    clocked(PH_DRAIN_FAST, td);
+  };
+
+  int nl = 0;           // listed images
+  int since_flush = 0;  // images listed since the last flush
+  // plane normals of the next 32 images, loaded one step ahead
+  float nx = 0.f, ny = 0.f, nz = 0.f;
+  auto load_normals = [&](int i) {
+    if (i < img1) {
+      const float *R = args.rot + 9 * (size_t)i;
+      nx = __ldg(R + 2);
+      ny = __ldg(R + 5);
+      nz = __ldg(R + 8);
+    }
+  };
+  load_normals(img0 + lane);
   for (int cs0 = img0;; cs0 += 32) {
     const bool last = cs0 >= img1;
     if (!last) {
+      // cull: an image is listed if its plane passes within a of the footprint box
       const long long tc = tick();
-      nl = cull_step(args, imgs, img_stride, s_list, nl, cs0, img1, cx, cy, cz, HX, HY, hz, ext,
-                     col_in_any(g, fx0, fy0));
+      const int i = cs0 + lane;
+      const float d = nx * cx + ny * cy + nz * cz;
+      const float supp = fabsf(nx) * HX + fabsf(ny) * HY + fabsf(nz) * HZ;
+      const bool keep = i < img1 && fabsf(d) <= g.a + supp + 1e-3f;
+      load_normals(i + 32);
+      const unsigned bk = __ballot_sync(FULL, keep);
+      if (keep) s_idx[nl + __popc(bk & lt)] = i;
+      nl += __popc(bk);
       __syncwarp();
-      if (prof && lane == 0) ph[PH_CULL] += (unsigned long long)(clock64() - tc);
+      clocked(PH_CULL, tc);
     }
-    if (last || nl > lcap - 32) {
-      if (prof && lane == 0) ph[PH_LIST_IMAGES] += (unsigned long long)nl;
-      for (int li = 0; li < nl; ++li) {
-        generate(li);
-        drain(false);
-        if (++since_flush >= GATHER_FLUSH) {
-          drain(true);
-          const long long tf = tick();
-          flush_partials<ZC, FW>(args, s_acc, fx0, fy0, z0, to_scratch);
-          if (prof && lane == 0) ph[PH_FLUSH] += (unsigned long long)(clock64() - tf);
-          since_flush = 0;
-        }
+    // the next step lists at most 32 images
+    if (nl > lcap - 32 || (last && nl > 0)) {
+      for (int head = 0; head < nl;) {
+        int ne = 0;
+        head += build(head, nl, ne);
+        count(PH_LIST_IMAGES, ne);
+        if (ne > 0) fetch(0);
+        for (int li = 0; li < ne; ++li) entry(li, ne);
       }
-      // the list is rebuilt next: nothing may refer to its entries afterwards
-      drain(true);
+      since_flush += nl;
       nl = 0;
+      if (since_flush > GATHER_FLUSH - 64) {
+        const long long tf = tick();
+        g2_flush<FW>(args, s_acc, fx0, fy0, z0, to_scratch);
+        clocked(PH_FLUSH, tf);
+        since_flush = 0;
+      }
     }
     if (last) break;
   }
   const long long tf = tick();
-  flush_partials<ZC, FW>(args, s_acc, fx0, fy0, z0, to_scratch);
-  if (prof && lane == 0) {
-    ph[PH_FLUSH] += (unsigned long long)(clock64() - tf);
-    ph[PH_WARP_CYCLES] = (unsigned long long)(clock64() - t_start);
-    for (int k = 0; k < PH_COUNT; ++k)
-      if (ph[k]) atomicAdd(args.phase + k, ph[k]);
-  }
+  if (since_flush) g2_flush<FW>(args, s_acc, fx0, fy0, z0, to_scratch);
+  clocked(PH_FLUSH, tf);
+  clocked(PH_WARP_CYCLES, t_start);
 }
 
-// One CTA per work unit (args.units[blockIdx.x]); warps run independently.
-// MINW: resident warps per SM the register allocation must allow (16, 20 or
-// 24: at most 128, 102 or 85 registers per thread).  FW, FOLD: see
-// gather2_warp.
-template <int BX, int BY, int ZC, int F16, int MINW, int FW = 8, int FOLD = 0>
-__global__ void __launch_bounds__(BX * BY, MINW * 32 / (BX * BY))
-gather2_kernel(const InsertArgs args) {
+// One warp per CTA: CTA b takes footprint b % W of work unit args.units[b / W]
+// (W footprints a brick).  Warps of one brick never wait for one another, but a
+// CTA holds its shared memory until its last warp ends: with two and four warps
+// a CTA 17 % of the resident warp slots stood idle.  MINW: resident warps per SM
+// the register allocation must allow (16: at most 128 registers per thread, and
+// what shared memory holds; more warps than that are not resident).  FW, FOLD:
+// see gather2_warp.
+template <int BX, int BY, int BZ, int F16, int MINW, int FW = 8, int FOLD = 0>
+__global__ void __launch_bounds__(32, MINW)
+gather2_kernel(const __grid_constant__ InsertArgs args) {
   extern __shared__ __align__(16) unsigned char smem[];
-  const int warp = threadIdx.x >> 5;
-  gather2_warp<BX, BY, ZC, F16, FW, FOLD>(args, args, args.images,
-                                smem + (size_t)warp * gather2_warp_smem<ZC>(args.chunk),
-                                args.units[blockIdx.x], warp);
+  constexpr int W = g2_warps<BX, BY, BZ, FW>();
+  gather2_warp<BX, BY, BZ, F16, FW, FOLD>(args, args, args.images, smem,
+                                          args.units[blockIdx.x / W], (int)(blockIdx.x % W));
 }
 
-// Several batches in one launch: CTA b takes work item p.items[b] =
-// {bx | by << 10 | bz << 20, split word, batch, slot} and copies its batch's
-// arguments p.descs[batch] to shared memory; geometry, weight polynomial and
-// list capacity, common to the launch's batches, are read from p.base (kernel
-// parameters: constant operands in the inner loops).
-template <int BX, int BY, int ZC, int F16, int MINW, int FW = 8, int FOLD = 0>
-__global__ void __launch_bounds__(BX * BY, MINW * 32 / (BX * BY))
-gather2_multi_kernel(const MultiLaunch p) {
-  constexpr int NT = BX * BY;
+// Several batches in one launch: CTA b takes footprint b % W of work item
+// p.items[b / W] = {bx | by << 10 | bz << 20, split word, batch, slot} of batch
+// p.descs[batch]; geometry, weight polynomial and list capacity, common to the
+// launch's batches, are read from p.base (kernel parameters: constant operands
+// in the inner loops), the batch's own arguments (rotations, volume) from its
+// descriptor.
+template <int BX, int BY, int BZ, int F16, int MINW, int FW = 8, int FOLD = 0>
+__global__ void __launch_bounds__(32, MINW)
+gather2_multi_kernel(const __grid_constant__ MultiLaunch p) {
   extern __shared__ __align__(16) unsigned char smem[];
-  const int tid = threadIdx.x, warp = tid >> 5;
-  InsertArgs *s_args = reinterpret_cast<InsertArgs *>(smem);
-  const int4 it = p.items[blockIdx.x];
-  const int *src = reinterpret_cast<const int *>(p.descs + it.z);
-  int *dst = reinterpret_cast<int *>(s_args);
-  for (int i = tid; i < (int)(sizeof(InsertArgs) / 4); i += NT) dst[i] = src[i];
-  __syncthreads();
+  constexpr int W = g2_warps<BX, BY, BZ, FW>();
+  const int4 it = p.items[blockIdx.x / W];
   const int4 unit = make_int4(it.x & 1023, (it.x >> 10) & 1023, (it.x >> 20) & 1023, it.y);
-  gather2_warp<BX, BY, ZC, F16, FW, FOLD>(
-      *s_args, p.base, p.images[it.w],
-      smem + GATHER_ARGS_BYTES + (size_t)warp * gather2_warp_smem<ZC>(p.base.chunk), unit, warp);
+  gather2_warp<BX, BY, BZ, F16, FW, FOLD>(p.descs[it.z], p.base, p.images[it.w], smem, unit,
+                                          (int)(blockIdx.x % W));
 }
 
 }  // namespace fr

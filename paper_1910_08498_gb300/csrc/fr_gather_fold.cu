@@ -1,7 +1,7 @@
 // fr_gather_fold.cu -- the direct-drain gather instantiated for the fold
 // columns |x| <= floor(a) (FOLD): bricks one 4-column footprint wide
-// (4 x 32 x 8, four 4 x 8 warp footprints stacked in y), the fold predicate
-// tested per candidate, 4 x 4 boxes (a < 2), polynomial weights.  Launched
+// (4 x 32 x 8, four 4 x 8 x 8 warp footprints stacked in y), the fold predicate
+// tested per pixel, 4 x 4 boxes (a < 2), polynomial weights.  Launched
 // beside the main direct-drain launch, which covers x >= floor(a) + 1: for one
 // batch, or for the work items of several batches in one launch.
 #include "fr_gather2.cuh"
@@ -11,7 +11,8 @@ namespace fr {
 namespace {
 constexpr int FBX = 4, FBY = 32, FZC = 8, FFW = 4;
 constexpr int FOLD_MINW = 16;  // resident warps per SM the registers allow
-constexpr size_t fold_smem(int chunk) { return (size_t)(FBX * FBY / 32) * gather2_warp_smem<FZC>(chunk); }
+constexpr int FOLD_WARPS = g2_warps<FBX, FBY, FZC, FFW>();
+constexpr size_t fold_smem(int chunk) { return gather2_warp_smem<FFW, 1>(chunk); }
 }  // namespace
 
 GatherShape fold_shape() { return GatherShape{FBX, FBY, FZC}; }
@@ -23,18 +24,18 @@ static cudaError_t launch_fold(const InsertArgs &a, cudaStream_t st) {
   cudaError_t e = allow_dynamic_smem((const void *)fn, smem);
   if (e != cudaSuccess) return e;
   if (a.nunits <= 0) return cudaSuccess;
-  fn<<<a.nunits, FBX * FBY, smem, st>>>(a);
+  fn<<<a.nunits * FOLD_WARPS, 32, smem, st>>>(a);
   return cudaGetLastError();
 }
 
 template <int F16>
 static cudaError_t launch_fold_multi(const MultiLaunch &p, cudaStream_t st) {
   auto fn = gather2_multi_kernel<FBX, FBY, FZC, F16, FOLD_MINW, FFW, 1>;
-  const size_t smem = GATHER_ARGS_BYTES + fold_smem(p.base.chunk);
+  const size_t smem = fold_smem(p.base.chunk);
   cudaError_t e = allow_dynamic_smem((const void *)fn, smem);
   if (e != cudaSuccess) return e;
   if (p.nitems <= 0) return cudaSuccess;
-  return launch_multi((const void *)fn, p, FBX * FBY, smem, st);
+  return launch_multi((const void *)fn, p, FOLD_WARPS, 32, smem, st);
 }
 
 cudaError_t launch_gather_fold_multi(int f16, const MultiLaunch &p, cudaStream_t st) {

@@ -144,8 +144,8 @@ struct PersistentLaunch {
 cudaError_t launch_gather_persistent(int shape_id, int kb, int f16, const PersistentLaunch &p,
                                      cudaStream_t st);
 
-// One launch over the work items of several batches, one CTA per item (the
-// hardware block scheduler hands out the items, heaviest first).  The
+// One launch over the work items of several batches, one CTA per warp footprint
+// of an item (the hardware block scheduler hands them out, heaviest first).  The
 // batches of one launch share S, blob, dtype and configuration: what they
 // share stays in the kernel parameters (base), the rest is read per batch.
 constexpr int MULTI_MAX = 64;  // batches per multi-batch launch
@@ -157,9 +157,10 @@ struct MultiLaunch {
   int priority;              // launch priority (cudaLaunchAttributePriority), 0 = the stream's
   const void *images[MULTI_MAX];  // images of the launch's batches, by slot (read in the inner loop)
 };
-// launch kernel fn (taking one MultiLaunch) with p.nitems CTAs, at p.priority
-cudaError_t launch_multi(const void *fn, const MultiLaunch &p, int threads, size_t smem,
-                         cudaStream_t st);
+// launch kernel fn (taking one MultiLaunch) with per_item CTAs for each of
+// p.nitems work items, at p.priority
+cudaError_t launch_multi(const void *fn, const MultiLaunch &p, int per_item, int threads,
+                         size_t smem, cudaStream_t st);
 // the direct-drain gather (fold columns excluded), FP32 or FP16 images
 cudaError_t launch_gather2_multi(int shape_id, int minw, int f16, const MultiLaunch &p,
                                  cudaStream_t st);

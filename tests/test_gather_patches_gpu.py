@@ -1,0 +1,58 @@
+"""GPU parity of the direct-drain gather at the edges of its pixel patches.
+
+A patch holds at most 17 x 17 stored pixels, copied 16 columns and 2 rows at a
+time and clamped into the half plane.  The sizes put every edge inside small
+volumes: images narrower than a patch (S = 8 .. 30), row lengths S/2 + 1 that
+are even (16-byte rows) and odd, patches that wrap at k_y = 0 and cross
+k_x = 0, footprints cut by the volume's border, an odd number of images, and
+blobs from less than one voxel to the widest 4-wide box.  Tolerance: the
+library's parity bar (2e-5 of the largest value, FP32 accumulation of at most
+40 images; FP16 images against the oracle fed the rounded values)."""
+import numpy as np
+import pytest
+import torch
+
+from paper_1910_08498_gb300 import inputs
+from tests.helpers import TOL_F32, gpu_insert, oracle_insert, rel_err, worst
+
+pytestmark = pytest.mark.gpu
+
+
+def _batch(S, n, seed):
+    img, rot = inputs.make_batch(S, n, seed)
+    perm = inputs.proper_signed_permutations()
+    rot[:5] = perm[[0, 5, 11, 17, 22]]  # planes along the axes: runs of every z level or none
+    return img, rot
+
+
+@pytest.mark.parametrize("f16", [False, True])
+@pytest.mark.parametrize("a", [0.6, 1.0, 1.5, 1.999])
+@pytest.mark.parametrize("S", [8, 10, 14, 16, 18, 30, 32, 34, 46])
+def test_patch_edges_match_oracle(S, a, f16):
+    a = float(np.float32(a))
+    batches = [_batch(S, 33, 7 * S)]
+    V, W, _ = gpu_insert(S, batches, a=a, tuning=False, f16=f16)
+    Vr, Wr, _ = oracle_insert(S, batches, a=a, f16=f16)
+    assert rel_err(V, Vr) <= TOL_F32, worst(V, Vr, S)
+    assert rel_err(W, Wr) <= TOL_F32, worst(W, Wr, S)
+
+
+def test_pixels_outside_the_blob_do_not_reach_a_voxel():
+    """One infinite pixel: only the voxels within the radius of it are not finite."""
+    S = 32
+    img, rot = inputs.make_batch(S, 2, 5)
+    img[1, 3, 7] = complex(float("inf"), 0.0)
+    V, W, _ = gpu_insert(S, [(img, rot)], tuning=False)
+    q = rot[1].double() @ torch.tensor([7.0, 3.0, 0.0], dtype=torch.float64)
+    if rot[1, 0, 0] * 7 + rot[1, 0, 1] * 3 < 0:
+        q = -q
+    D, H = S + 1, S // 2
+    g = np.arange(D) - H
+    z, y, x = np.meshgrid(g, g, g, indexing="ij")
+    r2 = (x - float(q[0])) ** 2 + (y - float(q[1])) ** 2 + (z - float(q[2])) ** 2
+    a2 = float(np.float32(1.9)) ** 2
+    inside = (r2 <= a2 - 1e-4).ravel()
+    outside = (r2 > a2 + 1e-4).ravel()
+    assert not np.isfinite(V[inside]).any()
+    assert np.isfinite(V[outside]).all()
+    assert np.isfinite(W).all()
