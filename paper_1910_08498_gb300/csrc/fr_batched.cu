@@ -125,11 +125,11 @@ int build_plan(Plan &pl, fr_ctx *const *ctxs, const void *const *images, const i
   for (int b = 0; b < nb; ++b) {
     if (n[b] == 0) continue;
     fr_ctx *c = ctxs[b];
-    const Config &k = config_space()[cfg[b]];
+    const Config k = effective_config(c, cfg[b]);
     const int f16 = dtypes[b] == FR_F16 ? 1 : 0;
     const bool poly_ok = c->poly_err < 1e-6;
-    if (k.algo == ALGO_GATHER2 && poly_ok && c->g.KB == 4) {
-      groups[GKey(ALGO_GATHER2, k.shape, 4, f16, k.chunk, k.minw, c->S, c->g.a, c->g.alpha)]
+    if (k.algo == ALGO_GATHER2 && poly_ok) {
+      groups[GKey(ALGO_GATHER2, k.shape, c->g.KB, f16, k.chunk, k.minw, c->S, c->g.a, c->g.alpha)]
           .push_back(b);
     } else if (k.algo == ALGO_GATHER && k.wmode == W_POLY && poly_ok) {
       groups[GKey(ALGO_GATHER, k.shape, c->g.KB, f16, k.chunk, 0, 0, 0.f, 0.f)].push_back(b);
@@ -179,7 +179,7 @@ int build_plan(Plan &pl, fr_ctx *const *ctxs, const void *const *images, const i
     };
     auto fold_loads = [&](const fr_ctx *c, int nn, double target, std::vector<UnitLoad> &out,
                           int &split) {
-      return brick_unit_loads(c, fold_shape(), c->g.xa0, -c->g.xa0, nn, target, FOLD_UNITS_PER_SM,
+      return brick_unit_loads(c, fold_shape(c->g.KB), c->g.xa0, -c->g.xa0, nn, target, FOLD_UNITS_PER_SM,
                               out, split);
     };
     // pooled splitting target of the main items: total expected load over
@@ -368,7 +368,7 @@ int prime_plan(const Plan &pl, fr_ctx *const *ctxs, const int *dtypes, const std
     if (e != cudaSuccess) return cuda_err(e);
   }
   for (int b : pl.sequential) {
-    const Config &k = config_space()[cfg[b]];
+    const Config k = effective_config(ctxs[b], cfg[b]);
     InsertArgs a = base_args(ctxs[b]);
     a.f16 = dtypes[b] == FR_F16;
     a.chunk = k.chunk;

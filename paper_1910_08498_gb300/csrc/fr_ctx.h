@@ -67,6 +67,8 @@ InsertArgs base_args(const fr_ctx *c);
 int ensure_scratch(fr_ctx *c);
 // create the context's side stream and fork/join events if it has none yet
 int ensure_side_stream(fr_ctx *c);
+// configuration id as this context runs it (its kernel family)
+Config effective_config(const fr_ctx *c, int id);
 // gather work unit with its expected load (images it scans)
 struct UnitLoad {
   double load;

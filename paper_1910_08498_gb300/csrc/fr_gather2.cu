@@ -89,7 +89,7 @@ cudaError_t launch_multi(const void *fn, const MultiLaunch &p, int per_item, int
 
 size_t gather2_smem_bytes(const GatherShape &sh, int chunk) {
   (void)sh;  // one warp per CTA
-  return gather2_warp_smem<8, 0>(chunk);
+  return gather2_warp_smem<8, 4, 0>(chunk);
 }
 
 // brick shapes: columns in x, columns in y, voxels per column (z)
@@ -114,7 +114,7 @@ cudaError_t launch_gather2_multi_shape2(int minw, int f16, const MultiLaunch &p,
 
 cudaError_t launch_gather2_multi(int shape_id, int minw, int f16, const MultiLaunch &p,
                                  cudaStream_t st) {
-  if (p.base.chunk > 64 || p.base.g.KB != 4) return cudaErrorInvalidValue;
+  if (p.base.chunk > 128) return cudaErrorInvalidValue;
   switch (shape_id) {
     case 0: return launch_gather2_multi_shape0(minw, f16, p, st);
     case 1: return launch_gather2_multi_shape1(minw, f16, p, st);
@@ -125,8 +125,8 @@ cudaError_t launch_gather2_multi(int shape_id, int minw, int f16, const MultiLau
 
 cudaError_t launch_gather2(int shape_id, int minw, const InsertArgs &a, cudaStream_t st,
                            int query_only, KernelInfo *info) {
-  if (a.g.KB != 4 || a.chunk > 64) return cudaErrorInvalidValue;
-  // two-pixel row loads: the images must be 16-byte aligned (fr_insert checks it)
+  if (a.chunk > 128) return cudaErrorInvalidValue;
+  // pixel copies of eight bytes: fr_insert checks for 16-byte aligned images
   if (reinterpret_cast<uintptr_t>(a.images) & 15u) return cudaErrorInvalidValue;
   switch (shape_id) {
     case 0: return launch_gather2_shape0(minw, a, st, query_only, info);

@@ -17,9 +17,10 @@
 //    8-bit tag per item (column, z level) at positions from a warp scan;
 //  * evaluation: 32 items a round, one per lane: u = R^T v from the footprint
 //    centre's compensated projection, the 4 x 4 candidate box at rint(u - 1.5)
-//    (it covers [u - a, u + a] for every a < 2), clamped into the patch (rows
-//    and columns moved in by the clamp lie outside the blob and are masked), its
-//    16 pixels from the patch, the Chebyshev weight polynomial in
+//    (it covers [u - a, u + a] for every a < 2; for 2 <= a < 3 the 6 x 6 box at
+//    rint(u - 2.5)), clamped into the patch (rows and columns moved in by the
+//    clamp lie outside the blob and are masked), its pixels from the patch, the
+//    Chebyshev weight polynomial in
 //    x = 2 r^2 / a^2 - 1 for two candidates at a time with packed FP32x2 FMAs
 //    (masked to 0 outside r <= a), and the complex and weight sums added to the
 //    voxel's partial sums with plain loads and stores: the items of one entry
@@ -48,7 +49,7 @@
 // that three of four lanes hold fold columns: there a stored pixel k counts in
 // the entry as stored when it is not folded and in the reflected entry when it
 // is (exact sign of R00 k_x + R01 k_y, found once per pixel of the patch and
-// kept as one bit).  Polynomial weights only, 4 x 4 boxes only (a < 2).
+// kept as one bit).  Polynomial weights only.
 #pragma once
 
 #include "fr_gather.cuh"
@@ -58,27 +59,31 @@ namespace fr {
 constexpr int G2_ENTRIES = 16;  // records built and processed at a time
 constexpr int G2_REC = 16;      // floats of a record
 
-// Geometry of the warp footprint FW x 8 x 8 and of its pixel patches.
-template <int FW>
+// Geometry of the warp footprint FW x 8 x 8 and of its pixel patches, for
+// KB x KB candidate boxes (KB = 4: a < 2, KB = 6: a < 3).
+template <int FW, int KB>
 struct G2Shape {
   static constexpr int FH = 8, ZC = 8;
   static constexpr int NC = FW * FH / 32;               // columns per lane
   static constexpr int WV = FW * FH * ZC;               // voxels
   static constexpr float HX = 0.5f * (FW - 1), HY = 0.5f * (FH - 1), HZ = 0.5f * (ZC - 1);
-  // a box reaches 2 pixels past u, and u lies within the footprint's radius
-  // (6.07; 5.17 for FW = 4) of the centre: at most 17 (15) columns
-  static constexpr int PW = FW == 8 ? 17 : 15;          // patch columns and rows
+  // a box reaches KB / 2 pixels past u, and u lies within the footprint's
+  // radius (6.07; 5.17 for FW = 4) of the centre: at most 17 (KB = 6: 19;
+  // FW = 4: 15) columns
+  static constexpr int PW = (FW == 8 ? 13 : 11) + KB;   // patch columns and rows
+  static constexpr int XC = PW > 16 ? PW - 16 : 0;      // columns past the first 16
   static constexpr int PITCH = 20;                      // = 4 modulo 16 eight-byte banks
   static constexpr int PATCH = PW * PITCH;              // pixels of a patch
+  static_assert(PW <= PITCH && (XC == 0 || XC == 1 || XC == 3), "patch rows");
 };
 
 // Per-warp shared memory: records, partial sums, patches, image list, fold
 // bits, tags.
-template <int FW, int FOLD>
+template <int FW, int KB, int FOLD>
 __host__ __device__ constexpr size_t gather2_warp_smem(int chunk) {
-  using SH = G2Shape<FW>;
+  using SH = G2Shape<FW, KB>;
   return ((size_t)G2_REC * G2_ENTRIES * 4 + (size_t)3 * SH::WV * 4 + (size_t)2 * SH::PATCH * 8 +
-          (size_t)chunk * 4 + (FOLD ? (size_t)2 * 16 * 4 : 0) + (size_t)(SH::WV + 32) + 15) &
+          (size_t)chunk * 4 + (FOLD ? (size_t)2 * SH::PITCH * 4 : 0) + (size_t)(SH::WV + 32) + 15) &
          ~(size_t)15;
 }
 
@@ -87,62 +92,100 @@ __device__ __forceinline__ void cp_async8(uint32_t dst, const void *src) {
 }
 __device__ __forceinline__ void cp_async_wait_all() { asm volatile("cp.async.wait_all;" ::: "memory"); }
 
-// The 4 x 4 box of an item: pixels p[l * PITCH + j], u at (dx, dy) from pixel
+// Candidates of a fold column's box within rounding of the blob edge (FP32 r^2
+// within 1e-5 a^2 of a^2), decided as the real numbers do: with a lattice
+// distance a (a = 2, or a signed permutation for the rotation) the DC pixel
+// and others sit there for every image.  k0: the box's first stored pixel.
+template <int PITCH, int KB>
+__device__ __noinline__ void g2_ties(const float2 *cp, const float2 *p, float dx, float dy,
+                                     float uz2, float cs, const unsigned *rows, int shift,
+                                     const float4 e1, const float4 e2, int3 v, int2 k0, float a,
+                                     float &ar, float &ai, float &aw) {
+  for (int r = 0; r < KB; ++r)
+    for (int j = 0; j < KB; ++j) {
+      const float ex = dx - (float)j, ey = dy - (float)r;
+      const float x = fmaf(cs, fmaf(ex, ex, fmaf(ey, ey, uz2)), -1.0f);
+      if (fabsf(x - 1.0f) > 2e-5f || !((rows[r] >> (shift + j)) & 1u) ||
+          !exact_r2_le_a2(v.x, v.y, v.z, e1.x, e1.y, e1.z, e2.x, e2.y, e2.z, k0.x + j, k0.y + r, a))
+        continue;
+      float w = cp[POLY_N - 1].x;
+      for (int k = POLY_N - 2; k >= 0; --k) w = fmaf(w, fminf(x, 1.0f), cp[k].x);
+      const float2 q = p[r * PITCH + j];
+      ar = fmaf(w, q.x, ar);
+      ai = fmaf(w, q.y, ai);
+      aw += w;
+    }
+}
+
+// The KB x KB box of an item: pixels p[l * PITCH + j], u at (dx, dy) from pixel
 // (0, 0), u_z^2 = uz2; returns the sums of w p (complex) and of w over the
 // candidates with r <= a.  FOLD: candidate (j, l) counts only if bit j of
-// rows[l] >> shift is set.
-template <int PITCH, int FOLD>
-__device__ __forceinline__ void g2_box(const float2 *cp, const float2 *p, float dx, float dy,
+// rows[l] >> shift is set; with KB = 6 (a >= 2) candidates within rounding of
+// the blob edge are left out, and whether there are any is returned (g2_ties).
+template <int PITCH, int KB, int FOLD>
+__device__ __forceinline__ bool g2_box(const float2 *cp, const float2 *p, float dx, float dy,
                                        float uz2, float cs, float sq, float &ar, float &ai,
                                        float &aw, const unsigned *rows, int shift) {
-  constexpr int NP = POLY_N;
+  constexpr int NP = POLY_N, KP = KB / 2, RP = KB == 4 ? 4 : 3;
   // cp: coefficient pairs (c_k, c_k), kernel-parameter constants
   // scaled column offsets sq (dx - j): x = (sq dx)^2 + cs (dy^2 + u_z^2) - 1
   const float2 S2 = make_float2(sq, sq), C2 = make_float2(cs, cs);
   const float2 DX = make_float2(dx, dx), DY = make_float2(dy, dy);
-  const float2 d01 = __fmul2_rn(__fadd2_rn(DX, make_float2(0.0f, -1.0f)), S2);
-  const float2 d23 = __fmul2_rn(__fadd2_rn(DX, make_float2(-2.0f, -3.0f)), S2);
+  float2 d[KP];
+#pragma unroll
+  for (int j = 0; j < KP; ++j)
+    d[j] = __fmul2_rn(__fadd2_rn(DX, make_float2(-2.0f * j, -2.0f * j - 1.0f)), S2);
   const float U = fmaf(cs, uz2, -1.0f);
   const float2 UU = make_float2(U, U);
-  // all 16 polynomials advance together: eight independent chains of packed
-  // FMAs (row by row, two chains, the FMA pipe waits for their latency)
-  float2 x[8], h[8];
-#pragma unroll
-  for (int r = 0; r < 4; ++r) {
-    const float2 EY = r ? __fadd2_rn(DY, make_float2(-(float)r, -(float)r)) : DY;
-    const float2 YY = __ffma2_rn(__fmul2_rn(C2, EY), EY, UU);
-    x[2 * r] = __ffma2_rn(d01, d01, YY);
-    x[2 * r + 1] = __ffma2_rn(d23, d23, YY);
-  }
-#pragma unroll
-  for (int i = 0; i < 8; ++i) h[i] = __ffma2_rn(cp[NP - 1], x[i], cp[NP - 2]);
-#pragma unroll
-  for (int k = NP - 3; k >= 0; --k)
-#pragma unroll
-    for (int i = 0; i < 8; ++i) h[i] = __ffma2_rn(h[i], x[i], cp[k]);
   ar = 0.f;
   ai = 0.f;
   aw = 0.f;
+  bool ties = false;
 #pragma unroll
-  for (int r = 0; r < 4; ++r) {
-    const float2 p0 = p[r * PITCH], p1 = p[r * PITCH + 1], p2 = p[r * PITCH + 2],
-                 p3 = p[r * PITCH + 3];
-    bool i0 = x[2 * r].x <= 1.0f, i1 = x[2 * r].y <= 1.0f, i2 = x[2 * r + 1].x <= 1.0f,
-         i3 = x[2 * r + 1].y <= 1.0f;
-    if (FOLD) {
-      const unsigned m = rows[r] >> shift;
-      i0 = i0 && (m & 1u);
-      i1 = i1 && (m & 2u);
-      i2 = i2 && (m & 4u);
-      i3 = i3 && (m & 8u);
+  for (int r0 = 0; r0 < KB; r0 += RP) {
+    // all polynomials of RP rows advance together: eight or nine independent
+    // chains of packed FMAs (row by row the FMA pipe waits for their latency).
+    // With a constant as its third operand a packed FMA runs at the full rate
+    // (74 TFLOP/s measured; with three register pairs 44).
+    float2 x[RP * KP], h[RP * KP];
+#pragma unroll
+    for (int r = 0; r < RP; ++r) {
+      const float2 EY = r0 + r ? __fadd2_rn(DY, make_float2(-(float)(r0 + r), -(float)(r0 + r))) : DY;
+      const float2 YY = __ffma2_rn(__fmul2_rn(C2, EY), EY, UU);
+#pragma unroll
+      for (int j = 0; j < KP; ++j) x[r * KP + j] = __ffma2_rn(d[j], d[j], YY);
     }
-    // predicated accumulation: no select, and no pixel outside the blob is used
-    const float2 wa = h[2 * r], wb = h[2 * r + 1];
-    if (i0) { ar = fmaf(wa.x, p0.x, ar); ai = fmaf(wa.x, p0.y, ai); aw += wa.x; }
-    if (i1) { ar = fmaf(wa.y, p1.x, ar); ai = fmaf(wa.y, p1.y, ai); aw += wa.y; }
-    if (i2) { ar = fmaf(wb.x, p2.x, ar); ai = fmaf(wb.x, p2.y, ai); aw += wb.x; }
-    if (i3) { ar = fmaf(wb.y, p3.x, ar); ai = fmaf(wb.y, p3.y, ai); aw += wb.y; }
+#pragma unroll
+    for (int i = 0; i < RP * KP; ++i) h[i] = __ffma2_rn(cp[NP - 1], x[i], cp[NP - 2]);
+#pragma unroll
+    for (int k = NP - 3; k >= 0; --k)
+#pragma unroll
+      for (int i = 0; i < RP * KP; ++i) h[i] = __ffma2_rn(h[i], x[i], cp[k]);
+#pragma unroll
+    for (int r = 0; r < RP; ++r) {
+      const unsigned m = FOLD ? rows[r0 + r] >> shift : 0u;
+#pragma unroll
+      for (int j = 0; j < KB; ++j) {
+        const float2 xx = x[r * KP + j / 2], hh = h[r * KP + j / 2];
+        const float xv = j & 1 ? xx.y : xx.x, w = j & 1 ? hh.y : hh.x;
+        const float2 q = p[(r0 + r) * PITCH + j];
+        bool in = xv <= 1.0f;
+        if (FOLD) in = in && ((m >> j) & 1u);
+        if (FOLD && KB == 6) {
+          const bool tie = fabsf(xv - 1.0f) <= 2e-5f;
+          ties = ties || tie;
+          in = in && !tie;
+        }
+        // predicated accumulation: no select, and no pixel outside the blob is used
+        if (in) {
+          ar = fmaf(w, q.x, ar);
+          ai = fmaf(w, q.y, ai);
+          aw += w;
+        }
+      }
+    }
   }
+  return ties;
 }
 
 // Fold a warp's partial sums (s_acc: [3][WV], slot (y FW + x) 8 + z) into HBM
@@ -151,10 +194,10 @@ __device__ __forceinline__ void g2_box(const float2 *cp, const float2 *p, float 
 // scratch with atomics (merged after the launch).  The loads of four z levels
 // are issued together: one after the other, their latency made a flush take
 // four times as long.
-template <int FW>
+template <int FW, int KB>
 __device__ __noinline__ void g2_flush(const InsertArgs &args, float *s_acc, int fx0, int fy0,
                                       int z0, bool to_scratch) {
-  using SH = G2Shape<FW>;
+  using SH = G2Shape<FW, KB>;
   constexpr int WV = SH::WV, ZC = SH::ZC, ZG = 4;
   const Geom &g = args.g;
   const int lane = threadIdx.x & 31;
@@ -216,16 +259,16 @@ __host__ __device__ constexpr int g2_warps() {
 // in the inner loops.  FOLD = 0: the bricks tile x >= floor(a) + 1; FOLD = 1:
 // they tile x >= -floor(a) and only the fold columns |x| <= floor(a) are
 // computed, with the fold predicate tested per candidate.
-template <int BX, int BY, int BZ, int F16, int FW = 8, int FOLD = 0>
+template <int BX, int BY, int BZ, int F16, int KB = 4, int FW = 8, int FOLD = 0>
 __device__ __forceinline__ void gather2_warp(const InsertArgs &args, const InsertArgs &cst,
                                              const void *images, unsigned char *wsmem,
                                              const int4 unit, const int warp) {
-  using SH = G2Shape<FW>;
+  using SH = G2Shape<FW, KB>;
   constexpr int FH = SH::FH, ZC = SH::ZC, WV = SH::WV, PW = SH::PW, PITCH = SH::PITCH,
-                NC = SH::NC;
+                NC = SH::NC, XC = SH::XC;
   static_assert((FW == 8 || FW == 4) && BX % FW == 0 && BY % FH == 0 && BZ % ZC == 0,
                 "warp footprints are 8 x 8 x 8 or 4 x 8 x 8 voxels");
-  static_assert(PW <= 17 && PW <= PITCH && (!FOLD || PW <= 16), "patch rows");
+  constexpr float HB = 0.5f * KB;  // a box reaches HB pixels past u
   constexpr int ESZ = F16 ? 4 : 8;
   constexpr float HX = SH::HX, HY = SH::HY, HZ = SH::HZ;
   constexpr unsigned FULL = 0xffffffffu;
@@ -237,7 +280,7 @@ __device__ __forceinline__ void gather2_warp(const InsertArgs &args, const Inser
   const int fy0 = -g.H + unit.y * BY + wy * FH;
   const int z0 = -g.H + unit.z * BZ + wz * ZC;
   const int lcap = cst.chunk;
-  if (lcap < 32 || lcap > 64) {  // the image list holds lcap entries
+  if (lcap < 32 || lcap > 128) {  // the image list holds lcap entries
     if (lane == 0) set_err(args.err, DERR_RANGE);
     return;
   }
@@ -246,8 +289,8 @@ __device__ __forceinline__ void gather2_warp(const InsertArgs &args, const Inser
   float *s_acc = reinterpret_cast<float *>(s_rec + G2_REC / 4 * G2_ENTRIES);        // [3][WV]
   float2 *s_patch = reinterpret_cast<float2 *>(s_acc + 3 * WV);                     // [2][PATCH]
   int *s_idx = reinterpret_cast<int *>(s_patch + 2 * SH::PATCH);                    // [lcap]
-  unsigned *s_bits = reinterpret_cast<unsigned *>(s_idx + lcap);                    // FOLD: [2][16]
-  unsigned char *s_tag = reinterpret_cast<unsigned char *>(s_bits + (FOLD ? 32 : 0));  // [WV + 32]
+  unsigned *s_bits = reinterpret_cast<unsigned *>(s_idx + lcap);                    // FOLD: [2][PITCH]
+  unsigned char *s_tag = reinterpret_cast<unsigned char *>(s_bits + (FOLD ? 2 * PITCH : 0));  // [WV + 32]
 
   const int split = unit.w & 0xffff, nsplit = (unit.w >> 16) & 0x3fff;
   const bool to_scratch = nsplit > 1 || ((unit.w >> 30) & 1);
@@ -340,14 +383,14 @@ __device__ __forceinline__ void gather2_warp(const InsertArgs &args, const Inser
           const int ccx = h ? -cxi : cxi, ccy = h ? -cyi : cyi;
           // pixels that the boxes can reach, inside the stored half plane [0, H]
           // x [-H, H - 1]; at least one whole box, at most PW x PW
-          const float far = 4096.0f, wx_ = sx + 2.01f, wy_ = sy + 2.01f;
+          const float far = 4096.0f, wx_ = sx + (HB + 0.01f), wy_ = sy + (HB + 0.01f);
           const int lox = ccx + (int)fminf(fmaxf(ceilf(ffx - wx_), -far), far);
           const int hix = ccx + (int)fminf(fmaxf(floorf(ffx + wx_), -far), far);
           const int loy = ccy + (int)fminf(fmaxf(ceilf(ffy - wy_), -far), far);
           const int hiy = ccy + (int)fminf(fmaxf(floorf(ffy + wy_), -far), far);
           const int px = max(0, min(lox, g.H + 1 - PW)), py = max(-g.H, min(loy, g.H - PW));
-          const int pw = min(max(min(hix, g.H) - px + 1, 4), min(PW, g.H + 1 - px));
-          const int ph = min(max(min(hiy, g.H - 1) - py + 1, 4), min(PW, g.H - py));
+          const int pw = min(max(min(hix, g.H) - px + 1, KB), min(PW, g.H + 1 - px));
+          const int ph = min(max(min(hiy, g.H - 1) - py + 1, KB), min(PW, g.H - py));
           const int rpx = max(-127, min(px - ccx, 127)), rpy = max(-127, min(py - ccy, 127));
           s_rec[o * 4 + 0] = make_float4(mx, my, mz, uz);
           s_rec[o * 4 + 1] = make_float4(sg * e1x, sg * e1y, sg * e1z, ffx);
@@ -364,11 +407,12 @@ __device__ __forceinline__ void gather2_warp(const InsertArgs &args, const Inser
   };
 
   // Patch copies: 16 columns x 2 rows a step (rows past the patch repeat its
-  // last row), then column 16.
-  constexpr int RG = (PW + 1) / 2;
+  // last row), then the columns past 16 (4 of them x 8 rows a step, or one).
+  constexpr int RG = (PW + 1) / 2, XL = XC == 3 ? 4 : 1, XR = XC == 0 ? 0 : (PW * XL + 31) / 32;
+  const int xc = lane % XL, xr = lane / XL;
   const int pc = lane & 15, pr = lane >> 4;
   const int row_bytes = g.NX * ESZ;
-  __half2 stage[F16 ? RG + 1 : 1];
+  __half2 stage[F16 ? RG + XR : 1];
   // start copying the patch of entry li (FP32: into its patch; FP16: into registers)
   auto fetch = [&](int li) {
     const int4 q = reinterpret_cast<const int4 *>(s_rec)[li * 4 + 3];
@@ -395,12 +439,16 @@ __device__ __forceinline__ void gather2_warp(const InsertArgs &args, const Inser
         else if (2 * r + 1 < PW || pr == 0) cp_async8(dst + 2 * r * PITCH * 8, src);
       }
     }
-    if (PW > 16 && pw > 16) {
-      const int ky = py + min(lane, ph1);
-      const unsigned char *src = img + (ky + (ky < 0 ? g.S : 0)) * row_bytes + 16 * ESZ;
-      if (F16) stage[RG] = __ldg(reinterpret_cast<const __half2 *>(src));
-      else if (lane < PW)
-        cp_async8(dst + (lane * PITCH + 16 - pr * PITCH - pc) * 8, src);
+    if (XC > 0 && pw > 16) {
+      const int cx = min(16 + xc, pw - 1) - 16;
+#pragma unroll
+      for (int k = 0; k < XR; ++k) {
+        const int row = xr + k * (32 / XL), ky = py + min(row, ph1);
+        const unsigned char *src = img + (ky + (ky < 0 ? g.S : 0)) * row_bytes + (16 + cx) * ESZ;
+        if (F16) stage[RG + k] = __ldg(reinterpret_cast<const __half2 *>(src));
+        else if (row < PW && xc < XC)
+          cp_async8(dst + (row * PITCH + 16 + xc - pr * PITCH - pc) * 8, src);
+      }
     }
   };
   // FP16: convert the staged pixels into entry li's patch
@@ -409,8 +457,14 @@ __device__ __forceinline__ void gather2_warp(const InsertArgs &args, const Inser
 #pragma unroll
     for (int r = 0; r < RG; ++r)
       if (2 * r + 1 < PW || pr == 0) dst[2 * r * PITCH] = __half22float2(stage[r]);
-    if (PW > 16 && pw > 16 && lane < PW)
-      dst[lane * PITCH + 16 - pr * PITCH - pc] = __half22float2(stage[RG]);
+    if (XC > 0 && pw > 16) {
+#pragma unroll
+      for (int k = 0; k < XR; ++k) {
+        const int row = xr + k * (32 / XL);
+        if (row < PW && xc < XC)
+          dst[row * PITCH + 16 + xc - pr * PITCH - pc] = __half22float2(stage[RG + k]);
+      }
+    }
   };
 
   // one entry: its items, then their rounds
@@ -420,8 +474,8 @@ __device__ __forceinline__ void gather2_warp(const InsertArgs &args, const Inser
     const int4 q3 = reinterpret_cast<const int4 *>(s_rec)[li * 4 + 3];
     const int rpx = (int)(signed char)(q3.x & 255), rpy = (int)(signed char)((q3.x >> 8) & 255);
     const int pw = (q3.x >> 16) & 255, ph = (int)((unsigned)q3.x >> 24);
-    const float lox = (float)rpx, hix = (float)(rpx + pw - 4);
-    const float loy = (float)rpy, hiy = (float)(rpy + ph - 4);
+    const float lox = (float)rpx, hix = (float)(rpx + pw - KB);
+    const float loy = (float)rpy, hiy = (float)(rpy + ph - KB);
     const float2 *patch = s_patch + (li & 1) * SH::PATCH;
     if (F16) {
       land(li, pw);
@@ -442,7 +496,7 @@ __device__ __forceinline__ void gather2_warp(const InsertArgs &args, const Inser
           if (fold_pred(r00, r01, px + t + s - 1, py + lane) != up) t += s;
         const unsigned before = t > 30 ? 0x7fffffffu : (1u << t) - 1u;
         const unsigned folded = up ? ~before : before;
-        s_bits[(li & 1) * 16 + lane] = refl ? folded : ~folded;
+        s_bits[(li & 1) * PITCH + lane] = refl ? folded : ~folded;
       }
     }
     // z levels t of each column with |u_z| <= a, u_z = b + m_z t: t within a /
@@ -526,19 +580,25 @@ __device__ __forceinline__ void gather2_warp(const InsertArgs &args, const Inser
       const float uz = fmaf(q0.z, sdz, fmaf(q0.y, sdy, fmaf(q0.x, sdx, q0.w)));
       const float ux = fmaf(q1.z, sdz, fmaf(q1.y, sdy, fmaf(q1.x, sdx, q1.w)));
       const float uy = fmaf(q2.z, sdz, fmaf(q2.y, sdy, fmaf(q2.x, sdx, q2.w)));
-      // box origin: the nearest integer to u - 1.5 (by adding 1.5 2^23), clamped
-      const float ox = fminf(fmaxf(__fadd_rn(__fadd_rn(ux - 1.5f, kR), -kR), lox), hix);
-      const float oy = fminf(fmaxf(__fadd_rn(__fadd_rn(uy - 1.5f, kR), -kR), loy), hiy);
+      // box origin: the nearest integer to u - 1.5 (2.5; by adding 1.5 2^23), clamped
+      constexpr float HO = HB - 0.5f;
+      const float ox = fminf(fmaxf(__fadd_rn(__fadd_rn(ux - HO, kR), -kR), lox), hix);
+      const float oy = fminf(fmaxf(__fadd_rn(__fadd_rn(uy - HO, kR), -kR), loy), hiy);
       const unsigned at = __float_as_uint(fmaf(oy, (float)PITCH, __fadd_rn(ox, kR))) + base;
       const unsigned *rows = s_bits;
       int shift = 0;
       if (FOLD) {
         shift = (int)(ox - lox);
-        rows += (li & 1) * 16 + (int)(oy - loy);
+        rows += (li & 1) * PITCH + (int)(oy - loy);
       }
       float ar, ai, aw;
-      g2_box<PITCH, FOLD>(cst.poly2, patch + at, ux - ox, uy - oy, uz * uz, cs, sq, ar, ai, aw,
-                          rows, shift);
+      const bool ties = g2_box<PITCH, KB, FOLD>(cst.poly2, patch + at, ux - ox, uy - oy, uz * uz, cs,
+                                                sq, ar, ai, aw, rows, shift);
+      if (FOLD && KB == 6 && ties)
+        g2_ties<PITCH, KB>(cst.poly2, patch + at, ux - ox, uy - oy, uz * uz, cs, rows, shift, q1,
+                           q2, make_int3(fx0 + (slot / ZC) % FW, fy0 + slot / (ZC * FW), z0 + slot % ZC),
+                           make_int2((q3.y & 0xffff) + shift, (q3.y >> 16) + (int)(oy - loy)), g.a, ar,
+                           ai, aw);
       if (h < total) {
         s_acc[slot] = tr + ar;
         s_acc[WV + slot] = fmaf(sgn, ai, ti);
@@ -590,9 +650,9 @@ __device__ __forceinline__ void gather2_warp(const InsertArgs &args, const Inser
       }
       since_flush += nl;
       nl = 0;
-      if (since_flush > GATHER_FLUSH - 64) {
+      if (since_flush > GATHER_FLUSH - lcap) {
         const long long tf = tick();
-        g2_flush<FW>(args, s_acc, fx0, fy0, z0, to_scratch);
+        g2_flush<FW, KB>(args, s_acc, fx0, fy0, z0, to_scratch);
         clocked(PH_FLUSH, tf);
         since_flush = 0;
       }
@@ -600,7 +660,7 @@ __device__ __forceinline__ void gather2_warp(const InsertArgs &args, const Inser
     if (last) break;
   }
   const long long tf = tick();
-  if (since_flush) g2_flush<FW>(args, s_acc, fx0, fy0, z0, to_scratch);
+  if (since_flush) g2_flush<FW, KB>(args, s_acc, fx0, fy0, z0, to_scratch);
   clocked(PH_FLUSH, tf);
   clocked(PH_WARP_CYCLES, t_start);
 }
@@ -612,12 +672,12 @@ __device__ __forceinline__ void gather2_warp(const InsertArgs &args, const Inser
 // the register allocation must allow (16: at most 128 registers per thread, and
 // what shared memory holds; more warps than that are not resident).  FW, FOLD:
 // see gather2_warp.
-template <int BX, int BY, int BZ, int F16, int MINW, int FW = 8, int FOLD = 0>
+template <int BX, int BY, int BZ, int F16, int MINW, int KB = 4, int FW = 8, int FOLD = 0>
 __global__ void __launch_bounds__(32, MINW)
 gather2_kernel(const __grid_constant__ InsertArgs args) {
   extern __shared__ __align__(16) unsigned char smem[];
   constexpr int W = g2_warps<BX, BY, BZ, FW>();
-  gather2_warp<BX, BY, BZ, F16, FW, FOLD>(args, args, args.images, smem,
+  gather2_warp<BX, BY, BZ, F16, KB, FW, FOLD>(args, args, args.images, smem,
                                           args.units[blockIdx.x / W], (int)(blockIdx.x % W));
 }
 
@@ -627,14 +687,14 @@ gather2_kernel(const __grid_constant__ InsertArgs args) {
 // launch's batches, are read from p.base (kernel parameters: constant operands
 // in the inner loops), the batch's own arguments (rotations, volume) from its
 // descriptor.
-template <int BX, int BY, int BZ, int F16, int MINW, int FW = 8, int FOLD = 0>
+template <int BX, int BY, int BZ, int F16, int MINW, int KB = 4, int FW = 8, int FOLD = 0>
 __global__ void __launch_bounds__(32, MINW)
 gather2_multi_kernel(const __grid_constant__ MultiLaunch p) {
   extern __shared__ __align__(16) unsigned char smem[];
   constexpr int W = g2_warps<BX, BY, BZ, FW>();
   const int4 it = p.items[blockIdx.x / W];
   const int4 unit = make_int4(it.x & 1023, (it.x >> 10) & 1023, (it.x >> 20) & 1023, it.y);
-  gather2_warp<BX, BY, BZ, F16, FW, FOLD>(p.descs[it.z], p.base, p.images[it.w], smem, unit,
+  gather2_warp<BX, BY, BZ, F16, KB, FW, FOLD>(p.descs[it.z], p.base, p.images[it.w], smem, unit,
                                           (int)(blockIdx.x % W));
 }
 

@@ -3,4 +3,5 @@
 #define FR2_BX 16
 #define FR2_BY 16
 #define FR2_ZC 8
+#define FR2_WIDE
 #include "fr_gather2_launch.inc"

@@ -1,7 +1,7 @@
 // fr_gather_fold.cu -- the direct-drain gather instantiated for the fold
-// columns |x| <= floor(a) (FOLD): bricks one 4-column footprint wide
-// (4 x 32 x 8, four 4 x 8 x 8 warp footprints stacked in y), the fold predicate
-// tested per pixel, 4 x 4 boxes (a < 2), polynomial weights.  Launched
+// columns |x| <= floor(a) (FOLD): bricks one footprint wide, 4 columns (8 for
+// 2 <= a < 3) x 32 x 8, four warp footprints stacked in y, the fold predicate
+// tested per pixel, polynomial weights.  Launched
 // beside the main direct-drain launch, which covers x >= floor(a) + 1: for one
 // batch, or for the work items of several batches in one launch.
 #include "fr_gather2.cuh"
@@ -9,44 +9,49 @@
 namespace fr {
 
 namespace {
-constexpr int FBX = 4, FBY = 32, FZC = 8, FFW = 4;
+constexpr int FBY = 32, FZC = 8;
 constexpr int FOLD_MINW = 16;  // resident warps per SM the registers allow
-constexpr int FOLD_WARPS = g2_warps<FBX, FBY, FZC, FFW>();
-constexpr size_t fold_smem(int chunk) { return gather2_warp_smem<FFW, 1>(chunk); }
+// three fold columns for a < 2 (a footprint 4 wide), five for 2 <= a < 3
+template <int KB>
+constexpr int fold_width() { return KB == 4 ? 4 : 8; }
 }  // namespace
 
-GatherShape fold_shape() { return GatherShape{FBX, FBY, FZC}; }
+GatherShape fold_shape(int kb) { return GatherShape{kb == 4 ? fold_width<4>() : fold_width<6>(), FBY, FZC}; }
 
-template <int F16>
+template <int F16, int KB>
 static cudaError_t launch_fold(const InsertArgs &a, cudaStream_t st) {
-  auto fn = gather2_kernel<FBX, FBY, FZC, F16, FOLD_MINW, FFW, 1>;
-  const size_t smem = fold_smem(a.chunk);
+  constexpr int FW = fold_width<KB>();
+  auto fn = gather2_kernel<FW, FBY, FZC, F16, FOLD_MINW, KB, FW, 1>;
+  const size_t smem = gather2_warp_smem<FW, KB, 1>(a.chunk);
   cudaError_t e = allow_dynamic_smem((const void *)fn, smem);
   if (e != cudaSuccess) return e;
   if (a.nunits <= 0) return cudaSuccess;
-  fn<<<a.nunits * FOLD_WARPS, 32, smem, st>>>(a);
+  fn<<<a.nunits * g2_warps<FW, FBY, FZC, FW>(), 32, smem, st>>>(a);
   return cudaGetLastError();
 }
 
-template <int F16>
+template <int F16, int KB>
 static cudaError_t launch_fold_multi(const MultiLaunch &p, cudaStream_t st) {
-  auto fn = gather2_multi_kernel<FBX, FBY, FZC, F16, FOLD_MINW, FFW, 1>;
-  const size_t smem = fold_smem(p.base.chunk);
+  constexpr int FW = fold_width<KB>();
+  auto fn = gather2_multi_kernel<FW, FBY, FZC, F16, FOLD_MINW, KB, FW, 1>;
+  const size_t smem = gather2_warp_smem<FW, KB, 1>(p.base.chunk);
   cudaError_t e = allow_dynamic_smem((const void *)fn, smem);
   if (e != cudaSuccess) return e;
   if (p.nitems <= 0) return cudaSuccess;
-  return launch_multi((const void *)fn, p, FOLD_WARPS, 32, smem, st);
+  return launch_multi((const void *)fn, p, g2_warps<FW, FBY, FZC, FW>(), 32, smem, st);
 }
 
 cudaError_t launch_gather_fold_multi(int f16, const MultiLaunch &p, cudaStream_t st) {
-  if (p.base.g.KB != 4 || p.base.chunk > 64) return cudaErrorInvalidValue;
-  return f16 ? launch_fold_multi<1>(p, st) : launch_fold_multi<0>(p, st);
+  if (p.base.chunk > 128) return cudaErrorInvalidValue;
+  if (p.base.g.KB == 4) return f16 ? launch_fold_multi<1, 4>(p, st) : launch_fold_multi<0, 4>(p, st);
+  return f16 ? launch_fold_multi<1, 6>(p, st) : launch_fold_multi<0, 6>(p, st);
 }
 
 cudaError_t launch_gather_fold(const InsertArgs &a, cudaStream_t st) {
-  if (a.g.KB != 4 || a.chunk > 64) return cudaErrorInvalidValue;
+  if (a.chunk > 128) return cudaErrorInvalidValue;
   if (reinterpret_cast<uintptr_t>(a.images) & 15u) return cudaErrorInvalidValue;
-  return a.f16 ? launch_fold<1>(a, st) : launch_fold<0>(a, st);
+  if (a.g.KB == 4) return a.f16 ? launch_fold<1, 4>(a, st) : launch_fold<0, 4>(a, st);
+  return a.f16 ? launch_fold<1, 6>(a, st) : launch_fold<0, 6>(a, st);
 }
 
 }  // namespace fr

@@ -126,8 +126,8 @@ cudaError_t launch_debug_blob(const InsertArgs &a, const float *r2, int m, int m
 int num_gather_shapes();
 GatherShape gather_shape(int id);
 // the direct-drain gather over the fold columns |x| <= floor(a) only, in
-// bricks of fold_shape() (one 4-column footprint wide), polynomial weights
-GatherShape fold_shape();
+// bricks of fold_shape(KB) (one footprint wide), polynomial weights
+GatherShape fold_shape(int kb);
 cudaError_t launch_gather_fold(const InsertArgs &a, cudaStream_t st);
 // dynamic shared memory a gather launch needs
 size_t gather_smem_bytes(const GatherShape &sh, int wmode, int lut_n, int chunk);

@@ -192,6 +192,23 @@ double gather_unit_loads(const fr_ctx *c, int shape, int n, double target,
                           any_split);
 }
 
+// The kernel family a configuration runs with on this context.  For 6 x 6
+// boxes (2 <= a < 3) the per-voxel gather's polynomial-weight configurations of
+// 8-deep bricks run the direct-drain gather of the same brick (shapes 0 and 1
+// of both families): on GB300 at S = 96, 777 FP32 images, a = 2.5, an insert
+// takes 0.79 ms instead of 2.39.  Tables and A&S weights, 4-deep bricks and images
+// too small for a 6 x 6 box in the half plane (S < 10) stay with the per-voxel
+// gather; so does a < 2, where the direct-drain gather has its own
+// configurations.
+Config effective_config(const fr_ctx *c, int id) {
+  Config cfg = config_space()[id];
+  if (cfg.algo == ALGO_GATHER && cfg.wmode == W_POLY && c->g.KB == 6 && cfg.shape <= 1 && c->g.H >= 5) {
+    cfg.algo = ALGO_GATHER2;
+    cfg.minw = 16;
+  }
+  return cfg;
+}
+
 // Work units of a gather launch of this batch alone, heaviest first (so the
 // largest ones start first), cached on the device per (shape, n).
 static int gather_units(fr_ctx *c, const Config &cfg, int n, InsertArgs &a,
@@ -216,7 +233,8 @@ static int gather_units(fr_ctx *c, const Config &cfg, int n, InsertArgs &a,
     // bricks one footprint wide, split finely (they are few and heavy)
     brick_unit_loads(c, gather2_shape(cfg.shape), 1 - c->g.xa0, c->g.H, n, 0.0, MAIN_UNITS_PER_SM,
                      us, any_split);
-    brick_unit_loads(c, fold_shape(), c->g.xa0, -c->g.xa0, n, 0.0, FOLD_UNITS_PER_SM, fs, fsplit);
+    brick_unit_loads(c, fold_shape(c->g.KB), c->g.xa0, -c->g.xa0, n, 0.0, FOLD_UNITS_PER_SM, fs,
+                     fsplit);
   } else {
     gather_unit_loads(c, cfg.shape, n, 0.0, us, any_split);
   }
@@ -262,7 +280,7 @@ static void gather_geometry(const fr_ctx *c, const Config &cfg, InsertArgs &a) {
 // Allocate and upload whatever a launch of configuration id on n images
 // needs (work units, scratch), so that the launch itself only enqueues work.
 int prepare_config(fr_ctx *c, int id, int n) {
-  const Config &cfg = config_space()[id];
+  const Config cfg = effective_config(c, id);
   InsertArgs a = base_args(c);
   if (cfg.algo == ALGO_GATHER || cfg.algo == ALGO_GATHER2) {
     const int4 *fold = nullptr;
@@ -281,7 +299,7 @@ int prepare_config(fr_ctx *c, int id, int n) {
 // Enqueue the insertion of n images with configuration id; no timing.
 int run_config(fr_ctx *c, int id, const void *images, int f16, const float *rot, int n,
                cudaStream_t st) {
-  const Config &cfg = config_space()[id];
+  const Config cfg = effective_config(c, id);
   InsertArgs a = base_args(c);
   a.images = images;
   a.f16 = f16;
@@ -718,7 +736,7 @@ int fr_config_features(int id, int S, int n, float a, float *out16) {
 int fr_insert_launches(fr_ctx *c, int id, int n, int *out) {
   if (!c || !out || n < 1 || id < 0 || id >= (int)config_space().size())
     return FR_ERR_INVALID_ARG;
-  const Config &cfg = config_space()[id];
+  const Config cfg = effective_config(c, id);
   if (cfg.algo == ALGO_SCATTER) {
     *out = 2 * ((n + cfg.sub - 1) / cfg.sub);  // scatter + merge per sub-batch
     return FR_OK;

@@ -1,11 +1,11 @@
 """GPU parity of the direct-drain gather at the edges of its pixel patches.
 
-A patch holds at most 17 x 17 stored pixels, copied 16 columns and 2 rows at a
+A patch holds at most 19 x 19 stored pixels, copied 16 columns and 2 rows at a
 time and clamped into the half plane.  The sizes put every edge inside small
 volumes: images narrower than a patch (S = 8 .. 30), row lengths S/2 + 1 that
 are even (16-byte rows) and odd, patches that wrap at k_y = 0 and cross
 k_x = 0, footprints cut by the volume's border, an odd number of images, and
-blobs from less than one voxel to the widest 4-wide box.  Tolerance: the
+blobs from less than one voxel to the widest 6-wide box.  Tolerance: the
 library's parity bar (2e-5 of the largest value, FP32 accumulation of at most
 40 images; FP16 images against the oracle fed the rounded values)."""
 import numpy as np
@@ -26,7 +26,7 @@ def _batch(S, n, seed):
 
 
 @pytest.mark.parametrize("f16", [False, True])
-@pytest.mark.parametrize("a", [0.6, 1.0, 1.5, 1.999])
+@pytest.mark.parametrize("a", [0.6, 1.0, 1.5, 1.999, 2.0, 2.5, 2.999])
 @pytest.mark.parametrize("S", [8, 10, 14, 16, 18, 30, 32, 34, 46])
 def test_patch_edges_match_oracle(S, a, f16):
     a = float(np.float32(a))
