@@ -76,19 +76,29 @@ struct UnitLoad {
 };
 double gather_unit_loads(const fr_ctx *c, int shape, int n, double target,
                          std::vector<UnitLoad> &out, int &any_split);
+// Expected images of one work unit, given the total over all bricks.
+// Per-voxel gather: the total over per_sm units per SM, at least 16.  Direct-drain
+// gather (direct = true): the same, but at least 8 images (a unit's fixed cost, its
+// partial sums cleared and written back, is about one image's work per 512
+// voxels), or fewer, down to 2, while the units would not fill 8 per SM.
+// Measured on GB300 (insert time; floors of 16 / 8 / 4 / 2 images): S = 32, 64
+// images 57 / 45 / 36 / 30 us; S = 64, 200 images 112 / 86 / 85 / 85 us; S = 96,
+// 500 images at 18 images a unit 242 us, at 6 images 255.
+double unit_share(double total, int sms, int per_sm, bool direct);
 // work units of bricks of shape sh tiling x in [x0, x1] (all y, z), split so
-// that no unit exceeds `target` expected images (target <= 0: the total over
-// per_sm units per SM, at least UNIT_MIN_LOAD), into at most 64 units of at
-// least SPLIT_MIN_IMAGES images per brick; returns the total expected load
-constexpr double UNIT_MIN_LOAD = 16.0;
-constexpr int SPLIT_MIN_IMAGES = 8;
-// units per SM of the direct-drain gather's main launch and of its fold-column
-// launch (the fold bricks are few and every plane crosses the central ones:
-// fine splits keep that launch's serial path inside the main launch's time)
-constexpr int MAIN_UNITS_PER_SM = 32;
+// that no unit exceeds `target` expected images (target <= 0: unit_share of the
+// total), into at most 64 units per brick of at least 2 images (per-voxel
+// gather: 8), unsplit below 16 images; returns the total expected load.
+// Units per SM of the direct-drain gather's main launch (32 / 64 / 96 / 128
+// measured at S = 128, n = 1000: 651 / 631 / 627 / 636 us; S = 256, n = 5000: 9.37
+// / 9.69 / 9.11 / 9.50 ms) and of its fold-column launch (the fold bricks are few
+// and every plane crosses the central ones: fine splits keep that launch's serial
+// path inside the main launch's time; 4 to 12 measured alike).
+constexpr int MAIN_UNITS_PER_SM = 96;
 constexpr int FOLD_UNITS_PER_SM = 8;
 double brick_unit_loads(const fr_ctx *c, const GatherShape &sh, int x0, int x1, int n,
-                        double target, int per_sm, std::vector<UnitLoad> &out, int &any_split);
+                        double target, int per_sm, bool direct, std::vector<UnitLoad> &out,
+                        int &any_split);
 // drop cached batched-insertion plans that refer to c (called by fr_destroy)
 void batched_forget(const fr_ctx *c);
 // release the reconstruction buffers of c (called by fr_destroy)

@@ -136,15 +136,19 @@ int ensure_scratch(fr_ctx *c) {
 // crossed, within a + (brick radius) r, by a fraction min(1, (a + r) / d) of
 // uniformly oriented planes through the origin, so its expected image count is
 // n min(1, (a + r) / d).  Bricks whose count exceeds a target share are split
-// into several units, each taking a contiguous range of the images.  `target`
-// <= 0 selects the share of one launch of this batch alone (total load over
-// per_sm units per SM, at least UNIT_MIN_LOAD).  Every plane crosses the
-// bricks at the centre, whose warps take the images of their unit one after
-// another: the split floor bounds that serial path (at most 64 units per
-// brick, at least SPLIT_MIN_IMAGES images each).  Returns the units with
-// their expected loads, unsorted.
+// into several units, each taking a contiguous range of the images.  Every
+// plane crosses the bricks at the centre, whose warps take the images of their
+// unit one after another: the split floor bounds that serial path.  Returns the
+// units with their expected loads, unsorted.
+double unit_share(double total, int sms, int per_sm, bool direct) {
+  const double share = total / (std::max(sms, 1) * (double)per_sm);
+  if (!direct) return std::max(16.0, share);
+  return std::max(share, std::min(8.0, std::max(2.0, total / (std::max(sms, 1) * 8.0))));
+}
+
 double brick_unit_loads(const fr_ctx *c, const GatherShape &sh, int x0, int x1, int n,
-                        double target, int per_sm, std::vector<UnitLoad> &out, int &any_split) {
+                        double target, int per_sm, bool direct, std::vector<UnitLoad> &out,
+                        int &any_split) {
   const Geom &g = c->g;
   const int nbx = (x1 - x0 + sh.bx) / sh.bx, nby = (g.D + sh.by - 1) / sh.by,
             nbz = (g.D + sh.zc - 1) / sh.zc;
@@ -168,8 +172,9 @@ double brick_unit_loads(const fr_ctx *c, const GatherShape &sh, int x0, int x1, 
   if (target <= 0) {
     int sms = 0;
     cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, c->device);
-    target = std::max(UNIT_MIN_LOAD, total / (std::max(sms, 1) * (double)per_sm));
+    target = unit_share(total, sms, per_sm, direct);
   }
+  const int most = n < 16 ? 1 : std::min(64, n / (direct ? 2 : 8));
   out.clear();
   out.reserve(load.size() + 64);
   any_split = 0;
@@ -178,7 +183,7 @@ double brick_unit_loads(const fr_ctx *c, const GatherShape &sh, int x0, int x1, 
       for (int bx = 0; bx < nbx; ++bx) {
         const double l = load[((size_t)bz * nby + by) * nbx + bx];
         int ns = (int)std::ceil(l / target);
-        ns = std::max(1, std::min(ns, std::min(64, std::max(1, n / SPLIT_MIN_IMAGES))));
+        ns = std::max(1, std::min(ns, most));
         if (ns > 1) any_split = 1;
         for (int s = 0; s < ns; ++s)
           out.push_back(UnitLoad{l / ns, make_int4(bx, by, bz, s | (ns << 16))});
@@ -188,7 +193,7 @@ double brick_unit_loads(const fr_ctx *c, const GatherShape &sh, int x0, int x1, 
 
 double gather_unit_loads(const fr_ctx *c, int shape, int n, double target,
                          std::vector<UnitLoad> &out, int &any_split) {
-  return brick_unit_loads(c, gather_shape(shape), c->g.xa0, c->g.H, n, target, 32, out,
+  return brick_unit_loads(c, gather_shape(shape), c->g.xa0, c->g.H, n, target, 32, false, out,
                           any_split);
 }
 
@@ -232,9 +237,9 @@ static int gather_units(fr_ctx *c, const Config &cfg, int n, InsertArgs &a,
     // columns x in [-floor(a), floor(a)] go to its fold-column launch in
     // bricks one footprint wide, split finely (they are few and heavy)
     brick_unit_loads(c, gather2_shape(cfg.shape), 1 - c->g.xa0, c->g.H, n, 0.0, MAIN_UNITS_PER_SM,
-                     us, any_split);
-    brick_unit_loads(c, fold_shape(c->g.KB), c->g.xa0, -c->g.xa0, n, 0.0, FOLD_UNITS_PER_SM, fs,
-                     fsplit);
+                     true, us, any_split);
+    brick_unit_loads(c, fold_shape(c->g.KB), c->g.xa0, -c->g.xa0, n, 0.0, FOLD_UNITS_PER_SM, true,
+                     fs, fsplit);
   } else {
     gather_unit_loads(c, cfg.shape, n, 0.0, us, any_split);
   }
