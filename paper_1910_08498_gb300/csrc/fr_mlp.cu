@@ -8,6 +8,7 @@
 
 #include <algorithm>
 #include <cmath>
+#include <mutex>
 #include <numeric>
 #include <random>
 #include <vector>
@@ -26,135 +27,233 @@ constexpr int OFF_W3 = OFF_B2 + MLP_H;
 constexpr int OFF_B3 = OFF_W3 + MLP_H;
 static_assert(OFF_B3 + 1 == MLP_NPARAM, "parameter layout");
 
-constexpr int ROWS = 32;  // rows per CTA; one CTA of MLP_H threads (one per hidden unit)
+// Forward and backward: CTAs of 256 threads, thread (j, q) = (tid & 63, tid >> 6)
+// being hidden unit j for every fourth row of a tile of at most ROWS rows.  The
+// layers are latency bound (a few microseconds of arithmetic on 152 SMs), so the
+// rows are spread over all SMs (at least ROWS_MIN a tile), a unit's weights sit in
+// registers (rows of W2 for the forward pass, columns for the deltas: read at
+// every step from shared memory, unpadded, they cost a 32-way bank conflict), and the activations are read as broadcast 16-byte groups.  2970 rows:
+// forward 41 -> 7 us, backward with its reduction 76 -> 21 us (cold caches).
+constexpr int ROWS = 32, ROWS_MIN = 4, MLP_T = 256, MLP_Q = MLP_T / MLP_H;
+constexpr int MLP_GRID = 304;  // CTAs of a backward launch at most (partial gradients kept per CTA)
 
-struct MlpSmem {
-  float P[MLP_NPARAM];
-  float x[ROWS][MLP_IN];
-  float h1[ROWS][MLP_H];
-  float h2[ROWS][MLP_H];
-  float d2[ROWS][MLP_H];  // dL/dz2
-  float d1[ROWS][MLP_H];  // dL/dz1
+struct MlpTile {
+  __align__(16) float x[ROWS][MLP_IN];
+  __align__(16) float h1[ROWS][MLP_H];
+  __align__(16) float h2[ROWS][MLP_H];
+  __align__(16) float d2[ROWS][MLP_H];  // dL/dz2
+  __align__(16) float d1[ROWS][MLP_H];  // dL/dz1
+  float w1[MLP_H][MLP_IN + 1];  // padded: a row or a column per lane without bank conflicts
+  float w2[MLP_H][MLP_H + 1];
+  float w3[MLP_H];
   float y[ROWS];
   float dy[ROWS];
 };
 
-__device__ void mlp_tile_forward(MlpSmem &s, int nrows) {
-  const int j = threadIdx.x;  // hidden unit
-  for (int r = 0; r < nrows; ++r) {
-    float z = s.P[OFF_B1 + j];
+// rows of a tile: as few as spread m rows over the SMs
+static int mlp_rows(int m) {
+  const int r = (m + device_sm_count() - 1) / device_sm_count();
+  return r < ROWS_MIN ? ROWS_MIN : r > ROWS ? ROWS : r;
+}
+static int mlp_grid(int m) {
+  const int tiles = (m + mlp_rows(m) - 1) / mlp_rows(m);
+  return tiles < MLP_GRID ? tiles : MLP_GRID;
+}
+
+// f(r, b + sum_k w[k] v[r][k]) for the thread's rows r = q, q + 4, ... < nrows, k
+// ascending, four rows at a time: four independent chains of FMAs (v's rows are
+// 16-byte aligned and read by broadcast)
+template <int N, class F>
+__device__ __forceinline__ void mlp_dots(const float (&w)[N], const float (*v)[N], float b, int q,
+                                         int nrows, F f) {
+  for (int r = q; r < nrows; r += 4 * MLP_Q) {
+    float z[4] = {b, b, b, b};
 #pragma unroll
-    for (int k = 0; k < MLP_IN; ++k) z = fmaf(s.P[OFF_W1 + j * MLP_IN + k], s.x[r][k], z);
-    s.h1[r][j] = fmaxf(z, 0.f);
+    for (int k = 0; k < N; k += 4)
+#pragma unroll
+      for (int i = 0; i < 4; ++i) {
+        const int ri = min(r + i * MLP_Q, nrows - 1);
+        const float4 u = *reinterpret_cast<const float4 *>(v[ri] + k);
+        z[i] = fmaf(w[k], u.x, z[i]);
+        z[i] = fmaf(w[k + 1], u.y, z[i]);
+        z[i] = fmaf(w[k + 2], u.z, z[i]);
+        z[i] = fmaf(w[k + 3], u.w, z[i]);
+      }
+#pragma unroll
+    for (int i = 0; i < 4; ++i)
+      if (r + i * MLP_Q < nrows) f(r + i * MLP_Q, z[i]);
   }
+}
+
+// activations and outputs of one tile's nrows rows; w1, w2: rows j of W1, W2
+__device__ __forceinline__ void mlp_tile_forward(MlpTile &s, const float (&w1)[MLP_IN], float b1,
+                                                 const float (&w2)[MLP_H], float b2, float b3,
+                                                 const float *X, int r0, int nrows) {
+  const int tid = threadIdx.x, j = tid & (MLP_H - 1), q = tid / MLP_H;
+  for (int i = tid; i < nrows * MLP_IN; i += MLP_T) (&s.x[0][0])[i] = X[(size_t)r0 * MLP_IN + i];
   __syncthreads();
-  for (int r = 0; r < nrows; ++r) {
-    float z = s.P[OFF_B2 + j];
-#pragma unroll 16
-    for (int k = 0; k < MLP_H; ++k) z = fmaf(s.P[OFF_W2 + j * MLP_H + k], s.h1[r][k], z);
-    s.h2[r][j] = fmaxf(z, 0.f);
-  }
+  mlp_dots(w1, s.x, b1, q, nrows, [&](int r, float z) { s.h1[r][j] = fmaxf(z, 0.f); });
   __syncthreads();
-  if (j < nrows) {
-    float z = s.P[OFF_B3];
-    for (int k = 0; k < MLP_H; ++k) z = fmaf(s.P[OFF_W3 + k], s.h2[j][k], z);
-    s.y[j] = z;
-  }
+  mlp_dots(w2, s.h1, b2, q, nrows, [&](int r, float z) { s.h2[r][j] = fmaxf(z, 0.f); });
+  __syncthreads();
+  // output layer: eight lanes a row
+  const int r = tid / 8, c = tid & 7;
+  float z = 0.f;
+  if (r < nrows)
+#pragma unroll
+    for (int k = 0; k < 8; ++k) z = fmaf(s.w3[c + 8 * k], s.h2[r][c + 8 * k], z);
+#pragma unroll
+  for (int o = 4; o > 0; o >>= 1) z += __shfl_down_sync(0xffffffffu, z, o, 8);
+  if (r < nrows && c == 0) s.y[r] = z + b3;
   __syncthreads();
 }
 
-__device__ void load_tile(MlpSmem &s, const float *P, const float *X, int r0, int nrows) {
-  for (int i = threadIdx.x; i < MLP_NPARAM; i += blockDim.x) s.P[i] = P[i];
-  for (int i = threadIdx.x; i < ROWS * MLP_IN; i += blockDim.x) {
-    int r = i / MLP_IN, k = i % MLP_IN;
-    s.x[r][k] = r < nrows ? X[(size_t)(r0 + r) * MLP_IN + k] : 0.f;
+__device__ __forceinline__ void mlp_weights(const float *P, float (&w1)[MLP_IN], float &b1,
+                                            float (&w2)[MLP_H], float &b2, float &b3, MlpTile &s) {
+  const int j = threadIdx.x & (MLP_H - 1);
+  // every load in flight before the first store (one after the other: 8 us)
+  constexpr int L1 = MLP_H * MLP_IN / MLP_T, L2 = MLP_H * MLP_H / MLP_T;
+  float t1[L1], t2[L2];
+#pragma unroll
+  for (int k = 0; k < L1; ++k) t1[k] = __ldg(P + OFF_W1 + k * MLP_T + threadIdx.x);
+#pragma unroll
+  for (int k = 0; k < L2; ++k) t2[k] = __ldg(P + OFF_W2 + k * MLP_T + threadIdx.x);
+  b1 = __ldg(P + OFF_B1 + j);
+  b2 = __ldg(P + OFF_B2 + j);
+  b3 = __ldg(P + OFF_B3);
+  if (threadIdx.x < MLP_H) s.w3[j] = __ldg(P + OFF_W3 + j);
+#pragma unroll
+  for (int k = 0; k < L1; ++k) {
+    const int i = k * MLP_T + threadIdx.x;
+    s.w1[i / MLP_IN][i % MLP_IN] = t1[k];
+  }
+#pragma unroll
+  for (int k = 0; k < L2; ++k) {
+    const int i = k * MLP_T + threadIdx.x;
+    s.w2[i / MLP_H][i % MLP_H] = t2[k];
   }
   __syncthreads();
+#pragma unroll
+  for (int k = 0; k < MLP_IN; ++k) w1[k] = s.w1[j][k];
+#pragma unroll
+  for (int k = 0; k < MLP_H; ++k) w2[k] = s.w2[j][k];
 }
 
-__global__ void __launch_bounds__(MLP_H) mlp_forward_kernel(const float *P, const float *X, int m,
-                                                            float *Y) {
+__global__ void __launch_bounds__(MLP_T) mlp_forward_kernel(const float *P, const float *X, int m,
+                                                            int rows, float *Y) {
   extern __shared__ __align__(16) unsigned char raw[];
-  MlpSmem &s = *reinterpret_cast<MlpSmem *>(raw);
-  const int r0 = blockIdx.x * ROWS;
-  const int nrows = min(ROWS, m - r0);
-  load_tile(s, P, X, r0, nrows);
-  mlp_tile_forward(s, nrows);
+  MlpTile &s = *reinterpret_cast<MlpTile *>(raw);
+  float w1[MLP_IN], w2[MLP_H], b1, b2, b3;
+  mlp_weights(P, w1, b1, w2, b2, b3, s);
+  const int r0 = blockIdx.x * rows, nrows = min(rows, m - r0);
+  mlp_tile_forward(s, w1, b1, w2, b2, b3, X, r0, nrows);
   if ((int)threadIdx.x < nrows) Y[r0 + threadIdx.x] = s.y[threadIdx.x];
 }
 
-// Per-CTA partial gradient (and partial loss) of L = (1/m) sum (y - t)^2 into
-// work[blockIdx.x][MLP_NPARAM + 1]; summed in fixed order by mlp_reduce_kernel.
-__global__ void __launch_bounds__(MLP_H) mlp_backward_kernel(const float *P, const float *X,
-                                                             const float *T, int m, float *work) {
+// Partial gradient (and partial loss) of L = (1/m) sum (y - t)^2 over the CTA's
+// tiles blockIdx.x, blockIdx.x + gridDim.x, ... into work[blockIdx.x][MLP_NPARAM
+// + 1]; summed in fixed order by mlp_reduce_kernel.  Thread (j, q) holds the
+// gradients of W2[j][16 q ..], W1[j][4 q ..] and, for q = 0, of unit j's biases
+// and W3[j].
+__global__ void __launch_bounds__(MLP_T) mlp_backward_kernel(const float *P, const float *X,
+                                                             const float *T, int m, int rows,
+                                                             float *work) {
   extern __shared__ __align__(16) unsigned char raw[];
-  MlpSmem &s = *reinterpret_cast<MlpSmem *>(raw);
-  const int r0 = blockIdx.x * ROWS;
-  const int nrows = min(ROWS, m - r0);
-  const int j = threadIdx.x;
-  load_tile(s, P, X, r0, nrows);
-  mlp_tile_forward(s, nrows);
-  float *G = work + (size_t)blockIdx.x * (MLP_NPARAM + 1);
+  MlpTile &s = *reinterpret_cast<MlpTile *>(raw);
+  const int tid = threadIdx.x, j = tid & (MLP_H - 1), q = tid / MLP_H;
+  float w1[MLP_IN], w2[MLP_H], b1, b2, b3;
+  mlp_weights(P, w1, b1, w2, b2, b3, s);
+  float c2[MLP_H];  // column j of W2
+#pragma unroll
+  for (int k = 0; k < MLP_H; ++k) c2[k] = s.w2[k][j];
+  constexpr int N2 = MLP_H / MLP_Q, N1 = MLP_IN / MLP_Q;
+  float g2[N2] = {}, g1[N1] = {}, gb1 = 0.f, gb2 = 0.f, gw3 = 0.f, gb3 = 0.f, loss = 0.f;
   const float inv_m = 1.0f / (float)m;
-  if (j < nrows) {
-    float e = s.y[j] - T[r0 + j];
-    s.dy[j] = 2.f * e * inv_m;
-    s.y[j] = e * e * inv_m;  // reuse as the per-row loss term
-  }
-  __syncthreads();
-  // output layer
-  {
-    float gw3 = 0.f;
-    for (int r = 0; r < nrows; ++r) gw3 = fmaf(s.dy[r], s.h2[r][j], gw3);
-    G[OFF_W3 + j] = gw3;
-    const float w3 = s.P[OFF_W3 + j];
-    for (int r = 0; r < nrows; ++r) s.d2[r][j] = s.h2[r][j] > 0.f ? s.dy[r] * w3 : 0.f;
-  }
-  if (j == 0) {
-    float gb3 = 0.f, l = 0.f;
-    for (int r = 0; r < nrows; ++r) { gb3 += s.dy[r]; l += s.y[r]; }
-    G[OFF_B3] = gb3;
-    G[MLP_NPARAM] = l;
-  }
-  __syncthreads();
-  // hidden layer 2: dW2[j][k] = sum_r d2[r][j] h1[r][k]; dz1[r][k] = [h1>0] sum_j W2[j][k] d2[r][j]
-  {
-    float gb2 = 0.f;
-    for (int r = 0; r < nrows; ++r) gb2 += s.d2[r][j];
-    G[OFF_B2 + j] = gb2;
-    for (int k = 0; k < MLP_H; ++k) {
-      float g = 0.f;
-      for (int r = 0; r < nrows; ++r) g = fmaf(s.d2[r][j], s.h1[r][k], g);
-      G[OFF_W2 + j * MLP_H + k] = g;
+  for (long long first = (long long)blockIdx.x * rows; first < m; first += (long long)gridDim.x * rows) {
+    const int r0 = (int)first, nrows = min(rows, m - r0);
+    mlp_tile_forward(s, w1, b1, w2, b2, b3, X, r0, nrows);
+    if (tid < nrows) {
+      const float e = s.y[tid] - T[r0 + tid];
+      s.dy[tid] = 2.f * e * inv_m;
+      s.y[tid] = e * e * inv_m;  // the row's loss term
     }
-    // thread j now plays input unit k = j of layer 2
+    __syncthreads();
+    const float w3 = s.w3[j];
+    for (int r = q; r < nrows; r += MLP_Q) s.d2[r][j] = s.h2[r][j] > 0.f ? s.dy[r] * w3 : 0.f;
+    __syncthreads();
+    // dW2[j][k] = sum_r d2[r][j] h1[r][k]; dz1[r][k] = [h1 > 0] sum_o W2[o][k] d2[r][o]
+#pragma unroll 4
     for (int r = 0; r < nrows; ++r) {
-      float d = 0.f;
-      for (int o = 0; o < MLP_H; ++o) d = fmaf(s.P[OFF_W2 + o * MLP_H + j], s.d2[r][o], d);
-      s.d1[r][j] = s.h1[r][j] > 0.f ? d : 0.f;
+      const float d = s.d2[r][j];
+      const float *h = s.h1[r] + q * N2;
+#pragma unroll
+      for (int k = 0; k < N2; k += 4) {
+        const float4 u = *reinterpret_cast<const float4 *>(h + k);
+        g2[k] = fmaf(d, u.x, g2[k]);
+        g2[k + 1] = fmaf(d, u.y, g2[k + 1]);
+        g2[k + 2] = fmaf(d, u.z, g2[k + 2]);
+        g2[k + 3] = fmaf(d, u.w, g2[k + 3]);
+      }
+      if (q == 0) {
+        gb2 += d;
+        gw3 = fmaf(s.dy[r], s.h2[r][j], gw3);
+      }
     }
+    mlp_dots(c2, s.d2, 0.f, q, nrows,
+             [&](int r, float z) { s.d1[r][j] = s.h1[r][j] > 0.f ? z : 0.f; });
+    if (tid == MLP_T - 1)
+      for (int r = 0; r < nrows; ++r) {
+        gb3 += s.dy[r];
+        loss += s.y[r];
+      }
+    __syncthreads();
+#pragma unroll 4
+    for (int r = 0; r < nrows; ++r) {
+      const float d = s.d1[r][j];
+      const float4 u = *reinterpret_cast<const float4 *>(s.x[r] + q * N1);
+      g1[0] = fmaf(d, u.x, g1[0]);
+      g1[1] = fmaf(d, u.y, g1[1]);
+      g1[2] = fmaf(d, u.z, g1[2]);
+      g1[3] = fmaf(d, u.w, g1[3]);
+      if (q == 0) gb1 += d;
+    }
+    __syncthreads();  // the tile is refilled
   }
-  __syncthreads();
-  // hidden layer 1
-  {
-    float gb1 = 0.f;
-    for (int r = 0; r < nrows; ++r) gb1 += s.d1[r][j];
+  static_assert(N1 == 4 && N2 % 4 == 0, "four thread groups");
+  float *G = work + (size_t)blockIdx.x * (MLP_NPARAM + 1);
+#pragma unroll
+  for (int k = 0; k < N2; ++k) G[OFF_W2 + j * MLP_H + q * N2 + k] = g2[k];
+#pragma unroll
+  for (int k = 0; k < N1; ++k) G[OFF_W1 + j * MLP_IN + q * N1 + k] = g1[k];
+  if (q == 0) {
     G[OFF_B1 + j] = gb1;
-    for (int k = 0; k < MLP_IN; ++k) {
-      float g = 0.f;
-      for (int r = 0; r < nrows; ++r) g = fmaf(s.d1[r][j], s.x[r][k], g);
-      G[OFF_W1 + j * MLP_IN + k] = g;
-    }
+    G[OFF_B2 + j] = gb2;
+    G[OFF_W3 + j] = gw3;
+  }
+  if (tid == MLP_T - 1) {
+    G[OFF_B3] = gb3;
+    G[MLP_NPARAM] = loss;
   }
 }
 
-__global__ void mlp_reduce_kernel(const float *work, int nblk, float *grad, float *loss) {
-  int i = blockIdx.x * blockDim.x + threadIdx.x;
-  if (i > MLP_NPARAM) return;
+// Sum the CTAs' partial gradients: eight groups of CTAs a parameter, then the
+// groups in order (fixed order: deterministic).
+__global__ void __launch_bounds__(256) mlp_reduce_kernel(const float *work, int nblk, float *grad,
+                                                         float *loss) {
+  __shared__ float part[8][32];
+  const int c = threadIdx.x & 31, gq = threadIdx.x >> 5;
+  const int i = blockIdx.x * 32 + c;
   float s = 0.f;
-  for (int b = 0; b < nblk; ++b) s += work[(size_t)b * (MLP_NPARAM + 1) + i];
-  if (i < MLP_NPARAM) grad[i] = s;
-  else if (loss) *loss = s;
+  if (i <= MLP_NPARAM)
+#pragma unroll 20
+    for (int b = gq; b < nblk; b += 8) s += work[(size_t)b * (MLP_NPARAM + 1) + i];
+  part[gq][c] = s;
+  __syncthreads();
+  if (gq == 0 && i <= MLP_NPARAM) {
+    for (int k = 1; k < 8; ++k) s += part[k][c];
+    if (i < MLP_NPARAM) grad[i] = s;
+    else if (loss) *loss = s;
+  }
 }
 
 __global__ void mlp_adam_kernel(float *P, const float *G, float *M1, float *M2, float lr, float b1,
@@ -170,19 +269,18 @@ __global__ void mlp_adam_kernel(float *P, const float *G, float *M1, float *M2, 
   P[i] -= lr * mh / (sqrtf(vh) + eps);
 }
 
-static size_t smem_bytes() { return sizeof(MlpSmem); }
-
 static bool set_attrs() {
-  return allow_dynamic_smem((const void *)mlp_forward_kernel, smem_bytes()) == cudaSuccess &&
-         allow_dynamic_smem((const void *)mlp_backward_kernel, smem_bytes()) == cudaSuccess;
+  return allow_dynamic_smem((const void *)mlp_forward_kernel, sizeof(MlpTile)) == cudaSuccess &&
+         allow_dynamic_smem((const void *)mlp_backward_kernel, sizeof(MlpTile)) == cudaSuccess;
 }
 
-size_t mlp_work_floats(int m) { return (size_t)((m + ROWS - 1) / ROWS) * (MLP_NPARAM + 1); }
+size_t mlp_work_floats(int m) { return (size_t)mlp_grid(m) * (MLP_NPARAM + 1); }
 
 cudaError_t mlp_forward(const float *params, const float *x, int m, float *y, cudaStream_t st) {
   if (m <= 0) return cudaSuccess;
   if (!set_attrs()) return cudaGetLastError();
-  mlp_forward_kernel<<<(m + ROWS - 1) / ROWS, MLP_H, smem_bytes(), st>>>(params, x, m, y);
+  const int rows = mlp_rows(m);
+  mlp_forward_kernel<<<(m + rows - 1) / rows, MLP_T, sizeof(MlpTile), st>>>(params, x, m, rows, y);
   return cudaGetLastError();
 }
 
@@ -190,9 +288,9 @@ cudaError_t mlp_backward(const float *params, const float *x, const float *t, in
                          float *loss, float *work, cudaStream_t st) {
   if (m <= 0) return cudaErrorInvalidValue;
   if (!set_attrs()) return cudaGetLastError();
-  int nblk = (m + ROWS - 1) / ROWS;
-  mlp_backward_kernel<<<nblk, MLP_H, smem_bytes(), st>>>(params, x, t, m, work);
-  mlp_reduce_kernel<<<(MLP_NPARAM + 1 + 255) / 256, 256, 0, st>>>(work, nblk, grad, loss);
+  const int nblk = mlp_grid(m);
+  mlp_backward_kernel<<<nblk, MLP_T, sizeof(MlpTile), st>>>(params, x, t, m, mlp_rows(m), work);
+  mlp_reduce_kernel<<<(MLP_NPARAM + 1 + 31) / 32, 256, 0, st>>>(work, nblk, grad, loss);
   return cudaGetLastError();
 }
 
@@ -202,6 +300,41 @@ cudaError_t mlp_adam(float *params, const float *grad, float *m1, float *m2, int
   mlp_adam_kernel<<<(MLP_NPARAM + 255) / 256, 256, 0, st>>>(params, grad, m1, m2, lr, b1, b2, eps,
                                                             c1, c2);
   return cudaGetLastError();
+}
+
+// Stream-ordered workspace of fr_mlp_backward, from a pool per device that keeps
+// up to WORK_KEEP bytes between calls (a gradient's partial sums are at most 6.5
+// MB): the default pool hands its memory back at every synchronisation, and a call
+// that follows one waited 170 us for new memory.
+static cudaError_t work_alloc(float **p, size_t bytes, cudaStream_t st) {
+  constexpr unsigned long long WORK_KEEP = 8ull << 20;
+  static std::mutex mu;
+  static std::vector<cudaMemPool_t> pools;  // by device ordinal
+  int dev = 0;
+  cudaError_t e = cudaGetDevice(&dev);
+  if (e != cudaSuccess) return e;
+  cudaMemPool_t pool = nullptr;
+  {
+    std::lock_guard<std::mutex> lk(mu);
+    if ((int)pools.size() <= dev) pools.resize(dev + 1, nullptr);
+    if (!pools[dev]) {
+      cudaMemPoolProps props{};
+      props.allocType = cudaMemAllocationTypePinned;
+      props.location.type = cudaMemLocationTypeDevice;
+      props.location.id = dev;
+      unsigned long long keep = WORK_KEEP;
+      if (cudaMemPoolCreate(&pools[dev], &props) != cudaSuccess ||
+          cudaMemPoolSetAttribute(pools[dev], cudaMemPoolAttrReleaseThreshold, &keep) != cudaSuccess) {
+        cudaGetLastError();
+        pools[dev] = nullptr;
+      }
+    }
+    pool = pools[dev];
+  }
+  void *q = nullptr;
+  e = pool ? cudaMallocFromPoolAsync(&q, bytes, pool, st) : cudaMallocAsync(&q, bytes, st);
+  *p = static_cast<float *>(q);
+  return e;
 }
 
 // He-uniform initialisation on the host from a seed.
@@ -264,8 +397,7 @@ int fr_mlp_backward(const float *params, const float *x, const float *target, in
                     float *loss, void *stream) {
   if (m < 1 || !params || !x || !target || !grad || !loss) return FR_ERR_INVALID_ARG;
   float *work = nullptr;
-  if (cudaMallocAsync(&work, mlp_work_floats(m) * sizeof(float), (cudaStream_t)stream) !=
-      cudaSuccess)
+  if (work_alloc(&work, mlp_work_floats(m) * sizeof(float), (cudaStream_t)stream) != cudaSuccess)
     return FR_ERR_OOM;
   cudaError_t e = mlp_backward(params, x, target, m, grad, loss, work, (cudaStream_t)stream);
   cudaFreeAsync(work, (cudaStream_t)stream);

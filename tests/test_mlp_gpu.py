@@ -83,3 +83,23 @@ def test_training_fits_a_smooth_target():
         assert float(np.mean((y - T) ** 2)) == pytest.approx(loss, rel=1e-3)
     finally:
         L.fr_destroy(ctx)
+
+
+@pytest.mark.parametrize("m", [1, 3, 4, 5, 31, 608, 609, 4865, 12000])
+def test_tile_edges_match_oracle(m):
+    """Row counts at the edges of the kernels' tiles: fewer rows than a tile, one
+    row past the rows an SM takes, more tiles than CTAs (each CTA then sums
+    several).  Tolerance: the other gradient tests' 2e-5 of the largest value
+    (FP32 sums of m terms of scale 1/m)."""
+    p, X, T = (a.astype(np.float32) for a in problem(40 + m, m))
+    ref, _ = mlp.forward(p, X)
+    Lr, gr = mlp.loss_and_grad(p, X, T)
+    y = torch.full((m + 1,), 7.0, device="cuda")
+    L.fr_mlp_forward(dev(p), dev(X), y[:m])
+    g = torch.empty(mlp.NPARAM, device="cuda")
+    loss = torch.empty(1, device="cuda")
+    L.fr_mlp_backward(dev(p), dev(X), dev(T), g, loss)
+    assert np.max(np.abs(y[:m].cpu().numpy() - ref)) <= 2e-5 * max(1.0, np.max(np.abs(ref)))
+    assert y[m].item() == 7.0
+    assert loss.item() == pytest.approx(Lr, rel=2e-5)
+    assert np.max(np.abs(g.cpu().numpy() - gr)) <= 2e-5 * max(1.0, np.max(np.abs(gr)))
