@@ -32,8 +32,10 @@ static_assert(OFF_B3 + 1 == MLP_NPARAM, "parameter layout");
 // layers are latency bound (a few microseconds of arithmetic on 152 SMs), so the
 // rows are spread over all SMs (at least ROWS_MIN a tile), a unit's weights sit in
 // registers (rows of W2 for the forward pass, columns for the deltas: read at
-// every step from shared memory, unpadded, they cost a 32-way bank conflict), and the activations are read as broadcast 16-byte groups.  2970 rows:
-// forward 41 -> 7 us, backward with its reduction 76 -> 21 us (cold caches).
+// every step from shared memory, unpadded, they cost a 32-way bank conflict),
+// and the activations are read as broadcast 16-byte groups.  2970 rows: forward
+// 41 -> 7 us, backward with its reduction 76 -> 21 us (cold caches; its row
+// loops unrolled by four it took 24).
 constexpr int ROWS = 32, ROWS_MIN = 4, MLP_T = 256, MLP_Q = MLP_T / MLP_H;
 constexpr int MLP_GRID = 304;  // CTAs of a backward launch at most (partial gradients kept per CTA)
 
@@ -182,7 +184,6 @@ __global__ void __launch_bounds__(MLP_T) mlp_backward_kernel(const float *P, con
     for (int r = q; r < nrows; r += MLP_Q) s.d2[r][j] = s.h2[r][j] > 0.f ? s.dy[r] * w3 : 0.f;
     __syncthreads();
     // dW2[j][k] = sum_r d2[r][j] h1[r][k]; dz1[r][k] = [h1 > 0] sum_o W2[o][k] d2[r][o]
-#pragma unroll 4
     for (int r = 0; r < nrows; ++r) {
       const float d = s.d2[r][j];
       const float *h = s.h1[r] + q * N2;
@@ -207,7 +208,6 @@ __global__ void __launch_bounds__(MLP_T) mlp_backward_kernel(const float *P, con
         loss += s.y[r];
       }
     __syncthreads();
-#pragma unroll 4
     for (int r = 0; r < nrows; ++r) {
       const float d = s.d1[r][j];
       const float4 u = *reinterpret_cast<const float4 *>(s.x[r] + q * N1);
@@ -245,7 +245,7 @@ __global__ void __launch_bounds__(256) mlp_reduce_kernel(const float *work, int 
   const int i = blockIdx.x * 32 + c;
   float s = 0.f;
   if (i <= MLP_NPARAM)
-#pragma unroll 20
+#pragma unroll 8
     for (int b = gq; b < nblk; b += 8) s += work[(size_t)b * (MLP_NPARAM + 1) + i];
   part[gq][c] = s;
   __syncthreads();
