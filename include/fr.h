@@ -177,9 +177,9 @@ int fr_insert(fr_ctx *ctx, const void *images, fr_dtype dtype, const float *rota
  * configurations share a kernel instantiation run in ONE launch over the
  * pooled work units (a brick and a share of a batch's images) of all of them,
  * heaviest units first, so uneven S and n share the GPU without a tail per
- * batch: the direct-drain gather as one CTA per unit (its fold columns in a
- * second launch on a high-priority side stream), the per-voxel gather as a
- * persistent kernel whose CTAs take units from a device counter.  Batches
+ * batch: the direct-drain gather as one CTA per warp footprint of a unit, the
+ * per-voxel gather as a persistent kernel whose CTAs take units from a device
+ * counter.  Batches
  * whose configuration has no multi-batch kernel (scatter, tabulated weights)
  * run their own launches after those.  A context that appears more than once
  * receives its sums through its scratch volume with atomics.  The first call

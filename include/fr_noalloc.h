@@ -3,9 +3,10 @@
  *
  * The paper has no counterpart of this call: it is a service entry point of
  * this library.  It runs the same insertion as fr_insert (the definition is
- * written out in fr.h) through the atomic scatter kernel, whose scratch
- * volume is a fixed array in the library's static device memory instead of a
- * cudaMalloc'd buffer.
+ * written out in fr.h) through the direct-drain gather, or the atomic scatter
+ * where that is the more exact one (a^2 within 1e-4 of an integer, alpha > 16, S
+ * < 10 with a >= 2) or the faster one (small batches), whose scratch volume is a fixed array in the library's
+ * static device memory instead of a cudaMalloc'd buffer.
  *
  * Who needs it: callers that must not enter the device allocator for the
  * duration of the call.  cudaMalloc and cudaFree can synchronise the device
@@ -37,8 +38,8 @@ extern "C" {
  *              returns FR_ERR_NOALLOC_LIMIT and enqueues nothing; an odd S
  *              returns FR_ERR_UNSUPPORTED, S < 8 FR_ERR_INVALID_ARG.
  *   a, alpha   blob radius (0 < a < 3) and taper (0 <= alpha <= 40); the
- *              weights are evaluated on the fly (Abramowitz & Stegun 9.8.1 /
- *              9.8.2 for I0).
+ *              weights are evaluated on the fly (the weight polynomial; in the
+ *              scatter Abramowitz & Stegun 9.8.1 / 9.8.2 for I0).
  *   images     device, [n][S][S/2+1] complex of `dtype` (layout of fr.h),
  *              16-byte aligned.
  *   rotations  device, [n][9] float32 (layout of fr.h).
@@ -62,7 +63,8 @@ extern "C" {
  * The first call on each device performs a one-time setup: it looks up the
  * scratch array's address with cudaGetSymbolAddress (which also loads the
  * library's device code on that device if lazy loading has not done so yet)
- * while that device is current, and caches it.  Make that first call before
+ * while that device is current, caches it, and allows the gather kernel its
+ * shared memory.  Make that first call before
  * any stream capture begins.
  *
  * The batch is added in sub-batches of 1024 images, each merged into V and W

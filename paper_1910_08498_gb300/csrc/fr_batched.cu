@@ -11,10 +11,9 @@
 //     polynomial, which stays a kernel parameter);
 //   * each group's work units (bricks and image splits, with expected loads)
 //     are pooled over its batches with one splitting target and ordered
-//     heaviest first.  A direct-drain group is one launch with a CTA per item,
-//     plus one launch of its fold-column instantiation over the items of the
-//     fold columns on a high-priority side stream beside it; a per-voxel gather
-//     group is one persistent launch whose CTAs take items from a device
+//     heaviest first.  A direct-drain group is one launch with a CTA per warp
+//     footprint of an item, the items of the fold columns first; a per-voxel
+//     gather group is one persistent launch whose CTAs take items from a device
 //     counter;
 //   * the per-batch launch arguments and the items are uploaded once into a
 //     device buffer the plan owns;
@@ -55,8 +54,8 @@ struct PlanKey {
 struct Group {
   int algo = ALGO_GATHER, shape = 0, kb = 4, f16 = 0, chunk = 64, minw = 0;
   PersistentLaunch launch{};  // per-voxel gather: persistent launch
-  MultiLaunch main{}, fold{};  // direct-drain gather: main and fold-column launches
-  int lane = 0;               // direct-drain gather: the stream its main launch runs on
+  MultiLaunch main{};         // direct-drain gather: its launch
+  int lane = 0;               // direct-drain gather: the stream its launch runs on
 };
 
 constexpr int MAX_LANES = 4;
@@ -68,13 +67,11 @@ struct Plan {
   std::vector<Group> groups;
   std::vector<InsertArgs> merges;    // scratch merges after the groups
   std::vector<int> sequential;       // batches run with their own launches
-  // direct-drain groups: their main launches on up to MAX_LANES streams side
-  // by side, the fold-column launches on a highest-priority stream; forked
-  // from and joined back into the caller's stream
+  // direct-drain groups: their launches on up to MAX_LANES streams side by side,
+  // forked from and joined back into the caller's stream
   std::vector<cudaStream_t> lanes;
-  cudaStream_t side = nullptr;
   cudaEvent_t ev_fork = nullptr;
-  std::vector<cudaEvent_t> ev_join;  // one per lane, then the side stream's
+  std::vector<cudaEvent_t> ev_join;  // one per lane
   cudaGraphExec_t exec = nullptr;
 };
 
@@ -87,11 +84,9 @@ void free_plan(Plan &p) {
   if (p.ev_fork) cudaEventDestroy(p.ev_fork);
   for (cudaEvent_t e : p.ev_join) cudaEventDestroy(e);
   for (cudaStream_t l : p.lanes) cudaStreamDestroy(l);
-  if (p.side) cudaStreamDestroy(p.side);
   cudaFree(p.dev);
   p.exec = nullptr;
   p.dev = nullptr;
-  p.side = nullptr;
   p.ev_fork = nullptr;
   p.ev_join.clear();
   p.lanes.clear();
@@ -134,7 +129,7 @@ int build_plan(Plan &pl, fr_ctx *const *ctxs, const void *const *images, const i
     } else if (k.algo == ALGO_GATHER && k.wmode == W_POLY && poly_ok) {
       groups[GKey(ALGO_GATHER, k.shape, c->g.KB, f16, k.chunk, 0, 0, 0.f, 0.f)].push_back(b);
     } else {
-      // its own launches: units, scratch and side stream ready before any capture
+      // its own launches: units and scratch ready before any capture
       int rc = prepare_config(c, cfg[b], n[b]);
       if (rc != FR_OK) return rc;
       pl.sequential.push_back(b);
@@ -143,7 +138,7 @@ int build_plan(Plan &pl, fr_ctx *const *ctxs, const void *const *images, const i
   const int sms = std::max(device_sm_count(), 1);
 
   std::vector<InsertArgs> descs(nb);  // each batch's own arguments
-  std::vector<std::vector<int4>> items;  // per group: main items, then (gather2) fold items
+  std::vector<std::vector<int4>> items;  // per group; gather2: fold items, then main items
   std::set<const fr_ctx *> merge_ctx;
   struct It { double load; int4 v; };
   auto order = [](std::vector<It> &its) {
@@ -161,8 +156,6 @@ int build_plan(Plan &pl, fr_ctx *const *ctxs, const void *const *images, const i
       glist.push_back({kv.first, std::vector<int>(kv.second.begin() + i,
                                                   kv.second.begin() + std::min(kv.second.size(), i + cap))});
   }
-  int greatest = 0, least = 0;
-  cudaDeviceGetStreamPriorityRange(&least, &greatest);
   int n_g2 = 0;
   for (auto &kv : glist) {
     Group gr;
@@ -207,7 +200,7 @@ int build_plan(Plan &pl, fr_ctx *const *ctxs, const void *const *images, const i
         for (const UnitLoad &u : tmp)
           fits.push_back(It{u.load, make_int4(u.unit.x | (u.unit.y << 10) | (u.unit.z << 20),
                                               u.unit.w | shared_bit, b, (int)slot)});
-        gr.main.images[slot] = gr.fold.images[slot] = images[b];
+        gr.main.images[slot] = images[b];
       }
       if (split || fsplit || shared) {
         int rc = ensure_scratch(c);
@@ -225,17 +218,19 @@ int build_plan(Plan &pl, fr_ctx *const *ctxs, const void *const *images, const i
       a.scratch = c->scratch;
       descs[b] = a;
     }
-    items.push_back(order(its));
+    std::vector<int4> ordered = order(its);
     if (g2) {
-      items.push_back(order(fits));
+      std::vector<int4> all = order(fits);
+      gr.main.nfold = (int)all.size();
+      gr.main.nitems = (int)ordered.size();
+      all.insert(all.end(), ordered.begin(), ordered.end());
+      ordered.swap(all);
       // the arguments the group's batches share (geometry, weights, list
-      // capacity): those of its first batch; the kernels read the rest per batch
-      InsertArgs base = descs[kv.second.front()];
-      gr.main.base = base;
-      gr.fold.base = base;
-      gr.fold.priority = greatest;
+      // capacity): those of its first batch; the kernel reads the rest per batch
+      gr.main.base = descs[kv.second.front()];
       gr.lane = n_g2++ % MAX_LANES;
     }
+    items.push_back(std::move(ordered));
     pl.groups.push_back(gr);
   }
   // device buffer: descriptors | items of each group | one counter per group
@@ -259,38 +254,29 @@ int build_plan(Plan &pl, fr_ctx *const *ctxs, const void *const *images, const i
                    cudaMemcpyHostToDevice);
     if (e != cudaSuccess) return cuda_err(e);
   }
-  size_t ii = 0;
   for (size_t gi = 0; gi < pl.groups.size(); ++gi) {
     Group &gr = pl.groups[gi];
     if (gr.algo == ALGO_GATHER2) {
-      gr.main.descs = gr.fold.descs = reinterpret_cast<const InsertArgs *>(d);
-      gr.main.items = reinterpret_cast<const int4 *>(d + item_off[ii]);
-      gr.main.nitems = (int)items[ii].size();
-      gr.fold.items = reinterpret_cast<const int4 *>(d + item_off[ii + 1]);
-      gr.fold.nitems = (int)items[ii + 1].size();
-      ii += 2;
+      gr.main.descs = reinterpret_cast<const InsertArgs *>(d);
+      gr.main.items = reinterpret_cast<const int4 *>(d + item_off[gi]);
     } else {
       PersistentLaunch &L = gr.launch;
       L.descs = reinterpret_cast<const InsertArgs *>(d);
-      L.items = reinterpret_cast<const int4 *>(d + item_off[ii]);
-      L.nitems = (int)items[ii].size();
+      L.items = reinterpret_cast<const int4 *>(d + item_off[gi]);
+      L.nitems = (int)items[gi].size();
       L.chunk = gr.chunk;
       L.counter = reinterpret_cast<unsigned *>(d + counter_off) + gi;
-      ii += 1;
     }
   }
   if (n_g2 > 0) {
-    int lo = 0, hi = 0;
-    e = cudaDeviceGetStreamPriorityRange(&lo, &hi);
-    if (e == cudaSuccess) e = cudaStreamCreateWithPriority(&pl.side, cudaStreamNonBlocking, hi);
-    if (e == cudaSuccess) e = cudaEventCreateWithFlags(&pl.ev_fork, cudaEventDisableTiming);
+    e = cudaEventCreateWithFlags(&pl.ev_fork, cudaEventDisableTiming);
     const int nl = std::min(n_g2, MAX_LANES);
     for (int l = 0; l < nl && e == cudaSuccess; ++l) {
       cudaStream_t s = nullptr;
       e = cudaStreamCreateWithFlags(&s, cudaStreamNonBlocking);
       if (e == cudaSuccess) pl.lanes.push_back(s);
     }
-    for (int l = 0; l <= nl && e == cudaSuccess; ++l) {
+    for (int l = 0; l < nl && e == cudaSuccess; ++l) {
       cudaEvent_t ev = nullptr;
       e = cudaEventCreateWithFlags(&ev, cudaEventDisableTiming);
       if (e == cudaSuccess) pl.ev_join.push_back(ev);
@@ -306,24 +292,18 @@ int build_plan(Plan &pl, fr_ctx *const *ctxs, const void *const *images, const i
 int enqueue_plan(const Plan &pl, fr_ctx *const *ctxs, const void *const *images, const int *dtypes,
                  const float *const *rotations, const int *n, const std::vector<int> &cfg,
                  cudaStream_t st) {
-  // direct-drain groups: fork the lanes and the side stream off st; the
-  // fold-column launches first, on the side stream (disjoint voxels; split
-  // and shared units add to the scratch with atomics, merged after the join)
+  // direct-drain groups: fork the lanes off st (split and shared units add to
+  // the scratch with atomics, merged after the join)
   cudaError_t e = cudaSuccess;
   const int nl = (int)pl.lanes.size();
-  if (pl.side) {
+  if (nl > 0) {
     e = cudaEventRecord(pl.ev_fork, st);
-    if (e == cudaSuccess) e = cudaStreamWaitEvent(pl.side, pl.ev_fork, 0);
     for (int l = 0; l < nl && e == cudaSuccess; ++l)
       e = cudaStreamWaitEvent(pl.lanes[l], pl.ev_fork, 0);
     for (const Group &gr : pl.groups)
       if (e == cudaSuccess && gr.algo == ALGO_GATHER2)
-        e = launch_gather_fold_multi(gr.f16, gr.fold, pl.side);
-    for (const Group &gr : pl.groups)
-      if (e == cudaSuccess && gr.algo == ALGO_GATHER2)
         e = launch_gather2_multi(gr.shape, gr.minw, gr.f16, gr.main, pl.lanes[gr.lane]);
     for (int l = 0; l < nl && e == cudaSuccess; ++l) e = cudaEventRecord(pl.ev_join[l], pl.lanes[l]);
-    if (e == cudaSuccess) e = cudaEventRecord(pl.ev_join[nl], pl.side);
     if (e != cudaSuccess) return cuda_err(e);
   }
   for (const Group &gr : pl.groups) {
@@ -332,10 +312,8 @@ int enqueue_plan(const Plan &pl, fr_ctx *const *ctxs, const void *const *images,
     if (e == cudaSuccess) e = launch_gather_persistent(gr.shape, gr.kb, gr.f16, gr.launch, st);
     if (e != cudaSuccess) return cuda_err(e);
   }
-  if (pl.side) {
-    for (int l = 0; l <= nl && e == cudaSuccess; ++l) e = cudaStreamWaitEvent(st, pl.ev_join[l], 0);
-    if (e != cudaSuccess) return cuda_err(e);
-  }
+  for (int l = 0; l < nl && e == cudaSuccess; ++l) e = cudaStreamWaitEvent(st, pl.ev_join[l], 0);
+  if (e != cudaSuccess) return cuda_err(e);
   for (const InsertArgs &m : pl.merges) {
     e = launch_merge_scratch(m, st);
     if (e != cudaSuccess) return cuda_err(e);
@@ -355,11 +333,8 @@ int prime_plan(const Plan &pl, fr_ctx *const *ctxs, const int *dtypes, const std
     cudaError_t e;
     if (gr.algo == ALGO_GATHER2) {
       MultiLaunch q = gr.main;
-      q.nitems = 0;
+      q.nitems = q.nfold = 0;
       e = launch_gather2_multi(gr.shape, gr.minw, gr.f16, q, nullptr);
-      q = gr.fold;
-      q.nitems = 0;
-      if (e == cudaSuccess) e = launch_gather_fold_multi(gr.f16, q, nullptr);
     } else {
       PersistentLaunch q = gr.launch;
       q.nitems = 0;
@@ -377,9 +352,6 @@ int prime_plan(const Plan &pl, fr_ctx *const *ctxs, const int *dtypes, const std
       e = launch_gather(k.shape, k.wmode, a, nullptr, 1, nullptr);
     } else if (k.algo == ALGO_GATHER2) {
       e = launch_gather2(k.shape, k.minw, a, nullptr, 1, nullptr);
-      InsertArgs f = a;
-      f.nunits = 0;
-      if (e == cudaSuccess) e = launch_gather_fold(f, nullptr);
     } else {
       e = launch_scatter(k.threads, k.wmode, a, nullptr, 1, nullptr);
     }

@@ -35,17 +35,13 @@ struct fr_ctx {
   struct Units {
     int shape = -1, n = -1, count = 0, any_split = 0, algo = 0;
     int4 *dev = nullptr;
-    // direct-drain gather: the units of its fold-column launch (|x| <=
-    // floor(a)), stored after the main units in dev
-    int fold_count = 0, fold_split = 0;
+    // direct-drain gather: the units of its fold columns (|x| <= floor(a)),
+    // stored after the main units in dev
+    int fold_count = 0;
     const int4 *fold = nullptr;
   };
   Units units[8];
   unsigned long long *d_phase = nullptr;  // gather phase counters (debug bit 1)
-  // side stream (highest priority) and fork/join events: the direct-drain
-  // gather's fold-column launch runs beside its main launch
-  cudaStream_t side = nullptr;
-  cudaEvent_t ev_fork = nullptr, ev_join = nullptr;
   // cost model
   float *d_mlp = nullptr;
   bool mlp_trained = false;
@@ -65,8 +61,6 @@ int key_bucket(int n);
 InsertArgs base_args(const fr_ctx *c);
 // allocate the context's float4 scratch volume if it has none yet
 int ensure_scratch(fr_ctx *c);
-// create the context's side stream and fork/join events if it has none yet
-int ensure_side_stream(fr_ctx *c);
 // configuration id as this context runs it (its kernel family)
 Config effective_config(const fr_ctx *c, int id);
 // gather work unit with its expected load (images it scans)
@@ -89,11 +83,11 @@ double unit_share(double total, int sms, int per_sm, bool direct);
 // that no unit exceeds `target` expected images (target <= 0: unit_share of the
 // total), into at most 64 units per brick of at least 2 images (per-voxel
 // gather: 8), unsplit below 16 images; returns the total expected load.
-// Units per SM of the direct-drain gather's main launch (32 / 64 / 96 / 128
+// Units per SM of the direct-drain gather's main bricks (32 / 64 / 96 / 128
 // measured at S = 128, n = 1000: 651 / 631 / 627 / 636 us; S = 256, n = 5000: 9.37
-// / 9.69 / 9.11 / 9.50 ms) and of its fold-column launch (the fold bricks are few
-// and every plane crosses the central ones: fine splits keep that launch's serial
-// path inside the main launch's time; 4 to 12 measured alike).
+// / 9.69 / 9.11 / 9.50 ms) and of its fold columns (the fold bricks are few and
+// every plane crosses the central ones: fine splits keep their serial path inside
+// the launch's time; 4 to 12 measured alike).
 constexpr int MAIN_UNITS_PER_SM = 96;
 constexpr int FOLD_UNITS_PER_SM = 8;
 double brick_unit_loads(const fr_ctx *c, const GatherShape &sh, int x0, int x1, int n,

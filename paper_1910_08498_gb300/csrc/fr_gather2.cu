@@ -71,25 +71,13 @@ int resident_ctas(const void *fn, int threads, size_t smem) {
   return per_sm;
 }
 
-cudaError_t launch_multi(const void *fn, const MultiLaunch &p, int per_item, int threads,
-                         size_t smem, cudaStream_t st) {
-  cudaLaunchConfig_t cfg{};
-  cfg.gridDim = dim3((unsigned)p.nitems * (unsigned)per_item);
-  cfg.blockDim = dim3((unsigned)threads);
-  cfg.dynamicSmemBytes = smem;
-  cfg.stream = st;
-  cudaLaunchAttribute attr[1];
-  attr[0].id = cudaLaunchAttributePriority;
-  attr[0].val.priority = p.priority;
-  cfg.attrs = attr;
-  cfg.numAttrs = p.priority != 0 ? 1 : 0;
-  void *params[] = {const_cast<MultiLaunch *>(&p)};
-  return cudaLaunchKernelExC(&cfg, fn, params);
-}
-
 size_t gather2_smem_bytes(const GatherShape &sh, int chunk) {
   (void)sh;  // one warp per CTA
-  return gather2_warp_smem<8, 4, 0>(chunk);
+  return gather2_smem<4>(chunk);
+}
+
+GatherShape fold_shape(int kb) {
+  return GatherShape{kb == 4 ? g2_fold_width<4>() : g2_fold_width<6>(), G2_FOLD_BY, G2_FOLD_BZ};
 }
 
 // brick shapes: columns in x, columns in y, voxels per column (z)

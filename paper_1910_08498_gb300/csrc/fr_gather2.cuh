@@ -42,11 +42,10 @@
 // every point of the extended plane within a of the voxel has (R c)_x > 0, so
 // a column c_x > 0 receives the stored pixel c, a column c_x < 0 the stored -c
 // conjugated, and the column c_x = 0 both (0, c_y) and, conjugated, (0, -c_y):
-// exactly what the two entries read.  The bricks of this kernel's main launch
-// tile x >= floor(a) + 1.  The fold columns |x| <= floor(a), where the fold
-// predicate itself has to be evaluated per pixel, are computed by a second
-// instantiation over those columns only (FOLD), in footprints 4 columns wide so
-// that three of four lanes hold fold columns: there a stored pixel k counts in
+// exactly what the two entries read.  The main bricks tile x >= floor(a) + 1.
+// The fold columns |x| <= floor(a), where the fold predicate itself has to be
+// evaluated per pixel, have units of their own (FOLD), in footprints 4 (8) columns
+// wide so that three of four (five of eight) lanes hold fold columns: there a stored pixel k counts in
 // the entry as stored when it is not folded and in the reflected entry when it
 // is (exact sign of R00 k_x + R01 k_y, found once per pixel of the patch and
 // kept as one bit).  Polynomial weights only.
@@ -188,14 +187,21 @@ __device__ __forceinline__ bool g2_box(const float2 *cp, const float2 *p, float 
   return ties;
 }
 
-// Fold a warp's partial sums (s_acc: [3][WV], slot (y FW + x) 8 + z) into HBM
-// and clear them: straight into the double-float accumulators (error-free
-// TwoSum) when the warp is the only writer of its voxels, else into the float4
-// scratch with atomics (merged after the launch).  The loads of four z levels
-// are issued together: one after the other, their latency made a flush take
-// four times as long.
+// Clear a warp's partial sums (16-byte aligned).
+template <int WV>
+__device__ __forceinline__ void g2_clear(float *s_acc, int lane) {
+#pragma unroll 4
+  for (int i = lane; i < 3 * WV / 4; i += 32)
+    reinterpret_cast<float4 *>(s_acc)[i] = make_float4(0.f, 0.f, 0.f, 0.f);
+}
+
+// Fold a warp's partial sums (s_acc: [3][WV], slot (y FW + x) 8 + z) into HBM:
+// straight into the double-float accumulators (error-free TwoSum) when the warp
+// is the only writer of its voxels, else into the float4 scratch with atomics
+// (merged after the launch).  The loads of four z levels are issued together:
+// one after the other, their latency made a flush take four times as long.
 template <int FW, int KB>
-__device__ __noinline__ void g2_flush(const InsertArgs &args, float *s_acc, int fx0, int fy0,
+__device__ __noinline__ void g2_flush(const InsertArgs &args, const float *s_acc, int fx0, int fy0,
                                       int z0, bool to_scratch) {
   using SH = G2Shape<FW, KB>;
   constexpr int WV = SH::WV, ZC = SH::ZC, ZG = 4;
@@ -207,16 +213,20 @@ __device__ __noinline__ void g2_flush(const InsertArgs &args, float *s_acc, int 
     const int col = (k / (ZC / ZG)) * 32 + lane, t0 = k % (ZC / ZG) * ZG;
     const int vx = fx0 + col % FW, vy = fy0 + col / FW;
     if (vx > g.H || vy > g.H) continue;
-    const float *s = s_acc + col * ZC + t0;
+    float s[3][ZG];  // four z levels of the three sums, as 16-byte groups
+#pragma unroll
+    for (int c = 0; c < 3; ++c) {
+      const float4 q = *reinterpret_cast<const float4 *>(s_acc + c * WV + col * ZC + t0);
+      s[c][0] = q.x, s[c][1] = q.y, s[c][2] = q.z, s[c][3] = q.w;
+    }
     const size_t slice = (size_t)g.D * g.NXa;
     const size_t v0 = ((size_t)(z0 + t0 + g.H) * g.D + (size_t)(vy + g.H)) * g.NXa + (size_t)(vx - g.xa0);
     if (to_scratch) {
+      float4 *q = args.scratch + v0;
 #pragma unroll
-      for (int t = 0; t < ZG; ++t) {
-        const float4 v = make_float4(s[t], s[WV + t], s[2 * WV + t], 0.f);
-        if (z0 + t0 + t <= g.H && (v.x != 0.f || v.y != 0.f || v.z != 0.f))
-          atomicAdd(args.scratch + v0 + t * slice, v);
-      }
+      for (int t = 0; t < ZG; ++t, q += slice)
+        if (z0 + t0 + t <= g.H && (s[0][t] != 0.f || s[1][t] != 0.f || s[2][t] != 0.f))
+          atomicAdd(q, make_float4(s[0][t], s[1][t], s[2][t], 0.f));
     } else {
       float h[3 * ZG], l[3 * ZG];
 #pragma unroll
@@ -230,20 +240,17 @@ __device__ __noinline__ void g2_flush(const InsertArgs &args, float *s_acc, int 
         }
 #pragma unroll
       for (int t = 0; t < ZG; ++t) {
-        const float add[3] = {s[t], s[WV + t], s[2 * WV + t]};
-        if (z0 + t0 + t > g.H || (add[0] == 0.f && add[1] == 0.f && add[2] == 0.f)) continue;
+        if (z0 + t0 + t > g.H || (s[0][t] == 0.f && s[1][t] == 0.f && s[2][t] == 0.f)) continue;
 #pragma unroll
         for (int c = 0; c < 3; ++c) {
           float *q = args.acc + c * args.plane + v0 + t * slice;
-          dd_add(h[3 * t + c], l[3 * t + c], add[c]);
+          dd_add(h[3 * t + c], l[3 * t + c], s[c][t]);
           q[0] = h[3 * t + c];
           q[3 * args.plane] = l[3 * t + c];
         }
       }
     }
   }
-  __syncwarp();
-  for (int i = lane; i < 3 * WV; i += 32) s_acc[i] = 0.f;
   __syncwarp();
 }
 
@@ -312,7 +319,7 @@ __device__ __forceinline__ void gather2_warp(const InsertArgs &args, const Inser
     tmax[c] = vx <= g.H && vy <= g.H && (!FOLD || vx <= -g.xa0) ? min(ZC - 1, g.H - z0) : -1;
   }
 
-  for (int i = lane; i < 3 * WV; i += 32) s_acc[i] = 0.f;
+  g2_clear<WV>(s_acc, lane);
   __syncwarp();
   // optional phase counters (fr_options.debug bit 1): cycles of cull, item
   // generation with the patches (PH_QUEUE), evaluation rounds (PH_DRAIN_FAST)
@@ -653,6 +660,8 @@ __device__ __forceinline__ void gather2_warp(const InsertArgs &args, const Inser
       if (since_flush > GATHER_FLUSH - lcap) {
         const long long tf = tick();
         g2_flush<FW, KB>(args, s_acc, fx0, fy0, z0, to_scratch);
+        g2_clear<WV>(s_acc, lane);
+        __syncwarp();
         clocked(PH_FLUSH, tf);
         since_flush = 0;
       }
@@ -665,37 +674,92 @@ __device__ __forceinline__ void gather2_warp(const InsertArgs &args, const Inser
   clocked(PH_WARP_CYCLES, t_start);
 }
 
-// One warp per CTA: CTA b takes footprint b % W of work unit args.units[b / W]
-// (W footprints a brick).  Warps of one brick never wait for one another, but a
-// CTA holds its shared memory until its last warp ends: with two and four warps
-// a CTA 17 % of the resident warp slots stood idle.  MINW: resident warps per SM
-// the register allocation must allow (16: at most 128 registers per thread, and
-// what shared memory holds; more warps than that are not resident).  FW, FOLD:
-// see gather2_warp.
-template <int BX, int BY, int BZ, int F16, int MINW, int KB = 4, int FW = 8, int FOLD = 0>
+// Bricks of the fold columns: one footprint wide (three fold columns for a < 2,
+// five for 2 <= a < 3), 32 x 8.
+template <int KB>
+__host__ __device__ constexpr int g2_fold_width() {
+  return KB == 4 ? 4 : 8;
+}
+constexpr int G2_FOLD_BY = 32, G2_FOLD_BZ = 8;
+
+// Dynamic shared memory of a launch: a warp of the main or the fold columns.
+template <int KB>
+__host__ __device__ constexpr size_t gather2_smem(int chunk) {
+  const size_t m = gather2_warp_smem<8, KB, 0>(chunk),
+               f = gather2_warp_smem<g2_fold_width<KB>(), KB, 1>(chunk);
+  return m > f ? m : f;
+}
+
+// Work unit k of a launch without a unit list: split k / (bricks) of brick k %
+// (bricks) of those that tile x in [x0, x1], of as many splits as its expected
+// images (brick_unit_loads' estimate) over unit_share; false if it has fewer.
+template <int BX, int BY, int BZ>
+__device__ __forceinline__ bool g2_implicit_unit(const InsertArgs &args, int x0, int x1, int k,
+                                                 int4 &unit) {
+  const Geom &g = args.g;
+  const int nbx = (x1 - x0 + BX) / BX, nby = (g.D + BY - 1) / BY, nbz = (g.D + BZ - 1) / BZ;
+  const int b = k % (nbx * nby * nbz), s = k / (nbx * nby * nbz);
+  const int bx = b % nbx, by = b / nbx % nby, bz = b / (nbx * nby);
+  const float hx = 0.5f * (BX - 1), hy = 0.5f * (BY - 1), hz = 0.5f * (BZ - 1);
+  const float cx = x0 + bx * BX + hx, cy = -g.H + by * BY + hy, cz = -g.H + bz * BZ + hz;
+  const float d = sqrtf(cx * cx + cy * cy + cz * cz), r = g.a + sqrtf(hx * hx + hy * hy + hz * hz);
+  const float load = args.n * ((d <= r ? 1.0f : r / d) + 0.02f);
+  const int ns = max(1, min((int)ceilf(load / args.unit_share), args.unit_most));
+  unit = make_int4(bx, by, bz, s | (ns << 16) | (1 << 30));
+  return s < ns;
+}
+
+// One warp per CTA: after the nfold units of the fold columns (the few heavy ones
+// first), CTA b takes footprint b % W of work unit args.units[b / W] (W footprints
+// a brick).  Warps of one brick never wait for one another, but a CTA holds its
+// shared memory until its last warp ends: with two and four warps a CTA 17 % of
+// the resident warp slots stood idle.  Both kinds of unit in one launch: as a
+// second kernel on a side stream the fold columns cost a fork and a join.  MINW:
+// resident warps per SM the register allocation must allow (16: at most 128
+// registers per thread, and what shared memory holds; more are not resident).
+template <int BX, int BY, int BZ, int F16, int MINW, int KB = 4>
 __global__ void __launch_bounds__(32, MINW)
 gather2_kernel(const __grid_constant__ InsertArgs args) {
   extern __shared__ __align__(16) unsigned char smem[];
-  constexpr int W = g2_warps<BX, BY, BZ, FW>();
-  gather2_warp<BX, BY, BZ, F16, KB, FW, FOLD>(args, args, args.images, smem,
-                                          args.units[blockIdx.x / W], (int)(blockIdx.x % W));
+  constexpr int FW = g2_fold_width<KB>(), W = g2_warps<BX, BY, BZ, 8>(),
+                WF = g2_warps<FW, G2_FOLD_BY, G2_FOLD_BZ, FW>();
+  const Geom &g = args.g;
+  const int nf = args.nfold * WF;
+  int4 unit;
+  if ((int)blockIdx.x < nf) {
+    const int k = blockIdx.x / WF;
+    if (args.units) unit = args.fold[k];
+    else if (!g2_implicit_unit<FW, G2_FOLD_BY, G2_FOLD_BZ>(args, g.xa0, -g.xa0, k, unit)) return;
+    gather2_warp<FW, G2_FOLD_BY, G2_FOLD_BZ, F16, KB, FW, 1>(args, args, args.images, smem, unit,
+                                                             (int)(blockIdx.x % WF));
+  } else {
+    const int b = (int)blockIdx.x - nf, k = b / W;
+    if (args.units) unit = args.units[k];
+    else if (!g2_implicit_unit<BX, BY, BZ>(args, 1 - g.xa0, g.H, k, unit)) return;
+    gather2_warp<BX, BY, BZ, F16, KB>(args, args, args.images, smem, unit, b % W);
+  }
 }
 
-// Several batches in one launch: CTA b takes footprint b % W of work item
-// p.items[b / W] = {bx | by << 10 | bz << 20, split word, batch, slot} of batch
-// p.descs[batch]; geometry, weight polynomial and list capacity, common to the
-// launch's batches, are read from p.base (kernel parameters: constant operands
-// in the inner loops), the batch's own arguments (rotations, volume) from its
+// Several batches in one launch: work items p.items[k] = {bx | by << 10 | bz <<
+// 20, split word, batch, slot} of batch p.descs[batch], first those of the fold
+// columns; geometry, weight polynomial and list capacity, common to the launch's
+// batches, are read from p.base (kernel parameters: constant operands in the
+// inner loops), the batch's own arguments (rotations, volume) from its
 // descriptor.
-template <int BX, int BY, int BZ, int F16, int MINW, int KB = 4, int FW = 8, int FOLD = 0>
+template <int BX, int BY, int BZ, int F16, int MINW, int KB = 4>
 __global__ void __launch_bounds__(32, MINW)
 gather2_multi_kernel(const __grid_constant__ MultiLaunch p) {
   extern __shared__ __align__(16) unsigned char smem[];
-  constexpr int W = g2_warps<BX, BY, BZ, FW>();
-  const int4 it = p.items[blockIdx.x / W];
+  constexpr int FW = g2_fold_width<KB>(), W = g2_warps<BX, BY, BZ, 8>(),
+                WF = g2_warps<FW, G2_FOLD_BY, G2_FOLD_BZ, FW>();
+  const int nf = p.nfold * WF, b = (int)blockIdx.x - nf;
+  const int4 it = p.items[b < 0 ? (int)blockIdx.x / WF : p.nfold + b / W];
   const int4 unit = make_int4(it.x & 1023, (it.x >> 10) & 1023, (it.x >> 20) & 1023, it.y);
-  gather2_warp<BX, BY, BZ, F16, KB, FW, FOLD>(p.descs[it.z], p.base, p.images[it.w], smem, unit,
-                                          (int)(blockIdx.x % W));
+  if (b < 0)
+    gather2_warp<FW, G2_FOLD_BY, G2_FOLD_BZ, F16, KB, FW, 1>(p.descs[it.z], p.base, p.images[it.w],
+                                                             smem, unit, (int)(blockIdx.x % WF));
+  else
+    gather2_warp<BX, BY, BZ, F16, KB>(p.descs[it.z], p.base, p.images[it.w], smem, unit, b % W);
 }
 
 }  // namespace fr

@@ -55,8 +55,15 @@ struct InsertArgs {
   // gather geometry
   int nbx, nby, nbz;    // bricks per axis
   int chunk;            // capacity of a warp's image list
-  const int4 *units;    // work units: (brick x, y, z, split | nsplit << 16), one per CTA
+  const int4 *units;    // work units: (brick x, y, z, split | nsplit << 16)
   int nunits;
+  // direct-drain gather: units of the fold columns, computed in the same launch.
+  // units == null (no list in device memory): each of nunits / nfold is one of
+  // unit_most splits of a brick, which uses as many as its load over unit_share
+  const int4 *fold;
+  int nfold;
+  float unit_share;
+  int unit_most;
   int any_split;        // 1 if some unit shares its brick with other units
   unsigned long long *phase;  // optional per-phase cycle and item counters (PH_*), or null
   // scatter
@@ -112,6 +119,8 @@ cudaError_t launch_scatter(int threads, int wmode, const InsertArgs &a, cudaStre
 cudaError_t launch_merge_scratch(const InsertArgs &a, cudaStream_t st);
 // 1 / (A&S 9.8.2 polynomial at 3.75 / alpha): the constant of the on-the-fly weights
 float otf_inv_pa(double alpha);
+// coefficients (power basis in x = 2 r^2 / a^2 - 1) of the weight polynomial
+void weight_polynomial(double alpha, float *poly);
 // record a CUDA error for fr_last_cuda_error
 void fr_note_cuda_error(int e);
 cudaError_t launch_finalize(const Geom &g, const float *acc, size_t plane, float2 *V, float *W,
@@ -125,10 +134,9 @@ cudaError_t launch_debug_blob(const InsertArgs &a, const float *r2, int m, int m
 // number of gather shapes and their geometry
 int num_gather_shapes();
 GatherShape gather_shape(int id);
-// the direct-drain gather over the fold columns |x| <= floor(a) only, in
-// bricks of fold_shape(KB) (one footprint wide), polynomial weights
+// bricks of the direct-drain gather's fold-column units (|x| <= floor(a)), one
+// footprint wide: 4 columns (8 for KB = 6) x 32 x 8
 GatherShape fold_shape(int kb);
-cudaError_t launch_gather_fold(const InsertArgs &a, cudaStream_t st);
 // dynamic shared memory a gather launch needs
 size_t gather_smem_bytes(const GatherShape &sh, int wmode, int lut_n, int chunk);
 size_t gather_persistent_smem_bytes(const GatherShape &sh, int chunk);
@@ -152,20 +160,14 @@ constexpr int MULTI_MAX = 64;  // batches per multi-batch launch
 struct MultiLaunch {
   InsertArgs base;           // common arguments: geometry, weights, list capacity
   const InsertArgs *descs;   // device, one per batch (images, rot, n, acc, scratch, err)
-  const int4 *items;         // device, {bx | by << 10 | bz << 20, split word, batch, slot}
+  const int4 *items;         // device, {bx | by << 10 | bz << 20, split word, batch, slot}:
+  int nfold;                 // nfold items of the fold columns, then nitems of the rest
   int nitems;
-  int priority;              // launch priority (cudaLaunchAttributePriority), 0 = the stream's
   const void *images[MULTI_MAX];  // images of the launch's batches, by slot (read in the inner loop)
 };
-// launch kernel fn (taking one MultiLaunch) with per_item CTAs for each of
-// p.nitems work items, at p.priority
-cudaError_t launch_multi(const void *fn, const MultiLaunch &p, int per_item, int threads,
-                         size_t smem, cudaStream_t st);
-// the direct-drain gather (fold columns excluded), FP32 or FP16 images
+// the direct-drain gather, FP32 or FP16 images
 cudaError_t launch_gather2_multi(int shape_id, int minw, int f16, const MultiLaunch &p,
                                  cudaStream_t st);
-// the direct-drain gather over the fold columns
-cudaError_t launch_gather_fold_multi(int f16, const MultiLaunch &p, cudaStream_t st);
 
 // MLP kernels
 cudaError_t mlp_forward(const float *params, const float *x, int m, float *y, cudaStream_t st);

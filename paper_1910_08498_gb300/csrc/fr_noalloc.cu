@@ -1,8 +1,11 @@
-// fr_noalloc.cu -- fr_insert_noalloc: the atomic scatter insertion with its
-// scratch volume in a fixed array of static device memory, for callers that
-// must not enter the device allocator (they may be sharing the device with
-// latency-bound streams that a cudaMalloc/cudaFree would synchronise, or hold
-// all device memory in their own pool allocator).  Nothing here allocates:
+// fr_noalloc.cu -- fr_insert_noalloc: the insertion with its scratch volume in a
+// fixed array of static device memory, for callers that must not enter the
+// device allocator (they may be sharing the device with latency-bound streams
+// that a cudaMalloc/cudaFree would synchronise, or hold all device memory in
+// their own pool allocator).  The direct-drain gather runs without a unit list
+// (its CTAs work theirs out), every unit adding to the scratch; the atomic
+// scatter stays where the gather cannot decide as exactly or has no box (see
+// gather_here).  Nothing here allocates:
 // no cudaMalloc, no cudaFree, no allocating library routine; the scratch
 // address is looked up once per device with cudaGetSymbolAddress.
 #include <cuda_runtime.h>
@@ -12,6 +15,7 @@
 #include <cstdint>
 #include <mutex>
 
+#include "fr_ctx.h"
 #include "fr_device.cuh"
 #include "fr_internal.h"
 #include "fr_noalloc.h"
@@ -54,6 +58,53 @@ __global__ void noalloc_add_kernel(const Geom g, float4 *__restrict__ scratch,
       scratch[v] = make_float4(0.f, 0.f, 0.f, 0.f);
     }
   }
+}
+
+// The scatter decides r <= a as the real numbers do for every candidate; the
+// gather does only in the fold columns for a >= 2.  With a^2 within 1e-4 of an
+// integer whole lattices of candidates can sit on the blob's edge (the DC pixel
+// against the axes' voxels for every rotation), so such radii keep the scatter.
+// So does alpha > 16, where the weight polynomial is less accurate than the
+// scatter's Bessel approximations (2e-7), and an image too small for a box.
+// Small batches also stay: up to about 4e5 pixels (7e5 for 6 x 6 boxes) the
+// scatter is as fast or faster (S = 32, 100 images: 31 against 36 us; S = 64, 64
+// images, a = 2.5: 90 against 92), beyond it slower (S = 64, 2000 images: 931
+// against 558 us, a = 2.5: 2025 against 1253; S = 48, 600 FP16 images: 159
+// against 138).
+bool gather_here(const Geom &g, int n) {
+  const double a2 = (double)g.a * (double)g.a;
+  return std::fabs(a2 - std::round(a2)) > 1e-4 * a2 && g.alpha <= 16.0f && g.H >= g.KB - 1 &&
+         (double)n * g.S * g.NX >= (g.KB == 4 ? 4e5 : 7e5);
+}
+
+// weight polynomial of the last alpha asked for (12 numbers; no allocation)
+void cached_polynomial(float alpha, float *poly) {
+  static std::mutex mu;
+  static float last = -1.0f, c[POLY_N];
+  std::lock_guard<std::mutex> lk(mu);
+  if (alpha != last) {
+    weight_polynomial((double)alpha, c);
+    last = alpha;
+  }
+  std::copy(c, c + POLY_N, poly);
+}
+
+// Expected images over all bricks of shape sh that tile x in [x0, x1], for a
+// batch of n; *bricks: how many they are.
+double brick_images(const Geom &g, const GatherShape &sh, int x0, int x1, int n, int *bricks) {
+  const int nbx = (x1 - x0 + sh.bx) / sh.bx, nby = (g.D + sh.by - 1) / sh.by,
+            nbz = (g.D + sh.zc - 1) / sh.zc;
+  const double hx = 0.5 * (sh.bx - 1), hy = 0.5 * (sh.by - 1), hz = 0.5 * (sh.zc - 1);
+  const double r = g.a + std::sqrt(hx * hx + hy * hy + hz * hz);
+  double total = 0;
+  for (int b = 0; b < nbx * nby * nbz; ++b) {
+    const double cx = x0 + b % nbx * sh.bx + hx, cy = -g.H + b / nbx % nby * sh.by + hy,
+                 cz = -g.H + b / (nbx * nby) * sh.zc + hz;
+    const double d = std::sqrt(cx * cx + cy * cy + cz * cz);
+    total += n * ((d <= r ? 1.0 : r / d) + 0.02);
+  }
+  *bricks = nbx * nby * nbz;
+  return total;
 }
 
 int cuda_status(cudaError_t e) {
@@ -127,11 +178,31 @@ extern "C" int fr_insert_noalloc(int S, float a, float alpha, const void *images
   const int add_threads = 256;
   const int add_blocks = (int)std::min<size_t>((cells + add_threads - 1) / add_threads,
                                                (size_t)sms * 8);
+  constexpr int SHAPE = 1;  // 16 x 8 x 8 bricks
+  const bool gather_any = gather_here(g, std::min(n, NOALLOC_SUB));
+  if (gather_any) {
+    cached_polynomial(alpha, args.poly);
+    for (int k = 0; k < POLY_N; ++k) args.poly2[k] = make_float2(args.poly[k], args.poly[k]);
+    args.chunk = 64;
+    args.any_split = 1;
+  }
   for (int i0 = 0; i0 < n; i0 += NOALLOC_SUB) {
     args.n = std::min(NOALLOC_SUB, n - i0);
     args.images = static_cast<const unsigned char *>(images) + (size_t)i0 * img_bytes;
     args.rot = rotations + (size_t)i0 * 9;
-    e = launch_scatter(256, W_OTF, args, st, 0, nullptr);
+    if (gather_any && gather_here(g, args.n)) {
+      int bricks = 0, fold_bricks = 0;
+      const double total = brick_images(g, gather2_shape(SHAPE), 1 - g.xa0, g.H, args.n, &bricks);
+      brick_images(g, fold_shape(g.KB), g.xa0, -g.xa0, args.n, &fold_bricks);
+      args.unit_share = (float)unit_share(total, sms, MAIN_UNITS_PER_SM, true);
+      // splits of a central brick, which every image crosses
+      args.unit_most = std::max(1, std::min({64, args.n / 2, (int)std::ceil(1.02 * args.n / args.unit_share)}));
+      args.nunits = bricks * args.unit_most;
+      args.nfold = fold_bricks * args.unit_most;
+      e = launch_gather2(SHAPE, 16, args, st, 0, nullptr);
+    } else {
+      e = launch_scatter(256, W_OTF, args, st, 0, nullptr);
+    }
     if (e != cudaSuccess) return cuda_status(e);
     noalloc_add_kernel<<<add_blocks, add_threads, 0, st>>>(g, scratch, static_cast<float2 *>(V), W);
     e = cudaGetLastError();

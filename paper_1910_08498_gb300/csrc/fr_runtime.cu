@@ -79,6 +79,20 @@ void chebyshev_power_basis(F f, double *mono) {
 
 namespace fr {
 
+// the blob weight as a function of x = 2 r^2 / a^2 - 1 in [-1, 1]; depends on
+// alpha alone
+static double blob_of_x(double alpha, double i0a, double x) {
+  const double t = std::min(1.0, std::max(0.0, 0.5 * (x + 1.0)));  // (r/a)^2
+  return std::cyl_bessel_i(0.0, alpha * std::sqrt(1.0 - t)) / i0a;
+}
+
+void weight_polynomial(double alpha, float *poly) {
+  const double i0a = std::cyl_bessel_i(0.0, alpha);
+  double mono[POLY_N];
+  chebyshev_power_basis([&](double x) { return blob_of_x(alpha, i0a, x); }, mono);
+  for (int k = 0; k < POLY_N; ++k) poly[k] = (float)mono[k];
+}
+
 InsertArgs base_args(const fr_ctx *c) {
   InsertArgs a{};
   a.g = c->g;
@@ -112,16 +126,6 @@ bool alloc_fault(fr_ctx *c) {
   if (--c->alloc_countdown) return false;
   c->opt.fault_alloc = 0;  // one shot: a later fr_set_options from fr_get_options does not re-arm it
   return true;
-}
-
-int ensure_side_stream(fr_ctx *c) {
-  if (c->side) return FR_OK;
-  int lo = 0, hi = 0;
-  FR_CUDA(cudaDeviceGetStreamPriorityRange(&lo, &hi));
-  FR_CUDA(cudaStreamCreateWithPriority(&c->side, cudaStreamNonBlocking, hi));
-  FR_CUDA(cudaEventCreateWithFlags(&c->ev_fork, cudaEventDisableTiming));
-  FR_CUDA(cudaEventCreateWithFlags(&c->ev_join, cudaEventDisableTiming));
-  return FR_OK;
 }
 
 int ensure_scratch(fr_ctx *c) {
@@ -216,8 +220,7 @@ Config effective_config(const fr_ctx *c, int id) {
 
 // Work units of a gather launch of this batch alone, heaviest first (so the
 // largest ones start first), cached on the device per (shape, n).
-static int gather_units(fr_ctx *c, const Config &cfg, int n, InsertArgs &a,
-                        const int4 **fold = nullptr, int *nfold = nullptr, int *fold_split = nullptr) {
+static int gather_units(fr_ctx *c, const Config &cfg, int n, InsertArgs &a) {
   const int algo = cfg.algo == ALGO_GATHER2 ? ALGO_GATHER2 : ALGO_GATHER;
   for (int k = 0; k < 8; ++k) {
     fr_ctx::Units &u = c->units[k];
@@ -225,7 +228,8 @@ static int gather_units(fr_ctx *c, const Config &cfg, int n, InsertArgs &a,
       a.units = u.dev;
       a.nunits = u.count;
       a.any_split = u.any_split;
-      if (fold) { *fold = u.fold; *nfold = u.fold_count; *fold_split = u.fold_split; }
+      a.fold = u.fold;
+      a.nfold = u.fold_count;
       return FR_OK;
     }
   }
@@ -233,9 +237,9 @@ static int gather_units(fr_ctx *c, const Config &cfg, int n, InsertArgs &a,
   std::vector<UnitLoad> us, fs;
   int any_split = 0, fsplit = 0;
   if (algo == ALGO_GATHER2) {
-    // the direct-drain gather's bricks tile x in [floor(a) + 1, H]; the fold
-    // columns x in [-floor(a), floor(a)] go to its fold-column launch in
-    // bricks one footprint wide, split finely (they are few and heavy)
+    // the direct-drain gather's main bricks tile x in [floor(a) + 1, H]; the
+    // fold columns x in [-floor(a), floor(a)] have units in bricks one
+    // footprint wide, split finely (they are few and heavy)
     brick_unit_loads(c, gather2_shape(cfg.shape), 1 - c->g.xa0, c->g.H, n, 0.0, MAIN_UNITS_PER_SM,
                      true, us, any_split);
     brick_unit_loads(c, fold_shape(c->g.KB), c->g.xa0, -c->g.xa0, n, 0.0, FOLD_UNITS_PER_SM, true,
@@ -262,14 +266,14 @@ static int gather_units(fr_ctx *c, const Config &cfg, int n, InsertArgs &a,
   u.algo = algo;
   u.n = n;
   u.count = (int)us.size();
-  u.any_split = any_split;
+  u.any_split = any_split | fsplit;
   u.fold = u.dev + us.size();
   u.fold_count = (int)fs.size();
-  u.fold_split = fsplit;
   a.units = u.dev;
   a.nunits = u.count;
-  a.any_split = any_split;
-  if (fold) { *fold = u.fold; *nfold = u.fold_count; *fold_split = u.fold_split; }
+  a.any_split = u.any_split;
+  a.fold = u.fold;
+  a.nfold = u.fold_count;
   return FR_OK;
 }
 
@@ -288,15 +292,9 @@ int prepare_config(fr_ctx *c, int id, int n) {
   const Config cfg = effective_config(c, id);
   InsertArgs a = base_args(c);
   if (cfg.algo == ALGO_GATHER || cfg.algo == ALGO_GATHER2) {
-    const int4 *fold = nullptr;
-    int nfold = 0, fold_split = 0;
-    int rc = gather_units(c, cfg, n, a, &fold, &nfold, &fold_split);
+    int rc = gather_units(c, cfg, n, a);
     if (rc) return rc;
-    if (cfg.algo == ALGO_GATHER2) {
-      rc = ensure_side_stream(c);
-      if (rc) return rc;
-    }
-    return (a.any_split || fold_split) ? ensure_scratch(c) : FR_OK;
+    return a.any_split ? ensure_scratch(c) : FR_OK;
   }
   return ensure_scratch(c);
 }
@@ -312,40 +310,20 @@ int run_config(fr_ctx *c, int id, const void *images, int f16, const float *rot,
   a.n = n;
   if (cfg.algo == ALGO_GATHER || cfg.algo == ALGO_GATHER2) {
     gather_geometry(c, cfg, a);
-    const int4 *fold = nullptr;
-    int nfold = 0, fold_split = 0;
-    int rc = gather_units(c, cfg, n, a, &fold, &nfold, &fold_split);
+    int rc = gather_units(c, cfg, n, a);
     if (rc) return rc;
-    if (cfg.algo == ALGO_GATHER2) a.any_split |= fold_split;
     if (a.any_split) {
       rc = ensure_scratch(c);
       if (rc) return rc;
       a.scratch = c->scratch;
     }
-    cudaError_t e;
-    if (cfg.algo == ALGO_GATHER2) {
-      // the fold columns: the fold-column instantiation, on the side stream
-      // so that its few heavy units run beside the main launch (disjoint
-      // voxels; split units add to the scratch with atomics, merged after both)
-      rc = ensure_side_stream(c);
-      if (rc) return rc;
-      InsertArgs f = a;
-      f.units = fold;
-      f.nunits = nfold;
-      e = cudaEventRecord(c->ev_fork, st);
-      if (e == cudaSuccess) e = cudaStreamWaitEvent(c->side, c->ev_fork, 0);
-      if (e == cudaSuccess) e = launch_gather_fold(f, c->side);
-      if (e == cudaSuccess) e = cudaEventRecord(c->ev_join, c->side);
-      if (e != cudaSuccess) return cuda_fail(e);
-      e = launch_gather2(cfg.shape, cfg.minw, a, st, 0, nullptr);
-      if (e == cudaSuccess) e = cudaStreamWaitEvent(st, c->ev_join, 0);
-    } else {
-      e = launch_gather(cfg.shape, cfg.wmode, a, st, 0, nullptr);
-    }
+    const cudaError_t e = cfg.algo == ALGO_GATHER2
+                              ? launch_gather2(cfg.shape, cfg.minw, a, st, 0, nullptr)
+                              : launch_gather(cfg.shape, cfg.wmode, a, st, 0, nullptr);
     if (e != cudaSuccess) return cuda_fail(e);
     if (a.any_split) {
-      e = launch_merge_scratch(a, st);
-      if (e != cudaSuccess) return cuda_fail(e);
+      const cudaError_t em = launch_merge_scratch(a, st);
+      if (em != cudaSuccess) return cuda_fail(em);
     }
     return FR_OK;
   }
@@ -554,13 +532,7 @@ int fr_create(int S, const fr_blob *blob, fr_ctx **out) {
 
   // polynomial weights: b as a function of x = 2 r^2 / a^2 - 1 in [-1, 1]
   {
-    auto bx = [&](double x) {
-      double t = std::min(1.0, std::max(0.0, 0.5 * (x + 1.0)));  // (r/a)^2
-      return std::cyl_bessel_i(0.0, alpha * std::sqrt(1.0 - t)) / i0a;
-    };
-    double mono[POLY_N];
-    chebyshev_power_basis(bx, mono);
-    for (int k = 0; k < POLY_N; ++k) c->poly[k] = (float)mono[k];
+    weight_polynomial(alpha, c->poly);
     // measured error of the FP32 even/odd evaluation the device performs
     double worst = 0;
     for (int i = 0; i <= 20000; ++i) {
@@ -572,7 +544,7 @@ int fr_create(int S, const fr_blob *blob, fr_ctx **out) {
         o = std::fma(o, y, c->poly[2 * k + 1]);
       }
       const float p = std::fma(o, x, e);
-      worst = std::max(worst, std::fabs((double)p - bx((double)x)));
+      worst = std::max(worst, std::fabs((double)p - blob_of_x(alpha, i0a, (double)x)));
     }
     c->poly_err = worst;
   }
@@ -596,9 +568,6 @@ int fr_destroy(fr_ctx *c) {
   cudaFree(c->d_phase);
   cudaFree(c->d_mlp);
   for (auto &u : c->units) cudaFree(u.dev);
-  if (c->ev_fork) cudaEventDestroy(c->ev_fork);
-  if (c->ev_join) cudaEventDestroy(c->ev_join);
-  if (c->side) cudaStreamDestroy(c->side);
   delete c;
   return FR_OK;
 }
@@ -747,14 +716,9 @@ int fr_insert_launches(fr_ctx *c, int id, int n, int *out) {
     return FR_OK;
   }
   InsertArgs a = base_args(c);
-  const int4 *fold = nullptr;
-  int nfold = 0, fold_split = 0;
-  int rc = gather_units(c, cfg, n, a, &fold, &nfold, &fold_split);
+  int rc = gather_units(c, cfg, n, a);
   if (rc) return rc;
-  if (cfg.algo == ALGO_GATHER2)  // main launch, fold-column launch, merge if split
-    *out = 2 + ((a.any_split || fold_split) ? 1 : 0);
-  else
-    *out = 1 + (a.any_split ? 1 : 0);
+  *out = 1 + (a.any_split ? 1 : 0);
   return FR_OK;
 }
 

@@ -12,6 +12,7 @@ import numpy as np
 import pytest
 import torch
 
+from paper_1910_08498_gb300 import _lib as L
 from paper_1910_08498_gb300 import inputs
 from tests.helpers import TOL_F32, gpu_insert, oracle_insert, rel_err, worst
 
@@ -35,6 +36,29 @@ def test_patch_edges_match_oracle(S, a, f16):
     Vr, Wr, _ = oracle_insert(S, batches, a=a, f16=f16)
     assert rel_err(V, Vr) <= TOL_F32, worst(V, Vr, S)
     assert rel_err(W, Wr) <= TOL_F32, worst(W, Wr, S)
+
+
+@pytest.mark.parametrize("f16", [False, True])
+@pytest.mark.parametrize("a", [0.6, 1.0, 1.5, 1.9, 2.5, 2.999])
+@pytest.mark.parametrize("S,n", [(8, 1), (8, 40), (10, 3), (16, 17), (30, 33), (46, 15), (64, 130), (64, 400),
+                                 (46, 700)])
+def test_no_allocation_call_matches_oracle(S, n, a, f16):
+    """Batches and radii that keep the scatter (small ones, a = 1), and the
+    gather with units worked out by the CTAs themselves.  700 images: FP32 sums
+    of a voxel's about 700 terms, within the bar by the scatter's own test of
+    1024-image sub-batches."""
+    a = float(np.float32(a))
+    img, rot = inputs.make_batch(S, n, 11 * S + n)
+    perm = inputs.proper_signed_permutations()
+    rot[:min(n, 3)] = perm[[3, 9, 20]][:min(n, 3)]
+    V = torch.zeros((S + 1) ** 3, dtype=torch.complex64, device="cuda")
+    W = torch.zeros((S + 1) ** 3, dtype=torch.float32, device="cuda")
+    dev = (inputs.to_half(img) if f16 else img).cuda()
+    assert L.fr_insert_noalloc(S, dev, rot.cuda(), V, W, a=a, alpha=15.0) == L.FR_OK
+    Vr, Wr, _ = oracle_insert(S, [(img, rot)], a=a, f16=f16)
+    Vn, Wn = V.cpu().numpy(), W.cpu().numpy()
+    assert rel_err(Vn, Vr) <= TOL_F32, worst(Vn, Vr, S)
+    assert rel_err(Wn, Wr) <= TOL_F32, worst(Wn, Wr, S)
 
 
 def test_pixels_outside_the_blob_do_not_reach_a_voxel():
