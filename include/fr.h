@@ -223,11 +223,12 @@ int fr_finalize(fr_ctx *ctx, void *V, float *W, void *stream);
  *          times (-1)^(kx + j) when center != 0 (the image origin taken at
  *          pixel (S/2, S/2) instead of (0, 0)); FR_F16 rounds to nearest half.
  *   n      0 <= n <= 2^24 (0: nothing).
- * The transforms are the CUDA toolkit's cuFFT (batched R2C, loaded at run
- * time; FR_ERR_UNSUPPORTED if it cannot be loaded), in chunks of about 256 MB
- * of spectra (at least 256 images); the sign and the FP16 conversion are a
- * kernel of this library.  Allocates on first use the plans and, for FR_F16,
- * a staging buffer of one chunk.
+ * For S = 64, 128 and 256 the transforms are this library's kernels; for other
+ * sizes the CUDA toolkit's cuFFT (batched R2C, loaded at run time;
+ * FR_ERR_UNSUPPORTED if it cannot be loaded) with the sign and the FP16
+ * conversion a kernel of this library.  Either way in chunks of about 256 MB
+ * of spectra (at least 256 images).  Allocates on first use the plans and, for
+ * FR_F16, a staging buffer of one chunk.
  * Work is enqueued on `stream`. */
 int fr_prepare_images(fr_ctx *ctx, const float *real, int n, int center, void *out,
                       fr_dtype dtype, void *stream);

@@ -121,6 +121,12 @@ cudaError_t launch_merge_scratch(const InsertArgs &a, cudaStream_t st);
 float otf_inv_pa(double alpha);
 // coefficients (power basis in x = 2 r^2 / a^2 - 1) of the weight polynomial
 void weight_polynomial(double alpha, float *poly);
+// images' transforms by this library's kernels (fr_fft.cu): whether there are any
+// for this size, and the transforms of m real images into out (float2 or half2
+// spectra), by way of spec (m S (S/2 + 1) float2; may be out itself for float2)
+bool fft_images_here(int S);
+cudaError_t fft_images(int S, const float *real, float2 *spec, int m, int center, void *out,
+                       int f16, cudaStream_t st);
 // record a CUDA error for fr_last_cuda_error
 void fr_note_cuda_error(int e);
 cudaError_t launch_finalize(const Geom &g, const float *acc, size_t plane, float2 *V, float *W,

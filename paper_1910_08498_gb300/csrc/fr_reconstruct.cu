@@ -222,14 +222,17 @@ extern "C" int fr_prepare_images(fr_ctx *c, const float *real, int n, int center
   if (!c || n < 0 || n > (1 << 24) || (dtype != FR_F32 && dtype != FR_F16)) return FR_ERR_INVALID_ARG;
   if (n == 0) return FR_OK;
   if (!real || !out || ((uintptr_t)out & 15) || ((uintptr_t)real & 15)) return FR_ERR_INVALID_ARG;
-  const Cufft &fft = cufft();
-  if (!fft.ok) return FR_ERR_UNSUPPORTED;
   cudaStream_t st = static_cast<cudaStream_t>(stream);
   const int S = c->S, NX = S / 2 + 1;
   const size_t px_real = (size_t)S * S, px_spec = (size_t)S * NX;
-  // images per transform: about 256 MB of spectra per cuFFT launch (fewer,
-  // larger launches measured faster than chunks of 256 images at S = 256),
-  // and at least 256 images
+  const bool own = fft_images_here(S);  // this library's kernels (fr_fft.cu), else cuFFT
+  if (!own && !cufft().ok) return FR_ERR_UNSUPPORTED;
+  const Cufft &fft = g_fft;
+  // images per transform: about 256 MB of spectra per launch (fewer, larger
+  // launches measured faster than chunks of 256 images at S = 256, and than
+  // chunks that stay in L2, with either library: 1100 images of 256^2 to FP16
+  // with this one's kernels take 206 us in one chunk, 230 in chunks of 48 MB,
+  // 290 of 24 MB), and at least 256 images
   const int CHUNK = (int)std::max<size_t>(256, ((size_t)256 << 20) / (px_spec * sizeof(float2)));
   const bool direct = dtype == FR_F32;  // FP32: transform straight into out
   if (!direct && !c->prep_ws) {
@@ -244,6 +247,17 @@ extern "C" int fr_prepare_images(fr_ctx *c, const float *real, int n, int center
   cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
   for (int i0 = 0; i0 < n; i0 += CHUNK) {
     const int m = std::min(CHUNK, n - i0);
+    if (own) {
+      char *dst = static_cast<char *>(out) + (size_t)i0 * px_spec * (direct ? 8 : 4);
+      cudaError_t e = fft_images(S, real + (size_t)i0 * px_real,
+                                 direct ? reinterpret_cast<float2 *>(dst) : c->prep_ws, m, center,
+                                 dst, !direct, st);
+      if (e != cudaSuccess) {
+        fr_note_cuda_error((int)e);
+        return FR_ERR_CUDA;
+      }
+      continue;
+    }
     const int slot = m == CHUNK ? 0 : 1;
     int rc = prep_plan(c, slot, m);
     if (rc != FR_OK) return rc;

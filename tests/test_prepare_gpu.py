@@ -24,7 +24,8 @@ def _real(S, n, seed):
 
 
 @pytest.mark.parametrize("S,n,center", [(32, 300, False), (32, 300, True), (48, 257, True), (64, 5, False),
-                                         (30, 301, True), (14, 9, True)])
+                                         (30, 301, True), (14, 9, True), (64, 1, True), (64, 259, True),
+                                         (128, 1, False), (128, 3, True), (256, 1, True), (256, 5, False)])
 def test_prepare_fp32(S, n, center):
     real = _real(S, n, S + n)
     ctx = L.fr_create(S)
@@ -39,7 +40,7 @@ def test_prepare_fp32(S, n, center):
     assert np.max(np.abs(got - ref)) <= 1e-5 * np.max(np.abs(ref))
 
 
-@pytest.mark.parametrize("S,n", [(32, 70), (30, 33)])
+@pytest.mark.parametrize("S,n", [(32, 70), (30, 33), (64, 7), (128, 5), (256, 3)])
 def test_prepare_fp16(S, n):
     real = _real(S, n, 5 + S)
     ctx = L.fr_create(S)
