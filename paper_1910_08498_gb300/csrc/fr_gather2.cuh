@@ -29,10 +29,12 @@
 // What bounds it.  Reading the boxes straight from global memory through L1 cost
 // 128 data-pipe wavefronts a round (32 boxes lie in about nine image rows) and
 // kept that pipe 90 % busy at 63 % issue: 13.4 ms for 5000 FP32 images of 256^2.
-// From the patches a round costs 51, and one 512-voxel footprint a warp (137
-// items an entry) halves the work per entry against 256 voxels: 9.6 ms, the
-// data pipe 71 %, FMA pipe 63 %, issue 65 % busy, about one third of the time in
-// the per-entry work (items, patch copies), the rest in the rounds.
+// From the patches a round costs about 50, and one 512-voxel footprint a warp
+// (137 items an entry) halves the work per entry against 256 voxels; with an
+// entry's last half round on two lanes an item and 14 candidates a box: 8.4 ms.
+// Now the instructions bound it: 74 % issue, of which a quarter are packed FMAs
+// that hold the FMA pipe for two cycles (60 % busy); shared memory 63 %.  About a
+// quarter of the time is per-entry work (copies 0.6 ms, tags 0.2, records 0.2).
 //
 // Half planes.  A stored pixel k sits at R k or, point-reflected and
 // conjugated, at -R k.  An image whose patch lies in k_x > 0 (or its mirror)
@@ -121,38 +123,38 @@ __device__ __noinline__ void g2_ties(const float2 *cp, const float2 *p, float dx
 // candidates with r <= a.  FOLD: candidate (j, l) counts only if bit j of
 // rows[l] >> shift is set; with KB = 6 (a >= 2) candidates within rounding of
 // the blob edge are left out, and whether there are any is returned (g2_ties).
-template <int PITCH, int KB, int FOLD>
+// ROWS < KB: only the box's first ROWS rows.
+template <int PITCH, int KB, int FOLD, int ROWS = KB>
 __device__ __forceinline__ bool g2_box(const float2 *cp, const float2 *p, float dx, float dy,
                                        float uz2, float cs, float sq, float &ar, float &ai,
                                        float &aw, const unsigned *rows, int shift) {
-  constexpr int NP = POLY_N, KP = KB / 2, RP = KB == 4 ? 4 : 3;
+  constexpr int NP = POLY_N, KP = KB / 2, RP = KB == 4 ? ROWS : 3;
   // cp: coefficient pairs (c_k, c_k), kernel-parameter constants
   // scaled column offsets sq (dx - j): x = (sq dx)^2 + cs (dy^2 + u_z^2) - 1
-  const float2 S2 = make_float2(sq, sq), C2 = make_float2(cs, cs);
-  const float2 DX = make_float2(dx, dx), DY = make_float2(dy, dy);
-  float2 d[KP];
+  float d[KB];
 #pragma unroll
-  for (int j = 0; j < KP; ++j)
-    d[j] = __fmul2_rn(__fadd2_rn(DX, make_float2(-2.0f * j, -2.0f * j - 1.0f)), S2);
+  for (int j = 0; j < KB; ++j) d[j] = sq * (dx - (float)j);
   const float U = fmaf(cs, uz2, -1.0f);
-  const float2 UU = make_float2(U, U);
   ar = 0.f;
   ai = 0.f;
   aw = 0.f;
   bool ties = false;
 #pragma unroll
-  for (int r0 = 0; r0 < KB; r0 += RP) {
+  for (int r0 = 0; r0 < ROWS; r0 += RP) {
     // all polynomials of RP rows advance together: eight or nine independent
     // chains of packed FMAs (row by row the FMA pipe waits for their latency).
     // With a constant as its third operand a packed FMA runs at the full rate
-    // (74 TFLOP/s measured; with three register pairs 44).
+    // (74 TFLOP/s measured; with three register pairs 44), so only the
+    // polynomial is packed.  Unpacked it took 9.5 ms instead of 8.7 (S = 256, n =
+    // 5000): 32 % more instructions at 83 % issue.
     float2 x[RP * KP], h[RP * KP];
 #pragma unroll
     for (int r = 0; r < RP; ++r) {
-      const float2 EY = r0 + r ? __fadd2_rn(DY, make_float2(-(float)(r0 + r), -(float)(r0 + r))) : DY;
-      const float2 YY = __ffma2_rn(__fmul2_rn(C2, EY), EY, UU);
+      const float ey = dy - (float)(r0 + r);
+      const float Y = fmaf(cs * ey, ey, U);
 #pragma unroll
-      for (int j = 0; j < KP; ++j) x[r * KP + j] = __ffma2_rn(d[j], d[j], YY);
+      for (int j = 0; j < KP; ++j)
+        x[r * KP + j] = make_float2(fmaf(d[2 * j], d[2 * j], Y), fmaf(d[2 * j + 1], d[2 * j + 1], Y));
     }
 #pragma unroll
     for (int i = 0; i < RP * KP; ++i) h[i] = __ffma2_rn(cp[NP - 1], x[i], cp[NP - 2]);
@@ -185,6 +187,73 @@ __device__ __forceinline__ bool g2_box(const float2 *cp, const float2 *p, float 
     }
   }
   return ties;
+}
+
+// The 4 x 4 box of an item outside the fold columns, in 14 candidates: of the four
+// corner pixels at most two, neighbours, lie within a < 2 of u.  (Opposite ones: the
+// squared distances add up to dx^2 + (3 - dx)^2 + dy^2 + (3 - dy)^2 >= 9 > 2 a^2.)
+// They are on the side of the box that u is nearest to: with e = |dx - 1.5| >= |dy -
+// 1.5| a corner of the far column is at least (1.5 + e)^2 + (1.5 - e)^2 >= 4.5 away.
+template <int PITCH>
+__device__ __forceinline__ void g2_box14(const float2 *cp, const float2 *p, float dx, float dy,
+                                         float uz2, float cs, float sq, float &ar, float &ai,
+                                         float &aw) {
+  constexpr int NP = POLY_N;
+  float d[4], Y[4];
+#pragma unroll
+  for (int k = 0; k < 4; ++k) d[k] = sq * (dx - (float)k);
+  const float U = fmaf(cs, uz2, -1.0f);
+#pragma unroll
+  for (int k = 0; k < 4; ++k) {
+    const float ey = dy - (float)k;
+    Y[k] = fmaf(cs * ey, ey, U);
+  }
+  // the two corners: distance m from u's near side, nn and nn - 3 along it
+  const float gx = fabsf(dx - 1.5f), gy = fabsf(dy - 1.5f);
+  const bool side = gx > gy;  // a column's two corners, else a row's
+  const float m = 1.5f - fmaxf(gx, gy), V = fmaf(cs * m, m, U);
+  const float nn = side ? dy : dx, n0 = sq * nn, n1 = sq * (nn - 3.0f);
+  const int ca = side ? (dx < 1.5f ? 0 : 3) : (dy < 1.5f ? 0 : 3 * PITCH);
+  const float2 *pa = p + ca, *pb = pa + (side ? 3 * PITCH : 3);
+  float2 x[7], h[7];
+  x[0] = make_float2(fmaf(d[1], d[1], Y[0]), fmaf(d[2], d[2], Y[0]));
+#pragma unroll
+  for (int r = 1; r < 3; ++r) {
+    x[2 * r - 1] = make_float2(fmaf(d[0], d[0], Y[r]), fmaf(d[1], d[1], Y[r]));
+    x[2 * r] = make_float2(fmaf(d[2], d[2], Y[r]), fmaf(d[3], d[3], Y[r]));
+  }
+  x[5] = make_float2(fmaf(d[1], d[1], Y[3]), fmaf(d[2], d[2], Y[3]));
+  x[6] = make_float2(fmaf(n0, n0, V), fmaf(n1, n1, V));
+#pragma unroll
+  for (int i = 0; i < 7; ++i) h[i] = __ffma2_rn(cp[NP - 1], x[i], cp[NP - 2]);
+#pragma unroll
+  for (int k = NP - 3; k >= 0; --k)
+#pragma unroll
+    for (int i = 0; i < 7; ++i) h[i] = __ffma2_rn(h[i], x[i], cp[k]);
+  ar = 0.f;
+  ai = 0.f;
+  aw = 0.f;
+  auto add = [&](float xv, float w, const float2 q) {
+    if (xv <= 1.0f) {
+      ar = fmaf(w, q.x, ar);
+      ai = fmaf(w, q.y, ai);
+      aw += w;
+    }
+  };
+  add(x[0].x, h[0].x, p[1]);
+  add(x[0].y, h[0].y, p[2]);
+#pragma unroll
+  for (int r = 1; r < 3; ++r) {
+    const float2 *q = p + r * PITCH;
+    add(x[2 * r - 1].x, h[2 * r - 1].x, q[0]);
+    add(x[2 * r - 1].y, h[2 * r - 1].y, q[1]);
+    add(x[2 * r].x, h[2 * r].x, q[2]);
+    add(x[2 * r].y, h[2 * r].y, q[3]);
+  }
+  add(x[5].x, h[5].x, p[3 * PITCH + 1]);
+  add(x[5].y, h[5].y, p[3 * PITCH + 2]);
+  add(x[6].x, h[6].x, *pa);
+  add(x[6].y, h[6].y, *pb);
 }
 
 // Clear a warp's partial sums (16-byte aligned).
@@ -568,15 +637,19 @@ __device__ __forceinline__ void gather2_warp(const InsertArgs &args, const Inser
     // arrive with it
     const float kM = 8388608.0f, kR = 12582912.0f;
     const unsigned base = (unsigned)-(rpy * PITCH + rpx) - 0x4b400000u;
-    // one round ahead: the tags are loaded (their buffer is a round longer)
-    unsigned next = s_tag[lane];
-#pragma unroll 1
-    for (int h = lane, left = total; left > 0; h += 32, left -= 32) {
+    // an item: where its box is and u relative to it
+    struct Item {
+      int slot;
+      const float2 *p;
+      float dx, dy, uz2;
+      const unsigned *rows;
+      int shift, row;
+    };
+    auto locate = [&](unsigned tag, int h) -> Item {
+      Item it;
       // the slot: of the first columns up to position tot0, of the second after
-      const int slot = (int)((next + h) & 255) + (NC == 2 && h >= tot0 ? 256 : 0);
-      next = s_tag[h + 32];
-      // the partial sums, read before the box: no other item of the entry adds to them
-      const float tr = s_acc[slot], ti = s_acc[WV + slot], tw = s_acc[2 * WV + slot];
+      const int slot = (int)((tag + h) & 255) + (NC == 2 && h >= tot0 ? 256 : 0);
+      it.slot = slot;
       // voxel offsets from the centre: bit fields of the slot placed in the
       // significand of 2^23, scaled and shifted (exactly)
       const float sdz = (__int_as_float(0x4b000000 | (slot & (ZC - 1))) - kM) - HZ;
@@ -591,25 +664,63 @@ __device__ __forceinline__ void gather2_warp(const InsertArgs &args, const Inser
       constexpr float HO = HB - 0.5f;
       const float ox = fminf(fmaxf(__fadd_rn(__fadd_rn(ux - HO, kR), -kR), lox), hix);
       const float oy = fminf(fmaxf(__fadd_rn(__fadd_rn(uy - HO, kR), -kR), loy), hiy);
-      const unsigned at = __float_as_uint(fmaf(oy, (float)PITCH, __fadd_rn(ox, kR))) + base;
-      const unsigned *rows = s_bits;
-      int shift = 0;
+      it.p = patch + (__float_as_uint(fmaf(oy, (float)PITCH, __fadd_rn(ox, kR))) + base);
+      it.dx = ux - ox;
+      it.dy = uy - oy;
+      it.uz2 = uz * uz;
+      it.rows = s_bits;
+      it.shift = it.row = 0;
       if (FOLD) {
-        shift = (int)(ox - lox);
-        rows += (li & 1) * PITCH + (int)(oy - loy);
+        it.shift = (int)(ox - lox);
+        it.row = (int)(oy - loy);
+        it.rows += (li & 1) * PITCH + it.row;
       }
+      return it;
+    };
+    // one round ahead: the tags are loaded (their buffer is a round longer)
+    unsigned next = s_tag[lane];
+    // the last round of at most 16 items takes two lanes an item, two rows of the
+    // box each (half of all entries end in one: 137 items on average)
+    constexpr bool HALF = KB == 4 && !FOLD;
+    int left = total;
+#pragma unroll 1
+    for (int h = lane; left > (HALF ? 16 : 0); h += 32, left -= 32) {
+      const Item it = locate(next, h);
+      next = s_tag[h + 32];
+      // the partial sums, read before the box: no other item of the entry adds to them
+      const float tr = s_acc[it.slot], ti = s_acc[WV + it.slot], tw = s_acc[2 * WV + it.slot];
       float ar, ai, aw;
-      const bool ties = g2_box<PITCH, KB, FOLD>(cst.poly2, patch + at, ux - ox, uy - oy, uz * uz, cs,
-                                                sq, ar, ai, aw, rows, shift);
+      bool ties = false;
+      if (HALF)
+        g2_box14<PITCH>(cst.poly2, it.p, it.dx, it.dy, it.uz2, cs, sq, ar, ai, aw);
+      else
+        ties = g2_box<PITCH, KB, FOLD>(cst.poly2, it.p, it.dx, it.dy, it.uz2, cs, sq, ar, ai, aw,
+                                       it.rows, it.shift);
       if (FOLD && KB == 6 && ties)
-        g2_ties<PITCH, KB>(cst.poly2, patch + at, ux - ox, uy - oy, uz * uz, cs, rows, shift, q1,
-                           q2, make_int3(fx0 + (slot / ZC) % FW, fy0 + slot / (ZC * FW), z0 + slot % ZC),
-                           make_int2((q3.y & 0xffff) + shift, (q3.y >> 16) + (int)(oy - loy)), g.a, ar,
-                           ai, aw);
+        g2_ties<PITCH, KB>(cst.poly2, it.p, it.dx, it.dy, it.uz2, cs, it.rows, it.shift, q1, q2,
+                           make_int3(fx0 + (it.slot / ZC) % FW, fy0 + it.slot / (ZC * FW), z0 + it.slot % ZC),
+                           make_int2((q3.y & 0xffff) + it.shift, (q3.y >> 16) + it.row), g.a, ar, ai, aw);
       if (h < total) {
-        s_acc[slot] = tr + ar;
-        s_acc[WV + slot] = fmaf(sgn, ai, ti);
-        s_acc[2 * WV + slot] = tw + aw;
+        s_acc[it.slot] = tr + ar;
+        s_acc[WV + it.slot] = fmaf(sgn, ai, ti);
+        s_acc[2 * WV + it.slot] = tw + aw;
+      }
+    }
+    if (HALF && left > 0) {
+      const int h = total - left + (lane & 15), half = lane >> 4;
+      const Item it = locate(s_tag[h], h);
+      const float tr = s_acc[it.slot], ti = s_acc[WV + it.slot], tw = s_acc[2 * WV + it.slot];
+      float ar, ai, aw;
+      g2_box<PITCH, KB, 0, KB / 2>(cst.poly2, it.p + half * (KB / 2 * PITCH), it.dx,
+                                   it.dy - (float)(half * (KB / 2)), it.uz2, cs, sq, ar, ai, aw,
+                                   it.rows, 0);
+      ar += __shfl_xor_sync(FULL, ar, 16);
+      ai += __shfl_xor_sync(FULL, ai, 16);
+      aw += __shfl_xor_sync(FULL, aw, 16);
+      if (lane < left) {
+        s_acc[it.slot] = tr + ar;
+        s_acc[WV + it.slot] = fmaf(sgn, ai, ti);
+        s_acc[2 * WV + it.slot] = tw + aw;
       }
     }
     __syncwarp();

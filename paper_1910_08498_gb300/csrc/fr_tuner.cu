@@ -105,11 +105,13 @@ int default_gather_config(const fr_ctx *c) {
 }
 
 int default_config(const fr_ctx *c) {
-  // the direct-drain gather, 16 x 8 x 8 CTA, registers for 24 warps per SM;
-  // where it cannot run (a >= 2), the per-voxel gather default
+  // the direct-drain gather, 16 x 8 x 8 bricks, registers for 16 warps per SM
+  // (what shared memory holds; the budgets for 20 and 24 measured 0 to 1 and 1 to
+  // 4 % slower at S = 128 .. 256, FP32 and FP16); where it cannot run (a >= 2),
+  // the per-voxel gather default
   const auto &sp = config_space();
   for (int i = 0; i < (int)sp.size(); ++i)
-    if (sp[i].algo == ALGO_GATHER2 && sp[i].shape == 1 && sp[i].minw == 24 && sp[i].chunk == 64 &&
+    if (sp[i].algo == ALGO_GATHER2 && sp[i].shape == 1 && sp[i].minw == 16 && sp[i].chunk == 64 &&
         config_valid(c, i))
       return i;
   for (int i = 0; i < (int)sp.size(); ++i)
