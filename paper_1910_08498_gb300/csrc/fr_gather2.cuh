@@ -93,6 +93,13 @@ __device__ __forceinline__ void cp_async8(uint32_t dst, const void *src) {
 }
 __device__ __forceinline__ void cp_async_wait_all() { asm volatile("cp.async.wait_all;" ::: "memory"); }
 
+// x . x - 1 for a nearly unit vector, to a few ulp of the difference
+__device__ __forceinline__ float dot3_less_one(float x, float y, float z) {
+  float hi, lo;
+  dot3_dd(x, y, z, x, y, z, hi, lo);
+  return (hi - 1.0f) + lo;
+}
+
 // Candidates of a fold column's box within rounding of the blob edge (FP32 r^2
 // within 1e-5 a^2 of a^2), decided as the real numbers do: with a lattice
 // distance a (a = 2, or a signed permutation for the rotation) the DC pixel
@@ -431,6 +438,23 @@ __device__ __forceinline__ void gather2_warp(const InsertArgs &args, const Inser
       dot3_dd(e1x, e1y, e1z, cx, cy, cz, hxx, lx);
       dot3_dd(e2x, e2y, e2z, cx, cy, cz, hyy, ly);
       dot3_dd(mx, my, mz, cx, cy, cz, hzz, lz);
+      if (args.ortho) {
+        // An FP32 rotation is orthonormal only to 6e-8, which moves u by up to 6e-8
+        // |c| from the coordinates of c on e1, e2 and its distance from their plane:
+        // corrected to first order in R^T R - 1, formed without cancellation.
+        const float d11 = dot3_less_one(e1x, e1y, e1z), d22 = dot3_less_one(e2x, e2y, e2z),
+                    d33 = dot3_less_one(mx, my, mz);
+        float d12, d13, d23, l12, l13, l23;
+        dot3_dd(e1x, e1y, e1z, e2x, e2y, e2z, d12, l12);
+        dot3_dd(e1x, e1y, e1z, mx, my, mz, d13, l13);
+        dot3_dd(e2x, e2y, e2z, mx, my, mz, d23, l23);
+        d12 += l12;
+        d13 += l13;
+        d23 += l23;
+        lx -= fmaf(d11, hxx, d12 * hyy);
+        ly -= fmaf(d12, hxx, d22 * hyy);
+        lz -= fmaf(d13, hxx, fmaf(d23, hyy, 0.5f * d33 * hzz));
+      }
       const float rx = rintf(hxx), ry = rintf(hyy);
       fx = (hxx - rx) + lx;  // hxx - rx is exact
       fy = (hyy - ry) + ly;

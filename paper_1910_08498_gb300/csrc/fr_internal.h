@@ -64,6 +64,11 @@ struct InsertArgs {
   int nfold;
   float unit_share;
   int unit_most;
+  // correct the projections for a rotation that FP32 rounding left short of
+  // orthonormal.  fr_insert_noalloc does, whose scatter places every sample to
+  // FP32 accuracy; fr_insert keeps the plain R^T c, so that a volume resumed from a
+  // checkpoint goes on with the same positions
+  int ortho;
   int any_split;        // 1 if some unit shares its brick with other units
   unsigned long long *phase;  // optional per-phase cycle and item counters (PH_*), or null
   // scatter

@@ -185,6 +185,7 @@ extern "C" int fr_insert_noalloc(int S, float a, float alpha, const void *images
     for (int k = 0; k < POLY_N; ++k) args.poly2[k] = make_float2(args.poly[k], args.poly[k]);
     args.chunk = 64;
     args.any_split = 1;
+    args.ortho = 1;
   }
   for (int i0 = 0; i0 < n; i0 += NOALLOC_SUB) {
     args.n = std::min(NOALLOC_SUB, n - i0);
