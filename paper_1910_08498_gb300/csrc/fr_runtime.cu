@@ -604,10 +604,11 @@ int fr_insert_batched(fr_ctx *const *ctxs, const void *const *images, const fr_d
 int fr_finalize(fr_ctx *c, void *V, float *W, void *stream) {
   if (!c || !V || !W) return FR_ERR_INVALID_ARG;
   cudaStream_t st = (cudaStream_t)stream;
-  FR_CUDA(cudaStreamSynchronize(st));
   if (c->last_stream && c->last_stream != st) FR_CUDA(cudaStreamSynchronize(c->last_stream));
+  // the error word in stream order: one wait instead of two
   int h = 0;
-  FR_CUDA(cudaMemcpy(&h, c->d_err, sizeof(int), cudaMemcpyDeviceToHost));
+  FR_CUDA(cudaMemcpyAsync(&h, c->d_err, sizeof(int), cudaMemcpyDeviceToHost, st));
+  FR_CUDA(cudaStreamSynchronize(st));
   cudaError_t e = launch_finalize(c->g, c->acc, c->plane, (float2 *)V, W, st);
   if (e != cudaSuccess) return cuda_fail(e);
   c->last_stream = st;
