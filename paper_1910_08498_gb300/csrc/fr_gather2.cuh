@@ -61,7 +61,7 @@ constexpr int G2_ENTRIES = 16;  // records built and processed at a time
 constexpr int G2_REC = 16;      // floats of a record
 
 // Geometry of the warp footprint FW x 8 x 8 and of its pixel patches, for
-// KB x KB candidate boxes (KB = 4: a < 2, KB = 6: a < 3).
+// KB x KB candidate boxes (KB = 4: a < 2, 5: a <= 2.5, 6: a < 3).
 template <int FW, int KB>
 struct G2Shape {
   static constexpr int FH = 8, ZC = 8;
@@ -69,13 +69,13 @@ struct G2Shape {
   static constexpr int WV = FW * FH * ZC;               // voxels
   static constexpr float HX = 0.5f * (FW - 1), HY = 0.5f * (FH - 1), HZ = 0.5f * (ZC - 1);
   // a box reaches KB / 2 pixels past u, and u lies within the footprint's
-  // radius (6.07; 5.17 for FW = 4) of the centre: at most 17 (KB = 6: 19;
-  // FW = 4: 15) columns
+  // radius (6.07; 5.17 for FW = 4) of the centre: at most 17 (KB = 5: 18, KB = 6:
+  // 19; FW = 4: 15) columns
   static constexpr int PW = (FW == 8 ? 13 : 11) + KB;   // patch columns and rows
   static constexpr int XC = PW > 16 ? PW - 16 : 0;      // columns past the first 16
   static constexpr int PITCH = 20;                      // = 4 modulo 16 eight-byte banks
   static constexpr int PATCH = PW * PITCH;              // pixels of a patch
-  static_assert(PW <= PITCH && (XC == 0 || XC == 1 || XC == 3), "patch rows");
+  static_assert(PW <= PITCH && XC <= 3, "patch rows");
 };
 
 // Per-warp shared memory: records, partial sums, patches, image list, fold
@@ -261,6 +261,87 @@ __device__ __forceinline__ void g2_box14(const float2 *cp, const float2 *p, floa
   add(x[5].y, h[5].y, p[3 * PITCH + 2]);
   add(x[6].x, h[6].x, *pa);
   add(x[6].y, h[6].y, *pb);
+}
+
+// The 5 x 5 box of an item outside the fold columns (2 <= a <= 2.5), in 23
+// candidates: of the corners only the two on the near side (see g2_box14: opposite
+// corners' squared distances add up to at least 16 > 2 a^2, a far corner is at least
+// 8 away).  Its origin rint(u - 2) leaves out at most a pixel at distance exactly
+// 2.5 along an axis.
+template <int PITCH>
+__device__ __forceinline__ void g2_box23(const float2 *cp, const float2 *p, float dx, float dy,
+                                         float uz2, float cs, float sq, float &ar, float &ai,
+                                         float &aw) {
+  constexpr int NP = POLY_N;
+  float d[5], Y[5];
+#pragma unroll
+  for (int k = 0; k < 5; ++k) d[k] = sq * (dx - (float)k);
+  const float U = fmaf(cs, uz2, -1.0f);
+#pragma unroll
+  for (int k = 0; k < 5; ++k) {
+    const float ey = dy - (float)k;
+    Y[k] = fmaf(cs * ey, ey, U);
+  }
+  // the two corners: distance m from u's near side, nn and nn - 4 along it
+  const float gx = fabsf(dx - 2.0f), gy = fabsf(dy - 2.0f);
+  const bool side = gx > gy;  // a column's two corners, else a row's
+  const float m = 2.0f - fmaxf(gx, gy), V = fmaf(cs * m, m, U);
+  const float nn = side ? dy : dx, n0 = sq * nn, n1 = sq * (nn - 4.0f);
+  const int ca = side ? (dx < 2.0f ? 0 : 4) : (dy < 2.0f ? 0 : 4 * PITCH);
+  const float2 *pa = p + ca, *pb = pa + (side ? 4 * PITCH : 4);
+  ar = 0.f;
+  ai = 0.f;
+  aw = 0.f;
+  auto add = [&](float xv, float w, const float2 q) {
+    if (xv <= 1.0f) {
+      ar = fmaf(w, q.x, ar);
+      ai = fmaf(w, q.y, ai);
+      aw += w;
+    }
+  };
+  auto at = [&](int r, int c) { return fmaf(d[c], d[c], Y[r]); };
+  // two passes of six packed polynomials (the last one's second half repeats)
+#pragma unroll
+  for (int pass = 0; pass < 2; ++pass) {
+    float2 x[6], h[6];
+    if (pass == 0) {
+      x[0] = make_float2(at(0, 1), at(0, 2));
+      x[1] = make_float2(at(0, 3), at(1, 0));
+      x[2] = make_float2(at(1, 1), at(1, 2));
+      x[3] = make_float2(at(1, 3), at(1, 4));
+      x[4] = make_float2(at(2, 0), at(2, 1));
+      x[5] = make_float2(at(2, 2), at(2, 3));
+    } else {
+      x[0] = make_float2(at(2, 4), at(3, 0));
+      x[1] = make_float2(at(3, 1), at(3, 2));
+      x[2] = make_float2(at(3, 3), at(3, 4));
+      x[3] = make_float2(at(4, 1), at(4, 2));
+      x[4] = make_float2(at(4, 3), fmaf(n0, n0, V));
+      x[5] = make_float2(fmaf(n1, n1, V), 2.0f);
+    }
+#pragma unroll
+    for (int i = 0; i < 6; ++i) h[i] = __ffma2_rn(cp[NP - 1], x[i], cp[NP - 2]);
+#pragma unroll
+    for (int k = NP - 3; k >= 0; --k)
+#pragma unroll
+      for (int i = 0; i < 6; ++i) h[i] = __ffma2_rn(h[i], x[i], cp[k]);
+    const float2 *r0 = p, *r1 = p + PITCH, *r2 = p + 2 * PITCH, *r3 = p + 3 * PITCH, *r4 = p + 4 * PITCH;
+    if (pass == 0) {
+      add(x[0].x, h[0].x, r0[1]), add(x[0].y, h[0].y, r0[2]);
+      add(x[1].x, h[1].x, r0[3]), add(x[1].y, h[1].y, r1[0]);
+      add(x[2].x, h[2].x, r1[1]), add(x[2].y, h[2].y, r1[2]);
+      add(x[3].x, h[3].x, r1[3]), add(x[3].y, h[3].y, r1[4]);
+      add(x[4].x, h[4].x, r2[0]), add(x[4].y, h[4].y, r2[1]);
+      add(x[5].x, h[5].x, r2[2]), add(x[5].y, h[5].y, r2[3]);
+    } else {
+      add(x[0].x, h[0].x, r2[4]), add(x[0].y, h[0].y, r3[0]);
+      add(x[1].x, h[1].x, r3[1]), add(x[1].y, h[1].y, r3[2]);
+      add(x[2].x, h[2].x, r3[3]), add(x[2].y, h[2].y, r3[4]);
+      add(x[3].x, h[3].x, r4[1]), add(x[3].y, h[3].y, r4[2]);
+      add(x[4].x, h[4].x, r4[3]), add(x[4].y, h[4].y, *pa);
+      add(x[5].x, h[5].x, *pb);
+    }
+  }
 }
 
 // Clear a warp's partial sums (16-byte aligned).
@@ -507,8 +588,8 @@ __device__ __forceinline__ void gather2_warp(const InsertArgs &args, const Inser
   };
 
   // Patch copies: 16 columns x 2 rows a step (rows past the patch repeat its
-  // last row), then the columns past 16 (4 of them x 8 rows a step, or one).
-  constexpr int RG = (PW + 1) / 2, XL = XC == 3 ? 4 : 1, XR = XC == 0 ? 0 : (PW * XL + 31) / 32;
+  // last row), then the columns past 16 (4, 2 or 1 of them, 32 pixels a step).
+  constexpr int RG = (PW + 1) / 2, XL = XC == 3 ? 4 : XC == 2 ? 2 : 1, XR = XC == 0 ? 0 : (PW * XL + 31) / 32;
   const int xc = lane % XL, xr = lane / XL;
   const int pc = lane & 15, pr = lane >> 4;
   const int row_bytes = g.NX * ESZ;
@@ -717,6 +798,8 @@ __device__ __forceinline__ void gather2_warp(const InsertArgs &args, const Inser
       bool ties = false;
       if (HALF)
         g2_box14<PITCH>(cst.poly2, it.p, it.dx, it.dy, it.uz2, cs, sq, ar, ai, aw);
+      else if (KB == 5)
+        g2_box23<PITCH>(cst.poly2, it.p, it.dx, it.dy, it.uz2, cs, sq, ar, ai, aw);
       else
         ties = g2_box<PITCH, KB, FOLD>(cst.poly2, it.p, it.dx, it.dy, it.uz2, cs, sq, ar, ai, aw,
                                        it.rows, it.shift);
@@ -852,7 +935,9 @@ __device__ __forceinline__ bool g2_implicit_unit(const InsertArgs &args, int x0,
 // second kernel on a side stream the fold columns cost a fork and a join.  MINW:
 // resident warps per SM the register allocation must allow (16: at most 128
 // registers per thread, and what shared memory holds; more are not resident).
-template <int BX, int BY, int BZ, int F16, int MINW, int KB = 4>
+// KB: box width of the fold columns (4, or 6 for a >= 2), KBM: of the main bricks (5
+// for 2 <= a <= 2.5).
+template <int BX, int BY, int BZ, int F16, int MINW, int KB = 4, int KBM = KB>
 __global__ void __launch_bounds__(32, MINW)
 gather2_kernel(const __grid_constant__ InsertArgs args) {
   extern __shared__ __align__(16) unsigned char smem[];
@@ -871,7 +956,7 @@ gather2_kernel(const __grid_constant__ InsertArgs args) {
     const int b = (int)blockIdx.x - nf, k = b / W;
     if (args.units) unit = args.units[k];
     else if (!g2_implicit_unit<BX, BY, BZ>(args, 1 - g.xa0, g.H, k, unit)) return;
-    gather2_warp<BX, BY, BZ, F16, KB>(args, args, args.images, smem, unit, b % W);
+    gather2_warp<BX, BY, BZ, F16, KBM>(args, args, args.images, smem, unit, b % W);
   }
 }
 
@@ -881,7 +966,7 @@ gather2_kernel(const __grid_constant__ InsertArgs args) {
 // batches, are read from p.base (kernel parameters: constant operands in the
 // inner loops), the batch's own arguments (rotations, volume) from its
 // descriptor.
-template <int BX, int BY, int BZ, int F16, int MINW, int KB = 4>
+template <int BX, int BY, int BZ, int F16, int MINW, int KB = 4, int KBM = KB>
 __global__ void __launch_bounds__(32, MINW)
 gather2_multi_kernel(const __grid_constant__ MultiLaunch p) {
   extern __shared__ __align__(16) unsigned char smem[];
@@ -894,7 +979,7 @@ gather2_multi_kernel(const __grid_constant__ MultiLaunch p) {
     gather2_warp<FW, G2_FOLD_BY, G2_FOLD_BZ, F16, KB, FW, 1>(p.descs[it.z], p.base, p.images[it.w],
                                                              smem, unit, (int)(blockIdx.x % WF));
   else
-    gather2_warp<BX, BY, BZ, F16, KB>(p.descs[it.z], p.base, p.images[it.w], smem, unit, b % W);
+    gather2_warp<BX, BY, BZ, F16, KBM>(p.descs[it.z], p.base, p.images[it.w], smem, unit, b % W);
 }
 
 }  // namespace fr

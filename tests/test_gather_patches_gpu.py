@@ -27,7 +27,7 @@ def _batch(S, n, seed):
 
 
 @pytest.mark.parametrize("f16", [False, True])
-@pytest.mark.parametrize("a", [0.6, 1.0, 1.5, 1.999, 2.0, 2.5, 2.999])
+@pytest.mark.parametrize("a", [0.6, 1.0, 1.5, 1.999, 2.0, 2.25, 2.5, 2.51, 2.999])
 @pytest.mark.parametrize("S", [8, 10, 14, 16, 18, 30, 32, 34, 46])
 def test_patch_edges_match_oracle(S, a, f16):
     a = float(np.float32(a))
