@@ -21,8 +21,9 @@
  *     tile of C, the group's C written back by one bulk store; tuned over TY,
  *     TX in {1, 2, 4}, the rounds of the CTA's threads per group (1, 2, 4,
  *     8) and the CTA size cap (128, 256) (72 configurations).
- * Any 4-byte aligned A, B, C are accepted (the bulk copies move the 16-byte
- * aligned interior of each block and plain loads and stores the ends).
+ * Any 4-byte aligned A, B, C are accepted (the bulk copies move whole
+ * 16-byte cells, plain loads and stores the ends that have none; the width of
+ * the loads from shared memory follows the alignment, n and k).
  * The tuner is the insertion's non-blocking scheme (Sec. 3.2): a call with
  * tuning on splits its batch into sub-batches, each computed with the next
  * configuration of the search and timed with CUDA events, harvested without

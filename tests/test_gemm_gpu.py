@@ -109,6 +109,29 @@ def test_bulk_copies_at_unaligned_offsets(m, n, k, off):
     assert L.fr_gemm_device_status() == L.FR_OK
 
 
+@pytest.mark.parametrize("m,n,k", [(2, 2, 2), (7, 6, 8), (10, 12, 6), (9, 16, 31), (23, 22, 21), (5, 7, 32)])
+@pytest.mark.parametrize("oa,ob,oc", [(0, 0, 0), (2, 0, 0), (1, 2, 2), (0, 3, 0), (0, 0, 1), (2, 2, 0)])
+def test_bulk_wide_loads_at_each_alignment(m, n, k, oa, ob, oc):
+    """A, B and C each start at their own offset in floats: the width of the
+    shared-memory loads follows it; the surroundings (NaN) are neither used nor written."""
+    batch = 211
+    A, B = _data(m, n, k, batch, 31 * m + n + k + oa + ob + oc)
+
+    def placed(x, off):
+        buf = torch.full((x.numel() + 8,), float("nan"), device="cuda")
+        buf[off:off + x.numel()] = x.reshape(-1).cuda()
+        return buf, buf[off:off + x.numel()].view(x.shape)
+
+    Ad, Bd = placed(A, oa)[1], placed(B, ob)[1]
+    for cfg in _bulk_configs(m, n, k):
+        buf, C = placed(torch.full((batch, m, n), float("nan")), oc)
+        L.fr_gemm_run_config(cfg, Ad, Bd, C)
+        torch.cuda.synchronize()
+        _check(C, A, B)
+        assert torch.isnan(buf[:oc]).all() and torch.isnan(buf[oc + C.numel():]).all()
+    assert L.fr_gemm_device_status() == L.FR_OK
+
+
 @pytest.mark.parametrize("batch", [1, 2, 3, 5, 4099])
 def test_bulk_copies_ragged_batches(batch):
     """Batches from one instance up to many groups per CTA (the last group partial)."""
