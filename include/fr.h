@@ -244,9 +244,10 @@ int fr_prepare_images(fr_ctx *ctx, const float *real, int n, int center, void *o
  * The paper does not spell the weighting out; the clip w_clip > 0 (1 is a
  * good value: a voxel met by about one blob of weight keeps its sum) keeps
  * the division away from zero.  Allocates, on first use, a half-spectrum
- * buffer (8 S^2 (S/2+1) bytes) and an inverse-FFT plan; the inverse FFT is
- * the CUDA toolkit's cuFFT, loaded at run time (FR_ERR_UNSUPPORTED if it
- * cannot be loaded).  Work is enqueued on `stream`.  Returns FR_OK,
+ * buffer (8 S^2 (S/2+1) bytes).  For S = 64 and 128 the transform is this
+ * library's; for other sizes the CUDA toolkit's cuFFT, loaded at run time
+ * (FR_ERR_UNSUPPORTED if it cannot be loaded), with a plan made on first use.
+ * `out` is 8-byte aligned.  Work is enqueued on `stream`.  Returns FR_OK,
  * FR_ERR_INVALID_ARG (null pointer, w_clip <= 0), FR_ERR_OOM, FR_ERR_CUDA. */
 int fr_reconstruct(fr_ctx *ctx, float *out, float w_clip, void *stream);
 

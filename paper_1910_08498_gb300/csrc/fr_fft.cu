@@ -1,4 +1,5 @@
-// fr_fft.cu -- the images' 2D transforms for S = 64, 128, 256: a kernel over the
+// fr_fft.cu -- the volume's inverse transform for S = 64 and 128 (below), and the
+// images' 2D transforms for S = 64, 128, 256: a kernel over the
 // rows (real to complex) and one over the columns that also centres the image and
 // converts to the insertion's dtype.
 //
@@ -210,6 +211,173 @@ fft_cols_kernel(const float2 *spec, int center, void *out) {
   }
 }
 
+// ---- the volume's inverse transform, S = 64 and 128, in two kernels: weighting and
+// the z lines; then a plane a CTA, its y lines and its x lines (complex to real).
+//
+// The data fit in L2, so what counts is the number of passes and the latency of
+// each; the general path takes four (weighting, then cuFFT's three).  S = 128: 9.7 +
+// 20.6 us in four launches -> 12.8 + 7.5 us.  The z kernel waits for the six sums' 27
+// MB (4 us of HBM traffic); with 16 points a thread instead of 8, and half the warps,
+// it took 14.4 us, with the loads behind a branch a point 19.9.
+// The transforms are the forward ones above, applied to the conjugate of F.  Column
+// kx = S / 2 is zero and left out.
+template <int S>
+struct VolShape {
+  static constexpr int M = S / 2;                   // columns kept
+  static constexpr int Z1 = 8, Z2 = S / Z1;         // z lines: Z2 threads of Z1 points
+  static constexpr int CB = S == 64 ? 16 : 32;      // columns of a CTA of the z lines
+  static constexpr int TZ = Z2 * CB;
+  static constexpr int N1 = S == 64 ? 8 : 16, N2 = 8;  // y lines
+  static constexpr int TP = N2 * M;                 // threads of a plane's CTA
+  static constexpr int R1 = 8, R2 = M / R1;         // x lines: R2 threads of R1 points
+  // float2 per group of R2 points and per row of a plane in shared memory: a half
+  // warp's rows and groups fall on different bank pairs
+  static constexpr int GP = R2 + 1, P = S == 64 ? 52 : 72;
+  static_assert(N1 * N2 == S && P >= M && P >= R1 * GP, "volume lines");
+};
+
+template <int S>
+__global__ void __launch_bounds__(VolShape<S>::TZ)
+volume_z_kernel(const Geom g, const float *__restrict__ acc, size_t plane, float w_clip, float inv_n,
+                float2 *__restrict__ spec) {
+  using V = VolShape<S>;
+  constexpr int M = V::M, N1 = V::Z1, N2 = V::Z2, CB = V::CB, NB = M / CB;
+  __shared__ float2 tw[S], buf[S * CB];
+  const int jy = blockIdx.x / NB, c0 = (blockIdx.x % NB) * CB;
+  const int ky = jy < M ? jy : jy - S;
+  const int t = threadIdx.x / CB, c = threadIdx.x % CB;
+  const int kx = c0 + c;
+  // conj(F) at (kx, ky, kz), 0 on the Nyquist planes.  All points' sums are read first,
+  // without a branch, so that the reads are in flight together; those of the mirrored
+  // point -v join where it is stored (the first few columns).
+  float2 v[N1];
+  float w[N1];
+  // point k is kz = t + N2 k, less S from k = N1 / 2 on: plane kz + S / 2
+  const float *p = acc + ((size_t)t * g.D + (size_t)(ky + M)) * g.NXa + (size_t)(kx - g.xa0);
+  const size_t dz = (size_t)N2 * g.D * g.NXa;
+#pragma unroll
+  for (int k = 0; k < N1; ++k) {
+    const float *q = p + (size_t)((k + N1 / 2) % N1) * dz;
+    v[k] = make_float2(q[0] + q[3 * plane], q[plane] + q[4 * plane]);
+    w[k] = q[2 * plane] + q[5 * plane];
+  }
+  if (-kx >= g.xa0) {
+    const float *pm = acc + ((size_t)(S - t) * g.D + (size_t)(M - ky)) * g.NXa + (size_t)(-kx - g.xa0);
+#pragma unroll
+    for (int k = 0; k < N1; ++k) {
+      const float *q = pm - (size_t)((k + N1 / 2) % N1) * dz;
+      v[k].x += q[0] + q[3 * plane];
+      v[k].y -= q[plane] + q[4 * plane];
+      w[k] += q[2 * plane] + q[5 * plane];
+    }
+  }
+#pragma unroll
+  for (int k = 0; k < N1; ++k) {
+    const float s = inv_n / fmaxf(w[k], w_clip);
+    const bool nyquist = jy == M || (k == N1 / 2 && t == 0);
+    v[k] = nyquist ? make_float2(0.f, 0.f) : make_float2(v[k].x * s, -(v[k].y * s));
+  }
+  fill_twiddles<S>(tw);
+  __syncthreads();
+  dft(v);
+#pragma unroll
+  for (int k = 0; k < N1; ++k) buf[(k * N2 + t) * CB + c] = k ? cmul(v[k], tw[(t * k) & (S - 1)]) : v[0];
+  __syncthreads();
+  if (t < N1) {
+    float2 u[N2];
+#pragma unroll
+    for (int n = 0; n < N2; ++n) u[n] = buf[(t * N2 + n) * CB + c];
+    dft(u);
+#pragma unroll
+    for (int k = 0; k < N2; ++k) spec[((size_t)(t + N1 * k) * S + jy) * M + c0 + c] = u[k];
+  }
+}
+
+template <int S>
+__global__ void __launch_bounds__(VolShape<S>::TP)
+volume_plane_kernel(const float2 *__restrict__ spec, float2 *__restrict__ out) {
+  using V = VolShape<S>;
+  constexpr int M = V::M, N1 = V::N1, N2 = V::N2, R1 = V::R1, R2 = V::R2, GP = V::GP, P = V::P;
+  extern __shared__ __align__(16) unsigned char raw[];
+  float2 *tw = reinterpret_cast<float2 *>(raw);
+  float2 *buf = tw + S;  // [S][P]
+  spec += (size_t)blockIdx.x * S * M;
+  out += (size_t)blockIdx.x * S * M;
+  {
+    const int t = threadIdx.x / M, c = threadIdx.x % M;
+    float2 v[N1];
+#pragma unroll
+    for (int k = 0; k < N1; ++k) v[k] = spec[(t + N2 * k) * M + c];
+    fill_twiddles<S>(tw);
+    __syncthreads();
+    dft(v);
+#pragma unroll
+    for (int k = 0; k < N1; ++k) buf[(k * N2 + t) * P + c] = k ? cmul(v[k], tw[(t * k) & (S - 1)]) : v[0];
+    __syncthreads();
+    float2 u[N1 / N2][N2];
+#pragma unroll
+    for (int i = 0; i < N1 / N2; ++i)
+#pragma unroll
+      for (int n = 0; n < N2; ++n) u[i][n] = buf[((t + N2 * i) * N2 + n) * P + c];
+    __syncthreads();
+#pragma unroll
+    for (int i = 0; i < N1 / N2; ++i) {
+      dft(u[i]);
+#pragma unroll
+      for (int k = 0; k < N2; ++k) buf[(t + N2 * i + N1 * k) * P + c] = u[i][k];
+    }
+    __syncthreads();
+  }
+  // x lines: with Y the row and W = W_S, x[2n] + i x[2n + 1] is the transform over M
+  // points of E + i O, E[k] = Y[k] + conj Y[M - k], O[k] = (Y[k] - conj Y[M - k]) W^k;
+  // Y[M] = 0, and Y[0] counts by its real part
+  const int t = threadIdx.x % R2;
+  for (int row = threadIdx.x / R2; row < S; row += V::TP / R2) {
+    float2 *b = buf + row * P;
+    float2 v[R1];
+#pragma unroll
+    for (int n = 0; n < R1; ++n) {
+      const int k = t + R2 * n;
+      float2 y = b[k], z = make_float2(0.f, 0.f);
+      if (k) z = b[M - k];
+      else y.y = 0.f;
+      const float2 o = cmul(make_float2(y.x - z.x, y.y + z.y), tw[k]);
+      v[n] = make_float2(y.x + z.x - o.y, y.y - z.y + o.x);
+    }
+    __syncwarp();
+    dft(v);
+#pragma unroll
+    for (int k = 0; k < R1; ++k) b[k * GP + t] = k ? cmul(v[k], tw[2 * t * k]) : v[0];  // W_M = W_S^2
+    __syncwarp();
+#pragma unroll
+    for (int j = 0; j < R1 / R2; ++j) {
+      float2 u[R2];
+#pragma unroll
+      for (int n = 0; n < R2; ++n) u[n] = b[(t + j * R2) * GP + n];
+      if constexpr (R2 == 8) dft(u);
+      else dft4(u[0], u[1], u[2], u[3]);
+#pragma unroll
+      for (int n = 0; n < R2; ++n) out[row * M + t + j * R2 + R1 * n] = u[n];
+    }
+  }
+}
+
+template <int S>
+cudaError_t run_volume(const Geom &g, const float *acc, size_t plane, float w_clip, float2 *spec,
+                       float *out, cudaStream_t st) {
+  using V = VolShape<S>;
+  // the plane kernel stores pairs of floats (cuFFT refuses such an output too)
+  if (reinterpret_cast<uintptr_t>(out) % sizeof(float2)) return cudaErrorInvalidValue;
+  const size_t smem = (size_t)(S + S * V::P) * sizeof(float2);
+  auto pk = volume_plane_kernel<S>;
+  cudaError_t e = allow_dynamic_smem((const void *)pk, smem);
+  if (e != cudaSuccess) return e;
+  const float inv_n = 1.0f / ((float)S * (float)S * (float)S);
+  volume_z_kernel<S><<<S * (V::M / V::CB), V::TZ, 0, st>>>(g, acc, plane, w_clip, inv_n, spec);
+  pk<<<S, V::TP, smem, st>>>(spec, reinterpret_cast<float2 *>(out));
+  return cudaGetLastError();
+}
+
 template <int S>
 cudaError_t run(const float *real, float2 *spec, int m, int center, void *out, int f16,
                 cudaStream_t st) {
@@ -230,6 +398,14 @@ cudaError_t run(const float *real, float2 *spec, int m, int center, void *out, i
 }
 
 }  // namespace
+
+bool fft_volume_here(int S) { return S == 64 || S == 128; }
+
+cudaError_t fft_volume(const Geom &g, const float *acc, size_t plane, float w_clip, float2 *spec,
+                       float *out, cudaStream_t st) {
+  return g.S == 64 ? run_volume<64>(g, acc, plane, w_clip, spec, out, st)
+                   : run_volume<128>(g, acc, plane, w_clip, spec, out, st);
+}
 
 bool fft_images_here(int S) { return S == 64 || S == 128 || S == 256; }
 

@@ -126,6 +126,10 @@ cudaError_t launch_merge_scratch(const InsertArgs &a, cudaStream_t st);
 float otf_inv_pa(double alpha);
 // coefficients (power basis in x = 2 r^2 / a^2 - 1) of the weight polynomial
 void weight_polynomial(double alpha, float *poly);
+// the weighting and inverse transform of fr_reconstruct; spec: S * S * S / 2 float2
+bool fft_volume_here(int S);
+cudaError_t fft_volume(const Geom &g, const float *acc, size_t plane, float w_clip, float2 *spec,
+                       float *out, cudaStream_t st);
 // images' transforms by this library's kernels (fr_fft.cu): whether there are any
 // for this size, and the transforms of m real images into out (float2 or half2
 // spectra), by way of spec (m S (S/2 + 1) float2; may be out itself for float2)

@@ -2,9 +2,10 @@
 // insertion, on the GPU: the forward transforms of the images (the step the
 // paper runs on the CPU before uploading), staged into the insertion's input
 // layout and dtype, and the last step, applying the weights W to G and
-// transforming back.  The staging and weighting kernels are this library's;
-// the FFTs are the vendor's plain R2C / C2R transforms (cuFFT), loaded at run
-// time so that libfr.so does not depend on them.
+// transforming back.  For the power-of-two sizes both go through this library's
+// transforms (fr_fft.cu); for the others the staging and weighting kernels are this
+// library's and the FFTs the vendor's plain R2C / C2R transforms (cuFFT), loaded
+// at run time so that libfr.so does not depend on them.
 //
 // Last step:
 //   Vs(v) = V(v) + conj(V(-v)),  Ws(v) = W(v) + W(-v)   (undo the half-space fold)
@@ -171,8 +172,9 @@ using namespace fr;
 
 extern "C" int fr_reconstruct(fr_ctx *c, float *out, float w_clip, void *stream) {
   if (!c || !out || !(w_clip > 0.f)) return FR_ERR_INVALID_ARG;
-  const Cufft &fft = cufft();
-  if (!fft.ok) return FR_ERR_UNSUPPORTED;
+  const bool own = fft_volume_here(c->S);  // this library's kernels (fr_fft.cu), else cuFFT
+  if (!own && !cufft().ok) return FR_ERR_UNSUPPORTED;
+  const Cufft &fft = g_fft;
   cudaStream_t st = static_cast<cudaStream_t>(stream);
   const Geom &g = c->g;
   const size_t nspec = (size_t)g.S * g.S * (g.H + 1);
@@ -183,7 +185,7 @@ extern "C" int fr_reconstruct(fr_ctx *c, float *out, float w_clip, void *stream)
       return FR_ERR_OOM;
     }
   }
-  if (c->fft_plan < 0) {
+  if (!own && c->fft_plan < 0) {
     cufftHandle h = 0;
     if (fft.plan3d(&h, g.S, g.S, g.S, CUFFT_C2R) != CUFFT_SUCCESS) return FR_ERR_CUDA;
     c->fft_plan = (int)h;
@@ -195,6 +197,15 @@ extern "C" int fr_reconstruct(fr_ctx *c, float *out, float w_clip, void *stream)
       fr_note_cuda_error((int)e);
       return FR_ERR_CUDA;
     }
+  }
+  if (own) {
+    cudaError_t e = fft_volume(g, c->acc, c->plane, w_clip, c->spec, out, st);
+    if (e != cudaSuccess) {
+      fr_note_cuda_error((int)e);
+      return FR_ERR_CUDA;
+    }
+    c->last_stream = st;
+    return FR_OK;
   }
   int sms = 0, dev = 0;
   cudaGetDevice(&dev);

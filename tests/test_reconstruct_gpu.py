@@ -48,6 +48,31 @@ def test_reconstruct_matches_reference_on_same_sums(S, n, a, w_clip):
     assert err <= 1e-5, err
 
 
+@pytest.mark.parametrize("S,n,a,w_clip", [(64, 30, 1.5, 1.0), (64, 20, 2.5, 0.05), (128, 24, A32, 1.0)])
+def test_own_volume_transform(S, n, a, w_clip):
+    """Sizes with this library's own transform, against the reference on the same
+    sums; an output at any 8-byte address, nothing written around it, one at 4 bytes refused."""
+    img, rot = inputs.make_batch(S, n, 90 + S)
+    V, W, f = _run(S, [(img, rot)], a, w_clip=w_clip)
+    ref = recon.reconstruct(S, V.astype(np.complex128), W.astype(np.float64), w_clip)
+    err = np.max(np.abs(f - ref)) / np.max(np.abs(ref))
+    assert err <= 1e-5, err
+    ctx = L.fr_create(S, a, ALPHA, 0, 10000)
+    try:
+        L.fr_set_options(ctx, tuning=0, forced_config=-1)
+        L.fr_insert(ctx, img.cuda(), rot.cuda())
+        buf = torch.full((S ** 3 + 4,), float("nan"), device="cuda")
+        L.fr_reconstruct(ctx, buf[2:2 + S ** 3], w_clip)
+        with pytest.raises(L.FrError):
+            L.fr_reconstruct(ctx, buf[1:1 + S ** 3], w_clip)
+        torch.cuda.synchronize()
+        assert torch.isnan(buf[:2]).all() and torch.isnan(buf[-2:]).all()
+        err = np.max(np.abs(buf[2:-2].cpu().numpy().reshape(S, S, S) - ref)) / np.max(np.abs(ref))
+        assert err <= 1e-5, err
+    finally:
+        L.fr_destroy(ctx)
+
+
 @pytest.mark.parametrize("f16", [False, True])
 def test_reconstruct_end_to_end(f16):
     S = 32
