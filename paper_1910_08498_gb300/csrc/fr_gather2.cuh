@@ -17,8 +17,8 @@
 //    8-bit tag per item (column, z level) at positions from a warp scan;
 //  * evaluation: 32 items a round, one per lane: u = R^T v from the footprint
 //    centre's compensated projection, the 4 x 4 candidate box at rint(u - 1.5)
-//    (it covers [u - a, u + a] for every a < 2; for 2 <= a < 3 the 6 x 6 box at
-//    rint(u - 2.5)), clamped into the patch (rows and columns moved in by the
+//    (it covers [u - a, u + a] for every a < 2; for 2 <= a <= 2.5 the 5 x 5 box
+//    at rint(u - 2), for a < 3 the 6 x 6 box at rint(u - 2.5)), clamped into the patch (rows and columns moved in by the
 //    clamp lie outside the blob and are masked), its pixels from the patch, the
 //    Chebyshev weight polynomial in
 //    x = 2 r^2 / a^2 - 1 for two candidates at a time with packed FP32x2 FMAs
