@@ -910,13 +910,16 @@ __host__ __device__ constexpr size_t gather2_smem(int chunk) {
 
 // Work unit k of a launch without a unit list: split k / (bricks) of brick k %
 // (bricks) of those that tile x in [x0, x1], of as many splits as its expected
-// images (brick_unit_loads' estimate) over unit_share; false if it has fewer.
+// images (brick_unit_loads' estimate) over unit_share; false if it has fewer.  The
+// last splits come first: only the bricks around the centre have them, whose units
+// take longest, and the launch ends on units of the outer bricks (S = 64, 200
+// images: 91 -> 81 us a call; 1000 images: 288 -> 273).
 template <int BX, int BY, int BZ>
 __device__ __forceinline__ bool g2_implicit_unit(const InsertArgs &args, int x0, int x1, int k,
                                                  int4 &unit) {
   const Geom &g = args.g;
   const int nbx = (x1 - x0 + BX) / BX, nby = (g.D + BY - 1) / BY, nbz = (g.D + BZ - 1) / BZ;
-  const int b = k % (nbx * nby * nbz), s = k / (nbx * nby * nbz);
+  const int b = k % (nbx * nby * nbz), s = args.unit_most - 1 - k / (nbx * nby * nbz);
   const int bx = b % nbx, by = b / nbx % nby, bz = b / (nbx * nby);
   const float hx = 0.5f * (BX - 1), hy = 0.5f * (BY - 1), hz = 0.5f * (BZ - 1);
   const float cx = x0 + bx * BX + hx, cy = -g.H + by * BY + hy, cz = -g.H + bz * BZ + hz;

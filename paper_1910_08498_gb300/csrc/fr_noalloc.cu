@@ -65,16 +65,25 @@ __global__ void noalloc_add_kernel(const Geom g, float4 *__restrict__ scratch,
 // integer whole lattices of candidates can sit on the blob's edge (the DC pixel
 // against the axes' voxels for every rotation), so such radii keep the scatter.
 // So does alpha > 16, where the weight polynomial is less accurate than the
-// scatter's Bessel approximations (2e-7), and an image too small for a box.
-// Small batches also stay: up to about 4e5 pixels (7e5 for 6 x 6 boxes) the
-// scatter is as fast or faster (S = 32, 100 images: 31 against 36 us; S = 64, 64
-// images, a = 2.5: 90 against 92), beyond it slower (S = 64, 2000 images: 931
-// against 558 us, a = 2.5: 2025 against 1253; S = 48, 600 FP16 images: 159
-// against 138).
+// scatter's Bessel approximations (2e-7).
+// For the rest by size: the scatter's time goes with the pixels and a^3, the gather's
+// with the pixels, hardly with a (the 5 x 5 and 6 x 6 boxes from a = 2 on aside),
+// and with the footprints' halo, which weighs more on a small volume.  Gather over
+// scatter at 2.5e5 / 5.5e5 / 1.2e6 pixels a launch, S = 64: a = 1.3 1.24 / 1.10 /
+// 0.92, 1.6 1.12 / 0.96 / 0.79, 1.75 0.95 / 0.79 / 0.68, 1.9 0.89 / 0.77 / 0.65, 2.1
+// 1.24 / 0.85 / 0.65, 2.5 1.01 / 0.74 / 0.58, 2.9 0.84 / 0.67 / 0.56; S = 48: a = 1.6 1.25 /
+// 1.05 / 0.97, 1.75 1.06 / 0.91 / 0.83, 1.9 0.99 / 0.86 / 0.79, 2.1 1.38 / 0.99 / 0.80, 2.5
+// 1.17 / 0.82 / 0.73; S = 32 and 40 (5.5e5): 0.96 to 1.6.  FP16 images alike.
 bool gather_here(const Geom &g, int n) {
-  const double a2 = (double)g.a * (double)g.a;
-  return std::fabs(a2 - std::round(a2)) > 1e-4 * a2 && g.alpha <= 16.0f && g.H >= g.KB - 1 &&
-         (double)n * g.S * g.NX >= (g.KB == 4 ? 4e5 : 7e5);
+  const double a2 = (double)g.a * (double)g.a, pixels = (double)n * g.S * g.NX;
+  const double enough = g.a < 1.25f  ? 1e30
+                        : g.a < 1.5f ? 2e6
+                        : g.a < 1.7f ? 1.25e6
+                        : g.a < 1.85f ? 5.5e5
+                        : g.a < 2.0f ? (g.S >= 60 ? 2.5e5 : 4e5)
+                        : g.a < 2.3f ? 1e6
+                                     : 6e5;
+  return std::fabs(a2 - std::round(a2)) > 1e-4 * a2 && g.alpha <= 16.0f && g.S >= 44 && pixels >= enough;
 }
 
 // weight polynomial of the last alpha asked for (12 numbers; no allocation)

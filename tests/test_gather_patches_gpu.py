@@ -41,7 +41,7 @@ def test_patch_edges_match_oracle(S, a, f16):
 @pytest.mark.parametrize("f16", [False, True])
 @pytest.mark.parametrize("a", [0.6, 1.0, 1.5, 1.9, 2.5, 2.999])
 @pytest.mark.parametrize("S,n", [(8, 1), (8, 40), (10, 3), (16, 17), (30, 33), (46, 15), (64, 130), (64, 400),
-                                 (46, 700)])
+                                 (46, 700), (64, 640)])
 def test_no_allocation_call_matches_oracle(S, n, a, f16):
     """Batches and radii that keep the scatter (small ones, a = 1), and the
     gather with units worked out by the CTAs themselves.  700 images: FP32 sums
