@@ -31,7 +31,8 @@
 // kept that pipe 90 % busy at 63 % issue: 13.4 ms for 5000 FP32 images of 256^2.
 // From the patches a round costs about 50, and one 512-voxel footprint a warp
 // (137 items an entry) halves the work per entry against 256 voxels; with an
-// entry's last half round on two lanes an item and 14 candidates a box: 8.4 ms.
+// entry's last half round on two lanes an item and 14 candidates a box: 8.4 ms; with
+// the phase counters in a kernel of their own: 8.2 ms.
 // Now the instructions bound it: 74 % issue, of which a quarter are packed FMAs
 // that hold the FMA pipe for two cycles (60 % busy); shared memory 63 %.  About a
 // quarter of the time is per-entry work (copies 0.6 ms, tags 0.2, records 0.2).
@@ -423,7 +424,7 @@ __host__ __device__ constexpr int g2_warps() {
 // in the inner loops.  FOLD = 0: the bricks tile x >= floor(a) + 1; FOLD = 1:
 // they tile x >= -floor(a) and only the fold columns |x| <= floor(a) are
 // computed, with the fold predicate tested per candidate.
-template <int BX, int BY, int BZ, int F16, int KB = 4, int FW = 8, int FOLD = 0>
+template <int BX, int BY, int BZ, int F16, int KB = 4, int FW = 8, int FOLD = 0, int PROF = 0>
 __device__ __forceinline__ void gather2_warp(const InsertArgs &args, const InsertArgs &cst,
                                              const void *images, unsigned char *wsmem,
                                              const int4 unit, const int warp) {
@@ -478,10 +479,12 @@ __device__ __forceinline__ void gather2_warp(const InsertArgs &args, const Inser
 
   g2_clear<WV>(s_acc, lane);
   __syncwarp();
-  // optional phase counters (fr_options.debug bit 1): cycles of cull, item
-  // generation with the patches (PH_QUEUE), evaluation rounds (PH_DRAIN_FAST)
-  // and flushes, item and round counts, added by lane 0
-  const bool prof = args.phase != nullptr;
+  // PROF: phase counters (fr_options.debug bit 1), cycles of cull, item generation
+  // with the patches (PH_QUEUE), evaluation rounds (PH_DRAIN_FAST) and flushes, item
+  // and round counts, added by lane 0.  In kernels of their own: tests of a flag cost
+  // the others 12 registers and 3 % (2500 images of 256^2: 4.29 -> 4.17 ms without;
+  // 1000 of 128^2: 584 -> 564 us; 777 of 96^2, a = 2.5: 608 -> 588 us)
+  const bool prof = PROF && args.phase != nullptr;
   auto tick = [&]() -> long long { return prof ? clock64() : 0; };
   auto count = [&](int what, long long v) {
     if (prof && lane == 0) atomicAdd(args.phase + what, (unsigned long long)v);
@@ -940,7 +943,7 @@ __device__ __forceinline__ bool g2_implicit_unit(const InsertArgs &args, int x0,
 // registers per thread, and what shared memory holds; more are not resident).
 // KB: box width of the fold columns (4, or 6 for a >= 2), KBM: of the main bricks (5
 // for 2 <= a <= 2.5).
-template <int BX, int BY, int BZ, int F16, int MINW, int KB = 4, int KBM = KB>
+template <int BX, int BY, int BZ, int F16, int MINW, int KB = 4, int KBM = KB, int PROF = 0>
 __global__ void __launch_bounds__(32, MINW)
 gather2_kernel(const __grid_constant__ InsertArgs args) {
   extern __shared__ __align__(16) unsigned char smem[];
@@ -953,13 +956,13 @@ gather2_kernel(const __grid_constant__ InsertArgs args) {
     const int k = blockIdx.x / WF;
     if (args.units) unit = args.fold[k];
     else if (!g2_implicit_unit<FW, G2_FOLD_BY, G2_FOLD_BZ>(args, g.xa0, -g.xa0, k, unit)) return;
-    gather2_warp<FW, G2_FOLD_BY, G2_FOLD_BZ, F16, KB, FW, 1>(args, args, args.images, smem, unit,
-                                                             (int)(blockIdx.x % WF));
+    gather2_warp<FW, G2_FOLD_BY, G2_FOLD_BZ, F16, KB, FW, 1, PROF>(args, args, args.images, smem, unit,
+                                                                   (int)(blockIdx.x % WF));
   } else {
     const int b = (int)blockIdx.x - nf, k = b / W;
     if (args.units) unit = args.units[k];
     else if (!g2_implicit_unit<BX, BY, BZ>(args, 1 - g.xa0, g.H, k, unit)) return;
-    gather2_warp<BX, BY, BZ, F16, KBM>(args, args, args.images, smem, unit, b % W);
+    gather2_warp<BX, BY, BZ, F16, KBM, 8, 0, PROF>(args, args, args.images, smem, unit, b % W);
   }
 }
 

@@ -61,6 +61,32 @@ def test_no_allocation_call_matches_oracle(S, n, a, f16):
     assert rel_err(Wn, Wr) <= TOL_F32, worst(Wn, Wr, S)
 
 
+@pytest.mark.parametrize("f16", [False, True])
+@pytest.mark.parametrize("a", [1.9, 2.5, 2.999])
+@pytest.mark.parametrize("config", [47, 49])
+def test_phase_counting_kernel_computes_the_same_sums(config, a, f16):
+    """The counters run in kernels of their own; 12 images are not split, so the
+    sums of two runs are the same bits."""
+    if a >= 2:
+        config = -1  # the default's wide boxes
+    S, n = 30, 12
+    img, rot = _batch(S, n, 3)
+    out = []
+    for debug in (0, 2):
+        ctx = L.fr_create(S, float(np.float32(a)), 15.0, 0, 10000)
+        try:
+            L.fr_set_options(ctx, tuning=0, forced_config=config, debug=debug)
+            L.fr_insert(ctx, (inputs.to_half(img) if f16 else img).cuda(), rot.cuda())
+            V = torch.empty((S + 1) ** 3, dtype=torch.complex64, device="cuda")
+            W = torch.empty((S + 1) ** 3, dtype=torch.float32, device="cuda")
+            L.fr_finalize(ctx, V, W)
+            out.append((V.cpu(), W.cpu(), sum(L.fr_debug_phase_counters(ctx).values())))
+        finally:
+            L.fr_destroy(ctx)
+    assert torch.equal(out[0][0], out[1][0]) and torch.equal(out[0][1], out[1][1])
+    assert out[0][2] == 0 and out[1][2] > 0
+
+
 def test_pixels_outside_the_blob_do_not_reach_a_voxel():
     """One infinite pixel: only the voxels within the radius of it are not finite."""
     S = 32
