@@ -129,14 +129,14 @@ __device__ __noinline__ void g2_ties(const float2 *cp, const float2 *p, float dx
 // The KB x KB box of an item: pixels p[l * PITCH + j], u at (dx, dy) from pixel
 // (0, 0), u_z^2 = uz2; returns the sums of w p (complex) and of w over the
 // candidates with r <= a.  FOLD: candidate (j, l) counts only if bit j of
-// rows[l] >> shift is set; with KB = 6 (a >= 2) candidates within rounding of
+// rows[l] >> shift is set; with KB > 4 (a >= 2) candidates within rounding of
 // the blob edge are left out, and whether there are any is returned (g2_ties).
 // ROWS < KB: only the box's first ROWS rows.
 template <int PITCH, int KB, int FOLD, int ROWS = KB>
 __device__ __forceinline__ bool g2_box(const float2 *cp, const float2 *p, float dx, float dy,
                                        float uz2, float cs, float sq, float &ar, float &ai,
                                        float &aw, const unsigned *rows, int shift) {
-  constexpr int NP = POLY_N, KP = KB / 2, RP = KB == 4 ? ROWS : 3;
+  constexpr int NP = POLY_N, RP = KB == 4 ? ROWS : 3, NX = (RP * KB + 1) / 2;
   // cp: coefficient pairs (c_k, c_k), kernel-parameter constants
   // scaled column offsets sq (dx - j): x = (sq dx)^2 + cs (dy^2 + u_z^2) - 1
   float d[KB];
@@ -155,32 +155,39 @@ __device__ __forceinline__ bool g2_box(const float2 *cp, const float2 *p, float 
     // (74 TFLOP/s measured; with three register pairs 44), so only the
     // polynomial is packed.  Unpacked it took 9.5 ms instead of 8.7 (S = 256, n =
     // 5000): 32 % more instructions at 83 % issue.
-    float2 x[RP * KP], h[RP * KP];
+    // Candidate (r, j) of the rows is half i % 2 of pair i / 2, i = r KB + j.  The fold
+    // columns' 5 x 5 box (2 <= a <= 2.5) takes 8 + 5 pairs, the 6 x 6 box 9 + 9: an insert
+    // of 777 images, S = 96, a = 2.5, 588 -> 546 us.
+    const int nc = (ROWS - r0 < RP ? ROWS - r0 : RP) * KB;  // a constant, unrolled
+    float2 x[NX], h[NX];
 #pragma unroll
-    for (int r = 0; r < RP; ++r) {
-      const float ey = dy - (float)(r0 + r);
-      const float Y = fmaf(cs * ey, ey, U);
-#pragma unroll
-      for (int j = 0; j < KP; ++j)
-        x[r * KP + j] = make_float2(fmaf(d[2 * j], d[2 * j], Y), fmaf(d[2 * j + 1], d[2 * j + 1], Y));
+    for (int i = 0; i < 2 * NX; ++i) {
+      const float ey = dy - (float)(r0 + i / KB), dj = d[i % KB];
+      const float xv = i < nc ? fmaf(dj, dj, fmaf(cs * ey, ey, U)) : 0.f;
+      if (i & 1) x[i / 2].y = xv;
+      else x[i / 2].x = xv;
     }
 #pragma unroll
-    for (int i = 0; i < RP * KP; ++i) h[i] = __ffma2_rn(cp[NP - 1], x[i], cp[NP - 2]);
+    for (int i = 0; i < NX; ++i)
+      if (2 * i < nc) h[i] = __ffma2_rn(cp[NP - 1], x[i], cp[NP - 2]);
 #pragma unroll
     for (int k = NP - 3; k >= 0; --k)
 #pragma unroll
-      for (int i = 0; i < RP * KP; ++i) h[i] = __ffma2_rn(h[i], x[i], cp[k]);
+      for (int i = 0; i < NX; ++i)
+        if (2 * i < nc) h[i] = __ffma2_rn(h[i], x[i], cp[k]);
 #pragma unroll
     for (int r = 0; r < RP; ++r) {
+      if (r * KB >= nc) continue;
       const unsigned m = FOLD ? rows[r0 + r] >> shift : 0u;
 #pragma unroll
       for (int j = 0; j < KB; ++j) {
-        const float2 xx = x[r * KP + j / 2], hh = h[r * KP + j / 2];
-        const float xv = j & 1 ? xx.y : xx.x, w = j & 1 ? hh.y : hh.x;
+        const int i = r * KB + j;
+        const float2 xx = x[i / 2], hh = h[i / 2];
+        const float xv = i & 1 ? xx.y : xx.x, w = i & 1 ? hh.y : hh.x;
         const float2 q = p[(r0 + r) * PITCH + j];
         bool in = xv <= 1.0f;
         if (FOLD) in = in && ((m >> j) & 1u);
-        if (FOLD && KB == 6) {
+        if (FOLD && KB > 4) {
           const bool tie = fabsf(xv - 1.0f) <= 2e-5f;
           ties = ties || tie;
           in = in && !tie;
@@ -674,8 +681,8 @@ __device__ __forceinline__ void gather2_warp(const InsertArgs &args, const Inser
         const float r00 = refl ? -q1.x : q1.x, r01 = refl ? -q2.x : q2.x;
         const int px = q3.y & 0xffff, py = q3.y >> 16;
         const bool up = r00 < 0.f;  // the predicate (folded) turns true along the row, else false
-        int t = 0;                  // columns before the turn, 0 .. 31
-#pragma unroll
+        int t = 0;                  // columns before the turn, 0 .. 31 (not unrolled: the code is cold)
+#pragma unroll 1
         for (int s = 16; s > 0; s >>= 1)
           if (fold_pred(r00, r01, px + t + s - 1, py + lane) != up) t += s;
         const unsigned before = t > 30 ? 0x7fffffffu : (1u << t) - 1u;
@@ -799,14 +806,14 @@ __device__ __forceinline__ void gather2_warp(const InsertArgs &args, const Inser
       const float tr = s_acc[it.slot], ti = s_acc[WV + it.slot], tw = s_acc[2 * WV + it.slot];
       float ar, ai, aw;
       bool ties = false;
-      if (HALF)
+      if (KB == 4 && !FOLD)
         g2_box14<PITCH>(cst.poly2, it.p, it.dx, it.dy, it.uz2, cs, sq, ar, ai, aw);
-      else if (KB == 5)
+      else if (KB == 5 && !FOLD)
         g2_box23<PITCH>(cst.poly2, it.p, it.dx, it.dy, it.uz2, cs, sq, ar, ai, aw);
       else
         ties = g2_box<PITCH, KB, FOLD>(cst.poly2, it.p, it.dx, it.dy, it.uz2, cs, sq, ar, ai, aw,
                                        it.rows, it.shift);
-      if (FOLD && KB == 6 && ties)
+      if (FOLD && KB > 4 && ties)
         g2_ties<PITCH, KB>(cst.poly2, it.p, it.dx, it.dy, it.uz2, cs, it.rows, it.shift, q1, q2,
                            make_int3(fx0 + (it.slot / ZC) % FW, fy0 + it.slot / (ZC * FW), z0 + it.slot % ZC),
                            make_int2((q3.y & 0xffff) + it.shift, (q3.y >> 16) + it.row), g.a, ar, ai, aw);
@@ -821,9 +828,9 @@ __device__ __forceinline__ void gather2_warp(const InsertArgs &args, const Inser
       const Item it = locate(s_tag[h], h);
       const float tr = s_acc[it.slot], ti = s_acc[WV + it.slot], tw = s_acc[2 * WV + it.slot];
       float ar, ai, aw;
-      g2_box<PITCH, KB, 0, KB / 2>(cst.poly2, it.p + half * (KB / 2 * PITCH), it.dx,
-                                   it.dy - (float)(half * (KB / 2)), it.uz2, cs, sq, ar, ai, aw,
-                                   it.rows, 0);
+      g2_box<PITCH, KB, FOLD, KB / 2>(cst.poly2, it.p + half * (KB / 2 * PITCH), it.dx,
+                                      it.dy - (float)(half * (KB / 2)), it.uz2, cs, sq, ar, ai, aw,
+                                      it.rows + half * (KB / 2), it.shift);
       ar += __shfl_xor_sync(FULL, ar, 16);
       ai += __shfl_xor_sync(FULL, ai, 16);
       aw += __shfl_xor_sync(FULL, aw, 16);
@@ -941,8 +948,8 @@ __device__ __forceinline__ bool g2_implicit_unit(const InsertArgs &args, int x0,
 // second kernel on a side stream the fold columns cost a fork and a join.  MINW:
 // resident warps per SM the register allocation must allow (16: at most 128
 // registers per thread, and what shared memory holds; more are not resident).
-// KB: box width of the fold columns (4, or 6 for a >= 2), KBM: of the main bricks (5
-// for 2 <= a <= 2.5).
+// KB: what the launch's geometry and shared memory are for (4, or 6 for a >= 2), KBM:
+// width of the boxes (5 for 2 <= a <= 2.5).
 template <int BX, int BY, int BZ, int F16, int MINW, int KB = 4, int KBM = KB, int PROF = 0>
 __global__ void __launch_bounds__(32, MINW)
 gather2_kernel(const __grid_constant__ InsertArgs args) {
@@ -956,7 +963,7 @@ gather2_kernel(const __grid_constant__ InsertArgs args) {
     const int k = blockIdx.x / WF;
     if (args.units) unit = args.fold[k];
     else if (!g2_implicit_unit<FW, G2_FOLD_BY, G2_FOLD_BZ>(args, g.xa0, -g.xa0, k, unit)) return;
-    gather2_warp<FW, G2_FOLD_BY, G2_FOLD_BZ, F16, KB, FW, 1, PROF>(args, args, args.images, smem, unit,
+    gather2_warp<FW, G2_FOLD_BY, G2_FOLD_BZ, F16, KBM, FW, 1, PROF>(args, args, args.images, smem, unit,
                                                                    (int)(blockIdx.x % WF));
   } else {
     const int b = (int)blockIdx.x - nf, k = b / W;
@@ -982,7 +989,7 @@ gather2_multi_kernel(const __grid_constant__ MultiLaunch p) {
   const int4 it = p.items[b < 0 ? (int)blockIdx.x / WF : p.nfold + b / W];
   const int4 unit = make_int4(it.x & 1023, (it.x >> 10) & 1023, (it.x >> 20) & 1023, it.y);
   if (b < 0)
-    gather2_warp<FW, G2_FOLD_BY, G2_FOLD_BZ, F16, KB, FW, 1>(p.descs[it.z], p.base, p.images[it.w],
+    gather2_warp<FW, G2_FOLD_BY, G2_FOLD_BZ, F16, KBM, FW, 1>(p.descs[it.z], p.base, p.images[it.w],
                                                              smem, unit, (int)(blockIdx.x % WF));
   else
     gather2_warp<BX, BY, BZ, F16, KBM>(p.descs[it.z], p.base, p.images[it.w], smem, unit, b % W);

@@ -205,7 +205,7 @@ double gather_unit_loads(const fr_ctx *c, int shape, int n, double target,
 // boxes (2 <= a < 3) the per-voxel gather's polynomial-weight configurations of
 // 8-deep bricks run the direct-drain gather of the same brick (shapes 0 and 1
 // of both families): on GB300 at S = 96, 777 FP32 images, a = 2.5, an insert
-// takes 0.66 ms instead of 2.39.  Tables and A&S weights, 4-deep bricks and images
+// takes 0.60 ms instead of 2.39.  Tables and A&S weights, 4-deep bricks and images
 // too small for a 6 x 6 box in the half plane (S < 10) stay with the per-voxel
 // gather; so does a < 2, where the direct-drain gather has its own
 // configurations.
