@@ -5,9 +5,11 @@
 //
 // The general path (cuFFT rows, cuFFT columns, then a staging pass) moves the
 // spectra through HBM three times; here the columns' kernel does the staging's
-// work.  1100 real images of 256^2, centred, to FP16: 323 -> 205 us.  Rows 97 us
-// for 1016 images (the L1 data pipe 88 % busy with the shared-memory exchanges; 80
-// us of HBM traffic), columns 97 us (60 us of HBM traffic; two CTAs of 90 KB an SM).
+// work.  1100 real images of 256^2, centred, to FP16: 323 -> 203 us.  For 1016 images
+// the rows take 94 us (80 us of HBM traffic; 97 with the partners of the last step
+// exchanged through shared memory, whose data pipe was 88 % busy; S = 64, 1500
+// images: 25 -> 23 us in all), the columns 97 us (60 us of HBM traffic; two CTAs of
+// 90 KB an SM; narrower blocks, three CTAs of 68 KB, took 123).
 //
 // Transforms by Cooley-Tukey with two factors (N = N1 N2): a thread takes N1 points
 // n2 + N2 n1, transforms them in registers (radix 4 and 2 steps), multiplies by
@@ -132,29 +134,31 @@ __global__ void __launch_bounds__(RowShape<S>::T) fft_rows_kernel(const float2 *
   for (int j = 0; j < J; ++j)
 #pragma unroll
     for (int n = 0; n < M2; ++n) u[j][n] = b[(t + j * M2) * SH::GP + n];
-  __syncwarp();
 #pragma unroll
   for (int j = 0; j < J; ++j) {
     if constexpr (M2 == 8) dft(u[j]);
     else dft4(u[j][0], u[j][1], u[j][2], u[j][3]);
-#pragma unroll
-    for (int n = 0; n < M2; ++n) b[t + j * M2 + N1 * n] = u[j][n];
   }
-  __syncwarp();
-  if (!in) return;
+  // Z[k], k = t + M2 j + N1 n, is u[j][n]; its partner Z[M - k] is lane (M2 - t) % M2's
+  // u[J - 1 - j][M2 - 1 - n], but lane 0's partners are its own.  By shuffles: half the
+  // shared-memory wavefronts of another exchange.
+  const int peer = (threadIdx.x & 31 & ~(M2 - 1)) | ((M2 - t) & (M2 - 1));
   float2 *dst = out + row * NX;
-  // X[k] and X[M - k] together: with e, d the two halves and q = W^k d, X[k] = e - i
-  // q and X[M - k] = conj(e) - i conj(q)
 #pragma unroll
-  for (int i = 0; i < N1 / 2; ++i) {
-    const int k = t + M2 * i;
-    const float2 z = b[k], y = b[(M - k) & (M - 1)];
-    const float2 e = make_float2(0.5f * (z.x + y.x), 0.5f * (z.y - y.y));  // (Z + conj Y) / 2
-    const float2 q = cmul(make_float2(0.5f * (z.x - y.x), 0.5f * (z.y + y.y)), tw[k]);
-    dst[k] = make_float2(e.x + q.y, e.y - q.x);
-    dst[M - k] = make_float2(e.x - q.y, -e.y - q.x);
-  }
-  if (t == 0) dst[M / 2] = make_float2(b[M / 2].x, -b[M / 2].y);  // W^(M/2) = -i
+  for (int j = 0; j < J; ++j)
+#pragma unroll
+    for (int n = 0; n < M2; ++n) {
+      const float2 z = u[j][n], g = u[J - 1 - j][M2 - 1 - n];
+      const float2 own = j ? u[(J - j) % J][M2 - 1 - n] : u[0][(M2 - n) % M2];
+      float2 y = make_float2(__shfl_sync(0xffffffffu, g.x, peer), __shfl_sync(0xffffffffu, g.y, peer));
+      if (t == 0) y = own;
+      const int k = t + M2 * j + N1 * n;
+      // X[k] = e - i q, e = (Z[k] + conj Z[M - k]) / 2, q = W^k (Z[k] - conj Z[M - k]) / 2
+      const float2 e = make_float2(0.5f * (z.x + y.x), 0.5f * (z.y - y.y));
+      const float2 q = cmul(make_float2(0.5f * (z.x - y.x), 0.5f * (z.y + y.y)), tw[k]);
+      if (in) dst[k] = make_float2(e.x + q.y, e.y - q.x);
+    }
+  if (in && t == 0) dst[M] = make_float2(u[0][0].x - u[0][0].y, 0.f);
 }
 
 // ---- columns: S points, S = N1 N2, of CB columns a CTA; centring and conversion
