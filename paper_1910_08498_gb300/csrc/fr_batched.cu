@@ -52,7 +52,7 @@ struct PlanKey {
 };
 
 struct Group {
-  int algo = ALGO_GATHER, shape = 0, kb = 4, f16 = 0, chunk = 64, minw = 0;
+  int algo = ALGO_GATHER, shape = 0, kb = 4, f16 = 0, chunk = 64;
   PersistentLaunch launch{};  // per-voxel gather: persistent launch
   MultiLaunch main{};         // direct-drain gather: its launch
   int lane = 0;               // direct-drain gather: the stream its launch runs on
@@ -115,7 +115,7 @@ int build_plan(Plan &pl, fr_ctx *const *ctxs, const void *const *images, const i
   // group the batches a multi-batch kernel can take: the direct-drain gather
   // by (configuration, dtype, S, blob), the persistent per-voxel gather by
   // (shape, box width, dtype, list capacity)
-  using GKey = std::tuple<int, int, int, int, int, int, int, float, float>;
+  using GKey = std::tuple<int, int, int, int, int, int, float, float>;
   std::map<GKey, std::vector<int>> groups;
   for (int b = 0; b < nb; ++b) {
     if (n[b] == 0) continue;
@@ -124,10 +124,10 @@ int build_plan(Plan &pl, fr_ctx *const *ctxs, const void *const *images, const i
     const int f16 = dtypes[b] == FR_F16 ? 1 : 0;
     const bool poly_ok = c->poly_err < 1e-6;
     if (k.algo == ALGO_GATHER2 && poly_ok) {
-      groups[GKey(ALGO_GATHER2, k.shape, c->g.KB, f16, k.chunk, k.minw, c->S, c->g.a, c->g.alpha)]
+      groups[GKey(ALGO_GATHER2, k.shape, c->g.KB, f16, k.chunk, c->S, c->g.a, c->g.alpha)]
           .push_back(b);
     } else if (k.algo == ALGO_GATHER && k.wmode == W_POLY && poly_ok) {
-      groups[GKey(ALGO_GATHER, k.shape, c->g.KB, f16, k.chunk, 0, 0, 0.f, 0.f)].push_back(b);
+      groups[GKey(ALGO_GATHER, k.shape, c->g.KB, f16, k.chunk, 0, 0.f, 0.f)].push_back(b);
     } else {
       // its own launches: units and scratch ready before any capture
       int rc = prepare_config(c, cfg[b], n[b]);
@@ -161,7 +161,7 @@ int build_plan(Plan &pl, fr_ctx *const *ctxs, const void *const *images, const i
     Group gr;
     int S_ = 0;
     float a_ = 0.f, alpha_ = 0.f;
-    std::tie(gr.algo, gr.shape, gr.kb, gr.f16, gr.chunk, gr.minw, S_, a_, alpha_) = kv.first;
+    std::tie(gr.algo, gr.shape, gr.kb, gr.f16, gr.chunk, S_, a_, alpha_) = kv.first;
     const bool g2 = gr.algo == ALGO_GATHER2;
     const GatherShape sh = g2 ? gather2_shape(gr.shape) : gather_shape(gr.shape);
     auto main_loads = [&](const fr_ctx *c, int nn, double target, std::vector<UnitLoad> &out,
@@ -302,7 +302,7 @@ int enqueue_plan(const Plan &pl, fr_ctx *const *ctxs, const void *const *images,
       e = cudaStreamWaitEvent(pl.lanes[l], pl.ev_fork, 0);
     for (const Group &gr : pl.groups)
       if (e == cudaSuccess && gr.algo == ALGO_GATHER2)
-        e = launch_gather2_multi(gr.shape, gr.minw, gr.f16, gr.main, pl.lanes[gr.lane]);
+        e = launch_gather2_multi(gr.shape, gr.f16, gr.main, pl.lanes[gr.lane]);
     for (int l = 0; l < nl && e == cudaSuccess; ++l) e = cudaEventRecord(pl.ev_join[l], pl.lanes[l]);
     if (e != cudaSuccess) return cuda_err(e);
   }
@@ -334,7 +334,7 @@ int prime_plan(const Plan &pl, fr_ctx *const *ctxs, const int *dtypes, const std
     if (gr.algo == ALGO_GATHER2) {
       MultiLaunch q = gr.main;
       q.nitems = q.nfold = 0;
-      e = launch_gather2_multi(gr.shape, gr.minw, gr.f16, q, nullptr);
+      e = launch_gather2_multi(gr.shape, gr.f16, q, nullptr);
     } else {
       PersistentLaunch q = gr.launch;
       q.nitems = 0;
@@ -351,7 +351,7 @@ int prime_plan(const Plan &pl, fr_ctx *const *ctxs, const int *dtypes, const std
     if (k.algo == ALGO_GATHER) {
       e = launch_gather(k.shape, k.wmode, a, nullptr, 1, nullptr);
     } else if (k.algo == ALGO_GATHER2) {
-      e = launch_gather2(k.shape, k.minw, a, nullptr, 1, nullptr);
+      e = launch_gather2(k.shape, a, nullptr, 1, nullptr);
     } else {
       e = launch_scatter(k.threads, k.wmode, a, nullptr, 1, nullptr);
     }

@@ -89,37 +89,37 @@ GatherShape gather2_shape(int id) {
   return id >= 0 && id < num_gather2_shapes() ? kShapes2[id] : GatherShape{0, 0, 0};
 }
 
-cudaError_t launch_gather2_shape0(int minw, const InsertArgs &a, cudaStream_t st, int query_only,
+cudaError_t launch_gather2_shape0(const InsertArgs &a, cudaStream_t st, int query_only,
                                   KernelInfo *info);
-cudaError_t launch_gather2_shape1(int minw, const InsertArgs &a, cudaStream_t st, int query_only,
+cudaError_t launch_gather2_shape1(const InsertArgs &a, cudaStream_t st, int query_only,
                                   KernelInfo *info);
-cudaError_t launch_gather2_shape2(int minw, const InsertArgs &a, cudaStream_t st, int query_only,
+cudaError_t launch_gather2_shape2(const InsertArgs &a, cudaStream_t st, int query_only,
                                   KernelInfo *info);
 
-cudaError_t launch_gather2_multi_shape0(int minw, int f16, const MultiLaunch &p, cudaStream_t st);
-cudaError_t launch_gather2_multi_shape1(int minw, int f16, const MultiLaunch &p, cudaStream_t st);
-cudaError_t launch_gather2_multi_shape2(int minw, int f16, const MultiLaunch &p, cudaStream_t st);
+cudaError_t launch_gather2_multi_shape0(int f16, const MultiLaunch &p, cudaStream_t st);
+cudaError_t launch_gather2_multi_shape1(int f16, const MultiLaunch &p, cudaStream_t st);
+cudaError_t launch_gather2_multi_shape2(int f16, const MultiLaunch &p, cudaStream_t st);
 
-cudaError_t launch_gather2_multi(int shape_id, int minw, int f16, const MultiLaunch &p,
+cudaError_t launch_gather2_multi(int shape_id, int f16, const MultiLaunch &p,
                                  cudaStream_t st) {
   if (p.base.chunk > 128) return cudaErrorInvalidValue;
   switch (shape_id) {
-    case 0: return launch_gather2_multi_shape0(minw, f16, p, st);
-    case 1: return launch_gather2_multi_shape1(minw, f16, p, st);
-    case 2: return launch_gather2_multi_shape2(minw, f16, p, st);
+    case 0: return launch_gather2_multi_shape0(f16, p, st);
+    case 1: return launch_gather2_multi_shape1(f16, p, st);
+    case 2: return launch_gather2_multi_shape2(f16, p, st);
     default: return cudaErrorInvalidValue;
   }
 }
 
-cudaError_t launch_gather2(int shape_id, int minw, const InsertArgs &a, cudaStream_t st,
+cudaError_t launch_gather2(int shape_id, const InsertArgs &a, cudaStream_t st,
                            int query_only, KernelInfo *info) {
   if (a.chunk > 128) return cudaErrorInvalidValue;
   // pixel copies of eight bytes: fr_insert checks for 16-byte aligned images
   if (reinterpret_cast<uintptr_t>(a.images) & 15u) return cudaErrorInvalidValue;
   switch (shape_id) {
-    case 0: return launch_gather2_shape0(minw, a, st, query_only, info);
-    case 1: return launch_gather2_shape1(minw, a, st, query_only, info);
-    case 2: return launch_gather2_shape2(minw, a, st, query_only, info);
+    case 0: return launch_gather2_shape0(a, st, query_only, info);
+    case 1: return launch_gather2_shape1(a, st, query_only, info);
+    case 2: return launch_gather2_shape2(a, st, query_only, info);
     default: return cudaErrorInvalidValue;
   }
 }

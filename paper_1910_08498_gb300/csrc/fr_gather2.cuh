@@ -945,13 +945,12 @@ __device__ __forceinline__ bool g2_implicit_unit(const InsertArgs &args, int x0,
 // a brick).  Warps of one brick never wait for one another, but a CTA holds its
 // shared memory until its last warp ends: with two and four warps a CTA 17 % of
 // the resident warp slots stood idle.  Both kinds of unit in one launch: as a
-// second kernel on a side stream the fold columns cost a fork and a join.  MINW:
-// resident warps per SM the register allocation must allow (16: at most 128
-// registers per thread, and what shared memory holds; more are not resident).
-// KB: what the launch's geometry and shared memory are for (4, or 6 for a >= 2), KBM:
+// second kernel on a side stream the fold columns cost a fork and a join.  Shared
+// memory holds 16 CTAs an SM, so the registers are bounded for 16 (a bound for 24, 80
+// registers, spills: 8.5 ms instead of 8.2 for 5000 images of 256^2).  KB: what the launch's geometry and shared memory are for (4, or 6 for a >= 2), KBM:
 // width of the boxes (5 for 2 <= a <= 2.5).
-template <int BX, int BY, int BZ, int F16, int MINW, int KB = 4, int KBM = KB, int PROF = 0>
-__global__ void __launch_bounds__(32, MINW)
+template <int BX, int BY, int BZ, int F16, int KB = 4, int KBM = KB, int PROF = 0>
+__global__ void __launch_bounds__(32, 16)
 gather2_kernel(const __grid_constant__ InsertArgs args) {
   extern __shared__ __align__(16) unsigned char smem[];
   constexpr int FW = g2_fold_width<KB>(), W = g2_warps<BX, BY, BZ, 8>(),
@@ -979,8 +978,8 @@ gather2_kernel(const __grid_constant__ InsertArgs args) {
 // batches, are read from p.base (kernel parameters: constant operands in the
 // inner loops), the batch's own arguments (rotations, volume) from its
 // descriptor.
-template <int BX, int BY, int BZ, int F16, int MINW, int KB = 4, int KBM = KB>
-__global__ void __launch_bounds__(32, MINW)
+template <int BX, int BY, int BZ, int F16, int KB = 4, int KBM = KB>
+__global__ void __launch_bounds__(32, 16)
 gather2_multi_kernel(const __grid_constant__ MultiLaunch p) {
   extern __shared__ __align__(16) unsigned char smem[];
   constexpr int FW = g2_fold_width<KB>(), W = g2_warps<BX, BY, BZ, 8>(),

@@ -102,11 +102,10 @@ struct GatherShape {
 // launchers implemented in the .cu files
 cudaError_t launch_gather(int shape_id, int wmode, const InsertArgs &a, cudaStream_t st,
                           int query_only, KernelInfo *info);
-// direct-drain gather (fr_gather2.cuh): brick shape id of gather2_shape(),
-// register budget for minw (16, 20, 24) resident warps per SM
+// direct-drain gather (fr_gather2.cuh): brick shape id of gather2_shape()
 int num_gather2_shapes();
 GatherShape gather2_shape(int id);
-cudaError_t launch_gather2(int shape_id, int minw, const InsertArgs &a, cudaStream_t st,
+cudaError_t launch_gather2(int shape_id, const InsertArgs &a, cudaStream_t st,
                            int query_only, KernelInfo *info);
 size_t gather2_smem_bytes(const GatherShape &sh, int chunk);
 // allow a kernel `smem` bytes of dynamic shared memory on the current device
@@ -181,8 +180,7 @@ struct MultiLaunch {
   const void *images[MULTI_MAX];  // images of the launch's batches, by slot (read in the inner loop)
 };
 // the direct-drain gather, FP32 or FP16 images
-cudaError_t launch_gather2_multi(int shape_id, int minw, int f16, const MultiLaunch &p,
-                                 cudaStream_t st);
+cudaError_t launch_gather2_multi(int shape_id, int f16, const MultiLaunch &p, cudaStream_t st);
 
 // MLP kernels
 cudaError_t mlp_forward(const float *params, const float *x, int m, float *y, cudaStream_t st);

@@ -209,7 +209,7 @@ extern "C" int fr_insert_noalloc(int S, float a, float alpha, const void *images
       args.unit_most = std::max(1, std::min({64, args.n / 2, (int)std::ceil(1.02 * args.n / args.unit_share)}));
       args.nunits = bricks * args.unit_most;
       args.nfold = fold_bricks * args.unit_most;
-      e = launch_gather2(SHAPE, 16, args, st, 0, nullptr);
+      e = launch_gather2(SHAPE, args, st, 0, nullptr);
     } else {
       e = launch_scatter(256, W_OTF, args, st, 0, nullptr);
     }

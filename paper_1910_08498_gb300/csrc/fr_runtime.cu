@@ -211,10 +211,8 @@ double gather_unit_loads(const fr_ctx *c, int shape, int n, double target,
 // configurations.
 Config effective_config(const fr_ctx *c, int id) {
   Config cfg = config_space()[id];
-  if (cfg.algo == ALGO_GATHER && cfg.wmode == W_POLY && c->g.KB == 6 && cfg.shape <= 1 && c->g.H >= 5) {
+  if (cfg.algo == ALGO_GATHER && cfg.wmode == W_POLY && c->g.KB == 6 && cfg.shape <= 1 && c->g.H >= 5)
     cfg.algo = ALGO_GATHER2;
-    cfg.minw = 16;
-  }
   return cfg;
 }
 
@@ -318,7 +316,7 @@ int run_config(fr_ctx *c, int id, const void *images, int f16, const float *rot,
       a.scratch = c->scratch;
     }
     const cudaError_t e = cfg.algo == ALGO_GATHER2
-                              ? launch_gather2(cfg.shape, cfg.minw, a, st, 0, nullptr)
+                              ? launch_gather2(cfg.shape, a, st, 0, nullptr)
                               : launch_gather(cfg.shape, cfg.wmode, a, st, 0, nullptr);
     if (e != cudaSuccess) return cuda_fail(e);
     if (a.any_split) {

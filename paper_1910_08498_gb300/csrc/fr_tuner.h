@@ -46,7 +46,9 @@ struct Config {
   int chunk;    // gather: capacity of a warp's shared-memory image list
   int threads;  // scatter: block size
   int sub;      // scatter: images per atomic sub-batch (merged after each)
-  int minw = 0; // direct-drain gather: resident warps per SM the registers allow (16, 20, 24)
+  // direct-drain gather: 16, 20 or 24.  Resident warps per SM whose registers were
+  // to fit; all run the same kernel, of which shared memory holds 16
+  int minw = 0;
 };
 
 const std::vector<Config> &config_space();
