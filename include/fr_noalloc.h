@@ -4,10 +4,10 @@
  * The paper has no counterpart of this call: it is a service entry point of
  * this library.  It runs the same insertion as fr_insert (the definition is
  * written out in fr.h) through the direct-drain gather, or the atomic scatter
- * where that is the more exact one (a^2 within 1e-4 of an integer, alpha > 16)
- * or the faster one (small images, batches and radii), whose scratch volume is a
- * fixed array in the library's static device memory instead of a cudaMalloc'd
- * buffer.
+ * where that is the more exact one (a^2 within 1e-4 of an integer; the blob's
+ * edge weight 1 / I0(alpha) above 3e-6; alpha > 16) or the faster one (small
+ * images, batches and radii), whose scratch volume is a fixed array in the
+ * library's static device memory instead of a cudaMalloc'd buffer.
  *
  * Who needs it: callers that must not enter the device allocator for the
  * duration of the call.  cudaMalloc and cudaFree can synchronise the device

@@ -61,10 +61,16 @@ __global__ void noalloc_add_kernel(const Geom g, float4 *__restrict__ scratch,
 }
 
 // The scatter decides r <= a as the real numbers do for every candidate; the
-// gather does only in the fold columns for a >= 2.  With a^2 within 1e-4 of an
-// integer whole lattices of candidates can sit on the blob's edge (the DC pixel
-// against the axes' voxels for every rotation), so such radii keep the scatter.
-// So does alpha > 16, where the weight polynomial is less accurate than the
+// gather does only in the fold columns for a >= 2.  A candidate that rounding puts on
+// the wrong side of the edge costs its weight b(a) = 1 / I0(alpha): at alpha = 0 a
+// whole pixel, at alpha = 15 2.9e-6 of one.  At most eight pixels of an image lie at
+// one distance < 3 from a voxel (four below 1.58), and the voxel that all n images meet
+// holds W > 1.1 n (n), so with b(a) <= 3e-6 even all of them wrong at once, in every
+// image, make 2e-5 of the largest W.  Larger b(a) keep the scatter (a = sqrt(3.6),
+// rotations by the 3-4-5 angle: by the gather, V is off by 0.17 of its largest value at
+// alpha = 0, 1.2e-3 at 8).  So do a^2 within 1e-4 of an integer, where whole lattices of
+// candidates can sit on the edge (the DC pixel against the axes' voxels for every
+// rotation), and alpha > 16, where the weight polynomial is less accurate than the
 // scatter's Bessel approximations (2e-7).
 // For the rest by size: the scatter's time goes with the pixels and a^3, the gather's
 // with the pixels, hardly with a (the 5 x 5 and 6 x 6 boxes from a = 2 on aside),
@@ -74,7 +80,8 @@ __global__ void noalloc_add_kernel(const Geom g, float4 *__restrict__ scratch,
 // 1.24 / 0.85 / 0.65, 2.5 1.01 / 0.74 / 0.58, 2.9 0.84 / 0.67 / 0.56; S = 48: a = 1.6 1.25 /
 // 1.05 / 0.97, 1.75 1.06 / 0.91 / 0.83, 1.9 0.99 / 0.86 / 0.79, 2.1 1.38 / 0.99 / 0.80, 2.5
 // 1.17 / 0.82 / 0.73; S = 32 and 40 (5.5e5): 0.96 to 1.6.  FP16 images alike.
-bool gather_here(const Geom &g, int n) {
+constexpr float EDGE_WEIGHT_MAX = 3e-6f;  // alpha >= 14.99
+bool gather_here(const Geom &g, float edge_weight, int n) {
   const double a2 = (double)g.a * (double)g.a, pixels = (double)n * g.S * g.NX;
   const double enough = g.a < 1.25f  ? 1e30
                         : g.a < 1.5f ? 2e6
@@ -83,7 +90,8 @@ bool gather_here(const Geom &g, int n) {
                         : g.a < 2.0f ? (g.S >= 60 ? 2.5e5 : 4e5)
                         : g.a < 2.3f ? 1e6
                                      : 6e5;
-  return std::fabs(a2 - std::round(a2)) > 1e-4 * a2 && g.alpha <= 16.0f && g.S >= 44 && pixels >= enough;
+  return std::fabs(a2 - std::round(a2)) > 1e-4 * a2 && edge_weight <= EDGE_WEIGHT_MAX && g.alpha <= 16.0f &&
+         g.S >= 44 && pixels >= enough;
 }
 
 // weight polynomial of the last alpha asked for (12 numbers; no allocation)
@@ -188,7 +196,7 @@ extern "C" int fr_insert_noalloc(int S, float a, float alpha, const void *images
   const int add_blocks = (int)std::min<size_t>((cells + add_threads - 1) / add_threads,
                                                (size_t)sms * 8);
   constexpr int SHAPE = 1;  // 16 x 8 x 8 bricks
-  const bool gather_any = gather_here(g, std::min(n, NOALLOC_SUB));
+  const bool gather_any = gather_here(g, args.inv_i0a, std::min(n, NOALLOC_SUB));
   if (gather_any) {
     cached_polynomial(alpha, args.poly);
     for (int k = 0; k < POLY_N; ++k) args.poly2[k] = make_float2(args.poly[k], args.poly[k]);
@@ -200,7 +208,7 @@ extern "C" int fr_insert_noalloc(int S, float a, float alpha, const void *images
     args.n = std::min(NOALLOC_SUB, n - i0);
     args.images = static_cast<const unsigned char *>(images) + (size_t)i0 * img_bytes;
     args.rot = rotations + (size_t)i0 * 9;
-    if (gather_any && gather_here(g, args.n)) {
+    if (gather_any && gather_here(g, args.inv_i0a, args.n)) {
       int bricks = 0, fold_bricks = 0;
       const double total = brick_images(g, gather2_shape(SHAPE), 1 - g.xa0, g.H, args.n, &bricks);
       brick_images(g, fold_shape(g.KB), g.xa0, -g.xa0, args.n, &fold_bricks);

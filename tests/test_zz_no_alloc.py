@@ -106,3 +106,53 @@ def test_noalloc_fp16_images():
     Wn = W.cpu().numpy().astype(np.float64)
     assert rel_err(Vn, Vr) <= TOL_F16 and rel_err(Wn, Wr) <= TOL_F16
     assert rel_err(Vn, V16) <= TOL_F32 and rel_err(Wn, W16) <= TOL_F32
+
+
+def _lattice_rotations(n):
+    """Rotations by the 3-4-5 angle about each axis, turned by the signed
+    permutations: for a^2 = 3.6 pixels lie at distance a from voxels, to rounding,
+    all over the volume."""
+    c, s = 0.6, 0.8
+    turns = [np.array(m) for m in ([[c, -s, 0], [s, c, 0], [0, 0, 1]], [[1, 0, 0], [0, c, -s], [0, s, c]],
+                                   [[c, 0, s], [0, 1, 0], [-s, 0, c]])]
+    perms = inputs.proper_signed_permutations().double().numpy()
+    rots = [p @ t for t in turns for p in perms]
+    return torch.tensor(np.stack([rots[i % len(rots)] for i in range(n)]), dtype=torch.float32)
+
+
+def _noalloc(S, img, rot, a, alpha):
+    V = torch.zeros((S + 1) ** 3, dtype=torch.complex64, device="cuda")
+    W = torch.zeros((S + 1) ** 3, dtype=torch.float32, device="cuda")
+    assert L.fr_insert_noalloc(S, img.cuda(), rot.cuda(), V, W, a=a, alpha=alpha) == L.FR_OK
+    return V.cpu().numpy().astype(np.complex128), W.cpu().numpy().astype(np.float64)
+
+
+@pytest.mark.gpu
+@pytest.mark.parametrize("alpha", [0.0, 2.0, 8.0, 15.0])
+@pytest.mark.parametrize("a,lattice", [(3.6 ** 0.5, True), (A32, False), (6.4 ** 0.5, True)])
+def test_noalloc_decides_the_blob_edge_for_every_taper(a, lattice, alpha):
+    """b(a) = 1 / I0(alpha) is 1 at alpha = 0: a candidate at the blob's edge that
+    is decided wrongly then costs a whole pixel.  Sizes and radii at which the
+    gather is the faster kernel."""
+    S, n = L.FR_NOALLOC_MAX_S, 400
+    a = float(np.float32(a))
+    img, rot = inputs.make_batch(S, n, 45)
+    if lattice:
+        rot = _lattice_rotations(n)
+    V, W = _noalloc(S, img, rot, a, alpha)
+    Vr, Wr, _ = oracle_insert(S, [(img, rot)], a=a, alpha=alpha)
+    assert rel_err(V, Vr) <= TOL_F32, worst(V, Vr, S)
+    assert rel_err(W, Wr) <= TOL_F32, worst(W, Wr, S)
+
+
+@pytest.mark.gpu
+@pytest.mark.parametrize("tail", [20, 300])
+def test_noalloc_sub_batches_of_both_kernels(tail):
+    """A full sub-batch by the gather, then a tail that is small enough for the
+    scatter or large enough for the gather."""
+    S, n = L.FR_NOALLOC_MAX_S, 1024 + tail
+    img, rot = inputs.make_batch(S, n, 46)
+    V, W = _noalloc(S, img, rot, A32, ALPHA)
+    Vr, Wr, _ = oracle_insert(S, [(img, rot)])
+    assert rel_err(V, Vr) <= TOL_F32, worst(V, Vr, S)
+    assert rel_err(W, Wr) <= TOL_F32, worst(W, Wr, S)
