@@ -61,12 +61,12 @@ extern "C" {
  * same device) race on it and both results are wrong: the caller must order
  * them (one stream, or events between streams).
  *
- * The first call on each device performs a one-time setup: it looks up the
- * scratch array's address with cudaGetSymbolAddress (which also loads the
- * library's device code on that device if lazy loading has not done so yet)
- * while that device is current, caches it, and allows the gather kernel its
- * shared memory.  Make that first call before
- * any stream capture begins.
+ * The first call on each device (of any size, dtype and blob, with n > 0)
+ * performs a one-time setup while that device is current: it looks up the
+ * scratch array's address with cudaGetSymbolAddress and caches it, loads the
+ * code of every kernel that a later call can launch, and allows the gather
+ * kernels their shared memory.  Make that first call before any stream
+ * capture begins.
  *
  * The batch is added in sub-batches of 1024 images, each merged into V and W
  * before the next: if a launch fails part way (FR_ERR_CUDA), the sub-batches

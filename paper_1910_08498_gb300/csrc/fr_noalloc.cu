@@ -7,7 +7,7 @@
 // scatter stays where the gather cannot decide as exactly or has no box (see
 // gather_here).  Nothing here allocates:
 // no cudaMalloc, no cudaFree, no allocating library routine; the scratch
-// address is looked up once per device with cudaGetSymbolAddress.
+// address is looked up and every kernel loaded in the device's first call.
 #include <cuda_runtime.h>
 
 #include <algorithm>
@@ -124,6 +124,38 @@ double brick_images(const Geom &g, const GatherShape &sh, int x0, int x1, int n,
   return total;
 }
 
+constexpr int GATHER_SHAPE = 1;  // 16 x 8 x 8 bricks
+constexpr int GATHER_CHUNK = 64;
+
+// Everything a later call would otherwise set up on its way: the code of each kernel
+// that some call can launch (cudaFuncGetAttributes loads it), the gather's shared
+// memory attribute and the host-side caches behind both.  Once per device, under
+// g_mu.
+cudaError_t setup_device(DeviceSlot &slot) {
+  void *p = nullptr;
+  cudaError_t e = cudaGetSymbolAddress(&p, g_noalloc_scratch);
+  cudaFuncAttributes fa{};
+  if (e == cudaSuccess) e = cudaFuncGetAttributes(&fa, noalloc_add_kernel);
+  for (float a : {1.9f, 2.25f, 2.75f}) {  // 4 x 4, 5 x 5 and 6 x 6 boxes
+    InsertArgs q{};
+    q.g.a = a;
+    q.g.KB = a < 2.0f ? 4 : 6;
+    q.chunk = GATHER_CHUNK;
+    KernelInfo info{};
+    for (q.f16 = 0; q.f16 < 2 && e == cudaSuccess; ++q.f16) {
+      e = launch_gather2(GATHER_SHAPE, q, nullptr, 1, &info);
+      if (e == cudaSuccess) e = cudaFuncGetAttributes(&fa, info.fn);
+    }
+    if (e == cudaSuccess) e = launch_scatter(256, W_OTF, q, nullptr, 1, &info);
+    if (e == cudaSuccess) e = cudaFuncGetAttributes(&fa, info.fn);
+  }
+  if (e != cudaSuccess) return e;
+  device_sm_count();
+  slot.scratch = static_cast<float4 *>(p);
+  slot.ready = true;
+  return cudaSuccess;
+}
+
 int cuda_status(cudaError_t e) {
   fr_note_cuda_error((int)e);
   return FR_ERR_CUDA;
@@ -155,11 +187,8 @@ extern "C" int fr_insert_noalloc(int S, float a, float alpha, const void *images
     std::lock_guard<std::mutex> lk(g_mu);
     DeviceSlot &slot = g_slots[dev];
     if (!slot.ready) {
-      void *p = nullptr;
-      e = cudaGetSymbolAddress(&p, g_noalloc_scratch);
+      e = setup_device(slot);
       if (e != cudaSuccess) return cuda_status(e);
-      slot.scratch = static_cast<float4 *>(p);
-      slot.ready = true;
     }
     scratch = slot.scratch;
   }
@@ -195,12 +224,11 @@ extern "C" int fr_insert_noalloc(int S, float a, float alpha, const void *images
   const int add_threads = 256;
   const int add_blocks = (int)std::min<size_t>((cells + add_threads - 1) / add_threads,
                                                (size_t)sms * 8);
-  constexpr int SHAPE = 1;  // 16 x 8 x 8 bricks
   const bool gather_any = gather_here(g, args.inv_i0a, std::min(n, NOALLOC_SUB));
   if (gather_any) {
     cached_polynomial(alpha, args.poly);
     for (int k = 0; k < POLY_N; ++k) args.poly2[k] = make_float2(args.poly[k], args.poly[k]);
-    args.chunk = 64;
+    args.chunk = GATHER_CHUNK;
     args.any_split = 1;
     args.ortho = 1;
   }
@@ -210,14 +238,14 @@ extern "C" int fr_insert_noalloc(int S, float a, float alpha, const void *images
     args.rot = rotations + (size_t)i0 * 9;
     if (gather_any && gather_here(g, args.inv_i0a, args.n)) {
       int bricks = 0, fold_bricks = 0;
-      const double total = brick_images(g, gather2_shape(SHAPE), 1 - g.xa0, g.H, args.n, &bricks);
+      const double total = brick_images(g, gather2_shape(GATHER_SHAPE), 1 - g.xa0, g.H, args.n, &bricks);
       brick_images(g, fold_shape(g.KB), g.xa0, -g.xa0, args.n, &fold_bricks);
       args.unit_share = (float)unit_share(total, sms, MAIN_UNITS_PER_SM, true);
       // splits of a central brick, which every image crosses
       args.unit_most = std::max(1, std::min({64, args.n / 2, (int)std::ceil(1.02 * args.n / args.unit_share)}));
       args.nunits = bricks * args.unit_most;
       args.nfold = fold_bricks * args.unit_most;
-      e = launch_gather2(SHAPE, args, st, 0, nullptr);
+      e = launch_gather2(GATHER_SHAPE, args, st, 0, nullptr);
     } else {
       e = launch_scatter(256, W_OTF, args, st, 0, nullptr);
     }

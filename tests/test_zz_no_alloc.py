@@ -156,3 +156,60 @@ def test_noalloc_sub_batches_of_both_kernels(tail):
     Vr, Wr, _ = oracle_insert(S, [(img, rot)])
     assert rel_err(V, Vr) <= TOL_F32, worst(V, Vr, S)
     assert rel_err(W, Wr) <= TOL_F32, worst(W, Wr, S)
+
+
+_SETUP_CHILD = """
+import torch
+from paper_1910_08498_gb300 import _lib as L
+from paper_1910_08498_gb300 import inputs
+
+def args(S, n, f16):
+    img, rot = inputs.make_batch(S, n, 47)
+    img = (inputs.to_half(img) if f16 else img).cuda()
+    return S, img, rot.cuda(), torch.zeros((S + 1) ** 3, dtype=torch.complex64, device="cuda"), \
+        torch.zeros((S + 1) ** 3, dtype=torch.float32, device="cuda")
+
+small = args(16, 4, False)
+calls = [(args(64, 400, f16), a) for f16 in (False, True) for a in (1.9, 2.25, 2.9)]
+calls += [(args(32, 30, f16), a) for f16 in (False, True) for a in (1.9, 2.25)]
+L.fr_insert_noalloc(*small)  # the first call on the device: all of the setup
+torch.cuda.synchronize()
+free0, _ = torch.cuda.mem_get_info()
+for c, a in calls:
+    L.fr_insert_noalloc(*c, a=a)
+    torch.cuda.synchronize()
+    print(free0 - torch.cuda.mem_get_info()[0])
+"""
+
+
+@pytest.mark.gpu
+def test_noalloc_first_call_is_the_whole_setup():
+    """In a fresh process, after one small call (which runs the scatter): calls of
+    every kernel variant load no code, so that they change no free memory."""
+    import os
+    import subprocess
+    import sys
+    root = os.path.dirname(os.path.dirname(os.path.abspath(__file__)))
+    r = subprocess.run([sys.executable, "-c", _SETUP_CHILD], cwd=root, capture_output=True, text=True, timeout=300,
+                       env=dict(os.environ, PYTHONPATH=root, CUDA_MODULE_LOADING="LAZY"))
+    assert r.returncode == 0, r.stderr[-2000:]
+    assert r.stdout.split() == ["0"] * 10, r.stdout
+
+
+@pytest.mark.gpu
+def test_noalloc_call_can_be_captured():
+    """The gather's call in a graph, replayed into the same V, W."""
+    S, n = L.FR_NOALLOC_MAX_S, 300
+    img, rot = inputs.make_batch(S, n, 48)
+    V, W = _noalloc(S, img, rot, A32, ALPHA)
+    img, rot = img.cuda(), rot.cuda()
+    Vg = torch.zeros((S + 1) ** 3, dtype=torch.complex64, device="cuda")
+    Wg = torch.zeros((S + 1) ** 3, dtype=torch.float32, device="cuda")
+    g = torch.cuda.CUDAGraph()
+    torch.cuda.synchronize()
+    with torch.cuda.graph(g):
+        L.fr_insert_noalloc(S, img, rot, Vg, Wg, a=A32, alpha=ALPHA)
+    for _ in range(2):
+        g.replay()
+    torch.cuda.synchronize()
+    assert rel_err(Vg.cpu().numpy(), 2 * V) <= TOL_F32 and rel_err(Wg.cpu().numpy(), 2 * W) <= TOL_F32
