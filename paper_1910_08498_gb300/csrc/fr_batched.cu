@@ -17,11 +17,12 @@
 //     counter;
 //   * the per-batch launch arguments and the items are uploaded once into a
 //     device buffer the plan owns;
-//   * after the groups, the float4 scratch of every context that received
-//     split (or shared) units is merged.
+//   * after the groups, the sums of split (or shared) units are merged: a
+//     direct-drain batch's slabs, in the order of its units, and the float4
+//     scratch of every context that per-voxel gather units added to.
 // A context that appears in several batches of one call has all of its units
-// routed through its scratch (atomics), so concurrent units never race on its
-// accumulators.  Batches whose configuration no multi-batch kernel takes
+// routed through slabs of their own (direct-drain) or its scratch (per-voxel,
+// atomics), so concurrent units never race on its accumulators.  Batches whose configuration no multi-batch kernel takes
 // (scatter, tabulated weights, a context whose polynomial weights are not
 // accurate enough) run their own configuration's launches, in order, after
 // the groups.
@@ -66,6 +67,7 @@ struct Plan {
   void *dev = nullptr;               // descriptors, items, counters (owned)
   std::vector<Group> groups;
   std::vector<InsertArgs> merges;    // scratch merges after the groups
+  std::vector<std::pair<InsertArgs, SlabMerge>> slab_merges;
   std::vector<int> sequential;       // batches run with their own launches
   // direct-drain groups: their launches on up to MAX_LANES streams side by side,
   // forked from and joined back into the caller's stream
@@ -140,6 +142,10 @@ int build_plan(Plan &pl, fr_ctx *const *ctxs, const void *const *images, const i
   std::vector<InsertArgs> descs(nb);  // each batch's own arguments
   std::vector<std::vector<int4>> items;  // per group; gather2: fold items, then main items
   std::set<const fr_ctx *> merge_ctx;
+  // direct-drain batches with slabs: the merge's list, its place in the buffer later
+  struct Slabs { int b; SlabMerge m; std::vector<int4> list; };
+  std::vector<Slabs> slabs;
+  std::map<const fr_ctx *, SlabNeed> needs;  // of all of a context's batches together
   struct It { double load; int4 v; };
   auto order = [](std::vector<It> &its) {
     std::stable_sort(its.begin(), its.end(), [](const It &p, const It &q) { return p.load > q.load; });
@@ -192,20 +198,32 @@ int build_plan(Plan &pl, fr_ctx *const *ctxs, const void *const *images, const i
       const bool shared = uses[c] > 1;
       const int shared_bit = shared ? (1 << 30) : 0;
       main_loads(c, n[b], target, tmp, split);
-      for (const UnitLoad &u : tmp)
-        its.push_back(It{u.load, make_int4(u.unit.x | (u.unit.y << 10) | (u.unit.z << 20),
-                                           u.unit.w | shared_bit, b, (int)slot)});
       if (g2) {
+        Slabs sl{b, {}, {}};
+        SlabNeed &need = needs[c];
+        auto put = [&](const GatherShape &shape, int fw, std::vector<It> &to) {
+          assign_slabs(tmp, shape, fw, n[b], shared, need, sl.list);
+          for (const UnitLoad &u : tmp)
+            to.push_back(It{u.load, make_int4(u.unit.x, u.unit.w | shared_bit, b | ((int)slot << 24), u.unit.y)});
+        };
+        sl.m.main = sh;
+        put(sh, 8, its);
+        sl.m.nmain = (int)sl.list.size();
+        sl.m.fold = fold_shape(c->g.KB);
         fold_loads(c, n[b], 0.0, tmp, fsplit);
-        for (const UnitLoad &u : tmp)
-          fits.push_back(It{u.load, make_int4(u.unit.x | (u.unit.y << 10) | (u.unit.z << 20),
-                                              u.unit.w | shared_bit, b, (int)slot)});
+        put(sl.m.fold, sl.m.fold.bx, fits);
+        sl.m.nfold = (int)sl.list.size() - sl.m.nmain;
+        if (!sl.list.empty()) slabs.push_back(std::move(sl));
         gr.main.images[slot] = images[b];
-      }
-      if (split || fsplit || shared) {
-        int rc = ensure_scratch(c);
-        if (rc != FR_OK) return rc;
-        merge_ctx.insert(c);
+      } else {
+        for (const UnitLoad &u : tmp)
+          its.push_back(It{u.load, make_int4(u.unit.x | (u.unit.y << 10) | (u.unit.z << 20),
+                                             u.unit.w | shared_bit, b, (int)slot)});
+        if (split || shared) {
+          int rc = ensure_scratch(c);
+          if (rc != FR_OK) return rc;
+          merge_ctx.insert(c);
+        }
       }
       InsertArgs a = base_args(c);
       a.images = images[b];
@@ -227,13 +245,20 @@ int build_plan(Plan &pl, fr_ctx *const *ctxs, const void *const *images, const i
       ordered.swap(all);
       // the arguments the group's batches share (geometry, weights, list
       // capacity): those of its first batch; the kernel reads the rest per batch
-      gr.main.base = descs[kv.second.front()];
+      gr.main.base = descs[kv.second.front()];  // (the slabs are in the descriptors)
       gr.lane = n_g2++ % MAX_LANES;
     }
     items.push_back(std::move(ordered));
     pl.groups.push_back(gr);
   }
-  // device buffer: descriptors | items of each group | one counter per group
+  for (int b = 0; b < nb; ++b) {
+    auto it = needs.find(ctxs[b]);
+    if (n[b] == 0 || it == needs.end() || it->second.blocks == 0) continue;
+    int rc = ensure_slabs(ctxs[b], it->second, descs[b]);
+    if (rc != FR_OK) return rc;
+  }
+  for (const Slabs &sl : slabs) items.push_back(sl.list);
+  // device buffer: descriptors | items of each group, merge lists | one counter per group
   size_t off = (size_t)nb * sizeof(InsertArgs);
   off = (off + 15) & ~(size_t)15;
   std::vector<size_t> item_off;
@@ -267,6 +292,10 @@ int build_plan(Plan &pl, fr_ctx *const *ctxs, const void *const *images, const i
       L.chunk = gr.chunk;
       L.counter = reinterpret_cast<unsigned *>(d + counter_off) + gi;
     }
+  }
+  for (size_t i = 0; i < slabs.size(); ++i) {
+    slabs[i].m.list = reinterpret_cast<const int4 *>(d + item_off[pl.groups.size() + i]);
+    pl.slab_merges.push_back({descs[slabs[i].b], slabs[i].m});
   }
   if (n_g2 > 0) {
     e = cudaEventCreateWithFlags(&pl.ev_fork, cudaEventDisableTiming);
@@ -316,6 +345,10 @@ int enqueue_plan(const Plan &pl, fr_ctx *const *ctxs, const void *const *images,
   if (e != cudaSuccess) return cuda_err(e);
   for (const InsertArgs &m : pl.merges) {
     e = launch_merge_scratch(m, st);
+    if (e != cudaSuccess) return cuda_err(e);
+  }
+  for (const auto &m : pl.slab_merges) {
+    e = launch_merge_slabs(m.first, m.second, st);
     if (e != cudaSuccess) return cuda_err(e);
   }
   for (int b : pl.sequential) {

@@ -125,6 +125,54 @@ static __device__ __noinline__ bool exact_r2_le_a2(int vx, int vy, int vz, float
   return dh + (de + (rl - al)) <= 0.0f;
 }
 
+// ---------------------------------------------------------------- slabs
+
+// The four voxels (one column, z levels z0 + 4 (lt & 1) ..) that float4 lt of a slab's
+// plane holds, and their place in an accumulator plane.  xmax: last column that counts.
+struct SlabVoxels {
+  bool in;
+  int levels;     // of the four, inside the volume
+  size_t v0, slice;
+  __device__ __forceinline__ SlabVoxels(const Geom &g, int fx0, int fy0, int z0, int FW, int xmax, int lt) {
+    const int col = lt >> 1, vx = fx0 + col % FW, vy = fy0 + col / FW, vz = z0 + (lt & 1) * 4;
+    levels = min(4, g.H - vz + 1);
+    in = vx <= xmax && vy <= g.H && levels > 0;
+    slice = (size_t)g.D * g.NXa;
+    v0 = in ? ((size_t)(vz + g.H) * g.D + (size_t)(vy + g.H)) * g.NXa + (size_t)(vx - g.xa0) : 0;
+  }
+  // sum c's pairs (zeros outside)
+  __device__ __forceinline__ void load(const InsertArgs &a, int c, float (&h)[4], float (&l)[4]) const {
+    const float *p = a.acc + c * a.plane + v0;
+#pragma unroll
+    for (int t = 0; t < 4; ++t, p += slice) {
+      h[t] = in && t < levels ? p[0] : 0.f;
+      l[t] = in && t < levels ? p[3 * a.plane] : 0.f;
+    }
+  }
+  __device__ __forceinline__ void store(const InsertArgs &a, int c, const float (&h)[4], const float (&l)[4]) const {
+    float *p = a.acc + c * a.plane + v0;
+#pragma unroll
+    for (int t = 0; t < 4; ++t, p += slice)
+      if (in && t < levels) {
+        const float s = h[t] + l[t];
+        p[0] = s;
+        p[3 * a.plane] = l[t] - (s - h[t]);
+      }
+  }
+};
+
+// h + l (h the FP32 sum, l the sum of its rounding errors) += x
+__device__ __forceinline__ void add4(float (&h)[4], float (&l)[4], const float4 x) {
+  const float v[4] = {x.x, x.y, x.z, x.w};
+#pragma unroll
+  for (int t = 0; t < 4; ++t) {
+    float s, e;
+    two_sum(h[t], v[t], s, e);
+    h[t] = s;
+    l[t] += e;
+  }
+}
+
 // ---------------------------------------------------------------- blob weights
 
 // Tabulated blob: nodes at r^2 = i a^2 / (lut_n - 1), linear interpolation in

@@ -360,11 +360,40 @@ __device__ __forceinline__ void g2_clear(float *s_acc, int lane) {
     reinterpret_cast<float4 *>(s_acc)[i] = make_float4(0.f, 0.f, 0.f, 0.f);
 }
 
-// Fold a warp's partial sums (s_acc: [3][WV], slot (y FW + x) 8 + z) into HBM:
-// straight into the double-float accumulators (error-free TwoSum) when the warp
-// is the only writer of its voxels, else into the float4 scratch with atomics
-// (merged after the launch).  The loads of four z levels are issued together:
-// one after the other, their latency made a flush take four times as long.
+// Put a warp's partial sums (s_acc: [3][WV], slot (y FW + x) 8 + z) into its slab, the
+// folds-th time: FP32 sums first, an FP32 pair by TwoSum when there are more.  The
+// merge after the launch adds the slabs of a brick's units to the accumulators in the
+// units' order, so the result rounds nothing away and is the same bits in every run.
+// (The units' FP32 sums added with atomics instead: 100 equal images left W 9e-7 off,
+// and most bricks are split.  Atomics into an FP64 scratch cost 11 % at S = 128.)
+template <int WV>
+__device__ __noinline__ void g2_flush_slab(const float *s_acc, float *slab, int folds) {
+  const int lane = threadIdx.x & 31;
+  __syncwarp();
+  const float4 *src = reinterpret_cast<const float4 *>(s_acc);
+  float4 *hi = reinterpret_cast<float4 *>(slab), *lo = hi + 3 * WV / 4;
+#pragma unroll 4
+  for (int i = lane; i < 3 * WV / 4; i += 32) {
+    float4 s = src[i];
+    if (folds > 0) {  // a slab of six planes (see slab_once)
+      float4 h = hi[i], l = folds > 1 ? lo[i] : make_float4(0.f, 0.f, 0.f, 0.f);
+      dd_add(h.x, l.x, s.x);
+      dd_add(h.y, l.y, s.y);
+      dd_add(h.z, l.z, s.z);
+      dd_add(h.w, l.w, s.w);
+      lo[i] = l;
+      s = h;
+    }
+    hi[i] = s;
+  }
+  __syncwarp();
+}
+
+// Fold a warp's partial sums into HBM: straight into the double-float accumulators
+// (error-free TwoSum) when the warp is the only writer of its voxels, else, where there
+// are no slabs, into the float4 scratch with atomics (merged after the launch).  The
+// loads of four z levels are issued together: one after the other, their latency made a
+// flush take four times as long.
 template <int FW, int KB>
 __device__ __noinline__ void g2_flush(const InsertArgs &args, const float *s_acc, int fx0, int fy0,
                                       int z0, bool to_scratch) {
@@ -428,13 +457,13 @@ __host__ __device__ constexpr int g2_warps() {
 // One warp's share of one work unit (see gather_warp for the unit word).
 // args: the batch's arguments; cst: the arguments its launch shares (geometry,
 // weight polynomial, list capacity) and images the batch's images, both read
-// in the inner loops.  FOLD = 0: the bricks tile x >= floor(a) + 1; FOLD = 1:
-// they tile x >= -floor(a) and only the fold columns |x| <= floor(a) are
-// computed, with the fold predicate tested per candidate.
+// in the inner loops; block: the unit's slab, if it is split.  FOLD = 0: the bricks
+// tile x >= floor(a) + 1; FOLD = 1: they tile x >= -floor(a) and only the fold
+// columns |x| <= floor(a) are computed, with the fold predicate tested per candidate.
 template <int BX, int BY, int BZ, int F16, int KB = 4, int FW = 8, int FOLD = 0, int PROF = 0>
 __device__ __forceinline__ void gather2_warp(const InsertArgs &args, const InsertArgs &cst,
                                              const void *images, unsigned char *wsmem,
-                                             const int4 unit, const int warp) {
+                                             const int4 unit, const int block, const int warp) {
   using SH = G2Shape<FW, KB>;
   constexpr int FH = SH::FH, ZC = SH::ZC, WV = SH::WV, PW = SH::PW, PITCH = SH::PITCH,
                 NC = SH::NC, XC = SH::XC;
@@ -484,6 +513,19 @@ __device__ __forceinline__ void gather2_warp(const InsertArgs &args, const Inser
     tmax[c] = vx <= g.H && vy <= g.H && (!FOLD || vx <= -g.xa0) ? min(ZC - 1, g.H - z0) : -1;
   }
 
+  int folds = 0;  // of the sums into the slab
+  auto flush = [&]() {
+    if (to_scratch && args.slab) {
+      if (folds > 0 && args.slab_planes < 6) {  // no room for a pair; slab_once rules it out
+        if (lane == 0) set_err(args.err, DERR_RANGE);
+        return;
+      }
+      const size_t b = (size_t)block + warp * (WV / SLAB_BLOCK);
+      g2_flush_slab<WV>(s_acc, args.slab + b * (size_t)(SLAB_BLOCK * args.slab_planes), folds++);
+    } else {
+      g2_flush<FW, KB>(args, s_acc, fx0, fy0, z0, to_scratch);
+    }
+  };
   g2_clear<WV>(s_acc, lane);
   __syncwarp();
   // PROF: phase counters (fr_options.debug bit 1), cycles of cull, item generation
@@ -887,7 +929,7 @@ __device__ __forceinline__ void gather2_warp(const InsertArgs &args, const Inser
       nl = 0;
       if (since_flush > GATHER_FLUSH - lcap) {
         const long long tf = tick();
-        g2_flush<FW, KB>(args, s_acc, fx0, fy0, z0, to_scratch);
+        flush();
         g2_clear<WV>(s_acc, lane);
         __syncwarp();
         clocked(PH_FLUSH, tf);
@@ -897,7 +939,14 @@ __device__ __forceinline__ void gather2_warp(const InsertArgs &args, const Inser
     if (last) break;
   }
   const long long tf = tick();
-  if (since_flush) g2_flush<FW, KB>(args, s_acc, fx0, fy0, z0, to_scratch);
+  if (since_flush) flush();
+  if (to_scratch && args.slab) {
+    if (slab_once(args.n, nsplit)) {  // one FP32 sum, no state to read: zeros if no image came
+      if (folds == 0) flush();
+    } else if (lane == 0) {
+      args.slab_state[block + warp * (WV / SLAB_BLOCK)] = min(folds, 2);
+    }
+  }
   clocked(PH_FLUSH, tf);
   clocked(PH_WARP_CYCLES, t_start);
 }
@@ -940,6 +989,11 @@ __device__ __forceinline__ bool g2_implicit_unit(const InsertArgs &args, int x0,
   return s < ns;
 }
 
+// A unit's brick, packed, and split word as gather2_warp takes them.
+__device__ __forceinline__ int4 g2_unpack(int brick, int word) {
+  return make_int4(brick & 1023, (brick >> 10) & 1023, (brick >> 20) & 1023, word);
+}
+
 // One warp per CTA: after the nfold units of the fold columns (the few heavy ones
 // first), CTA b takes footprint b % W of work unit args.units[b / W] (W footprints
 // a brick).  Warps of one brick never wait for one another, but a CTA holds its
@@ -957,24 +1011,28 @@ gather2_kernel(const __grid_constant__ InsertArgs args) {
                 WF = g2_warps<FW, G2_FOLD_BY, G2_FOLD_BZ, FW>();
   const Geom &g = args.g;
   const int nf = args.nfold * WF;
+  const bool fold = (int)blockIdx.x < nf;
+  const int b = fold ? blockIdx.x : blockIdx.x - nf, k = fold ? b / WF : b / W;
   int4 unit;
-  if ((int)blockIdx.x < nf) {
-    const int k = blockIdx.x / WF;
-    if (args.units) unit = args.fold[k];
-    else if (!g2_implicit_unit<FW, G2_FOLD_BY, G2_FOLD_BZ>(args, g.xa0, -g.xa0, k, unit)) return;
-    gather2_warp<FW, G2_FOLD_BY, G2_FOLD_BZ, F16, KBM, FW, 1, PROF>(args, args, args.images, smem, unit,
-                                                                   (int)(blockIdx.x % WF));
-  } else {
-    const int b = (int)blockIdx.x - nf, k = b / W;
-    if (args.units) unit = args.units[k];
-    else if (!g2_implicit_unit<BX, BY, BZ>(args, 1 - g.xa0, g.H, k, unit)) return;
-    gather2_warp<BX, BY, BZ, F16, KBM, 8, 0, PROF>(args, args, args.images, smem, unit, b % W);
+  int block = 0;
+  if (args.units) {
+    const int4 q = fold ? args.fold[k] : args.units[k];
+    unit = g2_unpack(q.x, q.w);
+    block = q.y;
+  } else if (fold ? !g2_implicit_unit<FW, G2_FOLD_BY, G2_FOLD_BZ>(args, g.xa0, -g.xa0, k, unit)
+                  : !g2_implicit_unit<BX, BY, BZ>(args, 1 - g.xa0, g.H, k, unit)) {
+    return;
   }
+  if (fold)
+    gather2_warp<FW, G2_FOLD_BY, G2_FOLD_BZ, F16, KBM, FW, 1, PROF>(args, args, args.images, smem, unit,
+                                                                   block, b % WF);
+  else
+    gather2_warp<BX, BY, BZ, F16, KBM, 8, 0, PROF>(args, args, args.images, smem, unit, block, b % W);
 }
 
 // Several batches in one launch: work items p.items[k] = {bx | by << 10 | bz <<
-// 20, split word, batch, slot} of batch p.descs[batch], first those of the fold
-// columns; geometry, weight polynomial and list capacity, common to the launch's
+// 20, split word, batch | slot << 24, slab} of batch p.descs[batch], first those of the
+// fold columns; geometry, weight polynomial and list capacity, common to the launch's
 // batches, are read from p.base (kernel parameters: constant operands in the
 // inner loops), the batch's own arguments (rotations, volume) from its
 // descriptor.
@@ -986,12 +1044,14 @@ gather2_multi_kernel(const __grid_constant__ MultiLaunch p) {
                 WF = g2_warps<FW, G2_FOLD_BY, G2_FOLD_BZ, FW>();
   const int nf = p.nfold * WF, b = (int)blockIdx.x - nf;
   const int4 it = p.items[b < 0 ? (int)blockIdx.x / WF : p.nfold + b / W];
-  const int4 unit = make_int4(it.x & 1023, (it.x >> 10) & 1023, (it.x >> 20) & 1023, it.y);
+  const int4 unit = g2_unpack(it.x, it.y);
+  const InsertArgs &args = p.descs[it.z & 0xffffff];
+  const void *images = p.images[(unsigned)it.z >> 24];
   if (b < 0)
-    gather2_warp<FW, G2_FOLD_BY, G2_FOLD_BZ, F16, KBM, FW, 1>(p.descs[it.z], p.base, p.images[it.w],
-                                                             smem, unit, (int)(blockIdx.x % WF));
+    gather2_warp<FW, G2_FOLD_BY, G2_FOLD_BZ, F16, KBM, FW, 1>(args, p.base, images, smem, unit, it.w,
+                                                             (int)(blockIdx.x % WF));
   else
-    gather2_warp<BX, BY, BZ, F16, KBM>(p.descs[it.z], p.base, p.images[it.w], smem, unit, b % W);
+    gather2_warp<BX, BY, BZ, F16, KBM>(args, p.base, images, smem, unit, it.w, b % W);
 }
 
 }  // namespace fr

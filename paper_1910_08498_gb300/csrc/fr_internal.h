@@ -55,7 +55,9 @@ struct InsertArgs {
   // gather geometry
   int nbx, nby, nbz;    // bricks per axis
   int chunk;            // capacity of a warp's image list
-  const int4 *units;    // work units: (brick x, y, z, split | nsplit << 16)
+  // work units: (brick x, y, z, split | nsplit << 16); direct-drain gather: (brick x |
+  // y << 10 | z << 20, slab, 0, split | nsplit << 16)
+  const int4 *units;
   int nunits;
   // direct-drain gather: units of the fold columns, computed in the same launch.
   // units == null (no list in device memory): each of nunits / nfold is one of
@@ -73,6 +75,14 @@ struct InsertArgs {
   unsigned long long *phase;  // optional per-phase cycle and item counters (PH_*), or null
   // scatter
   float4 *scratch;      // [z][y][x - xa0] (re, im, w, 0)
+  // direct-drain gather: slabs of the split units' partial sums (SLAB_BLOCK), the
+  // state of each footprint whose unit may fold its sums more than once (0: no sums, 1:
+  // FP32 sums, 2: FP32 pairs) at its first block, and the planes of a slab (3, or 6 if
+  // there are such units).  null:
+  // split units add to scratch
+  float *slab;
+  int *slab_state;
+  int slab_planes;
 };
 
 // Per-phase counters of the gather kernel (diagnostics, enabled by
@@ -98,6 +108,34 @@ struct KernelInfo {
 struct GatherShape {
   int bx, by, zc;       // brick: bx x by columns of zc voxels (one column per thread)
 };
+
+// Private partial sums of the direct-drain gather's split units.  A unit's slab number
+// counts blocks of SLAB_BLOCK voxels; its footprints follow one another, each of
+// footprint voxels / SLAB_BLOCK blocks and slab_planes planes (re, im, w, and their
+// low parts), a plane in the order of the warp's partial sums: (y, x, z).
+constexpr int SLAB_BLOCK = 256;
+// Whether a unit of one of ns splits of n images folds its sums at most once (a list
+// of 128 images or fewer is folded with the last)
+__host__ __device__ constexpr bool slab_once(int n, int ns) { return (n + ns - 1) / ns <= 128; }
+// What the merge of an insert's slabs reads: split bricks (brick x | y << 10 | z << 20,
+// first slab, splits, 1 if they have states), first nmain of the main shape, then nfold of
+// the fold columns
+struct SlabMerge {
+  const int4 *list;
+  int nmain, nfold;
+  GatherShape main, fold;
+};
+// warp footprints (fw x 8 x 8 voxels) of a brick
+__host__ __device__ constexpr int gather2_footprints(const GatherShape &sh, int fw) {
+  return sh.bx / fw * (sh.by / 8) * (sh.zc / 8);
+}
+// the slab memory of a launch: blocks of SLAB_BLOCK voxels, planes a block
+struct SlabNeed {
+  int blocks = 0, planes = 3;
+  size_t state_bytes() const { return ((size_t)blocks * sizeof(int) + 255) & ~(size_t)255; }
+  size_t bytes() const { return state_bytes() + (size_t)blocks * SLAB_BLOCK * planes * sizeof(float); }
+};
+cudaError_t launch_merge_slabs(const InsertArgs &a, const SlabMerge &m, cudaStream_t st);
 
 // launchers implemented in the .cu files
 cudaError_t launch_gather(int shape_id, int wmode, const InsertArgs &a, cudaStream_t st,
@@ -173,9 +211,11 @@ cudaError_t launch_gather_persistent(int shape_id, int kb, int f16, const Persis
 constexpr int MULTI_MAX = 64;  // batches per multi-batch launch
 struct MultiLaunch {
   InsertArgs base;           // common arguments: geometry, weights, list capacity
-  const InsertArgs *descs;   // device, one per batch (images, rot, n, acc, scratch, err)
-  const int4 *items;         // device, {bx | by << 10 | bz << 20, split word, batch, slot}:
-  int nfold;                 // nfold items of the fold columns, then nitems of the rest
+  const InsertArgs *descs;   // device, one per batch (images, rot, n, acc, slab, err)
+  // device, {bx | by << 10 | bz << 20, split word, batch | slot << 24, slab}: nfold items
+  // of the fold columns, then nitems of the rest
+  const int4 *items;
+  int nfold;
   int nitems;
   const void *images[MULTI_MAX];  // images of the launch's batches, by slot (read in the inner loop)
 };

@@ -119,6 +119,93 @@ __global__ void merge_scratch_kernel(const InsertArgs args) {
   }
 }
 
+// Add the slabs of the split bricks' units to the double-float accumulators (see
+// SlabMerge).  A part is 32 four-voxel groups of one of a footprint's sums, one a lane; of
+// the G warps that share it warp w takes the units w, w + G, ... in order, and the warps'
+// sums are added in order: the result does not depend on timing.  What counts is the
+// latency of the chains: the fold columns, whose bricks have up to 64 units, come first,
+// eight warps a part; the main bricks have as many warps a part as fill the SMs.  S = 128,
+// 1000 images: 45 us for 130 MB of slabs and 53 MB of accumulators; S = 32, 64 images: 8.6
+// us.  Summed by the brick's last unit inside the gather, S = 128 took 110 us more; with
+// all three sums a thread, or 2, 3 or 6 slabs in flight, alike or slower.
+constexpr int MERGE_WARPS = 8;  // a CTA
+
+// part b of the bricks `list` of shape sh, whose first columns are x0 + brick sh.bx and
+// whose last one that counts is xmax; s_sum: the partial sums of the CTA's warps
+template <int G>
+__device__ __forceinline__ void merge_part(const InsertArgs &args, const GatherShape sh, int FW, int x0, int xmax,
+                                           const int4 *list, int nlist, int b, float (*s_sum)[8][32]) {
+  const Geom &g = args.g;
+  const int lane = threadIdx.x & 31, group = (threadIdx.x >> 5) % G;
+  const int W = gather2_footprints(sh, FW), parts = FW / 2;  // parts of a footprint's sum
+  const bool some = b < nlist * W * parts * 3;
+  const int4 q = some ? list[b / (W * parts * 3)] : make_int4(0, 0, 0, 0);
+  const int c = b / parts % 3, warp = b / (parts * 3) % W, lt = b % parts * 32 + lane;
+  const int fx0 = x0 + (q.x & 1023) * sh.bx + warp % (sh.bx / FW) * FW;
+  const int fy0 = -g.H + ((q.x >> 10) & 1023) * sh.by + warp / (sh.bx / FW) % (sh.by / 8) * 8;
+  const int z0 = -g.H + ((q.x >> 20) & 1023) * sh.zc + warp / (sh.bx / FW * (sh.by / 8)) * 8;
+  SlabVoxels v(g, fx0, fy0, z0, FW, xmax, lt);
+  v.in = v.in && some;
+  float h[4] = {}, l[4] = {};
+  if (group == 0) v.load(args, c, h, l);
+  if (v.in) {
+    const int bpf = FW * 64 / SLAB_BLOCK, step = W * bpf, planes = args.slab_planes;
+    const int first = q.y + warp * bpf;
+    const float4 *slab = reinterpret_cast<const float4 *>(args.slab) + c * (FW * 16) + lt;
+    constexpr int U = 4;  // slabs in flight
+    for (int s0 = group; s0 < q.z; s0 += U * G) {
+      int state[U];
+      float4 x[U];
+#pragma unroll
+      for (int u = 0; u < U; ++u) {
+        const int s = s0 + u * G;
+        state[u] = s >= q.z ? 0 : q.w ? __ldg(args.slab_state + first + s * step) : 1;
+      }
+#pragma unroll
+      for (int u = 0; u < U; ++u)
+        if (state[u]) x[u] = __ldg(slab + (size_t)(first + (s0 + u * G) * step) * (SLAB_BLOCK / 4 * planes));
+#pragma unroll
+      for (int u = 0; u < U; ++u) {
+        if (state[u]) add4(h, l, x[u]);
+        if (state[u] == 2 && planes == 6) {
+          const float4 y = __ldg(slab + (size_t)(first + (s0 + u * G) * step) * (SLAB_BLOCK / 4 * planes) + FW * 48);
+          l[0] += y.x;
+          l[1] += y.y;
+          l[2] += y.z;
+          l[3] += y.w;
+        }
+      }
+    }
+  }
+  if (G > 1) {
+    s_sum += (threadIdx.x >> 5) / G * (G - 1);
+    if (group > 0)
+#pragma unroll
+      for (int k = 0; k < 4; ++k) s_sum[group - 1][k][lane] = h[k], s_sum[group - 1][4 + k][lane] = l[k];
+    __syncthreads();
+    if (group > 0) return;
+#pragma unroll 1
+    for (int o = 0; o < G - 1; ++o) {
+      add4(h, l, make_float4(s_sum[o][0][lane], s_sum[o][1][lane], s_sum[o][2][lane], s_sum[o][3][lane]));
+#pragma unroll
+      for (int k = 0; k < 4; ++k) l[k] += s_sum[o][4 + k][lane];
+    }
+  }
+  v.store(args, c, h, l);
+}
+
+template <int G>
+__global__ void __launch_bounds__(32 * MERGE_WARPS)
+merge_slabs_kernel(const __grid_constant__ InsertArgs args, const __grid_constant__ SlabMerge m, int fold_ctas) {
+  __shared__ float s_sum[MERGE_WARPS - 1][8][32];
+  const Geom &g = args.g;
+  if ((int)blockIdx.x < fold_ctas)
+    merge_part<MERGE_WARPS>(args, m.fold, m.fold.bx, g.xa0, -g.xa0, m.list + m.nmain, m.nfold, blockIdx.x, s_sum);
+  else
+    merge_part<G>(args, m.main, 8, 1 - g.xa0, g.H, m.list, m.nmain,
+                  ((int)blockIdx.x - fold_ctas) * (MERGE_WARPS / G) + (int)(threadIdx.x >> 5) / G, s_sum);
+}
+
 // ---------------------------------------------------------------- finalize (A9)
 __global__ void finalize_kernel(const Geom g, const float *__restrict__ acc, size_t plane,
                                 float2 *__restrict__ V, float *__restrict__ W) {
@@ -282,6 +369,24 @@ cudaError_t launch_merge_scratch(const InsertArgs &a, cudaStream_t st) {
   int threads = 256;
   merge_scratch_kernel<<<grid_for(a.plane, threads, sm_count() * 8), threads, 0, st>>>(a);
   return cudaGetLastError();
+}
+
+template <int G>
+static cudaError_t launch_merge_slabs_t(const InsertArgs &a, const SlabMerge &m, int fold, int main, cudaStream_t st) {
+  constexpr int PER = MERGE_WARPS / G;
+  merge_slabs_kernel<G><<<fold + (main + PER - 1) / PER, 32 * MERGE_WARPS, 0, st>>>(a, m, fold);
+  return cudaGetLastError();
+}
+
+cudaError_t launch_merge_slabs(const InsertArgs &a, const SlabMerge &m, cudaStream_t st) {
+  const int main = m.nmain * gather2_footprints(m.main, 8) * 12,
+            fold = m.nfold * gather2_footprints(m.fold, m.fold.bx) * (m.fold.bx / 2 * 3);
+  if (main + fold == 0) return cudaSuccess;
+  const int warps = main > 0 ? sm_count() * 48 / main : 1;
+  if (warps >= 8) return launch_merge_slabs_t<8>(a, m, fold, main, st);
+  if (warps >= 4) return launch_merge_slabs_t<4>(a, m, fold, main, st);
+  if (warps >= 2) return launch_merge_slabs_t<2>(a, m, fold, main, st);
+  return launch_merge_slabs_t<1>(a, m, fold, main, st);
 }
 
 cudaError_t launch_finalize(const Geom &g, const float *acc, size_t plane, float2 *V, float *W,

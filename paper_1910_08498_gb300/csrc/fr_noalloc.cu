@@ -126,6 +126,7 @@ double brick_images(const Geom &g, const GatherShape &sh, int x0, int x1, int n,
 
 constexpr int GATHER_SHAPE = 1;  // 16 x 8 x 8 bricks
 constexpr int GATHER_CHUNK = 64;
+constexpr int UNITS_PER_SM = 96;  // finer than fr_insert's, which have slabs to merge
 
 // Everything a later call would otherwise set up on its way: the code of each kernel
 // that some call can launch (cudaFuncGetAttributes loads it), the gather's shared
@@ -240,7 +241,7 @@ extern "C" int fr_insert_noalloc(int S, float a, float alpha, const void *images
       int bricks = 0, fold_bricks = 0;
       const double total = brick_images(g, gather2_shape(GATHER_SHAPE), 1 - g.xa0, g.H, args.n, &bricks);
       brick_images(g, fold_shape(g.KB), g.xa0, -g.xa0, args.n, &fold_bricks);
-      args.unit_share = (float)unit_share(total, sms, MAIN_UNITS_PER_SM, true);
+      args.unit_share = (float)unit_share(total, sms, UNITS_PER_SM, true);
       // splits of a central brick, which every image crosses
       args.unit_most = std::max(1, std::min({64, args.n / 2, (int)std::ceil(1.02 * args.n / args.unit_share)}));
       args.nunits = bricks * args.unit_most;

@@ -136,6 +136,44 @@ int ensure_scratch(fr_ctx *c) {
   return FR_OK;
 }
 
+int ensure_slabs(fr_ctx *c, const SlabNeed &need, InsertArgs &a) {
+  const size_t bytes = need.bytes();
+  if (bytes > c->slabs_bytes) {
+    if (alloc_fault(c)) return FR_ERR_OOM;
+    // at least half as much again, so that the buffers kept add up to three times the last
+    const size_t want = c->slabs_bytes ? std::max(bytes, c->slabs_bytes + c->slabs_bytes / 2) : bytes;
+    void *p = nullptr;
+    FR_CUDA(cudaMalloc(&p, want));
+    if (c->slabs) c->slabs_old.push_back(c->slabs);
+    c->slabs = p;
+    c->slabs_bytes = want;
+  }
+  a.slab_state = static_cast<int *>(c->slabs);
+  a.slab = reinterpret_cast<float *>(static_cast<unsigned char *>(c->slabs) + need.state_bytes());
+  a.slab_planes = need.planes;
+  return FR_OK;
+}
+
+void assign_slabs(std::vector<UnitLoad> &units, const GatherShape &sh, int fw, int n, bool all,
+                  SlabNeed &need, std::vector<int4> &merge) {
+  const int blocks = gather2_footprints(sh, fw) * (fw * 64 / SLAB_BLOCK);  // a unit's
+  for (UnitLoad &u : units) {  // a brick's units follow one another
+    const int brick = u.unit.x | (u.unit.y << 10) | (u.unit.z << 20);
+    const int s = u.unit.w & 0xffff, ns = (u.unit.w >> 16) & 0x3fff;
+    int first = 0;
+    if (ns > 1 || all) {
+      if (s == 0) {
+        const bool once = slab_once(n, ns);
+        merge.push_back(make_int4(brick, need.blocks, ns, once ? 0 : 1));
+        need.blocks += ns * blocks;
+        if (!once) need.planes = 6;
+      }
+      first = merge.back().y + s * blocks;
+    }
+    u.unit = make_int4(brick, first, 0, u.unit.w);
+  }
+}
+
 // Work units of a gather launch.  A brick at distance d from the centre is
 // crossed, within a + (brick radius) r, by a fraction min(1, (a + r) / d) of
 // uniformly oriented planes through the origin, so its expected image count is
@@ -216,9 +254,15 @@ Config effective_config(const fr_ctx *c, int id) {
   return cfg;
 }
 
+// The slabs of a unit list into a, and the list of its merge.
+static int unit_slabs(fr_ctx *c, const fr_ctx::Units &u, InsertArgs &a, SlabMerge *merge) {
+  if (merge) *merge = u.merge;
+  return u.need.blocks > 0 ? ensure_slabs(c, u.need, a) : FR_OK;
+}
+
 // Work units of a gather launch of this batch alone, heaviest first (so the
 // largest ones start first), cached on the device per (shape, n).
-static int gather_units(fr_ctx *c, const Config &cfg, int n, InsertArgs &a) {
+static int gather_units(fr_ctx *c, const Config &cfg, int n, InsertArgs &a, SlabMerge *merge = nullptr) {
   const int algo = cfg.algo == ALGO_GATHER2 ? ALGO_GATHER2 : ALGO_GATHER;
   for (int k = 0; k < 8; ++k) {
     fr_ctx::Units &u = c->units[k];
@@ -228,20 +272,28 @@ static int gather_units(fr_ctx *c, const Config &cfg, int n, InsertArgs &a) {
       a.any_split = u.any_split;
       a.fold = u.fold;
       a.nfold = u.fold_count;
-      return FR_OK;
+      return unit_slabs(c, u, a, merge);
     }
   }
   if (alloc_fault(c)) return FR_ERR_OOM;
   std::vector<UnitLoad> us, fs;
+  std::vector<int4> merges;
   int any_split = 0, fsplit = 0;
+  SlabNeed need;
+  SlabMerge mg{};
   if (algo == ALGO_GATHER2) {
     // the direct-drain gather's main bricks tile x in [floor(a) + 1, H]; the
     // fold columns x in [-floor(a), floor(a)] have units in bricks one
     // footprint wide, split finely (they are few and heavy)
     brick_unit_loads(c, gather2_shape(cfg.shape), 1 - c->g.xa0, c->g.H, n, 0.0, MAIN_UNITS_PER_SM,
                      true, us, any_split);
-    brick_unit_loads(c, fold_shape(c->g.KB), c->g.xa0, -c->g.xa0, n, 0.0, FOLD_UNITS_PER_SM, true,
-                     fs, fsplit);
+    mg.main = gather2_shape(cfg.shape);
+    mg.fold = fold_shape(c->g.KB);
+    brick_unit_loads(c, mg.fold, c->g.xa0, -c->g.xa0, n, 0.0, FOLD_UNITS_PER_SM, true, fs, fsplit);
+    assign_slabs(us, mg.main, 8, n, false, need, merges);
+    mg.nmain = (int)merges.size();
+    assign_slabs(fs, mg.fold, mg.fold.bx, n, false, need, merges);
+    mg.nfold = (int)merges.size() - mg.nmain;
   } else {
     gather_unit_loads(c, cfg.shape, n, 0.0, us, any_split);
   }
@@ -249,9 +301,10 @@ static int gather_units(fr_ctx *c, const Config &cfg, int n, InsertArgs &a) {
   std::stable_sort(us.begin(), us.end(), heavy_first);
   std::stable_sort(fs.begin(), fs.end(), heavy_first);
   std::vector<int4> host;
-  host.reserve(us.size() + fs.size());
+  host.reserve(us.size() + fs.size() + merges.size());
   for (const UnitLoad &x : us) host.push_back(x.unit);
   for (const UnitLoad &x : fs) host.push_back(x.unit);
+  host.insert(host.end(), merges.begin(), merges.end());
   // replace the oldest cached list
   fr_ctx::Units &slot = c->units[7];
   cudaFree(slot.dev);
@@ -267,12 +320,15 @@ static int gather_units(fr_ctx *c, const Config &cfg, int n, InsertArgs &a) {
   u.any_split = any_split | fsplit;
   u.fold = u.dev + us.size();
   u.fold_count = (int)fs.size();
+  mg.list = u.dev + us.size() + fs.size();
+  u.merge = mg;
+  u.need = need;
   a.units = u.dev;
   a.nunits = u.count;
   a.any_split = u.any_split;
   a.fold = u.fold;
   a.nfold = u.fold_count;
-  return FR_OK;
+  return unit_slabs(c, u, a, merge);
 }
 
 // Fill the launch geometry of configuration `cfg` into `a`.
@@ -292,7 +348,7 @@ int prepare_config(fr_ctx *c, int id, int n) {
   if (cfg.algo == ALGO_GATHER || cfg.algo == ALGO_GATHER2) {
     int rc = gather_units(c, cfg, n, a);
     if (rc) return rc;
-    return a.any_split ? ensure_scratch(c) : FR_OK;
+    return a.any_split && cfg.algo == ALGO_GATHER ? ensure_scratch(c) : FR_OK;
   }
   return ensure_scratch(c);
 }
@@ -308,19 +364,20 @@ int run_config(fr_ctx *c, int id, const void *images, int f16, const float *rot,
   a.n = n;
   if (cfg.algo == ALGO_GATHER || cfg.algo == ALGO_GATHER2) {
     gather_geometry(c, cfg, a);
-    int rc = gather_units(c, cfg, n, a);
+    const bool direct = cfg.algo == ALGO_GATHER2;
+    SlabMerge merge{};
+    int rc = gather_units(c, cfg, n, a, &merge);
     if (rc) return rc;
-    if (a.any_split) {
+    if (a.any_split && !direct) {
       rc = ensure_scratch(c);
       if (rc) return rc;
       a.scratch = c->scratch;
     }
-    const cudaError_t e = cfg.algo == ALGO_GATHER2
-                              ? launch_gather2(cfg.shape, a, st, 0, nullptr)
-                              : launch_gather(cfg.shape, cfg.wmode, a, st, 0, nullptr);
+    const cudaError_t e = direct ? launch_gather2(cfg.shape, a, st, 0, nullptr)
+                                 : launch_gather(cfg.shape, cfg.wmode, a, st, 0, nullptr);
     if (e != cudaSuccess) return cuda_fail(e);
     if (a.any_split) {
-      const cudaError_t em = launch_merge_scratch(a, st);
+      const cudaError_t em = direct ? launch_merge_slabs(a, merge, st) : launch_merge_scratch(a, st);
       if (em != cudaSuccess) return cuda_fail(em);
     }
     return FR_OK;
@@ -561,6 +618,8 @@ int fr_destroy(fr_ctx *c) {
   cudaFree(c->acc);
   cudaFree(c->lut);
   cudaFree(c->scratch);
+  cudaFree(c->slabs);
+  for (void *p : c->slabs_old) cudaFree(p);
   cudaFree(c->d_err);
   cudaFree(c->d_count);
   cudaFree(c->d_phase);

@@ -106,3 +106,33 @@ def test_pixels_outside_the_blob_do_not_reach_a_voxel():
     assert not np.isfinite(V[inside]).any()
     assert np.isfinite(V[outside]).all()
     assert np.isfinite(W).all()
+
+
+@pytest.mark.parametrize("f16", [False, True])
+@pytest.mark.parametrize("a", [1.9, 2.5, 2.999])
+def test_split_units_sums_are_not_rounded(a, f16):
+    """100 copies of one image: around the centre a unit takes two.  Its FP32 sum of at
+    most four terms (an image meets a voxel in up to two records) takes three roundings,
+    the single image's sum one, the export one: 5 x 2^-24 of a voxel's W; 50 units'
+    sums added in FP32 round 49 times more."""
+    S, n, a = 32, 100, float(np.float32(a))
+    img, rot = inputs.make_batch(S, 1, 9)
+    _, W1, _ = gpu_insert(S, [(img, rot)], a=a, tuning=False, f16=f16)
+    _, W, _ = gpu_insert(S, [(img.repeat(n, 1, 1), rot.repeat(n, 1, 1))], a=a, tuning=False, f16=f16)
+    g = np.abs(np.arange(S + 1) - S // 2) <= 2
+    near = (g[:, None, None] & g[:, None] & g).ravel()
+    assert W1[near].max() > 0
+    err = np.abs(W[near] - n * W1[near])
+    assert np.all(err <= 5 * 2.0 ** -24 * n * W1[near]), np.max(err / np.maximum(n * W1[near], 1e-30))
+
+
+@pytest.mark.parametrize("S,n,a", [(64, 640, 1.9), (48, 300, 2.25), (40, 200, 2.9), (16, 20000, 1.9)])
+def test_split_units_give_the_same_bits_every_time(S, n, a):
+    """The units of a brick are summed in their order (20,000 images: units that fold
+    their sums into their slab more than once)."""
+    img, rot = _batch(S, n, 13)
+    runs = [gpu_insert(S, [(img, rot)], a=float(np.float32(a)), tuning=False) for _ in range(3)]
+    for V, W, _ in runs[1:]:
+        assert np.array_equal(V, runs[0][0]) and np.array_equal(W, runs[0][1])
+    Vr, Wr, _ = oracle_insert(S, [(img, rot)], a=float(np.float32(a)))
+    assert rel_err(runs[0][0], Vr) <= TOL_F32 and rel_err(runs[0][1], Wr) <= TOL_F32
