@@ -104,16 +104,19 @@ __device__ __forceinline__ float dot3_less_one(float x, float y, float z) {
 // Candidates of a fold column's box within rounding of the blob edge (FP32 r^2
 // within 1e-5 a^2 of a^2), decided as the real numbers do: with a lattice
 // distance a (a = 2, or a signed permutation for the rotation) the DC pixel
-// and others sit there for every image.  k0: the box's first stored pixel.
+// and others sit there for every image.  k0: the box's first stored pixel.  x by g2_box's
+// operations: a candidate that rounding put into the band there and out of it here was
+// lost (a = 2.00001, signed permutations: two voxels of each image, b(a) each).
 template <int PITCH, int KB>
 __device__ __noinline__ void g2_ties(const float2 *cp, const float2 *p, float dx, float dy,
-                                     float uz2, float cs, const unsigned *rows, int shift,
+                                     float uz2, float cs, float sq, const unsigned *rows, int shift,
                                      const float4 e1, const float4 e2, int3 v, int2 k0, float a,
                                      float &ar, float &ai, float &aw) {
+  const float U = fmaf(cs, uz2, -1.0f);
   for (int r = 0; r < KB; ++r)
     for (int j = 0; j < KB; ++j) {
-      const float ex = dx - (float)j, ey = dy - (float)r;
-      const float x = fmaf(cs, fmaf(ex, ex, fmaf(ey, ey, uz2)), -1.0f);
+      const float d = sq * (dx - (float)j), ey = dy - (float)r;
+      const float x = fmaf(d, d, fmaf(cs * ey, ey, U));
       if (fabsf(x - 1.0f) > 2e-5f || !((rows[r] >> (shift + j)) & 1u) ||
           !exact_r2_le_a2(v.x, v.y, v.z, e1.x, e1.y, e1.z, e2.x, e2.y, e2.z, k0.x + j, k0.y + r, a))
         continue;
@@ -856,7 +859,7 @@ __device__ __forceinline__ void gather2_warp(const InsertArgs &args, const Inser
         ties = g2_box<PITCH, KB, FOLD>(cst.poly2, it.p, it.dx, it.dy, it.uz2, cs, sq, ar, ai, aw,
                                        it.rows, it.shift);
       if (FOLD && KB > 4 && ties)
-        g2_ties<PITCH, KB>(cst.poly2, it.p, it.dx, it.dy, it.uz2, cs, it.rows, it.shift, q1, q2,
+        g2_ties<PITCH, KB>(cst.poly2, it.p, it.dx, it.dy, it.uz2, cs, sq, it.rows, it.shift, q1, q2,
                            make_int3(fx0 + (it.slot / ZC) % FW, fy0 + it.slot / (ZC * FW), z0 + it.slot % ZC),
                            make_int2((q3.y & 0xffff) + it.shift, (q3.y >> 16) + it.row), g.a, ar, ai, aw);
       if (h < total) {

@@ -136,3 +136,17 @@ def test_split_units_give_the_same_bits_every_time(S, n, a):
         assert np.array_equal(V, runs[0][0]) and np.array_equal(W, runs[0][1])
     Vr, Wr, _ = oracle_insert(S, [(img, rot)], a=float(np.float32(a)))
     assert rel_err(runs[0][0], Vr) <= TOL_F32 and rel_err(runs[0][1], Wr) <= TOL_F32
+
+
+@pytest.mark.parametrize("a", [2.0, 2.00001, 5 ** 0.5, 2.236079, 8 ** 0.5, 2.8284414])
+def test_fold_columns_decide_the_edge_band_once(a):
+    """Signed permutations put whole lattices of candidates at the blob's edge, or 1e-5
+    a^2 inside it, where the box leaves them to the exact decision; alpha = 0 gives
+    each the weight 1."""
+    S, a = 24, float(np.float32(a))
+    rot = inputs.proper_signed_permutations()
+    img, _ = inputs.make_batch(S, rot.shape[0], 21)
+    V, W, _ = gpu_insert(S, [(img, rot)], a=a, alpha=0.0, tuning=False)
+    Vr, Wr, _ = oracle_insert(S, [(img, rot)], a=a, alpha=0.0)
+    assert rel_err(V, Vr) <= TOL_F32, worst(V, Vr, S)
+    assert rel_err(W, Wr) <= TOL_F32, worst(W, Wr, S)
