@@ -279,6 +279,8 @@ int build_plan(Plan &pl, fr_ctx *const *ctxs, const void *const *images, const i
                    cudaMemcpyHostToDevice);
     if (e != cudaSuccess) return cuda_err(e);
   }
+  e = setup_done();
+  if (e != cudaSuccess) return cuda_err(e);
   for (size_t gi = 0; gi < pl.groups.size(); ++gi) {
     Group &gr = pl.groups[gi];
     if (gr.algo == ALGO_GATHER2) {

@@ -173,6 +173,10 @@ cudaError_t fft_volume(const Geom &g, const float *acc, size_t plane, float w_cl
 bool fft_images_here(int S);
 cudaError_t fft_images(int S, const float *real, float2 *spec, int m, int center, void *out,
                        int f16, cudaStream_t st);
+// Waits for set-up work on the legacy stream (a memset, a copy from pageable memory, which
+// may return before it has reached the device): launches on non-blocking streams are not
+// ordered behind it.
+inline cudaError_t setup_done() { return cudaStreamSynchronize(cudaStreamLegacy); }
 // record a CUDA error for fr_last_cuda_error
 void fr_note_cuda_error(int e);
 cudaError_t launch_finalize(const Geom &g, const float *acc, size_t plane, float2 *V, float *W,

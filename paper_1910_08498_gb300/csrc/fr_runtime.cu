@@ -133,6 +133,7 @@ int ensure_scratch(fr_ctx *c) {
   if (alloc_fault(c)) return FR_ERR_OOM;
   FR_CUDA(cudaMalloc(&c->scratch, c->plane * sizeof(float4)));
   FR_CUDA(cudaMemset(c->scratch, 0, c->plane * sizeof(float4)));
+  FR_CUDA(setup_done());
   return FR_OK;
 }
 
@@ -313,6 +314,7 @@ static int gather_units(fr_ctx *c, const Config &cfg, int n, InsertArgs &a, Slab
   fr_ctx::Units &u = c->units[0];
   FR_CUDA(cudaMalloc(&u.dev, host.size() * sizeof(int4)));
   FR_CUDA(cudaMemcpy(u.dev, host.data(), host.size() * sizeof(int4), cudaMemcpyHostToDevice));
+  FR_CUDA(setup_done());
   u.shape = cfg.shape;
   u.algo = algo;
   u.n = n;
@@ -581,6 +583,7 @@ int fr_create(int S, const fr_blob *blob, fr_ctx **out) {
   e = cudaMalloc(&c->lut, N * sizeof(float2));
   if (e != cudaSuccess) return fail(cuda_fail(e));
   e = cudaMemcpy(c->lut, tab.data(), N * sizeof(float2), cudaMemcpyHostToDevice);
+  if (e == cudaSuccess) e = setup_done();  // the accumulators' clearing, too
   if (e != cudaSuccess) return fail(cuda_fail(e));
   c->inv_i0a = (float)(1.0 / i0a);
   c->inv_pa = alpha > 3.75 ? (float)(1.0 / as_982_host(3.75 / alpha)) : 1.0f;
@@ -679,6 +682,7 @@ static int state_copy(fr_ctx *c, void *dst, const void *src) {
   if (c->last_stream) FR_CUDA(cudaStreamSynchronize(c->last_stream));
   FR_CUDA(cudaDeviceSynchronize());
   FR_CUDA(cudaMemcpy(dst, src, fr_state_bytes(c), cudaMemcpyDefault));
+  FR_CUDA(setup_done());
   return FR_OK;
 }
 
@@ -826,6 +830,7 @@ int fr_last_device_error(fr_ctx *c) {
   int h = 0;
   FR_CUDA(cudaMemcpy(&h, c->d_err, sizeof(int), cudaMemcpyDeviceToHost));
   FR_CUDA(cudaMemset(c->d_err, 0, sizeof(int)));
+  FR_CUDA(setup_done());
   if (!h) return FR_OK;
   return (h & DERR_TIMEOUT) ? FR_ERR_TIMEOUT : FR_ERR_DEVICE_ASSERT;
 }
@@ -838,6 +843,7 @@ int fr_debug_phase_counters(fr_ctx *c, unsigned long long *out, int cap) {
   unsigned long long h[PH_COUNT];
   FR_CUDA(cudaMemcpy(h, c->d_phase, sizeof h, cudaMemcpyDeviceToHost));
   FR_CUDA(cudaMemset(c->d_phase, 0, sizeof h));
+  FR_CUDA(setup_done());
   for (int k = 0; k < cap && k < PH_COUNT; ++k) out[k] = h[k];
   return FR_OK;
 }

@@ -166,3 +166,28 @@ def test_bulk_gemm_wait_timeout_is_reported_and_recovers():
     As, Bs = A[idx].cpu().numpy(), B[idx].cpu().numpy()
     err = np.abs(C[idx].cpu().numpy().astype(np.float64) - gemm.bgemm(As, Bs))
     assert np.all(err <= gemm.fp32_error_bound(As, Bs) + 1e-30)
+
+
+@pytest.mark.parametrize("config", [-1, 13, 37])
+def test_first_insert_on_a_non_blocking_stream(config):
+    """A new context's first insert right behind its creation, on a stream that does not
+    wait for the default one: the unit list has arrived and the accumulators, scratch
+    and slabs are clear before it runs.  Default, per-voxel gather, scatter."""
+    S, n = 160, 20
+    img, rot = inputs.make_batch(S, n, 77)
+    Vr, Wr, _ = oracle_insert(S, [(img, rot)])
+    img_d, rot_d = img.cuda(), rot.cuda()
+    torch.cuda.synchronize()
+    stream = torch.cuda.Stream()
+    for _ in range(3):
+        ctx = L.fr_create(S)
+        try:
+            L.fr_set_options(ctx, tuning=0, forced_config=config)
+            L.fr_insert(ctx, img_d, rot_d, stream=stream)
+            V = torch.empty((S + 1) ** 3, dtype=torch.complex64, device="cuda")
+            W = torch.empty((S + 1) ** 3, dtype=torch.float32, device="cuda")
+            L.fr_finalize(ctx, V, W, stream=stream)
+            stream.synchronize()
+        finally:
+            L.fr_destroy(ctx)
+        assert rel_err(V.cpu().numpy(), Vr) <= TOL_F32 and rel_err(W.cpu().numpy(), Wr) <= TOL_F32
