@@ -132,7 +132,7 @@ int build_plan(Plan &pl, fr_ctx *const *ctxs, const void *const *images, const i
       groups[GKey(ALGO_GATHER, k.shape, c->g.KB, f16, k.chunk, 0, 0.f, 0.f)].push_back(b);
     } else {
       // its own launches: units and scratch ready before any capture
-      int rc = prepare_config(c, cfg[b], n[b]);
+      int rc = prepare_config(c, cfg[b], f16, n[b]);
       if (rc != FR_OK) return rc;
       pl.sequential.push_back(b);
     }

@@ -2,6 +2,7 @@
 // dispatch of the direct-drain gather (fr_gather2.cuh); the kernels are
 // instantiated per brick shape in fr_gather2_s<k>.cu.
 #include <mutex>
+#include <utility>
 #include <vector>
 
 #include "fr_gather2.cuh"
@@ -35,6 +36,21 @@ cudaError_t allow_dynamic_smem(const void *fn, size_t smem, int carveout) {
     if (d.dev == dev && d.fn == fn) { d.smem = smem; return cudaSuccess; }
   done.push_back(Entry{dev, fn, smem});
   return cudaSuccess;
+}
+
+cudaError_t load_kernel(const void *fn) {
+  static std::mutex mu;
+  static std::vector<std::pair<int, const void *>> done;
+  int dev = 0;
+  cudaError_t e = cudaGetDevice(&dev);
+  if (e != cudaSuccess) return e;
+  std::lock_guard<std::mutex> lk(mu);
+  for (const auto &d : done)
+    if (d.first == dev && d.second == fn) return cudaSuccess;
+  cudaFuncAttributes fa{};
+  e = cudaFuncGetAttributes(&fa, fn);
+  if (e == cudaSuccess) done.push_back({dev, fn});
+  return e;
 }
 
 int device_sm_count() {

@@ -150,6 +150,10 @@ size_t gather2_smem_bytes(const GatherShape &sh, int chunk);
 // (and, if carveout >= 0, set its preferred shared-memory carveout in percent);
 // remembered per device and kernel; thread-safe
 cudaError_t allow_dynamic_smem(const void *fn, size_t smem, int carveout = -1);
+// load a kernel's code on the current device if that has not happened yet (remembered
+// per device and kernel; thread-safe): lazily, its first launch would
+cudaError_t load_kernel(const void *fn);
+cudaError_t load_merge_kernels();
 // SM count of the current device (cached per device; thread-safe)
 int device_sm_count();
 // resident CTAs per SM of kernel fn with `threads` threads and `smem` bytes

@@ -389,6 +389,15 @@ cudaError_t launch_merge_slabs(const InsertArgs &a, const SlabMerge &m, cudaStre
   return launch_merge_slabs_t<1>(a, m, fold, main, st);
 }
 
+cudaError_t load_merge_kernels() {
+  cudaError_t e = cudaSuccess;
+  for (const void *fn : {(const void *)merge_scratch_kernel, (const void *)merge_slabs_kernel<1>,
+                         (const void *)merge_slabs_kernel<2>, (const void *)merge_slabs_kernel<4>,
+                         (const void *)merge_slabs_kernel<8>})
+    if (e == cudaSuccess) e = load_kernel(fn);
+  return e;
+}
+
 cudaError_t launch_finalize(const Geom &g, const float *acc, size_t plane, float2 *V, float *W,
                             cudaStream_t st) {
   size_t total = (size_t)g.D * g.D * g.D;

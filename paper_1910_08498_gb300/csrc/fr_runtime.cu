@@ -342,11 +342,22 @@ static void gather_geometry(const fr_ctx *c, const Config &cfg, InsertArgs &a) {
   a.nbz = (c->g.D + sh.zc - 1) / sh.zc;
 }
 
-// Allocate and upload whatever a launch of configuration id on n images
-// needs (work units, scratch), so that the launch itself only enqueues work.
-int prepare_config(fr_ctx *c, int id, int n) {
+// Load the code of, and allocate and upload whatever else, a launch of configuration id
+// on n images needs (work units, scratch), so that the launch itself only enqueues
+// work.  (A kernel's code, loaded by its first launch, cost a tuning step 0.9 ms, which
+// made the step's configuration look several times slower than it is.)
+int prepare_config(fr_ctx *c, int id, int f16, int n) {
   const Config cfg = effective_config(c, id);
   InsertArgs a = base_args(c);
+  a.f16 = f16;
+  a.chunk = cfg.chunk;
+  KernelInfo info{};
+  cudaError_t e = cfg.algo == ALGO_GATHER2  ? launch_gather2(cfg.shape, a, nullptr, 1, &info)
+                  : cfg.algo == ALGO_GATHER ? launch_gather(cfg.shape, cfg.wmode, a, nullptr, 1, &info)
+                                            : launch_scatter(cfg.threads, cfg.wmode, a, nullptr, 1, &info);
+  if (e == cudaSuccess) e = load_kernel(info.fn);
+  if (e == cudaSuccess) e = load_merge_kernels();
+  if (e != cudaSuccess) return cuda_fail(e);
   if (cfg.algo == ALGO_GATHER || cfg.algo == ALGO_GATHER2) {
     int rc = gather_units(c, cfg, n, a);
     if (rc) return rc;
@@ -469,7 +480,7 @@ int fr::do_insert_ctx(fr_ctx *c, const void *images, fr_dtype dtype, const float
     int rc = (c->opt.fault_config > 0 && s.config == c->opt.fault_config - 1) ? FR_ERR_LAUNCH : FR_OK;
     // host work of the step (work-unit list, scratch) before the timed region,
     // so that a configuration's first use is timed like its later ones
-    if (rc == FR_OK) rc = prepare_config(c, s.config, s.images);
+    if (rc == FR_OK) rc = prepare_config(c, s.config, f16, s.images);
     Timing tm = c->tuner.begin(st);
     if (rc == FR_OK) rc = run_config(c, s.config, img, f16, r, s.images, st);
     if (rc != FR_OK) {

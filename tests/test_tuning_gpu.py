@@ -203,3 +203,41 @@ def test_automatic_tuning_steps():
         L.fr_destroy(ctx)
     assert rep["evaluated"] == 7
     assert rel_err(V, Vr) <= TOL_F32 and rel_err(W, Wr) <= TOL_F32
+
+
+_FIRST_STEPS_CHILD = """
+import json
+import torch
+from paper_1910_08498_gb300 import _lib as L
+from paper_1910_08498_gb300 import inputs
+from paper_1910_08498_gb300.sweep import time_config
+
+img, rot = [t.cuda() for t in inputs.make_batch(64, 200, 170)]
+ctx = L.fr_create(64)
+L.fr_set_options(ctx, tuning=1, search=L.FR_SEARCH_EXHAUSTIVE, steps_per_insert=1)
+for _ in range(100):
+    L.fr_insert(ctx, img, rot)
+    torch.cuda.synchronize()
+    if L.fr_tuning_report(ctx)["tuned"]:
+        break
+first = {c: t for c, t, _ in L.fr_tuning_measurements(ctx)}
+print(json.dumps([[L.fr_describe_config(c), t, time_config(ctx, c, img, rot, 2.0)] for c, t in first.items()]))
+"""
+
+
+def test_tuning_times_no_kernel_loads():
+    """In a fresh process every kernel's first launch is a tuning step.  Its time is a
+    launch's, not a launch's and the loading of its code (0.9 ms against 0.05 to 0.3):
+    within a factor of three of the same configuration's later launches."""
+    import json
+    import os
+    import subprocess
+    import sys
+    root = os.path.dirname(os.path.dirname(os.path.abspath(__file__)))
+    r = subprocess.run([sys.executable, "-c", _FIRST_STEPS_CHILD], cwd=root, capture_output=True, text=True,
+                       timeout=300, env=dict(os.environ, PYTHONPATH=root, CUDA_MODULE_LOADING="LAZY"))
+    assert r.returncode == 0, r.stderr[-2000:]
+    times = json.loads(r.stdout)
+    assert len(times) >= 40
+    slow = [t for t in times if t[1] > 3 * t[2]]
+    assert not slow, slow
