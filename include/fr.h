@@ -121,7 +121,8 @@ typedef struct fr_options {
 typedef struct fr_report {
     int S;                  /* image size of the current key */
     int n_bucket;           /* batch-size bucket of the current key (log2 of n, rounded down) */
-    int space_size;         /* valid configurations for this key */
+    int space_size;         /* configurations the tuner tries for this key: valid ones,
+                               each launch once */
     int evaluated;          /* configurations measured so far */
     int tuned;              /* 1 once the search has finished */
     int best_config;        /* best configuration id so far (-1 if none) */

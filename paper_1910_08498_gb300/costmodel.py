@@ -8,8 +8,8 @@ trained with fr_mlp_train on the 16 configuration/workload features of
 fr_config_features against the log time relative to the workload's mean
 log time (ranking within a workload is all the tuner needs).
 
-Evaluation on a workload with N valid configurations and a budget of
-k = max(1, floor(N / 10)) evaluations (the tuner's default learned budget):
+Evaluation on a workload with N distinct configurations (each launch once, as
+the tuner tries them) and a budget of k = max(1, floor(N / 10)) evaluations (the tuner's default learned budget):
   learned   measure the k configurations the model ranks fastest, keep the
             fastest measured;
   random    k configurations drawn uniformly without replacement (the
@@ -65,10 +65,23 @@ def features(S, a, n, cfgs):
     return np.array([L.fr_config_features(c, S, n, a) for c in cfgs], dtype=np.float32)
 
 
+def distinct(S, a, n, t):
+    """The configurations of a workload's times t, each launch once (the first
+    id).  Launches differ in their features, but for the direct-drain gather's
+    warps per SM (feature 8), which all run the same kernel."""
+    first = {}
+    for c in sorted(t):
+        f = list(L.fr_config_features(c, S, n, a))
+        if f[0] == 0.5:
+            f[8] = 0.0
+        first.setdefault(tuple(f), c)
+    return sorted(first.values())
+
+
 def training_set(wl):
     X, y = [], []
     for (S, a, n), t in wl.items():
-        cfgs = sorted(t)
+        cfgs = distinct(S, a, n, t)
         lt = np.log(np.array([t[c] for c in cfgs]))
         X.append(features(S, a, n, cfgs))
         y.append(lt - lt.mean())
@@ -101,7 +114,8 @@ def random_expected_regret(times, k):
 def evaluate(ctx, wl, frac=0.10):
     out = []
     for (S, a, n), t in sorted(wl.items()):
-        cfgs = sorted(t)
+        cfgs = distinct(S, a, n, t)
+        t = {c: t[c] for c in cfgs}
         k = max(1, int(frac * len(cfgs) + 1e-9))
         pred = predict(ctx, S, a, n, cfgs)
         top = [cfgs[i] for i in np.argsort(pred, kind="stable")[:k]]
@@ -115,14 +129,14 @@ def evaluate(ctx, wl, frac=0.10):
     return out
 
 
-DEFAULT_CONFIGS = ("gather2 bx=16 by=8 zc=8 chunk=64 warps=24 w=poly",
+DEFAULT_CONFIGS = ("gather2 bx=16 by=8 zc=8 chunk=64 warps=16 w=poly",
                    "gather bx=16 by=16 zc=8 chunk=64 w=poly")
 
 
 def default_start(t):
     """The library's default configuration among the measured ones of a
-    workload: the direct-drain gather 16 x 8 x 8 where it runs (a < 2), else
-    the per-voxel gather 16 x 16 x 8."""
+    workload: the direct-drain gather 16 x 8 x 8 for a < 2, else the
+    configuration 16 x 16 x 8 of the per-voxel family."""
     desc = {L.fr_describe_config(c): c for c in t}
     for d in DEFAULT_CONFIGS:
         if d in desc:
@@ -138,6 +152,7 @@ def compare_searchers(wl, frac=0.10, seeds=20, start=None, learned=None):
     ncfg = L.fr_num_configs()
     rows = []
     for key, t in sorted(wl.items()):
+        t = {c: t[c] for c in distinct(*key, t)}
         table = [t.get(c, 0.0) for c in range(ncfg)]
         st = default_start(t) if start is None else start
         k = max(1, int(frac * len(t) + 1e-9))

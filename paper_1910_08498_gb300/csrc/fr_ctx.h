@@ -67,7 +67,7 @@ int key_bucket(int n);
 InsertArgs base_args(const fr_ctx *c);
 // allocate the context's float4 scratch volume if it has none yet
 int ensure_scratch(fr_ctx *c);
-// configuration id as this context runs it (its kernel family)
+// configuration id as this context runs it (see the other form)
 Config effective_config(const fr_ctx *c, int id);
 // gather work unit with its expected load (images it scans)
 struct UnitLoad {

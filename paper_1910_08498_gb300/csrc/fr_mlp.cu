@@ -360,7 +360,7 @@ std::vector<int> learned_order(fr_ctx *c, const TuneKey &k, const std::vector<in
   std::vector<float> feat((size_t)m * MLP_IN), pred(m);
   const int n_repr = (int)std::min<long long>(1LL << 24, (3LL << k.nb) / 2);  // bucket middle
   for (int i = 0; i < m; ++i)
-    config_features(config_space()[valid[i]], k.S, n_repr, k.a, &feat[(size_t)i * MLP_IN]);
+    config_features(effective_config(valid[i], k.S, k.a), k.S, n_repr, k.a, &feat[(size_t)i * MLP_IN]);
   float *dx = nullptr, *dy = nullptr;
   if (cudaMalloc(&dx, feat.size() * sizeof(float)) != cudaSuccess) return order;
   if (cudaMalloc(&dy, m * sizeof(float)) != cudaSuccess) { cudaFree(dx); return order; }

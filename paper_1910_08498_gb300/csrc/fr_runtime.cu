@@ -14,6 +14,7 @@
 #include <mutex>
 #include <random>
 #include <string>
+#include <tuple>
 #include <vector>
 
 #include "../../include/fr.h"
@@ -248,11 +249,24 @@ double gather_unit_loads(const fr_ctx *c, int shape, int n, double target,
 // too small for a 6 x 6 box in the half plane (S < 10) stay with the per-voxel
 // gather; so does a < 2, where the direct-drain gather has its own
 // configurations.
-Config effective_config(const fr_ctx *c, int id) {
+Config effective_config(int id, int S, float a) {
   Config cfg = config_space()[id];
-  if (cfg.algo == ALGO_GATHER && cfg.wmode == W_POLY && c->g.KB == 6 && cfg.shape <= 1 && c->g.H >= 5)
+  if (cfg.algo == ALGO_GATHER && cfg.wmode == W_POLY && a >= 2.0f && cfg.shape <= 1 && S >= 10)
     cfg.algo = ALGO_GATHER2;
   return cfg;
+}
+
+Config effective_config(const fr_ctx *c, int id) { return effective_config(id, c->S, c->g.a); }
+
+int config_tuned(const fr_ctx *c, int id) {
+  if (!config_valid(c, id)) return 0;
+  auto launch = [&](int k) {
+    const Config q = effective_config(c, k);
+    return std::make_tuple(q.algo, q.shape, q.wmode, q.chunk, q.threads, q.sub);
+  };
+  for (int k = 0; k < id; ++k)
+    if (launch(k) == launch(id)) return 0;
+  return 1;
 }
 
 // The slabs of a unit list into a, and the list of its merge.
@@ -776,7 +790,7 @@ int fr_config_valid(const fr_ctx *c, int id) { return config_valid(c, id); }
 
 int fr_config_features(int id, int S, int n, float a, float *out16) {
   if (id < 0 || id >= (int)config_space().size() || !out16) return FR_ERR_INVALID_ARG;
-  config_features(config_space()[id], S, n, a, out16);
+  config_features(effective_config(id, S, a), S, n, a, out16);
   return FR_OK;
 }
 

@@ -60,13 +60,20 @@ std::string describe(const Config &c) {
   return b;
 }
 
+// Generation of the kernels: counted up when they change so much that times measured
+// before say nothing about which configuration is the best.
+static const char kKernels[] = "kernels 2";
+
 unsigned long long space_hash() {
   unsigned long long h = 1469598103934665603ULL;  // FNV-1a
-  for (const Config &c : config_space())
-    for (char ch : describe(c)) {
+  auto add = [&](const std::string &s) {
+    for (char ch : s) {
       h ^= (unsigned char)ch;
       h *= 1099511628211ULL;
     }
+  };
+  for (const Config &c : config_space()) add(describe(c));
+  add(kKernels);
   return h;
 }
 
@@ -105,10 +112,9 @@ int default_gather_config(const fr_ctx *c) {
 }
 
 int default_config(const fr_ctx *c) {
-  // the direct-drain gather, 16 x 8 x 8 bricks, registers for 16 warps per SM
-  // (what shared memory holds; the budgets for 20 and 24 measured 0 to 1 and 1 to
-  // 4 % slower at S = 128 .. 256, FP32 and FP16); where it cannot run (a >= 2),
-  // the per-voxel gather default
+  // the direct-drain gather, 16 x 8 x 8 bricks; for a >= 2, where its own
+  // configurations are not offered, the per-voxel family's 16 x 16 x 8 with polynomial
+  // weights, which runs the direct-drain gather there (effective_config)
   const auto &sp = config_space();
   for (int i = 0; i < (int)sp.size(); ++i)
     if (sp[i].algo == ALGO_GATHER2 && sp[i].shape == 1 && sp[i].minw == 16 && sp[i].chunk == 64 &&
@@ -166,7 +172,7 @@ std::vector<int> learned_order(fr_ctx *c, const TuneKey &k, const std::vector<in
 std::vector<int> Tuner::search_order(const TuneKey &k, fr_ctx *c) {
   std::vector<int> valid;
   for (int i = 0; i < (int)config_space().size(); ++i)
-    if (config_valid(c, i)) valid.push_back(i);
+    if (config_tuned(c, i)) valid.push_back(i);
   const fr_options &o = c->opt;
   std::mt19937_64 rng(o.seed ^ ((unsigned long long)k.S << 20) ^ ((unsigned long long)k.nb << 8) ^
                       (unsigned long long)k.dtype);
@@ -201,7 +207,7 @@ KeyState &Tuner::state(const TuneKey &k, fr_ctx *c) {
     ks.key = k;
     ks.order = search_order(k, c);
     ks.space_size = 0;
-    for (int i = 0; i < (int)config_space().size(); ++i) ks.space_size += config_valid(c, i);
+    for (int i = 0; i < (int)config_space().size(); ++i) ks.space_size += config_tuned(c, i);
     if (current_ != nullptr) ++retunes_;
     current_ = &ks;
     return ks;
@@ -551,7 +557,7 @@ int Tuner::load(const char *path) {
     ks = KeyState();
     ks.key = k;
     ks.space_size = 0;
-    for (int i = 0; i < (int)config_space().size(); ++i) ks.space_size += config_valid(ctx_, i);
+    for (int i = 0; i < (int)config_space().size(); ++i) ks.space_size += config_tuned(ctx_, i);
     size_t m = s.find("\"meas\": [", b);
     size_t p = m + 9;
     while (p < e) {
@@ -573,7 +579,7 @@ int Tuner::load(const char *path) {
     // unmeasured configurations are searched next
     std::vector<int> order;
     for (int i = 0; i < (int)config_space().size(); ++i)
-      if (config_valid(ctx_, i) && !ks.meas.count(i)) order.push_back(i);
+      if (config_tuned(ctx_, i) && !ks.meas.count(i)) order.push_back(i);
     ks.order = tuned > 0 ? std::vector<int>() : order;
     ks.next = 0;
     update_best(ks);

@@ -47,14 +47,21 @@ struct Config {
   int threads;  // scatter: block size
   int sub;      // scatter: images per atomic sub-batch (merged after each)
   // direct-drain gather: 16, 20 or 24.  Resident warps per SM whose registers were
-  // to fit; all run the same kernel, of which shared memory holds 16
+  // to fit; all run the same kernel, of which shared memory holds 16.  The ids stay (a
+  // caller may force one), the tuner takes the first of each three
   int minw = 0;
 };
 
 const std::vector<Config> &config_space();
 std::string describe(const Config &c);
 unsigned long long space_hash();
-// 16 normalised features of (configuration, S, n, a) for the cost model
+// configuration id as contexts of image size S and blob radius a run it: for 2 <= a the
+// per-voxel gather's polynomial configurations of 8-deep bricks are the direct-drain
+// gather's
+Config effective_config(int id, int S, float a);
+// whether the tuner tries configuration id: valid, and no earlier id is the same launch
+int config_tuned(const fr_ctx *c, int id);
+// 16 normalised features of (configuration as it is run, S, n, a) for the cost model
 void config_features(const Config &c, int S, int n, float a, float *out16);
 int default_config(const fr_ctx *c);
 // the per-voxel gather's default (the persistent batched launches run that family)

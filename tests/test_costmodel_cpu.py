@@ -101,3 +101,36 @@ def test_walks_beat_random_on_a_smooth_landscape():
     rows = cm.compare_searchers(wl, frac=0.45, seeds=50, start=4)
     assert rows[0]["annealing"] < 0.2 and rows[0]["mcmc"] < 0.2
     assert rows[0]["random"] > 0.5
+
+
+def test_each_launch_is_tried_once():
+    """The three warp counts of a direct-drain brick and list are one launch; for
+    2 <= a six configurations of the per-voxel family run the direct-drain gather and
+    have its features."""
+    desc = [L.fr_describe_config(i) for i in range(L.fr_num_configs())]
+    for a in (1.5, 1.9):
+        left = cm.distinct(128, a, 1000, dict.fromkeys(range(len(desc)), 1.0))
+        assert len(left) == 48 and sum(desc[c].startswith("gather2") for c in left) == 4
+    wide = [i for i, s in enumerate(desc) if not s.startswith("gather2")]
+    assert cm.distinct(96, 2.5, 1000, dict.fromkeys(wide, 1.0)) == wide
+    direct = [desc[c] for c in wide if L.fr_config_features(c, 96, 1000, 2.5)[0] == 0.5]
+    assert len(direct) == 6 and all(" zc=8 " in s and s.endswith("w=poly") for s in direct)
+    assert all(L.fr_config_features(c, 96, 1000, 1.9)[0] != 0.5 for c in wide)
+    assert all(L.fr_config_features(c, 8, 1000, 2.5)[0] != 0.5 for c in wide)
+
+
+def test_shipped_model_measures_the_direct_drain_gather():
+    """The fastest family at every measured size and radius, also where the per-voxel
+    family's ids run it: it has to be within the model's default budget."""
+    from oracle import mlp
+    p = np.array(json.load(open(cm.PRETRAINED)), dtype=np.float64)
+    n_cfg = L.fr_num_configs()
+    desc = [L.fr_describe_config(i) for i in range(n_cfg)]
+    for S in (64, 96, 128, 160, 192, 256, 320):
+        for a in (1.5, 1.9, 2.5, 2.9):
+            ids = [i for i in range(n_cfg) if a < 2 or not desc[i].startswith("gather2")]
+            cfgs = cm.distinct(S, a, 1500, dict.fromkeys(ids, 1.0))
+            X = cm.features(S, a, 1500, cfgs)
+            y, _ = mlp.forward(p, X.astype(np.float64))
+            top = np.argsort(y, kind="stable")[:max(1, len(cfgs) // 10)]
+            assert any(X[i][0] == 0.5 for i in top), (S, a, [desc[cfgs[i]] for i in top])

@@ -8,8 +8,9 @@ import pytest
 import torch
 
 from paper_1910_08498_gb300 import _lib as L
+from paper_1910_08498_gb300 import costmodel as cm
 from paper_1910_08498_gb300 import inputs
-from tests.helpers import TOL_F32, oracle_insert, rel_err
+from tests.helpers import A32, TOL_F32, oracle_insert, rel_err
 
 pytestmark = pytest.mark.gpu
 
@@ -241,3 +242,34 @@ def test_tuning_times_no_kernel_loads():
     assert len(times) >= 40
     slow = [t for t in times if t[1] > 3 * t[2]]
     assert not slow, slow
+
+
+@pytest.mark.parametrize("a", [A32, 2.5])
+def test_search_tries_each_launch_once(a, tmp_path):
+    """An exhaustive search measures no two configurations that are the same launch, a
+    cache from before the present kernels (another space hash) is not taken over."""
+    S, n = 40, 64
+    img, rot = [t.cuda() for t in inputs.make_batch(S, n, 160)]
+    ctx = L.fr_create(S, a)
+    try:
+        L.fr_set_options(ctx, tuning=1, search=L.FR_SEARCH_EXHAUSTIVE, steps_per_insert=8)
+        _tune_until_done(ctx, img, rot)
+        rep = L.fr_tuning_report(ctx)
+        meas = L.fr_tuning_measurements(ctx)
+        times = {c: t for c, t, _ in meas}
+        assert sorted(times) == cm.distinct(S, a, n, times) and rep["space_size"] == len(times)
+        path = str(tmp_path / "cache.json")
+        L.fr_tuning_save(ctx, path)
+    finally:
+        L.fr_destroy(ctx)
+    saved = open(path).read()
+    for text, tuned in ((saved, 1), (saved.replace('"space_hash": "', '"space_hash": "0'), 0)):
+        open(path, "w").write(text)
+        ctx = L.fr_create(S, a)
+        try:
+            L.fr_set_options(ctx, tuning=1, search=L.FR_SEARCH_EXHAUSTIVE, steps_per_insert=8)
+            L.fr_tuning_load(ctx, path)
+            L.fr_insert(ctx, img, rot)
+            assert L.fr_tuning_report(ctx)["tuned"] == tuned
+        finally:
+            L.fr_destroy(ctx)
