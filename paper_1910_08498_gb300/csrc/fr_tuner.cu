@@ -224,14 +224,38 @@ KeyState &Tuner::state(const TuneKey &k, fr_ctx *c) {
 // Smaller steps put fewer images through slow configurations: over a stream of
 // 20 batches of 5000 images at S = 256, 32 steps per insert cost 20 % over the
 // oraculum where 4 steps cost 92 %, with the same configuration chosen.
-static int steps_for(const fr_ctx *c, int n, const fr_options &opt) {
-  if (opt.steps_per_insert > 0) return opt.steps_per_insert;
+static double auto_steps(const fr_ctx *c, int n) {
   constexpr double AUTO_STEP_UPDATES = 2e7;
-  constexpr int AUTO_STEPS_MAX = 32;
   const double per_image = (double)c->S * (c->S / 2 + 1) * (4.0 / 3.0) * 3.14159265358979 *
                            (double)c->g.a * c->g.a * c->g.a;
-  const double k = std::floor((double)n * per_image / AUTO_STEP_UPDATES);
-  return (int)std::max(1.0, std::min((double)AUTO_STEPS_MAX, k));
+  return std::floor((double)n * per_image / AUTO_STEP_UPDATES);
+}
+
+static int steps_for(const fr_ctx *c, int n, const fr_options &opt) {
+  if (opt.steps_per_insert > 0) return opt.steps_per_insert;
+  constexpr int AUTO_STEPS_MAX = 32;
+  return (int)std::max(1.0, std::min((double)AUTO_STEPS_MAX, auto_steps(c, n)));
+}
+
+// The direct-drain launches that screened within CLOSE of the fastest one (and it), beyond
+// the finalists, where an insert is several steps long: they differ in what a unit and a
+// list cost at a step's few images (S = 256: at 156 images 32-image lists are 1.16 times
+// faster than the default, at 5000 1.11 times slower).  At most three.
+static std::vector<int> close_launches(const fr_ctx *c, const KeyState &ks) {
+  constexpr double CLOSE = 1.3;
+  std::vector<std::pair<double, int>> v;
+  if (auto_steps(c, ks.insert_images) < 2) return {};
+  for (const auto &m : ks.meas)
+    if (m.second.images > 0 && !ks.invalid.count(m.first) &&
+        effective_config(c, m.first).algo == ALGO_GATHER2)
+      v.push_back({m.second.per_image(), m.first});
+  std::sort(v.begin(), v.end());
+  std::vector<int> out;
+  for (const auto &x : v)
+    if (x.first <= CLOSE * v[0].first && out.size() < 3 &&
+        std::find(ks.finalists.begin(), ks.finalists.end(), x.second) == ks.finalists.end())
+      out.push_back(x.second);
+  return out;
 }
 
 std::vector<Step> Tuner::plan(KeyState &ks, int n, const fr_options &opt) {
@@ -273,6 +297,7 @@ std::vector<Step> Tuner::plan(KeyState &ks, int n, const fr_options &opt) {
     ks.proposed += (int)cfgs.size();
     const int m = (int)cfgs.size();
     if (m > 1) ks.sub_steps = true;
+    ks.insert_images = n;
     const int base = n / m, extra = n % m;
     for (int i = 0; i < m; ++i) steps.push_back(Step{cfgs[i], base + (i < extra ? 1 : 0), true});
     return steps;
@@ -286,6 +311,7 @@ std::vector<Step> Tuner::plan(KeyState &ks, int n, const fr_options &opt) {
   }
   int k = std::min(std::min(kmax, remaining), n);
   if (k > 1) ks.sub_steps = true;
+  ks.insert_images = n;
   int base = n / k, extra = n % k;
   for (int i = 0; i < k; ++i) {
     int cfg = ks.order[ks.next++];
@@ -353,6 +379,7 @@ void Tuner::finish_if_done(KeyState &ks) {
       }
       std::sort(fam.begin(), fam.end());
       for (auto &x : fam) ks.finalists.push_back(x.second);
+      for (int c : close_launches(ctx_, ks)) ks.finalists.push_back(c);
     }
     if (ks.finalists.size() > 1) {
       ks.confirming = true;

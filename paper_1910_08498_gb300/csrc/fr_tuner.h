@@ -15,9 +15,10 @@
 // ranking kernel families on sub-batches can pick a family that is slower at
 // the batch's own size.  When the screening ran in sub-batch steps, the
 // fastest configuration of each kernel family is therefore run once more on
-// a whole insert, and the key's best is the fastest of those whole-insert
-// timings (within a family the per-launch costs are alike, so the
-// sub-batch ranking stands).
+// a whole insert, and so, where an insert is several steps long, is each
+// direct-drain launch that screened close to that family's fastest; the key's
+// best is the fastest of those whole-insert timings (elsewhere in a family the
+// per-launch costs are alike, so the sub-batch ranking stands).
 //
 // A key is (S, batch-size bucket, blob radius, image dtype): a change of image
 // size or of batch shape starts a new search (or reuses a cached one), which
@@ -116,8 +117,9 @@ struct KeyState {
   Walker walker;
   // confirmation on whole inserts (see the file comment)
   bool sub_steps = false;       // some screening step took part of an insert
+  int insert_images = 0;        // of the last insert that was screened on
   bool confirming = false, confirmed = false;
-  std::vector<int> finalists;   // the fastest screened configuration of each family
+  std::vector<int> finalists;   // the fastest screened configuration of each family, close ones
   size_t fin_next = 0;
   int fin_pending = 0;
   std::map<int, Meas> full;     // whole-insert timings of the finalists

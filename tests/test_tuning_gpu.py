@@ -10,6 +10,7 @@ import torch
 from paper_1910_08498_gb300 import _lib as L
 from paper_1910_08498_gb300 import costmodel as cm
 from paper_1910_08498_gb300 import inputs
+from paper_1910_08498_gb300.sweep import time_config
 from tests.helpers import A32, TOL_F32, oracle_insert, rel_err
 
 pytestmark = pytest.mark.gpu
@@ -273,3 +274,35 @@ def test_search_tries_each_launch_once(a, tmp_path):
             assert L.fr_tuning_report(ctx)["tuned"] == tuned
         finally:
             L.fr_destroy(ctx)
+
+
+def test_close_direct_drain_launches_are_confirmed():
+    """Inserts of several automatic steps: every direct-drain launch that screened
+    within 1.3 of the fastest runs one whole insert, after the families' fastest, and
+    the best is no slower than the default configuration (5 % for noise)."""
+    S, n = 256, 2500
+    img, rot = inputs.make_batch(S, n, 180, device="cuda")
+    ctx = L.fr_create(S)
+    try:
+        L.fr_set_options(ctx, tuning=0)
+        L.fr_insert(ctx, img, rot)
+        default = L.fr_tuning_report(ctx)["last_config"]
+        L.fr_set_options(ctx, tuning=1, search=L.FR_SEARCH_EXHAUSTIVE, steps_per_insert=0)
+        lasts = []
+        for _ in range(40):
+            L.fr_insert(ctx, img, rot)
+            torch.cuda.synchronize()
+            rep = L.fr_tuning_report(ctx)
+            lasts.append(rep["last_config"])
+            if rep["tuned"]:
+                break
+        assert rep["tuned"] == 1
+        meas = {c: t for c, t, _ in L.fr_tuning_measurements(ctx)}
+        best = rep["best_config"]
+        t = {c: time_config(ctx, c, img, rot) for c in {best, default}}
+    finally:
+        L.fr_destroy(ctx)
+    direct = sorted((c for c in meas if _family(c) == "gather2"), key=meas.get)
+    close = [c for c in direct[1:] if meas[c] <= 1.3 * meas[direct[0]]]
+    assert lasts[len(lasts) - len(close):] == close
+    assert t[best] <= 1.05 * t[default], (L.fr_describe_config(best), t)
