@@ -9,7 +9,11 @@ library's CUDA kernels).  The metric is voxel-updates/s: one update is one
 (pixel, voxel) pair with |v - q| <= a inside the volume, counted exactly by
 fr_count_updates.
 
-Phases (one JSON line at the end):
+The last line of the standard output is one short JSON line: the headline, the
+end-to-end figure and what they were measured on.  The whole record, with every
+phase below, is a JSON line on the standard error stream, or a file (--detail).
+
+Phases:
   untuned  the library's default configuration, no tuning;
   tuning   cold-start non-blocking dynamic tuning (exhaustive search, four
            configurations per insert) until the space is exhausted; reports
@@ -70,6 +74,8 @@ def parse():
     p.add_argument("--n", type=int, default=5000)
     p.add_argument("--batches", type=int, default=4, help="distinct resident batches, cycled")
     p.add_argument("--cpu-seconds", type=float, default=15.0, help="target oracle work for cpu_baseline")
+    p.add_argument("--detail", default=None, metavar="FILE",
+                   help="write the whole record there (default: a JSON line on the standard error stream)")
     p.add_argument("--no-cpu-baseline", action="store_true")
     p.add_argument("--no-e2e", action="store_true")
     p.add_argument("--no-batched", action="store_true", help="skip the uneven-batch workload")
@@ -281,6 +287,26 @@ def sample_errors(g, Vo, Wo):
     import numpy as np
     return {"err_V": float(np.max(np.abs(g["V"] - Vo)) / g["scale_v"]),
             "err_W": float(np.max(np.abs(g["W"] - Wo)) / g["scale_w"]), "voxels": len(g["pts"])}
+
+
+# ------------------------------------------------------------------ the line printed
+
+HEADLINE = ("metric", "value", "unit", "n_gpus", "steps", "warmup", "ms_per_step", "higher_is_better", "scaling",
+            "vs_baseline", "dtype", "data", "config", "gpu_launches", "clocks", "wall_s_timed")
+
+
+def headline(line):
+    """The short line: the headline's own keys, and of the end-to-end figure, the
+    untuned rate, the roofline and the CPU baseline what is needed to read them (some
+    readers keep no more than the end of a long output)."""
+    def pick(d, *keys):
+        return {k: d[k] for k in keys if k in d} if d else None
+    out = {k: line[k] for k in HEADLINE}
+    out["e2e"] = pick(line["e2e"], "value", "unit", "h2d_bytes_per_step", "d2h_bytes_per_step")
+    out["untuned"] = line["untuned"]
+    out["roofline"] = pick(line["roofline"], "bound", "achieved", "peak", "unit", "frac")
+    out["cpu_baseline"] = pick(line["cpu_baseline"], "value", "unit", "cores", "kind")
+    return out
 
 
 # ------------------------------------------------------------------ reference arm
@@ -719,7 +745,12 @@ def run_ours(args):
     }
     L.fr_destroy(ctx)
     if rank == 0:
-        print(json.dumps(line), flush=True)
+        if args.detail:
+            with open(args.detail, "w") as f:
+                json.dump(line, f)
+        else:
+            print(json.dumps(line), file=sys.stderr, flush=True)
+        print(json.dumps(headline(line)), flush=True)
     if world > 1:
         import torch.distributed as dist
         dist.destroy_process_group()
