@@ -199,3 +199,36 @@ def test_batched_equals_per_batch_inserts_on_uneven_sizes():
     finally:
         for c in per + bat:
             L.fr_destroy(c)
+
+
+@pytest.mark.parametrize("f16", [False, True])
+@pytest.mark.parametrize("a", [A32, 2.0, 2.25, 2.999])
+def test_batched_groups_of_direct_drain_batches(a, f16):
+    """Each box width in groups of several batches: one context twice (all of its
+    units in slabs, merged batch by batch), split and unsplit batches; captured, then
+    replayed after a larger insert of a context has replaced its slabs."""
+    a = float(np.float32(a))
+    spec = [(48, 120, 81, 0), (48, 300, 82, 1), (48, 90, 83, 0), (32, 12, 84, 2), (32, 400, 85, 3)]
+    ctxs = {}
+    for S, _, _, slot in spec:
+        if slot not in ctxs:
+            ctxs[slot] = (L.fr_create(S, a, ALPHA, 0, 10000), S)
+            L.fr_set_options(ctxs[slot][0], tuning=0)
+    more = inputs.make_batch(48, 700, 86)
+    try:
+        host = [inputs.make_batch(S, n, seed) for S, n, seed, _ in spec]
+        imgs = [(inputs.to_half(i) if f16 else i).cuda() for i, _ in host]
+        rots = [r.cuda() for _, r in host]
+        order = [ctxs[slot][0] for *_, slot in spec]
+        L.fr_insert_batched(order, imgs, rots, capture=1)
+        L.fr_insert(ctxs[1][0], (inputs.to_half(more[0]) if f16 else more[0]).cuda(), more[1].cuda())
+        L.fr_insert_batched(order, imgs, rots, capture=1)  # graph replay
+        for slot, (c, S) in ctxs.items():
+            mine = [b for b, sp in zip(host, spec) if sp[-1] == slot]
+            Vr, Wr, _ = oracle_insert(S, mine + mine + ([more] if slot == 1 else []), a=a, f16=f16)
+            V, W = _finalize(c, S)
+            assert rel_err(V, Vr) <= TOL_F32, (slot, rel_err(V, Vr), worst(V, Vr, S))
+            assert rel_err(W, Wr) <= TOL_F32, (slot, rel_err(W, Wr), worst(W, Wr, S))
+    finally:
+        for c, _ in ctxs.values():
+            L.fr_destroy(c)
