@@ -497,18 +497,17 @@ __device__ __forceinline__ int cull_step(const InsertArgs &args, const unsigned 
 }
 
 // Fold a warp's shared partial sums (s_acc: [3][32 ZC], slot lane * ZC + t for
-// the voxel (fx0 + lane % FW, fy0 + lane / FW, z0 + t); FW = 8 for the 8 x 4
-// footprint, 4 for the 4 x 8 one) into HBM and clear them:
+// the voxel (fx0 + lane % 8, fy0 + lane / 8, z0 + t)) into HBM and clear them:
 // straight into the double-float accumulators (error-free TwoSum) when the
 // warp is the only writer of its voxels, else into the float4 scratch with
 // atomics (merged after the launch).
-template <int ZC, int FW = 8>
+template <int ZC>
 __device__ __forceinline__ void flush_partials(const InsertArgs &args, float *s_acc, int fx0,
                                                int fy0, int z0, bool to_scratch) {
   constexpr int WV = 32 * ZC;
   const Geom &g = args.g;
   const int lane = threadIdx.x & 31;
-  const int vx = fx0 + lane % FW, vy = fy0 + lane / FW;
+  const int vx = fx0 + lane % 8, vy = fy0 + lane / 8;
   __syncwarp();
   if (vx <= g.H && vy <= g.H) {
 #pragma unroll
@@ -958,30 +957,6 @@ gather_persistent_kernel(const InsertArgs *__restrict__ descs, const int4 *__res
                                             unit, warp);
     __syncthreads();  // s_item and s_args are rewritten next
   }
-}
-
-// Several batches in one launch, one CTA per work item: CTA b takes
-// p.items[b] (encoded as for the persistent gather) and copies its batch's
-// arguments p.descs[batch] to shared memory; geometry, weights and list
-// capacity, common to the launch's batches, are read from p.base (kernel
-// parameters).  Weights on the fly.
-template <int BX, int BY, int ZC, int WMODE, int KB, int F16>
-__global__ void __launch_bounds__(BX * BY, 512 / (BX * BY))
-gather_multi_kernel(const MultiLaunch p) {
-  static_assert(WMODE != W_LUT, "the multi-batch gather evaluates weights on the fly");
-  constexpr int NT = BX * BY;
-  const int tid = threadIdx.x, warp = tid >> 5;
-  extern __shared__ __align__(16) unsigned char smem[];
-  InsertArgs *s_args = reinterpret_cast<InsertArgs *>(smem);
-  const int4 it = p.items[blockIdx.x];
-  const int *src = reinterpret_cast<const int *>(p.descs + it.z);
-  int *dst = reinterpret_cast<int *>(s_args);
-  for (int i = tid; i < (int)(sizeof(InsertArgs) / 4); i += NT) dst[i] = src[i];
-  __syncthreads();
-  const int4 unit = make_int4(it.x & 1023, (it.x >> 10) & 1023, (it.x >> 20) & 1023, it.y);
-  gather_warp<BX, BY, ZC, WMODE, KB, F16>(
-      *s_args, p.base, p.images[it.w], nullptr,
-      smem + GATHER_ARGS_BYTES + (size_t)warp * gather_warp_smem(ZC, p.base.chunk), unit, warp);
 }
 
 }  // namespace fr

@@ -99,18 +99,6 @@ void config_features(const Config &c, int S, int n, float a, float *f) {
   f[11] = a / 2.5f;
 }
 
-int default_gather_config(const fr_ctx *c) {
-  // the per-voxel gather, 16 x 16 x 8 CTA, polynomial weights, 64-image warp lists
-  const auto &sp = config_space();
-  for (int i = 0; i < (int)sp.size(); ++i)
-    if (sp[i].algo == ALGO_GATHER && sp[i].shape == 0 && sp[i].wmode == W_POLY &&
-        sp[i].chunk == 64 && config_valid(c, i))
-      return i;
-  for (int i = 0; i < (int)sp.size(); ++i)
-    if (sp[i].algo == ALGO_GATHER && config_valid(c, i)) return i;
-  return 0;
-}
-
 int default_config(const fr_ctx *c) {
   // the direct-drain gather, 16 x 8 x 8 bricks; for a >= 2, where its own
   // configurations are not offered, the per-voxel family's 16 x 16 x 8 with polynomial

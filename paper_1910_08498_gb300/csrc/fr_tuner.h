@@ -65,8 +65,6 @@ int config_tuned(const fr_ctx *c, int id);
 // 16 normalised features of (configuration as it is run, S, n, a) for the cost model
 void config_features(const Config &c, int S, int n, float a, float *out16);
 int default_config(const fr_ctx *c);
-// the per-voxel gather's default (the persistent batched launches run that family)
-int default_gather_config(const fr_ctx *c);
 int config_valid(const fr_ctx *c, int id);
 int run_config(fr_ctx *c, int id, const void *images, int f16, const float *rot, int n,
                cudaStream_t st);
