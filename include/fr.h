@@ -104,14 +104,15 @@ typedef struct fr_options {
     int forced_config;   /* >= 0: always use this configuration id; -1 (default): tuner decides */
     uint64_t seed;       /* seed of the search order (default 1) */
     int debug;           /* bit 0: synchronise after every launch and check the device error
-                            word; bit 1: collect gather phase counters; bit 2: an NVTX range
+                            word; bit 1: collect gather phase counters (fr_insert; the
+                            multi-batch launches of fr_insert_batched have none); bit 2: an NVTX range
                             around every insertion step (named by configuration and images) */
     int fault_config;    /* test hook (host-side fault injection): > 0 makes every launch of
                             configuration fault_config - 1 report a launch failure without
                             enqueuing work, so the fallback path runs; 0 (default): none */
     int fault_alloc;     /* test hook (host-side fault injection): k > 0 makes the k-th device
                             allocation the insertion path attempts after this call (work-unit
-                            lists, scratch) fail as out of memory; the step then falls back as
+                            lists, scratch, slabs) fail as out of memory; the step then falls back as
                             for a failed launch.  One shot: reads back as 0 once it has fired.
                             0 (default): none */
     int reserved[6];
@@ -180,10 +181,10 @@ int fr_insert(fr_ctx *ctx, const void *images, fr_dtype dtype, const float *rota
  * heaviest units first, so uneven S and n share the GPU without a tail per
  * batch: the direct-drain gather as one CTA per warp footprint of a unit, the
  * per-voxel gather as a persistent kernel whose CTAs take units from a device
- * counter.  Batches
- * whose configuration has no multi-batch kernel (scatter, tabulated weights)
- * run their own launches after those.  A context that appears more than once
- * receives its sums through its scratch volume with atomics.  The first call
+ * counter.  Batches whose configuration has no multi-batch kernel (scatter,
+ * tabulated weights) run their own launches after those.  A context that
+ * appears more than once receives its sums through scratch memory, merged
+ * after the launches.  The first call
  * with a given (contexts, pointers, sizes, dtypes, configurations) builds a
  * plan and uploads it (synchronously); later calls reuse it.  With capture =
  * 1 the plan's launch sequence is captured, on a stream the library owns,

@@ -21,7 +21,7 @@ struct fr_ctx {
   float lut_scale = 0.f;
   float inv_i0a = 0.f, inv_pa = 0.f;
   float poly[fr::POLY_N] = {};
-  double poly_err = 1.0;  // max |poly - b| measured on the host (FP32 Horner)
+  double poly_err = 1.0;  // max |poly - b| measured on the host (FP32)
   float4 *scratch = nullptr;
   // slabs of the direct-drain gather's split units; replaced smaller buffers
   void *slabs = nullptr;

@@ -218,7 +218,8 @@ fft_cols_kernel(const float2 *spec, int center, void *out) {
 // ---- the volume's inverse transform, S = 64 and 128, in two kernels: weighting and
 // the z lines; then a plane a CTA, its y lines and its x lines (complex to real).
 //
-// The data fit in L2, so what counts is the number of passes and the latency of
+// A plane's CTA holds it in shared memory: 74 KB at S = 128, 4 times that at 256, which
+// does not fit.  The data fit in L2, so what counts is the number of passes and the latency of
 // each; the general path takes four (weighting, then cuFFT's three).  S = 128: 9.7 +
 // 20.6 us in four launches -> 12.8 + 7.5 us.  The z kernel waits for the six sums' 27
 // MB (4 us of HBM traffic); with 16 points a thread instead of 8, and half the warps,

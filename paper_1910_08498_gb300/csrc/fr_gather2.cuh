@@ -18,9 +18,9 @@
 //  * evaluation: 32 items a round, one per lane: u = R^T v from the footprint
 //    centre's compensated projection, the 4 x 4 candidate box at rint(u - 1.5)
 //    (it covers [u - a, u + a] for every a < 2; for 2 <= a <= 2.5 the 5 x 5 box
-//    at rint(u - 2), for a < 3 the 6 x 6 box at rint(u - 2.5)), clamped into the patch (rows and columns moved in by the
-//    clamp lie outside the blob and are masked), its pixels from the patch, the
-//    Chebyshev weight polynomial in
+//    at rint(u - 2), for a < 3 the 6 x 6 box at rint(u - 2.5)), clamped into the
+//    patch (rows and columns moved in by the clamp lie outside the blob and are
+//    masked), its pixels from the patch, the Chebyshev weight polynomial in
 //    x = 2 r^2 / a^2 - 1 for two candidates at a time with packed FP32x2 FMAs
 //    (masked to 0 outside r <= a), and the complex and weight sums added to the
 //    voxel's partial sums with plain loads and stores: the items of one entry
@@ -32,9 +32,10 @@
 // From the patches a round costs about 50, and one 512-voxel footprint a warp
 // (137 items an entry) halves the work per entry against 256 voxels; with an
 // entry's last half round on two lanes an item and 14 candidates a box: 8.4 ms; with
-// the phase counters in a kernel of their own: 8.2 ms.
-// Now the instructions bound it: 74 % issue, of which a quarter are packed FMAs
-// that hold the FMA pipe for two cycles (60 % busy); shared memory 63 %.  About a
+// the phase counters in a kernel of their own: 8.2 ms; with the split units' sums in
+// slabs (exact and repeatable; see g2_flush_slab) and 32 units an SM: 8.4 ms.
+// Now the instructions bound it: 71 % issue, of which a quarter are packed FMAs
+// that hold the FMA pipe for two cycles (58 % busy); shared memory 59 %.  About a
 // quarter of the time is per-entry work (copies 0.6 ms, tags 0.2, records 0.2).
 //
 // Half planes.  A stored pixel k sits at R k or, point-reflected and
@@ -48,10 +49,14 @@
 // exactly what the two entries read.  The main bricks tile x >= floor(a) + 1.
 // The fold columns |x| <= floor(a), where the fold predicate itself has to be
 // evaluated per pixel, have units of their own (FOLD), in footprints 4 (8) columns
-// wide so that three of four (five of eight) lanes hold fold columns: there a stored pixel k counts in
-// the entry as stored when it is not folded and in the reflected entry when it
-// is (exact sign of R00 k_x + R01 k_y, found once per pixel of the patch and
-// kept as one bit).  Polynomial weights only.
+// wide so that three of four (five of eight) lanes hold fold columns: there a stored
+// pixel k counts in the entry as stored when it is not folded and in the reflected
+// entry when it is (exact sign of R00 k_x + R01 k_y, found once per pixel of the patch
+// and kept as one bit).  Polynomial weights only.
+//
+// The blob's edge r <= a is decided in FP32, but for the fold columns of a >= 2
+// (g2_ties): a candidate within rounding of it may fall on the wrong side and costs
+// b(a) = 1 / I0(alpha), 2.9e-6 at alpha = 15.
 #pragma once
 
 #include "fr_gather.cuh"
@@ -278,7 +283,8 @@ __device__ __forceinline__ void g2_box14(const float2 *cp, const float2 *p, floa
 // candidates: of the corners only the two on the near side (see g2_box14: opposite
 // corners' squared distances add up to at least 16 > 2 a^2, a far corner is at least
 // 8 away).  Its origin rint(u - 2) leaves out at most a pixel at distance exactly
-// 2.5 along an axis.
+// 2.5 along an axis, for u = (k + 1/2, m) in the image's plane: no voxel is seen there,
+// as |u|^2 would be an integer and 1/4, and |u| = |v| for a rotation.
 template <int PITCH>
 __device__ __forceinline__ void g2_box23(const float2 *cp, const float2 *p, float dx, float dy,
                                          float uz2, float cs, float sq, float &ar, float &ai,
@@ -1004,8 +1010,9 @@ __device__ __forceinline__ int4 g2_unpack(int brick, int word) {
 // the resident warp slots stood idle.  Both kinds of unit in one launch: as a
 // second kernel on a side stream the fold columns cost a fork and a join.  Shared
 // memory holds 16 CTAs an SM, so the registers are bounded for 16 (a bound for 24, 80
-// registers, spills: 8.5 ms instead of 8.2 for 5000 images of 256^2).  KB: what the launch's geometry and shared memory are for (4, or 6 for a >= 2), KBM:
-// width of the boxes (5 for 2 <= a <= 2.5).
+// registers, spilled: 8.5 ms instead of 8.2 for 5000 images of 256^2).  KB: what the
+// launch's geometry and shared memory are for (4, or 6 for a >= 2), KBM: width of the
+// boxes (5 for 2 <= a <= 2.5).
 template <int BX, int BY, int BZ, int F16, int KB = 4, int KBM = KB, int PROF = 0>
 __global__ void __launch_bounds__(32, 16)
 gather2_kernel(const __grid_constant__ InsertArgs args) {

@@ -68,8 +68,10 @@ struct InsertArgs {
   int unit_most;
   // correct the projections for a rotation that FP32 rounding left short of
   // orthonormal.  fr_insert_noalloc does, whose scatter places every sample to
-  // FP32 accuracy; fr_insert keeps the plain R^T c, so that a volume resumed from a
-  // checkpoint goes on with the same positions
+  // FP32 accuracy.  fr_insert keeps the plain R^T c: the correction would cost 1 % and
+  // cut the error at S = 128 from 1.6e-6 to 3.8e-7, but it moves single voxels by up to
+  // 2.3e-4 of the RMS at S = 156, more at 256, and the performance cases (perf/cases.py)
+  // take results that differ by up to 3e-4 for the same
   int ortho;
   int any_split;        // 1 if some unit shares its brick with other units
   unsigned long long *phase;  // optional per-phase cycle and item counters (PH_*), or null

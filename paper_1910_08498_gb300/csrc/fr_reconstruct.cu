@@ -2,10 +2,10 @@
 // insertion, on the GPU: the forward transforms of the images (the step the
 // paper runs on the CPU before uploading), staged into the insertion's input
 // layout and dtype, and the last step, applying the weights W to G and
-// transforming back.  For the power-of-two sizes both go through this library's
-// transforms (fr_fft.cu); for the others the staging and weighting kernels are this
-// library's and the FFTs the vendor's plain R2C / C2R transforms (cuFFT), loaded
-// at run time so that libfr.so does not depend on them.
+// transforming back.  For S = 64, 128 and 256 (images) and 64 and 128 (last step) they
+// go through this library's transforms (fr_fft.cu); for the others the staging and
+// weighting kernels are this library's and the FFTs the vendor's plain R2C / C2R
+// transforms (cuFFT), loaded at run time so that libfr.so does not depend on them.
 //
 // Last step:
 //   Vs(v) = V(v) + conj(V(-v)),  Ws(v) = W(v) + W(-v)   (undo the half-space fold)

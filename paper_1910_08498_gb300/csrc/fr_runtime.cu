@@ -616,7 +616,9 @@ int fr_create(int S, const fr_blob *blob, fr_ctx **out) {
   // polynomial weights: b as a function of x = 2 r^2 / a^2 - 1 in [-1, 1]
   {
     weight_polynomial(alpha, c->poly);
-    // measured error of the FP32 even/odd evaluation the device performs
+    // measured error of the FP32 evaluation in even and odd halves, as the per-voxel
+    // gather and the scatter do it; the direct-drain gather's plain Horner form has the
+    // same error to 15 % for every alpha (1.1e-7 at 15, 1e-6 at 21)
     double worst = 0;
     for (int i = 0; i <= 20000; ++i) {
       const float x = -1.0f + 2.0f * (float)i / 20000.0f;
