@@ -973,6 +973,7 @@ def run_stream(L, inputs, costmodel, dev, stream, batches256, updates256, n, f16
         img, rot = (batches256 if S == 256 else b192)[0]
         for _ in range(100):
             L.fr_insert(c, img, rot)
+            torch.cuda.synchronize()  # timings are harvested when they have arrived
             if L.fr_tuning_report(c)["tuned"]:
                 break
         best[S] = L.fr_tuning_report(c)["best_config"]
